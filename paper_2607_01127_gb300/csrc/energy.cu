@@ -3,35 +3,35 @@
 //
 // w_min is an order statistic, so it is found by a radix selection over the
 // 31-bit pattern u = bits(|w|) (non-negative floats order like their bit
-// patterns), three streaming passes over W:
-//   level 1: bucket u >> 23 (the exponent), 256 buckets;
-//   level 2: within the level-1 exponent, (u >> 11) & 0xfff, 4096 buckets;
-//   level 3: within the level-2 prefix u >> 11, u & 0x7ff, one value each.
-// Every value of a bucket shares its exponent e, so w^2 = m^2 * 2^(2e - 46)
-// with m the 24-bit significand: a bucket's energy is kept exactly as two
-// 64-bit integer sums (the high and low 24 bits of m^2), accumulated with
-// integer atomics in shared memory and flushed with integer atomics to global
-// memory, so the per-bucket sums do not depend on the order of the additions.
-// At level 1, where every weight lands in one of a few hot buckets, each warp
-// keeps its own copy of the 256 buckets and takes the distinct exponents of
-// its 32 values one at a time: their lanes add their parts with a warp
-// reduction (exact: 32 parts of 24 bits fit in 32 bits) and one lane adds the
-// sums to the warp's copy, without atomics; the copies are summed in a fixed
-// order at the end of the pass.
-// When eps is not tiny (eps > n * 2^-59, always so for the paper's 4e-3 and
-// 1e-6) level 1 instead follows an absmax pass and counts only the 31
-// exponents at and below that of w_max: each lane adds its values' m^2 to its
-// own 64-bit cells in shared memory (no collectives, no atomics, no fp64) and
-// folds them into registers every 256 values, long before a cell or a fold can
-// overflow.  Values below the window go to bucket 0 in the unit of bucket 1
-// (m^2 shifted right by twice the exponent difference; the truncation is below
-// 2^-106 of the total energy per value).  Each of them holds less than 2^-60
-// of the total energy, so their share is below n * 2^-60 < eps and the
-// crossing lies inside the window.
-// After each pass one CTA converts the bucket sums to fp64 and scans them in
-// ascending order from the energy below the bucket's prefix (a fixed-order
-// parallel scan): the first bucket whose cumulative share cum / total reaches
-// eps is the next prefix.  Level 1 also takes w_max and the non-finite flag.
+// patterns), three streaming passes over W, one CTA scanning the sums after each:
+//   1: energy per exponent u >> 23; also w_max and the non-finite flag;
+//   2: within the selected exponent, how many weights share (u >> 11) & 0xfff;
+//      their energies lie between the counts times the buckets' ends squared,
+//      which leaves a window of a few buckets for the crossing;
+//   3: the exact energy of the selected exponent's weights below that window, and
+//      how many weights have each value inside it.
+// Every value of an exponent e has w^2 = m^2 * 2^(2e - 46) with m the 24-bit
+// significand, so energies are kept exactly as integer sums of m^2 (high and low
+// 24 bits apart) and counts; only the scans' accumulation across buckets rounds
+// (fp64, ascending order of |w|).
+//
+// The passes read 235 MB for a 14336 x 4096 matrix, 35 us at the measured HBM
+// rate; every other pass runs from the end to the start, so that what the pass
+// before it left in L2 is read from there.
+//   Pass 1: each lane adds its values' m^2 to its own 64-bit cells in shared
+//     memory, one per exponent of a 32-exponent window that the CTA places at its
+//     first values (no collectives, no atomics); the few values outside go to
+//     256 exponent sums with shared-memory atomics.  A cell is folded into
+//     registers before 2^16 values (each m^2 < 2^48) could overflow it.
+//   Pass 2: 4096 counts with native 32-bit shared-memory atomics, for the weights
+//     of one exponent.
+//   Pass 3: registers, and shared-memory atomics for the few weights inside the
+//     window.
+// When the window does not fit (kWinBuckets), which takes a distribution whose
+// crossing lies in a nearly empty stretch above most of its exponent's weights (or
+// for 2^32 weights and more), `failed` is set and the caller runs the exact form of levels 2 and 3
+// (energy_hist_kernel): per-bucket energies with 64-bit atomics, 4096
+// sub-buckets and then 2048 single values.
 #include <math.h>
 #include <stdint.h>
 
@@ -45,9 +45,9 @@ constexpr int kScanThreads = 256;
 constexpr int kUnroll = 4;                       // float4 loads in flight per thread
 
 template <int LEVEL> struct Level;
-template <> struct Level<1> { static constexpr int NB = 256, COPIES = kHistThreads / 32; };
-template <> struct Level<2> { static constexpr int NB = 4096, COPIES = 1; };
-template <> struct Level<3> { static constexpr int NB = 2048, COPIES = 1; };
+template <> struct Level<1> { static constexpr int NB = 256; };
+template <> struct Level<2> { static constexpr int NB = 4096; };
+template <> struct Level<3> { static constexpr int NB = 2048; };
 static_assert(sizeof(EnergyState::hi) / sizeof(EnergyState::hi[0]) >= 4096, "bucket arrays");
 
 __device__ __forceinline__ float4 ld_stream4(const float4* p)
@@ -73,70 +73,23 @@ template <int LEVEL>
 __device__ __forceinline__ void add_one(uint32_t u, uint32_t prefix, unsigned long long* hi,
                                         unsigned long long* lo)
 {
-    const bool finite = u < 0x7f800000u;
-    if constexpr (LEVEL == 1) {
-        // every lane of the warp takes part (the loop trip count is uniform)
-        uint32_t h = 0, l = 0;
-        if (finite) msq_parts(u, h, l);
-        const uint32_t b = u >> 23;
-        // one round per distinct exponent in the warp (a handful for weights):
-        // the lanes of that exponent add their parts, the first of them adds
-        // the sums to this warp's copy of the buckets
-        const uint32_t lane = threadIdx.x & 31;
-        uint32_t todo = 0xffffffffu;
-        while (todo) {
-            const int first = __ffs(todo) - 1;
-            const uint32_t bb = __shfl_sync(0xffffffffu, b, first);
-            const uint32_t peers = __ballot_sync(0xffffffffu, b == bb);
-            const uint32_t sh = __reduce_add_sync(0xffffffffu, b == bb ? h : 0u);
-            const uint32_t sl = __reduce_add_sync(0xffffffffu, b == bb ? l : 0u);
-            if (lane == (uint32_t)first && (sh | sl)) {
-                hi[bb] += sh;
-                lo[bb] += sl;
-            }
-            todo &= ~peers;
-        }
-        __syncwarp();
-    } else {
-        const bool in = finite && (LEVEL == 2 ? (u >> 23) == prefix : (u >> 11) == prefix);
-        if (!in) return;
-        const uint32_t b = LEVEL == 2 ? ((u >> 11) & 0xfffu) : (u & 0x7ffu);
-        uint32_t h, l;
-        msq_parts(u, h, l);
-        if (h | l) {
-            atomicAdd(&hi[b], (unsigned long long)h);
-            atomicAdd(&lo[b], (unsigned long long)l);
-        }
+    const bool in = u < 0x7f800000u && (LEVEL == 2 ? (u >> 23) == prefix : (u >> 11) == prefix);
+    if (!in) return;
+    const uint32_t b = LEVEL == 2 ? ((u >> 11) & 0xfffu) : (u & 0x7ffu);
+    uint32_t h, l;
+    msq_parts(u, h, l);
+    if (h | l) {
+        atomicAdd(&hi[b], (unsigned long long)h);
+        atomicAdd(&lo[b], (unsigned long long)l);
     }
 }
 
-template <int LEVEL>
-__global__ void __launch_bounds__(kHistThreads) energy_hist_kernel(const float4* __restrict__ W, int64_t n4,
-                                                                   EnergyState* st, Workspace* ws)
+// Streams W in the grid's strides: kUnroll loads in flight per thread in whole
+// rounds (their number goes to take with each vector; whole warps take part),
+// then the rest (-1); from the end to the start when BACK.
+template <bool BACK, typename Take>
+__device__ __forceinline__ void stream(const float4* __restrict__ W, int64_t n4, Take&& take)
 {
-    constexpr int NB = Level<LEVEL>::NB, COPIES = Level<LEVEL>::COPIES;
-    extern __shared__ unsigned long long hist[];              // [COPIES][2][NB]
-    for (int i = threadIdx.x; i < 2 * NB * COPIES; i += kHistThreads) hist[i] = 0;
-    __syncthreads();
-    unsigned long long* hi = hist + (COPIES > 1 ? (threadIdx.x >> 5) * 2 * NB : 0);
-    unsigned long long* lo = hi + NB;
-    const uint32_t prefix = LEVEL == 1 ? 0u : st->prefix;
-    uint32_t umax = 0, bad = 0;
-    auto take = [&](const float4& v) {
-        const uint32_t u[4] = {__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu,
-                               __float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (LEVEL == 1) {
-                const bool nf = u[e] >= 0x7f800000u;
-                bad |= nf ? 1u : 0u;
-                umax = max(umax, nf ? 0u : u[e]);
-            }
-            add_one<LEVEL>(u[e], prefix, hi, lo);
-        }
-    };
-    // Whole rounds of kUnroll loads are taken by every thread of the grid
-    // (uniform trip count, so whole warps stay converged); the rest follows.
     const int64_t nthreads = (int64_t)gridDim.x * kHistThreads;
     const int64_t gtid = (int64_t)blockIdx.x * kHistThreads + threadIdx.x;
     const int64_t rounds = n4 / (nthreads * kUnroll);
@@ -144,154 +97,366 @@ __global__ void __launch_bounds__(kHistThreads) energy_hist_kernel(const float4*
         const int64_t base = r * nthreads * kUnroll + gtid;
         float4 v[kUnroll];
 #pragma unroll
-        for (int j = 0; j < kUnroll; ++j) v[j] = ld_stream4(W + base + j * nthreads);
-#pragma unroll
-        for (int j = 0; j < kUnroll; ++j) take(v[j]);
-    }
-    for (int64_t i0 = rounds * nthreads * kUnroll; i0 < n4; i0 += nthreads) {
-        // tail: whole warps iterate while any of their lanes has an element
-        const int64_t i = i0 + gtid;
-        const float4 v = i < n4 ? ld_stream4(W + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-        take(v);
-    }
-    if (LEVEL == 1) {
-        bad = __reduce_or_sync(0xffffffffu, bad);
-        umax = __reduce_max_sync(0xffffffffu, umax);
-        if ((threadIdx.x & 31) == 0) {
-            if (bad) atomicOr(&ws->nonfinite, 1u);
-            atomicMax(&ws->absmax_bits, umax);
+        for (int j = 0; j < kUnroll; ++j) {
+            const int64_t i = base + j * nthreads;
+            v[j] = ld_stream4(W + (BACK ? n4 - 1 - i : i));
         }
+#pragma unroll
+        for (int j = 0; j < kUnroll; ++j) take(v[j], r);
     }
+    for (int64_t i = rounds * nthreads * kUnroll + gtid; i < n4; i += nthreads)
+        take(ld_stream4(W + (BACK ? n4 - 1 - i : i)), (int64_t)-1);
+}
+
+// Exact levels 2 and 3 (see the top of the file).
+template <int LEVEL>
+__global__ void __launch_bounds__(kHistThreads) energy_hist_kernel(const float4* __restrict__ W, int64_t n4,
+                                                                   EnergyState* st)
+{
+    constexpr int NB = Level<LEVEL>::NB;
+    extern __shared__ unsigned long long hist[];              // [2][NB]
+    for (int i = threadIdx.x; i < 2 * NB; i += kHistThreads) hist[i] = 0;
+    __syncthreads();
+    unsigned long long *hi = hist, *lo = hist + NB;
+    const uint32_t prefix = st->prefix;
+    stream<LEVEL == 3>(W, n4, [&](const float4& v, int64_t) {
+        add_one<LEVEL>(__float_as_uint(v.x) & 0x7fffffffu, prefix, hi, lo);
+        add_one<LEVEL>(__float_as_uint(v.y) & 0x7fffffffu, prefix, hi, lo);
+        add_one<LEVEL>(__float_as_uint(v.z) & 0x7fffffffu, prefix, hi, lo);
+        add_one<LEVEL>(__float_as_uint(v.w) & 0x7fffffffu, prefix, hi, lo);
+    });
     __syncthreads();
     for (int i = threadIdx.x; i < NB; i += kHistThreads) {
-        unsigned long long sh = 0, sl = 0;
-#pragma unroll
-        for (int c = 0; c < COPIES; ++c) {
-            sh += hist[c * 2 * NB + i];
-            sl += hist[c * 2 * NB + NB + i];
-        }
-        if (sh) atomicAdd(&st->hi[i], sh);
-        if (sl) atomicAdd(&st->lo[i], sl);
+        if (hi[i]) atomicAdd(&st->hi[i], hi[i]);
+        if (lo[i]) atomicAdd(&st->lo[i], lo[i]);
     }
 }
 
 // 2^k as a double (normal range: k in [-1022, 1023]).
 __device__ __forceinline__ double pow2(int k) { return __longlong_as_double((long long)(1023 + k) << 52); }
 
-constexpr int kWin = 32;            // bucket 0: below the window; 1..31: exponent fields e_hi-30 .. e_hi
-constexpr int kFlushRounds = 16;    // 16 rounds x 16 values = 256 values per lane between folds
+constexpr int kWin = 32;                      // pass 1: exponents of a CTA's window
+constexpr int64_t kFoldRounds = 2048;         // rounds between folds: 2048 x 16 values per lane < 2^16
+constexpr int kWinBuckets = 7;                // pass 3: buckets of the window
+constexpr int kWinValues = kWinBuckets * 2048;
+static_assert(kWinValues % (4 * kScanThreads) == 0, "whole vectors per scanning thread");
+constexpr int kBelowHi = 4094, kBelowLo = 4095;   // lo[] slots of pass 3's energy below the window
+static_assert(kWinValues * 4 <= 8 * (4096 + 4094), "window counts share the bucket arrays");
 
-// Level 1 after an absmax pass: exponent window of w_max, lane-private cells.
-__global__ void __launch_bounds__(kHistThreads) energy_window_kernel(const float4* __restrict__ W, int64_t n4,
-                                                                     EnergyState* st, const Workspace* ws)
+// Pass 1 (see the top of the file).
+__global__ void __launch_bounds__(kHistThreads) energy_exponents_kernel(const float4* __restrict__ W, int64_t n4,
+                                                                        EnergyState* st, Workspace* ws)
 {
     extern __shared__ unsigned long long cells[];     // [warp][kWin][32 lanes]: sums of m^2
-    __shared__ unsigned long long wsum[kHistThreads / 32][2][kWin];
+    __shared__ unsigned long long shi[256], slo[256];
+    __shared__ uint32_t smax;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    unsigned long long* ce = cells + warp * kWin * 32;
-    for (int b = 0; b < kWin; ++b) ce[b * 32 + lane] = 0;
-    const int e_lo = (int)(ws->absmax_bits >> 23) - (kWin - 2);     // exponent field of bucket 1
-    unsigned long long acc_hi = 0, acc_lo = 0;        // bucket `lane` of this warp, folded so far
+    unsigned long long* ce = cells + warp * kWin * 32 + lane;
+    for (int b = 0; b < kWin; ++b) ce[b * 32] = 0;
+    for (int i = threadIdx.x; i < 256; i += kHistThreads) shi[i] = slo[i] = 0;
+    if (threadIdx.x == 0) smax = 0;
+    __syncthreads();
+    // window: up to one exponent above the largest of the CTA's first values
+    {
+        const int64_t i = (int64_t)blockIdx.x * kHistThreads + threadIdx.x;
+        uint32_t m = 0;
+        if (i < n4) {
+            const float4 v = ld_stream4(W + i);
+            const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const uint32_t u = __float_as_uint(w[e]) & 0x7fffffffu;
+                if (u < 0x7f800000u) m = max(m, u);
+            }
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) atomicMax(&smax, m);
+    }
+    __syncthreads();
+    const int top = (int)(smax >> 23) + 1;
+    const uint32_t e_lo = top > kWin ? (uint32_t)(top - (kWin - 1)) : 1u;     // exponent field of cell 0 (a normal one)
+    unsigned long long acc_hi = 0, acc_lo = 0;        // cell `lane` of this warp, folded so far
     auto fold = [&]() {
         __syncwarp();
-        // lane l collects bucket l from every lane's cells (rotated start); a
-        // cell holds < 2^56 (256 values of m^2 < 2^48), the 32 of them < 2^61,
-        // which is split into its high and low 24-bit parts
-        unsigned long long sum = 0;
+        // lane l collects cell l from every lane (rotated start), split before the
+        // lanes are added up: a cell may hold nearly 2^64
+        unsigned long long* row = cells + warp * kWin * 32 + lane * 32;
 #pragma unroll 8
-        for (int j = 0; j < 32; ++j) sum += ce[lane * 32 + ((j + lane) & 31)];
-        acc_hi += sum >> 24;
-        acc_lo += sum & 0xffffffull;
+        for (int j = 0; j < 32; ++j) {
+            const unsigned long long x = row[(j + lane) & 31];
+            acc_hi += x >> 24;
+            acc_lo += x & 0xffffffull;
+        }
         __syncwarp();
-        for (int b = 0; b < kWin; ++b) ce[b * 32 + lane] = 0;
+        for (int b = 0; b < kWin; ++b) ce[b * 32] = 0;
         __syncwarp();
     };
-    auto take = [&](const float4& v) {
+    uint32_t umax = 0;
+    int64_t folded = 0;
+    stream<false>(W, n4, [&](const float4& v, int64_t r) {
         const uint32_t u[4] = {__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu,
                                __float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu};
+        const uint32_t d[4] = {(u[0] >> 23) - e_lo, (u[1] >> 23) - e_lo, (u[2] >> 23) - e_lo, (u[3] >> 23) - e_lo};
+        umax = max(max(umax, max(u[0], u[1])), max(u[2], u[3]));
+        if (max(max(d[0], d[1]), max(d[2], d[3])) < (uint32_t)kWin) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (u[e] >= 0x7f800000u) continue;           // reported by the absmax pass
-            const int field = (int)(u[e] >> 23);
-            const int d = field - e_lo + 1;
-            const uint32_t mant = u[e] & 0x7fffffu;
-            const uint32_t m = field ? (mant | 0x800000u) : mant;
-            const int sh = d >= 1 ? 0 : 2 * (e_lo - (field ? field : 1));   // below the window
-            const unsigned long long sq = (unsigned long long)m * m;
-            ce[(d >= 1 ? d : 0) * 32 + lane] += sh < 64 ? (sq >> sh) : 0ull;
+            for (int e = 0; e < 4; ++e) {
+                const uint32_t m = (u[e] & 0x7fffffu) | 0x800000u;
+                ce[d[e] * 32] += (unsigned long long)m * m;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (d[e] < (uint32_t)kWin) {
+                    const uint32_t m = (u[e] & 0x7fffffu) | 0x800000u;
+                    ce[d[e] * 32] += (unsigned long long)m * m;
+                } else if (u[e] != 0 && u[e] < 0x7f800000u) {
+                    uint32_t h, l;
+                    msq_parts(u[e], h, l);
+                    atomicAdd(&shi[u[e] >> 23], (unsigned long long)h);
+                    atomicAdd(&slo[u[e] >> 23], (unsigned long long)l);
+                }
+            }
         }
-    };
-    const int64_t nthreads = (int64_t)gridDim.x * kHistThreads;
-    const int64_t gtid = (int64_t)blockIdx.x * kHistThreads + threadIdx.x;
-    const int64_t rounds = n4 / (nthreads * kUnroll);
-    for (int64_t r = 0; r < rounds; ++r) {
-        const int64_t base = r * nthreads * kUnroll + gtid;
-        float4 v[kUnroll];
-#pragma unroll
-        for (int j = 0; j < kUnroll; ++j) v[j] = ld_stream4(W + base + j * nthreads);
-#pragma unroll
-        for (int j = 0; j < kUnroll; ++j) take(v[j]);
-        if ((r % kFlushRounds) == kFlushRounds - 1) fold();
-    }
-    for (int64_t i0 = rounds * nthreads * kUnroll; i0 < n4; i0 += nthreads) {
-        const int64_t i = i0 + gtid;
-        if (i < n4) take(ld_stream4(W + i));
-    }
+        if (r - folded >= kFoldRounds) {              // the same for every lane of the warp
+            fold();
+            folded = r;
+        }
+    });
+    __syncwarp();
     fold();
-    // per warp: lane l holds bucket l
-    wsum[warp][0][lane] = acc_hi;
-    wsum[warp][1][lane] = acc_lo;
+    if (acc_hi) atomicAdd(&shi[e_lo + lane], acc_hi);
+    if (acc_lo) atomicAdd(&slo[e_lo + lane], acc_lo);
+    // umax saw non-finite patterns too: they order above every finite one
+    umax = __reduce_max_sync(0xffffffffu, umax);
+    if (lane == 0) {
+        if (umax >= 0x7f800000u) atomicOr(&ws->nonfinite, 1u);
+        else atomicMax(&ws->absmax_bits, umax);
+    }
     __syncthreads();
-    if (threadIdx.x < kWin) {
-        unsigned long long sh = 0, sl = 0;
-        for (int w = 0; w < kHistThreads / 32; ++w) {
-            sh += wsum[w][0][threadIdx.x];
-            sl += wsum[w][1][threadIdx.x];
-        }
-        if (sh) atomicAdd(&st->hi[threadIdx.x], sh);
-        if (sl) atomicAdd(&st->lo[threadIdx.x], sl);
+    for (int i = threadIdx.x; i < 256; i += kHistThreads) {
+        if (shi[i]) atomicAdd(&st->hi[i], shi[i]);
+        if (slo[i]) atomicAdd(&st->lo[i], slo[i]);
     }
 }
 
-// Scan of the window pass: bucket 0 is the energy below the window (in bucket
-// 1's unit), buckets 1..31 the window's exponents.
-__global__ void __launch_bounds__(32) energy_scan_window_kernel(EnergyState* st, const Workspace* ws, double eps)
+// Pass 2: weights of the selected exponent per sub-bucket (counts in st->hi, as
+// 32-bit words).
+__global__ void __launch_bounds__(kHistThreads) energy_count_kernel(const float4* __restrict__ W, int64_t n4,
+                                                                    EnergyState* st)
 {
-    __shared__ double en[kWin];
+    __shared__ uint32_t cnt[4096];
+    for (int i = threadIdx.x; i < 4096; i += kHistThreads) cnt[i] = 0;
+    __syncthreads();
+    const uint32_t prefix = st->prefix;
+    stream<true>(W, n4, [&](const float4& v, int64_t) {
+        const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t u = __float_as_uint(w[e]) & 0x7fffffffu;
+            if ((u >> 23) == prefix && u) atomicAdd(&cnt[(u >> 11) & 0xfffu], 1u);
+        }
+    });
+    __syncthreads();
+    uint32_t* out = reinterpret_cast<uint32_t*>(st->hi);
+    for (int i = threadIdx.x; i < 4096; i += kHistThreads)
+        if (cnt[i]) atomicAdd(&out[i], cnt[i]);
+}
+
+// Window of pass 3 from pass 2's counts: bucket b's values lie in [lo_b, lo_(b+1)),
+// so the cumulative energies have a lower and an upper bound; the crossing
+// bucket is at or after the first whose upper bound reaches eps and at or before the
+// first whose lower bound does.  Leaves the window's first bucket in wmin_bits and
+// its length in _pad, and clears the bucket arrays.
+__global__ void __launch_bounds__(kScanThreads) energy_window_scan_kernel(EnergyState* st, double eps)
+{
+    constexpr int PER = 4096 / kScanThreads;
+    __shared__ double part[2][2][kScanThreads];
+    __shared__ int first, last;
     const int t = threadIdx.x;
-    const int e_lo = (int)(ws->absmax_bits >> 23) - (kWin - 2);
-    {
-        const int field = t == 0 ? e_lo : e_lo + t - 1;
-        double x = 0.0;
-        if (field >= 0) {
-            const int e = (field ? field : 1) - 127;
-            x = ((double)st->hi[t] * 16777216.0 + (double)st->lo[t]) * pow2(2 * e - 46);
+    const uint32_t* cnt = reinterpret_cast<const uint32_t*>(st->hi);
+    const uint32_t field = st->prefix;
+    const int e = (field ? (int)field : 1) - 127;
+    const double unit = pow2(2 * e - 46);
+    // (significand at the start of bucket b)^2, exact
+    auto end_sq = [&](int b) {
+        const unsigned long long m = (field ? 8388608ull : 0ull) + 2048ull * b;
+        return m * m;
+    };
+    // This thread's buckets as exact integers (high and low 24 bits of the squares
+    // apart), one conversion each: fp64 runs at a 64th of the fp32 rate.
+    uint32_t n[PER];
+    unsigned long long sum[2][2] = {{0, 0}, {0, 0}};
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        n[j] = cnt[t * PER + j];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const unsigned long long sq = end_sq(t * PER + j + k);
+            sum[k][0] += n[j] * (sq >> 24);
+            sum[k][1] += n[j] * (sq & 0xffffffull);
         }
-        en[t] = x;
     }
-    __syncwarp();
+    double own[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) part[0][k][t] = own[k] = ((double)sum[k][0] * 16777216.0 + (double)sum[k][1]) * unit;
+    int cur = 0;
+    if (t == 0) { first = 4096; last = 4096; }
+    __syncthreads();
+    for (int off = 1; off < kScanThreads; off <<= 1) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            part[cur ^ 1][k][t] = t >= off ? part[cur][k][t] + part[cur][k][t - off] : part[cur][k][t];
+        cur ^= 1;
+        __syncthreads();
+    }
+    // the bounds' own rounding stays far below these margins
+    const double target = eps * st->total, below = st->below;
+    const double near = target * (1.0 - 0x1p-36), sure = target * (1.0 + 0x1p-36);
+    const double base[2] = {below + (t ? part[cur][0][t - 1] : 0.0), below + (t ? part[cur][1][t - 1] : 0.0)};
+    // the first of this thread's buckets whose cumulative bound k reaches x
+    auto reach = [&](int k, double x) {
+        if (!(base[k] + own[k] * (1.0 + 0x1p-40) >= x)) return 4096;
+        double cum = base[k];
+        for (int j = 0; j < PER; ++j) {
+            const int b = t * PER + j;
+            cum += (double)cnt[b] * (double)end_sq(b + k) * unit;
+            if (cnt[b] && cum >= x) return b;
+        }
+        return 4096;
+    };
+    const int f = reach(1, near), l = reach(0, sure);
+    if (f < 4096) atomicMin(&first, f);
+    if (l < 4096) atomicMin(&last, l);
+    __syncthreads();
+    uint32_t* words = reinterpret_cast<uint32_t*>(st->hi);
     if (t == 0) {
-        double total = 0.0;
-        for (int b = 0; b < kWin; ++b) total += en[b];
-        st->total = total;
-        double cum = 0.0;
-        int found = -1;
-        double before = 0.0;
-        const double near = eps * total * (1.0 - 0x1p-40);   // below this the share is surely < eps
-        for (int b = 0; b < kWin && found < 0; ++b) {
-            const double prev = cum;
-            cum += en[b];
-            if (en[b] > 0.0 && cum >= near && cum / total >= eps) {
-                found = b;
-                before = prev;
-            }
+        // without a sure bucket the crossing may be any up to the last
+        const int f0 = first, l0 = last < 4096 ? last : 4095;
+        const int len = f0 < 4096 ? l0 - f0 + 1 : 0;
+        if (len < 1 || len > kWinBuckets) st->failed = 1;
+        st->wmin_bits = (uint32_t)f0;
+        st->_pad = (uint32_t)(len < 1 || len > kWinBuckets ? 0 : len);
+    }
+    __syncthreads();
+    for (int i = t; i < 4 * 4096; i += kScanThreads) words[i] = 0;     // hi and lo, for pass 3
+}
+
+// Pass 3 (see the top of the file).
+__global__ void __launch_bounds__(kHistThreads) energy_values_kernel(const float4* __restrict__ W, int64_t n4,
+                                                                     EnergyState* st)
+{
+    extern __shared__ uint32_t cnt[];                    // [kWinValues]
+    __shared__ unsigned long long shi, slo;
+    const uint32_t prefix = st->prefix, len = st->_pad * 2048u;
+    if (len == 0) return;                                // no window: the exact form follows
+    const uint32_t win0 = (prefix << 23) | (st->wmin_bits << 11);        // first pattern of the window
+    for (uint32_t i = threadIdx.x; i < len; i += kHistThreads) cnt[i] = 0;
+    if (threadIdx.x == 0) shi = slo = 0;
+    __syncthreads();
+    const uint32_t span = win0 - (prefix << 23);
+    // energy below the window: one 64-bit sum per lane, split into high and low 24
+    // bits before 2^16 values of 2^48 could overflow it
+    const uint32_t lead = prefix ? 0x800000u : 0u;
+    unsigned long long acc = 0, hi = 0, lo = 0;
+    int64_t split = 0;
+    stream<false>(W, n4, [&](const float4& v, int64_t r) {
+        const float w[4] = {v.x, v.y, v.z, v.w};
+        uint32_t in[4];
+        bool any = false;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            // offset inside the exponent (wraps for smaller values)
+            in[e] = (__float_as_uint(w[e]) & 0x7fffffffu) - (prefix << 23);
+            const uint32_t m = in[e] < span ? in[e] | lead : 0u;
+            acc += (unsigned long long)m * m;
+            any |= in[e] - span < len;
         }
-        if (found <= 0) {
-            st->failed = 1;          // not reachable when eps > n * 2^-59
-            found = kWin - 1;
+        if (any)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (in[e] - span < len) atomicAdd(&cnt[in[e] - span], 1u);
+        if (r - split >= kFoldRounds) {
+            hi += acc >> 24;
+            lo += acc & 0xffffffull;
+            acc = 0;
+            split = r;
         }
-        st->below = before;
-        st->prefix = (uint32_t)(e_lo + found - 1);   // the exponent field, as level 1 leaves it
+    });
+    hi += acc >> 24;
+    lo += acc & 0xffffffull;
+    for (int o = 16; o; o >>= 1) {
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        lo += __shfl_xor_sync(0xffffffffu, lo, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&shi, hi);
+        atomicAdd(&slo, lo);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (shi) atomicAdd(&st->lo[kBelowHi], shi);
+        if (slo) atomicAdd(&st->lo[kBelowLo], slo);
+    }
+    uint32_t* out = reinterpret_cast<uint32_t*>(st->hi);
+    for (uint32_t i = threadIdx.x; i < len; i += kHistThreads)
+        if (cnt[i]) atomicAdd(&out[i], cnt[i]);
+}
+
+// The first value of the window whose cumulative share reaches eps.
+__global__ void __launch_bounds__(kScanThreads) energy_value_scan_kernel(EnergyState* st, double eps)
+{
+    constexpr int PER = kWinValues / kScanThreads;
+    __shared__ double part[2][kScanThreads];
+    __shared__ int found;
+    const int t = threadIdx.x, len = (int)st->_pad * 2048;
+    if (len == 0) return;
+    const uint32_t* cnt = reinterpret_cast<const uint32_t*>(st->hi);
+    const uint32_t prefix = st->prefix, start = st->wmin_bits << 11;
+    const int e = (prefix ? (int)prefix : 1) - 127;
+    const double unit = pow2(2 * e - 46);
+    auto sq_of = [&](int i) {
+        const uint32_t m = (start + (uint32_t)i) | (prefix ? 0x800000u : 0u);
+        return (unsigned long long)m * m;
+    };
+    unsigned long long hi = 0, lo = 0;                   // exact; one conversion per thread
+    const int i0 = t * PER, i1 = i0 + PER < len ? i0 + PER : len;
+    for (int i = i0; i < i1; i += 4) {
+        const uint4 n4 = *reinterpret_cast<const uint4*>(cnt + i);
+        const uint32_t n[4] = {n4.x, n4.y, n4.z, n4.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const unsigned long long sq = sq_of(i + k);
+            hi += n[k] * (sq >> 24);
+            lo += n[k] * (sq & 0xffffffull);
+        }
+    }
+    const double own = ((double)hi * 16777216.0 + (double)lo) * unit;
+    part[0][t] = own;
+    if (t == 0) found = kWinValues;
+    __syncthreads();
+    int cur = 0;
+    for (int off = 1; off < kScanThreads; off <<= 1) {
+        part[cur ^ 1][t] = t >= off ? part[cur][t] + part[cur][t - off] : part[cur][t];
+        cur ^= 1;
+        __syncthreads();
+    }
+    const double total = st->total, near = eps * total * (1.0 - 0x1p-40);
+    double cum = st->below + ((double)st->lo[kBelowHi] * 16777216.0 + (double)st->lo[kBelowLo]) * unit +
+                 (t ? part[cur][t - 1] : 0.0);
+    int f = kWinValues;
+    if (own > 0.0 && cum + own * (1.0 + 0x1p-40) >= near)
+        for (int i = i0; i < i1 && f == kWinValues; ++i) {
+            if (cnt[i] == 0) continue;
+            const double x = (double)cnt[i] * (double)sq_of(i) * unit;
+            cum += x;
+            if (x > 0.0 && cum >= near && cum / total >= eps) f = i;
+        }
+    if (f < kWinValues) atomicMin(&found, f);
+    __syncthreads();
+    if (t == 0) {
+        if (found == kWinValues) st->failed = 1;         // a rounding step short: the exact form settles it
+        st->wmin_bits = (prefix << 23) + start + (uint32_t)found;
     }
 }
 
@@ -382,21 +547,38 @@ __global__ void __launch_bounds__(kScanThreads) energy_scan_kernel(EnergyState* 
     }
 }
 
-template <int LEVEL>
-cudaError_t hist(const float* W, int64_t n4, EnergyState* st, Workspace* ws, int grid, cudaStream_t s)
+// Grid of a streaming pass: per_sm CTAs per SM, fewer for small inputs.
+int stream_grid(int64_t n4, int per_sm)
 {
-    constexpr size_t smem = 2 * sizeof(unsigned long long) * Level<LEVEL>::NB * Level<LEVEL>::COPIES;
-    static int configured[64] = {0};
+    const int sms = sm_count() > 0 ? sm_count() : 148;
+    const int64_t want = (n4 + kHistThreads * kUnroll - 1) / (kHistThreads * kUnroll), cap = (int64_t)per_sm * sms;
+    return (int)(want < cap ? (want > 0 ? want : 1) : cap);
+}
+
+// Dynamic shared memory opt-in, once per kernel and device.
+template <typename Kernel>
+cudaError_t allow_smem(Kernel k, size_t smem, int (&configured)[64])
+{
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!configured[dev] && smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(energy_hist_kernel<LEVEL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (!configured[dev]) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
+        configured[dev] = 1;
     }
-    configured[dev] = 1;
-    energy_hist_kernel<LEVEL><<<grid, kHistThreads, smem, s>>>(reinterpret_cast<const float4*>(W), n4, st, ws);
+    return cudaSuccess;
+}
+
+template <int LEVEL>
+cudaError_t hist(const float4* W, int64_t n4, EnergyState* st, cudaStream_t s)
+{
+    constexpr size_t smem = 2 * sizeof(unsigned long long) * Level<LEVEL>::NB;
+    static int configured[64] = {0};
+    cudaError_t e = allow_smem(energy_hist_kernel<LEVEL>, smem, configured);
+    if (e != cudaSuccess) return e;
+    energy_hist_kernel<LEVEL><<<stream_grid(n4, 3), kHistThreads, smem, s>>>(W, n4, st);
     return cudaGetLastError();
 }
 
@@ -405,39 +587,43 @@ cudaError_t hist(const float* W, int64_t n4, EnergyState* st, Workspace* ws, int
 cudaError_t launch_energy_range(const float* W, int64_t count, double eps, EnergyState* st, Workspace* ws,
                                 cudaStream_t s)
 {
+    const float4* W4 = reinterpret_cast<const float4*>(W);
     const int64_t n4 = count / 4;
-    const int sms = sm_count() > 0 ? sm_count() : 148;
-    int64_t want = (n4 + kHistThreads * kUnroll - 1) / (kHistThreads * kUnroll);
-    const int64_t cap = 3 * (int64_t)sms;
-    const int grid = (int)(want < cap ? (want > 0 ? want : 1) : cap);
-    cudaError_t e;
     const size_t bucket_bytes = sizeof st->hi + sizeof st->lo;
+    cudaError_t e;
     if ((e = cudaMemsetAsync(st, 0, sizeof(EnergyState), s)) != cudaSuccess) return e;
-    if (eps > (double)count * ldexp(1.0, -59)) {
-        // the crossing lies within 31 exponents of w_max's
-        if ((e = launch_absmax(W, count, ws, s)) != cudaSuccess) return e;
-        constexpr size_t smem = (size_t)(kHistThreads / 32) * kWin * 32 * sizeof(unsigned long long);
-        static int configured[64] = {0};
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-        if (!configured[dev]) {
-            e = cudaFuncSetAttribute(energy_window_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-            configured[dev] = 1;
-        }
-        energy_window_kernel<<<grid, kHistThreads, smem, s>>>(reinterpret_cast<const float4*>(W), n4, st, ws);
-        energy_scan_window_kernel<<<1, 32, 0, s>>>(st, ws, eps);
-    } else {
-        if ((e = hist<1>(W, n4, st, ws, grid, s)) != cudaSuccess) return e;
-        energy_scan_kernel<1><<<1, kScanThreads, 0, s>>>(st, eps);
+    static int configured1[64] = {0}, configured3[64] = {0};
+    constexpr size_t smem1 = (size_t)(kHistThreads / 32) * kWin * 32 * sizeof(unsigned long long);
+    constexpr size_t smem3 = (size_t)kWinValues * sizeof(uint32_t);
+    if ((e = allow_smem(energy_exponents_kernel, smem1, configured1)) != cudaSuccess) return e;
+    if ((e = allow_smem(energy_values_kernel, smem3, configured3)) != cudaSuccess) return e;
+    energy_exponents_kernel<<<stream_grid(n4, 3), kHistThreads, smem1, s>>>(W4, n4, st, ws);
+    energy_scan_kernel<1><<<1, kScanThreads, 0, s>>>(st, eps);
+    if (count >> 32) {                                   // beyond the passes' 32-bit counts
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        return cudaMemsetAsync(&st->failed, 1, 1, s);
     }
-    // levels 2 and 3 re-stream W and keep only the selected prefix
     if ((e = cudaMemsetAsync(st->hi, 0, bucket_bytes, s)) != cudaSuccess) return e;
-    if ((e = hist<2>(W, n4, st, ws, grid, s)) != cudaSuccess) return e;
+    energy_count_kernel<<<stream_grid(n4, 6), kHistThreads, 0, s>>>(W4, n4, st);
+    energy_window_scan_kernel<<<1, kScanThreads, 0, s>>>(st, eps);
+    energy_values_kernel<<<stream_grid(n4, 3), kHistThreads, smem3, s>>>(W4, n4, st);
+    energy_value_scan_kernel<<<1, kScanThreads, 0, s>>>(st, eps);
+    return cudaGetLastError();
+}
+
+// Levels 2 and 3 by exact bucket energies, after launch_energy_range left
+// `failed` set (its exponent and the energy below it stand).
+cudaError_t launch_energy_exact(const float* W, int64_t count, double eps, EnergyState* st, cudaStream_t s)
+{
+    const float4* W4 = reinterpret_cast<const float4*>(W);
+    const int64_t n4 = count / 4;
+    const size_t bucket_bytes = sizeof st->hi + sizeof st->lo;
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(st->hi, 0, bucket_bytes, s)) != cudaSuccess) return e;
+    if ((e = hist<2>(W4, n4, st, s)) != cudaSuccess) return e;
     energy_scan_kernel<2><<<1, kScanThreads, 0, s>>>(st, eps);
     if ((e = cudaMemsetAsync(st->hi, 0, bucket_bytes, s)) != cudaSuccess) return e;
-    if ((e = hist<3>(W, n4, st, ws, grid, s)) != cudaSuccess) return e;
+    if ((e = hist<3>(W4, n4, st, s)) != cudaSuccess) return e;
     energy_scan_kernel<3><<<1, kScanThreads, 0, s>>>(st, eps);
     return cudaGetLastError();
 }

@@ -21,17 +21,18 @@ constexpr size_t kWorkspaceBytes = sizeof(Workspace);
 
 // Device state of the energy-range selection (caller-provided scratch,
 // logq_energy_scratch_bytes() bytes): bucket energies of the current level as
-// exact integer sums of the high / low 24 bits of m^2, the total energy, the
-// energy below the selected prefix, the prefix and the result.
+// exact integer sums of the high / low 24 bits of m^2 (or 32-bit counts in the
+// same words), the total energy, the energy below the selected prefix, the
+// prefix and the result.
 struct EnergyState {
     unsigned long long hi[4096];
     unsigned long long lo[4096];
     double total;
     double below;
     uint32_t prefix;
-    uint32_t wmin_bits;
-    uint32_t failed;        // the window pass found the crossing below its window
-    uint32_t _pad;
+    uint32_t wmin_bits;     // the result; before it, the first bucket of pass 3's window
+    uint32_t failed;        // the window of the counting passes did not settle the crossing
+    uint32_t _pad;          // buckets of pass 3's window
 };
 
 // Decision boundaries handed to the quantise kernel (fp32, rounded up).
@@ -103,6 +104,7 @@ logq_status quantize_with(const float* W, int64_t N, int64_t K, int bits, double
 cudaError_t launch_absmax(const float* W, int64_t count, Workspace* ws, cudaStream_t s);
 cudaError_t launch_energy_range(const float* W, int64_t count, double eps, EnergyState* st, Workspace* ws,
                                 cudaStream_t s);
+cudaError_t launch_energy_exact(const float* W, int64_t count, double eps, EnergyState* st, cudaStream_t s);
 cudaError_t launch_quantize(const float* W, int64_t N, int64_t K, const QuantParams& p,
                             uint8_t* codes, Workspace* ws, cudaStream_t s);
 cudaError_t launch_gemv(const LinearArgs& a, cudaStream_t s);

@@ -338,11 +338,18 @@ logq_status logq_quantize_energy(const float* W, int64_t N, int64_t K, int bits,
         return LOGQ_ERR_CUDA;
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return LOGQ_ERR_CUDA;
     if (host_words[1]) return LOGQ_ERR_NONFINITE;
-    float fmax, fmin;
+    float fmax;
     memcpy(&fmax, &host_words[0], 4);
-    memcpy(&fmin, &sel[0], 4);
     if (!(fmax > 0.0f)) return LOGQ_ERR_INVALID_ARG;     // all-zero weights
-    if (sel[1]) return LOGQ_ERR_CUDA;                    // selection inconsistent (not expected)
+    if (sel[1]) {
+        // the counting passes left the crossing open (rare): exact bucket energies settle it
+        if ((e = launch_energy_exact(W, N * K, eps, st, s)) != cudaSuccess) return LOGQ_ERR_CUDA;
+        if ((e = cudaMemcpyAsync(sel, &st->wmin_bits, sizeof sel, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+            return LOGQ_ERR_CUDA;
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return LOGQ_ERR_CUDA;
+    }
+    float fmin;
+    memcpy(&fmin, &sel[0], 4);
     if (!(fmin > 0.0f)) return LOGQ_ERR_INVALID_ARG;
     if (!(fmin < fmax)) return LOGQ_ERR_INVALID_ARG;                      // Eq. (3) would give b = 1
     const int qmax = (1 << (bits - 1)) - 1;
