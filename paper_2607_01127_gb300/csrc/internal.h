@@ -35,13 +35,19 @@ struct EnergyState {
     uint32_t _pad;          // buckets of pass 3's window
 };
 
-// Decision boundaries handed to the quantise kernel (fp32, rounded up).
+// Decision boundaries handed to the quantise kernel: fp32, rounded up; or
+// (from_max) factor[j] = b^(j + 1/2 - q_max), with which the kernel itself forms
+// them from the largest |w| that an absmax pass left in the workspace:
+// thresh[j] = (fp64 product of that and factor[j], rounded up to fp32), the
+// arithmetic of logq_build_codebook.
 struct QuantParams {
     float thresh[128];
+    double factor[128];
+    double lambda;          // from_max: log2 of the boundaries' ratio
     int32_t qmax;
     int32_t bits;
     int32_t check_nonfinite;
-    int32_t _pad;
+    int32_t from_max;
 };
 
 // One quantised linear call after validation.

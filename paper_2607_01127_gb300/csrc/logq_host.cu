@@ -40,6 +40,18 @@ logq_status check_quantize_args(const float* W, int64_t N, int64_t K, int bits, 
     return LOGQ_OK;
 }
 
+// Boundaries over the range for a quantise kernel that forms them itself: the
+// factors logq_build_codebook multiplies the range by (exact shift).
+static void quant_factors(int bits, double base, QuantParams* p)
+{
+    memset(p, 0, sizeof *p);
+    p->bits = bits;
+    p->qmax = (1 << (bits - 1)) - 1;
+    p->from_max = 1;
+    p->lambda = log2(base);
+    for (int j = 0; j < p->qmax; ++j) p->factor[j] = pow(base, (double)j + 0.5 - (double)p->qmax);
+}
+
 // The quantisation itself, on a workspace record ws (device): Sec. 3.2 w_max
 // when range <= 0, the codebook (Eqs. (2), (4)), then Eq. (1) and packing;
 // one 8-byte readback and one stream synchronisation report non-finite
@@ -52,8 +64,25 @@ logq_status quantize_with(const float* W, int64_t N, int64_t K, int bits, double
 
     uint32_t host_words[2] = {0, 0};
     const bool auto_range = !(range > 0.0);
+    if (auto_range && flags == LOGQ_SHIFT_EXACT) {
+        // Sec. 3.2: w_max = max_i |w_i|, reduced on the device.  With the exact shift
+        // every boundary is w_max times a factor of the base, so the quantise
+        // kernel forms them itself and follows at once; w_max comes back afterwards.
+        QuantParams p;
+        quant_factors(bits, base, &p);
+        if ((e = launch_absmax(W, N * K, ws, s)) != cudaSuccess) return LOGQ_ERR_CUDA;
+        if ((e = launch_quantize(W, N, K, p, codes, ws, s)) != cudaSuccess) return LOGQ_ERR_CUDA;
+        if ((e = cudaMemcpyAsync(host_words, ws, sizeof host_words, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+            return LOGQ_ERR_CUDA;
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return LOGQ_ERR_CUDA;
+        if (host_words[1]) return LOGQ_ERR_NONFINITE;
+        float mx;
+        memcpy(&mx, &host_words[0], 4);
+        if (!(mx > 0.0f)) return LOGQ_ERR_INVALID_ARG;   // all-zero weights: no log range
+        return cb_out ? logq_build_codebook(bits, base, (double)mx, flags, cb_out) : LOGQ_OK;
+    }
     if (auto_range) {
-        // Sec. 3.2: w_max = max_i |w_i|, reduced on the device.
+        // The floor shift depends on log_b w_max as a whole number, settled on the host.
         if ((e = launch_absmax(W, N * K, ws, s)) != cudaSuccess) return LOGQ_ERR_CUDA;
         if ((e = cudaMemcpyAsync(host_words, ws, sizeof host_words, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
             return LOGQ_ERR_CUDA;

@@ -4,20 +4,32 @@
 // The quantiser assigns m = #{ j : |w| >= thresh[j] } against the fp32
 // decision boundaries of the codebook (rounded up from fp64), which for fp32
 // weights equals round(log_b|w| + s) clamped to [0, q_max].
+//
+// Over the reduced range the quantise kernel follows the absmax pass without a trip
+// to the host: it forms its boundaries from the maximum in the workspace (from_max,
+// estimate_setup).  The absmax pass walks W from the start and the quantise pass from
+// the end, so that it finds what the first left in L2.  Bound by HBM: the matrices of
+// a Llama-3.1-8B layer (872 MB of weights, 4 bits) take 560 us; 674 us
+// with the maximum read back in between and both passes from the start.
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
+
+#include <type_traits>
 
 #include "internal.h"
 
 namespace logq {
 namespace {
 
+// Level estimate of the kernels below.  from_max: the kernel forms t2 and C
+// itself (estimate_setup), the host gives K and factor.
 struct QuantEst {
     uint32_t t2[8];     // 2 x the boundaries' bit patterns; 0xffffffff after the last
     uint64_t C;         // fixed-point offset of the level estimate (two's complement)
     uint32_t K;         // fixed-point slope
-    uint32_t _pad;
+    int32_t from_max;
+    double factor[8];   // from_max: boundaries over the largest |w|
 };
 
 struct QuantEst8 {
@@ -25,7 +37,8 @@ struct QuantEst8 {
     uint32_t corr[64];  // log2(1 + f) - f (lower bound over each 1/64 of f), in units of 2^-24
     uint64_t C;         // fixed-point offset (two's complement), units of 2^-40 of a level
     uint32_t K;         // fixed-point slope
-    uint32_t _pad;
+    int32_t from_max;
+    double factor[128];
 };
 
 __device__ __forceinline__ float4 ld_stream(const float4* p)
@@ -90,6 +103,56 @@ __global__ void __launch_bounds__(256) absmax_kernel(const float4* __restrict__ 
     }
 }
 
+// The largest |w| an absmax pass left; 0 when there is none or a weight is not
+// finite (the caller reports either and the codes do not matter).
+__device__ __forceinline__ float max_of(const Workspace* ws)
+{
+    return ws->nonfinite ? 0.f : __uint_as_float(ws->absmax_bits);
+}
+
+// Boundary j of the codebook whose range is mx.
+__device__ __forceinline__ float boundary(float mx, double factor) { return __double2float_ru((double)mx * factor); }
+
+// A kernel's boundaries (2 x their bit patterns, NT2 of them, NB real ones) and
+// estimate offset in shared memory.  ONE is the unit of a level in the fixed
+// point.  Returns false when nothing is to be done (max_of), and leaves
+// *usable = 0 when the first boundary is below `least`, where the estimate does
+// not hold.
+template <int NB, int NT2, typename Est>
+__device__ __forceinline__ bool estimate_setup(const Est& q, const Workspace* ws, float least, double one, uint32_t* t2,
+                                               unsigned long long* C, int* usable)
+{
+    const int t = threadIdx.x;
+    const float mx = q.from_max ? max_of(ws) : 1.f;
+    if (!(mx > 0.f)) return false;
+    if (t < NT2) {
+        t2[t] = q.t2[t];
+        if (q.from_max) t2[t] = t < NB ? 2u * __float_as_uint(boundary(mx, q.factor[t])) : 0xffffffffu;
+    }
+    if (t == 0) {
+        *C = q.C;
+        *usable = 1;
+        if (q.from_max) {
+            // log2 of the first boundary in fp32: off by less than 2^-16, i.e. at most
+            // 0.0016 of a level (ratio 2^0.01) of the 0.05 that the bias leaves
+            const float t0 = boundary(mx, q.factor[0]), tl = boundary(mx, q.factor[NB - 1]);
+            const long long l0 = llrintf(log2f(t0) * 16777216.f) + (127ll << 24);
+            *C = (unsigned long long)((long long)(0.95 * one) - l0 * (long long)q.K);
+            *usable = t0 >= least && tl < __uint_as_float(0x7f800000u);
+        }
+    }
+    return true;
+}
+
+// Number of boundaries (2 x bit patterns) not above u2, for weights the estimate
+// does not serve.
+__device__ __forceinline__ uint32_t count_below(const uint32_t* t2, int n, uint32_t u2)
+{
+    uint32_t m = 0;
+    while ((int)m < n && u2 >= t2[m]) ++m;
+    return m;
+}
+
 // Magnitude index of one weight: the number of boundaries not above |w|.
 // Boundaries are positive fp32 values, so they compare like their bit
 // patterns; |w| is compared as bits too (a NaN counts as large and is
@@ -119,6 +182,17 @@ __device__ __forceinline__ uint32_t code_of(uint32_t bits, uint32_t m)
     return m != 0 ? (m | sign) : 0u;
 }
 
+// The boundaries' bit patterns (q_max 7 or 3) for the search kernels.
+__device__ __forceinline__ bool load_bounds(const QuantParams& p, const Workspace* ws, uint32_t (&t)[8])
+{
+    const float mx = p.from_max ? max_of(ws) : 1.f;
+    if (!(mx > 0.f)) return false;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        t[j] = __float_as_uint(!p.from_max ? p.thresh[j] : j < p.qmax ? boundary(mx, p.factor[j]) : INFINITY);
+    return true;
+}
+
 // 4-bit: each thread turns 8 consecutive weights into one 32-bit word
 // (k even in the low nibble of each byte).
 __global__ void __launch_bounds__(256) quantize4_kernel(const float4* __restrict__ W, int64_t nwords,
@@ -126,11 +200,10 @@ __global__ void __launch_bounds__(256) quantize4_kernel(const float4* __restrict
                                                         Workspace* ws)
 {
     uint32_t t[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) t[j] = __float_as_uint(p.thresh[j]);
+    if (!load_bounds(p, ws, t)) return;
     uint32_t umax = 0;                       // largest |w| bit pattern seen (non-finite check)
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nwords; i += stride) {
+    for (int64_t i = nwords - 1 - ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i >= 0; i -= stride) {
         const float4 a = ld_stream(W + 2 * i);
         const float4 b = ld_stream(W + 2 * i + 1);
         const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
@@ -165,11 +238,15 @@ __global__ void __launch_bounds__(256) quantize4e_kernel(const float4* __restric
                                                          uint32_t* __restrict__ out, Workspace* ws)
 {
     __shared__ uint32_t t2[8];
-    if (threadIdx.x < 8) t2[threadIdx.x] = q.t2[threadIdx.x];
+    __shared__ unsigned long long sC;
+    __shared__ int usable;
+    if (!estimate_setup<7, 8>(q, ws, 1.1754943508222875e-38f, 4294967296.0, t2, &sC, &usable)) return;
     __syncthreads();
+    const uint64_t C = sC;
     uint32_t umax = 0;                       // largest 2|w| bit pattern seen (non-finite check)
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nwords; i += stride) {
+    auto run = [&](auto estimate) {
+    for (int64_t i = nwords - 1 - ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i >= 0; i -= stride) {
         const float4 a = ld_stream(W + 2 * i);
         const float4 b = ld_stream(W + 2 * i + 1);
         const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
@@ -179,14 +256,18 @@ __global__ void __launch_bounds__(256) quantize4e_kernel(const float4* __restric
             const uint32_t bits = __float_as_uint(v[e]);
             const uint32_t u2 = bits << 1;   // 2|w|: the sign bit drops out
             if (CHECK) umax = max(umax, u2);
-            const uint64_t p = (uint64_t)u2 * q.K + q.C;
+            const uint64_t p = (uint64_t)u2 * q.K + C;
             const int mh = __vimin_s32_relu((int)(uint32_t)(p >> 32), 7);
-            mword |= ((uint32_t)mh + (u2 >= t2[mh] ? 1u : 0u)) << (4 * e);
+            const uint32_t m = decltype(estimate)::value ? (uint32_t)mh + (u2 >= t2[mh] ? 1u : 0u) : count_below(t2, 7, u2);
+            mword |= m << (4 * e);
             sword |= (bits >> 31) << (4 * e + 3);
         }
         // a sign bit only on nibbles whose magnitude is not 0 (m + 7 carries into bit 3)
         out[i] = mword | (sword & (mword + 0x77777777u) & 0x88888888u);
     }
+    };
+    if (usable) run(std::true_type());
+    else run(std::false_type());
     if (CHECK) {
         const uint32_t bad = __reduce_or_sync(0xffffffffu, umax >= 0xff000000u ? 1u : 0u);
         if (bad && (threadIdx.x & 31) == 0) atomicOr(&ws->nonfinite, 1u);
@@ -206,12 +287,16 @@ __global__ void __launch_bounds__(256) quantize8e_kernel(const float4* __restric
 {
     __shared__ uint32_t t2[128];
     __shared__ uint32_t corr[64];
-    if (threadIdx.x < 128) t2[threadIdx.x] = q.t2[threadIdx.x];
+    __shared__ unsigned long long sC;
+    __shared__ int usable;
+    if (!estimate_setup<127, 128>(q, ws, 7.52316384526264e-37f, 1099511627776.0, t2, &sC, &usable)) return;
     if (threadIdx.x < 64) corr[threadIdx.x] = q.corr[threadIdx.x];
     __syncthreads();
+    const uint64_t C = sC;
     uint32_t umax = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += stride) {
+    auto run = [&](auto estimate) {
+    for (int64_t i = n16 - 1 - ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i >= 0; i -= stride) {
         float4 v4[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) v4[j] = ld_stream(W + 4 * i + j);
@@ -225,15 +310,19 @@ __global__ void __launch_bounds__(256) quantize8e_kernel(const float4* __restric
                 const uint32_t bits = __float_as_uint(v[e]);
                 const uint32_t u2 = bits << 1;
                 if (CHECK) umax = max(umax, u2);
-                const uint64_t p = (uint64_t)(u2 + corr[(u2 >> 18) & 63]) * q.K + q.C;
+                const uint64_t p = (uint64_t)(u2 + corr[(u2 >> 18) & 63]) * q.K + C;
                 const int mh = __vimin_s32_relu((int)(uint32_t)(p >> 32) >> 8, 127);
-                mword |= ((uint32_t)mh + (u2 >= t2[mh] ? 1u : 0u)) << (8 * e);
+                const uint32_t m = decltype(estimate)::value ? (uint32_t)mh + (u2 >= t2[mh] ? 1u : 0u) : count_below(t2, 127, u2);
+                mword |= m << (8 * e);
                 sword |= (bits >> 31) << (8 * e + 7);
             }
             word[j] = mword | (sword & (mword + 0x7f7f7f7fu) & 0x80808080u);
         }
         out[i] = make_uint4(word[0], word[1], word[2], word[3]);
     }
+    };
+    if (usable) run(std::true_type());
+    else run(std::false_type());
     if (CHECK) {
         const uint32_t bad = __reduce_or_sync(0xffffffffu, umax >= 0xff000000u ? 1u : 0u);
         if (bad && (threadIdx.x & 31) == 0) atomicOr(&ws->nonfinite, 1u);
@@ -253,8 +342,7 @@ __global__ void __launch_bounds__(256) quantize3_kernel(const float4* __restrict
 {
     __shared__ float4 stage[8][256];
     uint32_t t[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) t[j] = __float_as_uint(p.thresh[j]);
+    if (!load_bounds(p, ws, t)) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     float4* st = stage[wid];
     uint32_t umax = 0;
@@ -338,8 +426,11 @@ __global__ void __launch_bounds__(kQ3eThreads) quantize3e_kernel(const float4* _
     constexpr int kWarps = kQ3eThreads / 32;
     __shared__ float4 stage[kWarps][2][256];
     __shared__ uint32_t t2[4];
-    if (threadIdx.x < 4) t2[threadIdx.x] = q.t2[threadIdx.x];
+    __shared__ unsigned long long sC;
+    __shared__ int usable;
+    if (!estimate_setup<3, 4>(q, ws, 1.1754943508222875e-38f, 4294967296.0, t2, &sC, &usable)) return;
     __syncthreads();
+    const uint64_t C = sC;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t umax = 0;                                             // largest 2|w| bit pattern seen
     constexpr uint32_t kLow = 0x1B6DB6DBu;                        // 0b011 in each of 10 slots
@@ -359,11 +450,13 @@ __global__ void __launch_bounds__(kQ3eThreads) quantize3e_kernel(const float4* _
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    int64_t gb = ((int64_t)blockIdx.x * kWarps + wid) * 32;
-    if (gb < ngroups) issue(0, gb);
-    for (int b = 0; gb < ngroups; b ^= 1) {
-        const int64_t gn = gb + wstride;
-        if (gn < ngroups) issue(b ^ 1, gn);
+    // batches from the end to the start
+    auto run = [&](auto estimate) {
+    int64_t gb = (ngroups - 1) / 32 * 32 - ((int64_t)blockIdx.x * kWarps + wid) * 32;
+    if (gb >= 0) issue(0, gb);
+    for (int b = 0; gb >= 0; b ^= 1) {
+        const int64_t gn = gb - wstride;
+        if (gn >= 0) issue(b ^ 1, gn);
         else asm volatile("cp.async.commit_group;" ::: "memory");   // keeps one group per batch
         asm volatile("cp.async.wait_group 1;" ::: "memory");         // this batch has landed
         __syncwarp();
@@ -382,9 +475,10 @@ __global__ void __launch_bounds__(kQ3eThreads) quantize3e_kernel(const float4* _
                     const uint32_t bits = __float_as_uint(w4[i]);
                     const uint32_t u2 = bits << 1;                  // 2|w|: the sign bit drops out
                     if (CHECK) umax = max(umax, u2);
-                    const uint64_t pe = (uint64_t)u2 * q.K + q.C;
+                    const uint64_t pe = (uint64_t)u2 * q.K + C;
                     const int mh = __vimin_s32_relu((int)(uint32_t)(pe >> 32), 3);
-                    const uint32_t val = (uint32_t)mh + (u2 >= t2[mh] ? 1u : 0u) + ((bits >> 31) << 2);
+                    const uint32_t m = decltype(estimate)::value ? (uint32_t)mh + (u2 >= t2[mh] ? 1u : 0u) : count_below(t2, 3, u2);
+                    const uint32_t val = m + ((bits >> 31) << 2);
                     if (e < 30) v[e / 10] += val << (3 * (e % 10));  // disjoint slots: add = or
                     else if (e == 30) c30 = val;
                     else c31 = val;
@@ -406,6 +500,9 @@ __global__ void __launch_bounds__(kQ3eThreads) quantize3e_kernel(const float4* _
         __syncwarp();                                  // stage b is refilled two batches on
         gb = gn;
     }
+    };
+    if (usable) run(std::true_type());
+    else run(std::false_type());
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     if (CHECK) {
         const uint32_t bad = __reduce_or_sync(0xffffffffu, umax >= 0xff000000u ? 1u : 0u);
@@ -421,11 +518,17 @@ __global__ void __launch_bounds__(256) quantize8_kernel(const float4* __restrict
                                                         Workspace* ws)
 {
     __shared__ uint32_t t[128];
-    if (threadIdx.x < 128) t[threadIdx.x] = threadIdx.x < 127 ? __float_as_uint(p.thresh[threadIdx.x]) : 0x7f800000u;
+    const float mx = p.from_max ? max_of(ws) : 1.f;
+    if (!(mx > 0.f)) return;
+    if (threadIdx.x < 128) {
+        float v = p.thresh[threadIdx.x];
+        if (p.from_max) v = boundary(mx, p.factor[threadIdx.x]);
+        t[threadIdx.x] = threadIdx.x < 127 ? __float_as_uint(v) : 0x7f800000u;
+    }
     __syncthreads();
     uint32_t umax = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += stride) {
+    for (int64_t i = n16 - 1 - ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i >= 0; i -= stride) {
         float4 v4[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) v4[j] = ld_stream(W + 4 * i + j);
@@ -468,6 +571,14 @@ __global__ void __launch_bounds__(256) quantize8_kernel(const float4* __restrict
 bool estimate_params(const QuantParams& p, QuantEst& q)
 {
     if (!((p.bits == 4 && p.qmax == 7) || (p.bits == 3 && p.qmax == 3))) return false;
+    memset(&q, 0, sizeof q);
+    if (p.from_max) {                    // the kernel looks at the first and last boundary
+        if (!(p.lambda >= 0.12) || !(p.lambda <= 3.0)) return false;
+        q.K = (uint32_t)nearbyint(256.0 / p.lambda);
+        q.from_max = 1;
+        for (int j = 0; j < 8; ++j) q.factor[j] = j < p.qmax ? p.factor[j] : 0.0;
+        return true;
+    }
     const int last = p.qmax - 1;
     const double t0 = p.thresh[0], tl = p.thresh[last];
     if (!(t0 >= 1.1754943508222875e-38) || !(tl > t0) || !isfinite(tl)) return false;
@@ -482,7 +593,6 @@ bool estimate_params(const QuantParams& p, QuantEst& q)
         if (j < p.qmax) memcpy(&b, &p.thresh[j], 4);
         q.t2[j] = j < p.qmax ? 2u * b : 0xffffffffu;
     }
-    q._pad = 0;
     return true;
 }
 
@@ -493,6 +603,19 @@ bool estimate_params(const QuantParams& p, QuantEst& q)
 bool estimate_params8(const QuantParams& p, QuantEst8& q)
 {
     if (p.bits != 8 || p.qmax != 127) return false;
+    memset(&q, 0, sizeof q);
+    for (int i = 0; i < 64; ++i) {
+        const double f0 = i / 64.0, f1 = (i + 1) / 64.0;
+        const double g0 = log2(1.0 + f0) - f0, g1 = log2(1.0 + f1) - f1;   // concave: minimum at an end
+        q.corr[i] = (uint32_t)floor(16777216.0 * (g0 < g1 ? g0 : g1));
+    }
+    if (p.from_max) {
+        if (!(p.lambda >= 0.01) || !(p.lambda <= 4.0)) return false;
+        q.K = (uint32_t)nearbyint(65536.0 / p.lambda);
+        q.from_max = 1;
+        for (int j = 0; j < 127; ++j) q.factor[j] = p.factor[j];
+        return true;
+    }
     const double t0 = p.thresh[0], tl = p.thresh[126];
     if (!(t0 >= 7.52316384526264e-37) || !(tl > t0) || !isfinite(tl)) return false;   // 2^-120
     const double l0 = log2(t0);
@@ -507,12 +630,6 @@ bool estimate_params8(const QuantParams& p, QuantEst8& q)
         q.t2[j] = 2u * b;
     }
     q.t2[127] = 0xffffffffu;
-    for (int i = 0; i < 64; ++i) {
-        const double f0 = i / 64.0, f1 = (i + 1) / 64.0;
-        const double g0 = log2(1.0 + f0) - f0, g1 = log2(1.0 + f1) - f1;   // concave: minimum at an end
-        q.corr[i] = (uint32_t)floor(16777216.0 * (g0 < g1 ? g0 : g1));
-    }
-    q._pad = 0;
     return true;
 }
 
