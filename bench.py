@@ -645,12 +645,6 @@ def time_skinny(logq, torch, dev, batches=(1, 4, 16), reps: int = 10):
     return out
 
 
-def _small_batch_on_tc(B: int) -> bool:
-    """Whether the library runs the 8B gate at batch B on the tensor cores: batches
-    9..16 (padded to 16 on the CUDA cores) do, batches up to 8 do not."""
-    return 9 <= B <= 16
-
-
 def fp32_peak_tflops(sm_mhz: float) -> float:
     """CUDA-core fp32 FMA rate: SMs x 128 lanes x 2 flops x clock."""
     import torch
@@ -763,7 +757,7 @@ def run_ours(args):
                             "(linears that read the same activations share a launch), chained: each "
                             "launch reads the previous launch's bf16 output; programmatic dependent "
                             "launch, each launch warms L2 with the next launch's codes when they are "
-                            "under 20 MiB"},
+                            "under 4 MiB"},
         "e2e": {"value": round(e2e_value, 1), "unit": "GB/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h},
         "gpu_launches": launches_per_step * args.steps,
@@ -794,14 +788,13 @@ def run_ours(args):
             line["skinny"] = {
                 f"B{B}": {"us": round(v["us"], 2), "gbs": round(v["gbs"], 1),
                           "hbm_frac": round(v["gbs"] / pk["hbm_gbs"], 4), "tflops": round(v["tflops"], 2),
-                          "path": "tensor cores" if _small_batch_on_tc(B) else "CUDA cores",
+                          "path": "decode kernel (lookups, warp-level tensor-core multiply-adds)",
                           "fp32_frac": round(v["tflops"] / fp32, 4)} for B, v in sk.items()}
             line["skinny"]["fp32_peak_tflops"] = round(fp32, 1)
             line["skinny"]["note"] = ("Llama-3.1-8B gate 14336x4096, 4-bit, bf16 in/out, 12 rotating code copies "
-                                      "(beyond L2), workspace of logq_linear_workspace_bytes; batch 16 runs on the "
-                                      "tensor cores (16-token tiles), batches 1 and 4 on the CUDA cores; fp32_frac "
-                                      "against SMs x 128 lanes x 2 flops x the median SM clock of the headline run "
-                                      "(the CUDA-core roof)")
+                                      "(beyond L2), workspace of logq_linear_workspace_bytes; fp32_frac against "
+                                      "SMs x 128 lanes x 2 flops x the median SM clock of the headline run (the "
+                                      "CUDA cores' fp32 rate, which the kernel does not use)")
         except Exception as e:
             line["skinny"] = {"error": str(e)[:200]}
     if rank == 0:

@@ -141,12 +141,13 @@ size_t logq_workspace_bytes(void);
 
 /* Bytes of workspace with which logq_linear (and logq_linear_grouped, per
  * matrix) runs a B x N x K product at full speed: logq_workspace_bytes() plus,
- * for products that run on the tensor cores, room for fp32 partial sums when
- * the output tiles are too few to fill the GPU and each tile's k range is split
- * over several CTAs (Y is then their fixed-order sum, a second kernel on the
- * same stream).  A smaller workspace (at least logq_workspace_bytes()) is
- * accepted: the call then splits less, or, for 4-bit batches of 8..16, keeps
- * the CUDA-core kernel.  0 for invalid sizes. */
+ * from batches of 8 (4 bits) or 5 (3 and 8 bits) on, room for fp32 partial sums
+ * when the output tiles are too few to fill the GPU and each tile's k range is
+ * split over several CTAs (Y is then their fixed-order sum, a second kernel on
+ * the same stream).  The decode kernel uses the same room for parts of K at
+ * batches of 9 and more.  A smaller workspace (at least
+ * logq_workspace_bytes()) is accepted: the call then splits less.  0 for
+ * invalid sizes. */
 size_t logq_linear_workspace_bytes(int64_t B, int64_t N, int64_t K, int bits);
 
 /*
@@ -173,12 +174,10 @@ logq_status logq_quantize(const float* W, int64_t N, int64_t K, int bits, double
  *   codes (device): packed as above for cb->bits.  X (device): x_dtype.
  *   Y (device): y_dtype in {LOGQ_F32, x_dtype}; a 16-bit Y is the fp32 sum
  *   rounded to nearest-even.  All device pointers 16-byte aligned.
- *   B <= 16 (4-bit) or B <= 4 (3- and 8-bit) runs the decode GEMV /
- *   skinny-GEMM kernel on CUDA cores; larger B runs the prefill GEMM kernel
- *   on the tensor cores (tcgen05), as do 4-bit batches of 8..16 when the
- *   workspace (see logq_linear_workspace_bytes) lets that launch keep at
- *   least half of the SMs busy.  Calls sharing a workspace must be ordered
- *   on one stream (partial sums may live in it).
+ *   B <= 16 runs the decode kernel, as does B <= 32 at 3 and 8 bits and, for
+ *   matrices of up to 32 M weights, at 4 bits; larger B runs the prefill GEMM
+ *   kernel (tcgen05).  Calls sharing a workspace must be ordered on one stream
+ *   (partial sums may live in it).
  * Asynchronous.  Errors: LOGQ_ERR_INVALID_ARG, LOGQ_ERR_UNSUPPORTED,
  * LOGQ_ERR_WORKSPACE, LOGQ_ERR_CUDA (launch).  A device-side wait that hit
  * its bound is reported later by logq_workspace_status. */
@@ -234,8 +233,9 @@ size_t logq_energy_scratch_bytes(void);
  *   eps in (0, 1].  wmin_out (host, may be NULL) receives w_min; cb_out (host,
  *   may be NULL) the codebook (its base is b, its range w_max).
  *   scratch: logq_energy_scratch_bytes() bytes of device memory.
- * Synchronises `stream` once after the range is known and once before
- * returning.
+ * Synchronises `stream` once after the range is known (twice where the counts
+ * of the selection leave w_min open and exact energies settle it) and once
+ * before returning.
  * Errors: those of logq_quantize; LOGQ_ERR_INVALID_ARG also when eps is not in
  * (0, 1], W is all zero, or w_min == w_max (a single magnitude holds the
  * required energy, so Eq. (3) gives b = 1: no logarithmic codebook exists);
@@ -320,10 +320,10 @@ typedef struct logq_linear_item {
  * e.g. the q/k/v or the gate/up projections of a transformer layer -- each
  * with its own per-tensor codebook (Sec. 3.1) and output: Y_i = X * What_i^T
  * (Sec. 3.3), in one call.  count is 1..4 and all items share the code width
- * of their codebooks.  With B <= 16 (4-bit) or B <= 4 (3-, 8-bit) the matrices
- * share a single decode-GEMV launch.  Larger B (and 4-bit batches of 8..16
- * that logq_linear would send to the tensor cores) runs one prefill launch
- * whose CTAs are divided among the matrices in proportion to their tiles,
+ * of their codebooks.  Batches that the decode kernel takes (as logq_linear,
+ * with the weights of all items) share a single launch of it.  Larger B runs
+ * one prefill launch whose CTAs are divided among the matrices in proportion to
+ * their tiles,
  * when its estimate beats one launch per matrix (small matrices such as k / v
  * projections then share the GPU with a larger one); otherwise one launch
  * each, as logq_linear.  The workspace holds the partial sums of split k
@@ -334,9 +334,9 @@ typedef struct logq_linear_item {
  * codes of the next layer -- a hint only: it is never read by the
  * computation and may be any readable device memory at any alignment (the
  * library prefetches the 16-byte aligned part inside it: the start rounded up
- * and the length down to whole 16-byte units).  A decode-GEMV launch ignores
- * a range of 20 MiB or more: codes that large stream at full rate when their
- * own launch reads them, and prefetching them would slow this one.  Asynchronous; errors
+ * and the length down to whole 16-byte units).  A decode launch ignores a
+ * range of 4 MiB or more: codes that large stream at full rate when their own
+ * launch reads them, and prefetching them would slow this one.  Asynchronous; errors
  * as logq_linear (LOGQ_ERR_INVALID_ARG also for count outside 1..4 or items
  * of different code widths).
  */

@@ -1,34 +1,49 @@
-// Decode GEMV / skinny GEMM on CUDA cores: Y[b][n] = sum_k X[b][k] * table[code(n, k)]
+// Decode kernel: Y[b][n] = sum_k X[b][k] * table[code(n, k)] for batches up to 32
 // (paper Sec. 3.3: dequantisation by lookup table instead of exponentiation).
 //
-// Design (CTAs of 8 or 16 warps, see the launch shapes below):
 //  * Pair table in shared memory.  Two codes (one byte at 4 bits, one 6-bit
 //    field at 3 bits) index a table whose entry is the bf16x2 / f16x2 pair of
-//    their dequantised values, signs included.  Each entry occupies a 256-byte
-//    row holding one copy per lane, so lane l always reads bank l: the lookups
-//    of a warp never conflict.  The table starts the dynamic shared memory at
-//    the fixed shared address kTabOff, so the byte offset of an entry,
-//    byte << 8 | 4 * lane, is one byte permute (prmt) of the code word and the
-//    table base is the load's immediate offset.
-//  * Each warp owns a fixed span of K (32 lanes x KW consecutive k) and keeps
-//    its activations for that span in registers for the whole kernel; it walks
-//    the rows of the CTA's row range, one 16-, 8- or 4-byte coalesced load of
-//    codes per lane and row (a warp reads a contiguous 512/256/128-byte run).
-//  * fp32 accumulation (mixed-precision fma with bf16/f16 operands), a
-//    reduce-scatter across the 32 lanes per round of rows, then a fixed-order
-//    sum over the spans in shared memory: results are bit-identical from run
-//    to run.
-//  * Batch-1 4-bit launches run 8-warp CTAs, two per SM (tiny ones one per
-//    SM): with programmatic dependent launch, a CTA of the next launch on the
-//    stream starts as soon as one of them leaves, and builds its table and
-//    issues its first code loads while the rest of this launch finishes.
-//    Other small launches run one 8-warp CTA per SM (room for the next
-//    launch's CTAs), other large ones one 16-warp CTA per SM.  Batches of 4
-//    and more hold more k per lane where registers allow (one CTA per SM), so
-//    that the cross-lane reduction of each row is shared by more multiply-adds.
-//  * Where it pays, the CTA's contiguous range of code rows is prefetched into
-//    L2 with bulk prefetches at kernel start; an optional warm-up range (the
-//    next launch's codes) is prefetched the same way when it is small.
+//    their dequantised values, signs included; at 8 bits one code per entry.
+//    Each entry occupies a 256-byte row holding one copy per lane, so lane l
+//    always reads bank l: the lookups of a warp never conflict.  The table starts
+//    the dynamic shared memory at the fixed shared address kTabOff, so the byte
+//    offset of an entry, byte << 8 | 4 * lane, is one byte permute (prmt) of the
+//    code word and the table base is the load's immediate offset.
+//  * Multiply-adds on the warp-level tensor-core instruction mma.sync m16n8k16:
+//    the looked-up pairs are its A fragments as they are (16 rows, k permuted
+//    alike in both operands), and B has 8 columns.  A batch of 1 needs one, so
+//    the others hold further segments of k: S segments x 8 / S batch rows, the 16
+//    MMA rows being 16 / S weight rows x S segments, of which the products on
+//    the matching columns are used.  This is not for the arithmetic rate
+//    (tcgen05 has far more, for operands in shared or tensor memory, which the
+//    lookups would have to be stored to first) but for the instruction count:
+//    one MMA takes the place of 8 fused multiply-adds per lane and of most of the
+//    cross-lane reduction, and batches up to 8 cost hardly more than 1.
+//  * Each warp owns a span of K and keeps its activations for it in registers;
+//    it walks the rows of the CTA's row range, T tiles of code loads in flight,
+//    each tile's registers refilled as soon as it is decoded.
+//  * fp32 accumulation: single MMAs up to batch 8 (chains of 2 above), their
+//    sums and everything after them added with rounding to nearest in a fixed
+//    order (bit-identical from run to run).  Longer chains lose bits (the tensor
+//    core truncates): against 64 bits fp32 outputs over 4096 k are 0.7e-7 (bf16)
+//    and 0.85e-7 (fp16) off, as with fp32 fused multiply-adds (0.7e-7, 0.9e-7);
+//    chains of 2 0.7e-7 and 0.9e-7, chains of 8 1.0e-7 and 1.9e-7.
+//  * Programmatic dependent launch: a CTA of the next launch on the stream starts
+//    as soon as one of these leaves, and issues its first code loads and builds
+//    its table meanwhile.  At batch 1 two 8-warp CTAs run per SM for that; larger
+//    batches, which hold more activations per lane, fill an SM with one CTA.
+//
+// What bounds it: the lookups (128 bytes of shared memory per 64 weights: 12 us
+// of an SM's shared-memory cycles for the 218 M weights of a Llama-3.1-8B layer,
+// against 16 us of HBM time for their codes at 4 bits) and, per launch, the
+// latency of a CTA's life (activations after the previous launch, first tile,
+// final sum: 2.5-3 us).  Per layer (q+k+v, o, gate+up, down chained, bf16), with
+// fused multiply-adds on the CUDA cores (batches up to 8; 16 as the tcgen05
+// prefill kernel at 3 and 8 bits above 4) before and now:
+//   4 bits, batch 1 / 2 / 4 / 8 / 16: 31.1 / 45.6 / 57.0 / 109 / 117 us before,
+//     30.7 / 34.3 / 41.8 / 49.1 / 64.4 now;
+//   3 bits, batch 1 / 4 / 16 / 32: 39.0 / 68.7 / 162 / 194 before, 35.8 / 45.5 / 75 / 130 now;
+//   8 bits, batch 1 / 4 / 16 / 32: 52.8 / 85.8 / 157 / 179 before, 48.2 / 64 / 96 / 144 now.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -41,90 +56,56 @@
 namespace logq {
 namespace {
 
-// Threads per CTA: 256 (two CTAs fit on an SM) for batch-1 4-bit launches,
-// small launches and batches of 4 and more, 512 (one per SM, all 16 warps
-// sharing one table) for the other large launches.
-constexpr int kSmallThreads = 256;
-constexpr int kLargeThreads = 512;
 constexpr int kTabStride = 256;               // bytes per pair-table entry
 // Shared address at which dynamic shared memory starts in a kernel without
 // static shared memory: the per-CTA reserved area comes first.
 constexpr uint32_t kTabOff = 1024;
 constexpr uint32_t kLvlOff = 128;             // levels staged in the free half of table row 0
-// Span partials: for batch 1-2 at 4 bits they live in the free upper halves
-// of the table's 256 rows (32 KiB), otherwise after the table.
-constexpr int kRedBytes = 32 * 1024;
-__host__ __device__ constexpr bool red_in_table(int bits, int B) { return bits == 4 && B <= 2; }
-constexpr int64_t kPrefetchCap = 1 << 20;     // bytes of codes prefetched per CTA up front
-constexpr int kMaxSmem = 256 * kTabStride + kRedBytes;
 constexpr int kMaxItems = 4;
-// Launches with at least this many bytes of codes run 16 warps per SM (4-bit
-// batch 1: as two CTAs): their main loop needs them to keep enough loads in
-// flight.  Smaller launches run 8 warps per SM, leaving the other half of the
-// SM to the next launch.  Warm-up ranges of this size or more are not
-// prefetched.
-#ifndef LOGQ_GEMV_SPLIT_BYTES
-#define LOGQ_GEMV_SPLIT_BYTES (20 << 20)
-#endif
-constexpr int64_t kSplitBytes = LOGQ_GEMV_SPLIT_BYTES;
-// Batch-1 4-bit launches below this many bytes of codes take 16 k per lane
-// (twice the spans, half the activations per lane): their few rows per warp
-// finish sooner after the activations arrive.
-#ifndef LOGQ_GEMV_TINY_BYTES
-#define LOGQ_GEMV_TINY_BYTES (4 << 20)
-#endif
-constexpr int64_t kTinyBytes = LOGQ_GEMV_TINY_BYTES;
-// Tiny batch-1 4-bit launches: CTAs per SM, and whether they prefetch their
-// own code rows into L2 (one CTA per SM with the prefetch measured best on the
-// 1B decode step; every other batch-1 4-bit launch runs two per SM without it).
-#ifndef LOGQ_GEMV_TINY_PER_SM
-#define LOGQ_GEMV_TINY_PER_SM 1
-#endif
-constexpr int kTinyPerSm = LOGQ_GEMV_TINY_PER_SM;
-#ifndef LOGQ_GEMV_TINY_OWN_PF
-#define LOGQ_GEMV_TINY_OWN_PF 1
-#endif
-// Shared-memory carveout of the batch-1/2 decode kernels, in percent of the
-// maximum: 58 % is 132 KiB, room for two CTAs of 64 KiB (plus their reserved
-// 1 KiB).  The rest of the 256 KiB per SM is L1, which also holds the data of
-// the code loads in flight, so a larger carveout slows the kernel down; one
-// setting for all of them spares the SMs a reconfiguration between launches.
-// Batches of 4 and more (two CTAs of up to 97 KiB) take the largest one.
-#ifndef LOGQ_GEMV_CARVEOUT
-#define LOGQ_GEMV_CARVEOUT 58
-#endif
+// Batches from kPartBatch up may share a row range among kMaxParts CTAs (each a
+// part of K): a CTA that takes several passes over K reads all of X, at batch 16
+// and K = 14336 458 KB against 190 KB of codes.  4096 x 14336 at batch 16 19.8 us
+// instead of 23.3, at batch 32 35.5 instead of 40.4; the partial sums need workspace.
+constexpr int64_t kPartBatch = 9, kMaxParts = 8;
+// Warm-up ranges of this size or more are not prefetched: a launch's end waits for
+// the prefetches it issued, and in a chain of launches that costs more than the
+// next one gains (a Llama-3.1-8B step of 128 launches: 981 us with 4 MiB, 990
+// with 20 MiB).
+constexpr int64_t kPrefetchBytes = 4 << 20;
 
 // One matrix of a grouped launch: all items share X, K, B and the code width.
 struct GemvItem {
     const uint8_t* codes;
     void* Y;
+    float* part;          // kparts > 1: partial sums [kparts][B][N] (caller's workspace)
     int32_t N;
     int32_t cta_begin;    // first CTA of this item
-    int32_t cta_count;    // CTAs assigned to it
-    int32_t rows_q;       // N / cta_count
-    int32_t rows_rem;     // N % cta_count (the first rows_rem CTAs take one more row)
-    int32_t _pad;
+    int32_t rows_q;       // rows per row range of this item
+    int32_t rows_rem;     // its first rows_rem row ranges take one more row
     uint32_t lvl16[16];   // code-indexed 16-bit levels (low half used)
 };
 
 struct GemvParams {
-    GemvItem item[kMaxItems];
     int32_t nitems;
     int32_t K;
     int32_t B;
     int32_t y_dtype;
     const uint16_t* X;
     uint32_t* err;        // workspace error word
-    int64_t row_bytes;
-    int32_t spans;        // S: spans of 32*KW k covering K
-    int32_t groups;       // G: warps sharing one span (row-parallel)
+    int32_t row_bytes;
+    int32_t blocks;       // blocks of a row
+    int32_t spans;        // spans of S J blocks covering K
+    int32_t kparts;       // CTAs that share a row range, each with part_spans of the spans
+    int32_t part_spans;
+    int32_t lg_groups;    // log2 of G, the warps sharing one span (row-parallel)
     int32_t span_cols;    // warps / G: spans in flight at once
     int32_t chunk_rows;   // rows reduced per shared-memory pass
+    int32_t pitch;        // floats from one set of partial sums to the next
+    int32_t _pad;
     const uint8_t* pf;    // optional L2 warm-up range (e.g. the next layer's codes)
     int64_t pf_bytes;
     int64_t pf_share;     // bytes of that range per CTA (multiple of 16)
-    int32_t own_pf;       // prefetch the CTA's own code rows into L2 at start
-    int32_t _pad;
+    GemvItem item[kMaxItems];
 };
 
 // 8-bit codes: their 256 code-indexed levels per matrix travel as a second
@@ -146,103 +127,77 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
     return r;
 }
 
-// Table entry at byte offset off from the table base.
+// Table entry at byte offset off from the table base.  Not volatile, so that
+// lookups move freely around the multiply-adds: what keeps them behind the
+// table's barrier is that every offset is made from a value defined after it.
 __device__ __forceinline__ uint32_t lds_tab(uint32_t off)
 {
     uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(off), "n"(kTabOff));
+    asm("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(off), "n"(kTabOff));
     return v;
 }
 
-template <int NW>
-struct CodeVec { uint32_t w[NW]; };
-
-template <int NW>
-__device__ __forceinline__ CodeVec<NW> ld_codes(const uint8_t* p)
+// A block is the k that four lanes hold, each its own run: 32 k (12 or 16 bytes of
+// codes), at 8 bits 16 k.
+__host__ __device__ constexpr int lane_k(int bits) { return bits == 8 ? 16 : 32; }
+__host__ __device__ constexpr int lane_words(int bits) { return bits == 3 ? 3 : 4; }
+// Batch rows that the 8 NTL columns hold beside S segments.
+__host__ __device__ constexpr int batch_cols(int S, int NTL) { return 8 * NTL / S; }
+// Accumulator chains per column tile: their length, and how many interleave
+// (registers allow fewer for more tiles).
+__host__ __device__ constexpr int chain_length(int NTL) { return NTL == 1 ? 1 : 2; }
+__host__ __device__ constexpr int chains_for(int bits, int S, int NTL)
 {
-    CodeVec<NW> c;
+    return NTL == 1 ? (bits == 4 && S <= 2 ? 4 : 8) : NTL == 2 ? 2 : 1;
+}
+constexpr int kMaxSmem = 226 * 1024;
+// Shared memory of partial sums after a table of tab bytes, per_sm CTAs on an SM.
+constexpr int64_t red_bytes(size_t tab, int per_sm) { return (int64_t)227 * 1024 / per_sm - 1024 - (int64_t)tab; }
+// Shared-memory carveout of the batch-1/2 kernels, in percent of the maximum:
+// 58 % is 132 KiB, room for two CTAs of 64 KiB (plus their reserved 1 KiB).
+// The rest of the 256 KiB per SM is L1, which also holds the data of the code
+// loads in flight; one setting for all of them spares the SMs a
+// reconfiguration between launches.
+constexpr int kCarveout = 58;
+
+// A lane's codes of a block: 16 bytes, or (3-bit) the three words of a 12-byte
+// group.  ALLOC: through L1 as usual; else without an L1 line.
+template <bool ALLOC, int NW>
+__device__ __forceinline__ void ld_codes(uint32_t (&w)[NW], const uint8_t* p)
+{
     if constexpr (NW == 4) {
-        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                     : "=r"(c.w[0]), "=r"(c.w[1]), "=r"(c.w[2]), "=r"(c.w[3]) : "l"(p));
-    } else if constexpr (NW == 2) {
-        asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];"
-                     : "=r"(c.w[0]), "=r"(c.w[1]) : "l"(p));
+        if constexpr (ALLOC)
+            asm volatile("ld.global.nc.v4.b32 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p));
+        else
+            asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "l"(p));
     } else {
 #pragma unroll
         for (int i = 0; i < NW; ++i)
-            asm volatile("ld.global.nc.L1::no_allocate.u32 %0, [%1];" : "=r"(c.w[i]) : "l"(p + 4 * i));
+            asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(w[i]) : "l"(p + 4 * i));
     }
-    return c;
 }
 
+// D (16 x 8, fp32) += A (16 x 16) * B (16 x 8): lane l = 4 g + t holds
+//   a0, a1: rows g, g + 8 at the first k pair of t; a2, a3: at the second one;
+//   b0, b1: column g at the first / second k pair of t;
+//   d0, d1: row g, columns 2t, 2t + 1; d2, d3: row g + 8.
 template <bool F16>
-__device__ __forceinline__ void fma_pair(float& a0, float& a1, uint32_t w, uint32_t x)
+__device__ __forceinline__ void mma(float (&d)[4], bool zero, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                    uint32_t b0, uint32_t b1)
 {
-    if constexpr (F16) {
-        asm("{.reg .b16 wl, wh, xl, xh;\n\t"
-            "mov.b32 {wl, wh}, %2;\n\t"
-            "mov.b32 {xl, xh}, %3;\n\t"
-            "fma.rn.f32.f16 %0, wl, xl, %0;\n\t"
-            "fma.rn.f32.f16 %1, wh, xh, %1;}"
-            : "+f"(a0), "+f"(a1) : "r"(w), "r"(x));
-    } else {
-        asm("{.reg .b16 wl, wh, xl, xh;\n\t"
-            "mov.b32 {wl, wh}, %2;\n\t"
-            "mov.b32 {xl, xh}, %3;\n\t"
-            "fma.rn.f32.bf16 %0, wl, xl, %0;\n\t"
-            "fma.rn.f32.bf16 %1, wh, xh, %1;}"
-            : "+f"(a0), "+f"(a1) : "r"(w), "r"(x));
-    }
-}
-
-// 8-bit: two looked-up entries (each holding its 16-bit value in both halves)
-// times one activation pair.
-template <bool F16>
-__device__ __forceinline__ void fma_two(float& a0, float& a1, uint32_t w0, uint32_t w1, uint32_t x)
-{
-    if constexpr (F16) {
-        asm("{.reg .b16 al, ah, bl, bh, xl, xh;\n\t"
-            "mov.b32 {al, ah}, %2;\n\t"
-            "mov.b32 {bl, bh}, %3;\n\t"
-            "mov.b32 {xl, xh}, %4;\n\t"
-            "fma.rn.f32.f16 %0, al, xl, %0;\n\t"
-            "fma.rn.f32.f16 %1, bl, xh, %1;}"
-            : "+f"(a0), "+f"(a1) : "r"(w0), "r"(w1), "r"(x));
-    } else {
-        asm("{.reg .b16 al, ah, bl, bh, xl, xh;\n\t"
-            "mov.b32 {al, ah}, %2;\n\t"
-            "mov.b32 {bl, bh}, %3;\n\t"
-            "mov.b32 {xl, xh}, %4;\n\t"
-            "fma.rn.f32.bf16 %0, al, xl, %0;\n\t"
-            "fma.rn.f32.bf16 %1, bl, xh, %1;}"
-            : "+f"(a0), "+f"(a1) : "r"(w0), "r"(w1), "r"(x));
-    }
-}
-
-// Reduce V per-lane values over the 32 lanes; afterwards lane l holds the
-// total of value index (l >> (5 - log2 V)) in a[0] (V <= 32, power of two).
-template <int V>
-__device__ __forceinline__ void reduce_scatter(float (&a)[V], int lane)
-{
-    int count = V;
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) {
-        if (count > 1) {
-            const int half = count / 2;
-            const bool upper = (lane & m) != 0;
-#pragma unroll
-            for (int i = 0; i < V / 2; ++i) {
-                if (i < half) {
-                    const float send = upper ? a[i] : a[i + half];
-                    const float keep = upper ? a[i + half] : a[i];
-                    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
-                }
-            }
-            count = half;
-        } else {
-            a[0] += __shfl_xor_sync(0xffffffffu, a[0], m);
-        }
-    }
+    const float c0 = zero ? 0.f : d[0], c1 = zero ? 0.f : d[1], c2 = zero ? 0.f : d[2], c3 = zero ? 0.f : d[3];
+    if constexpr (F16)
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+            "{%10,%11,%12,%13};"
+            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
+    else
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+            "{%10,%11,%12,%13};"
+            : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+            : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2), "f"(c3));
 }
 
 __device__ __forceinline__ void store_y(void* Y, int dtype, int64_t idx, float v)
@@ -256,90 +211,57 @@ __device__ __forceinline__ void store_y(void* Y, int dtype, int64_t idx, float v
     }
 }
 
-// Table offsets of the four pair entries of one 4-bit code word: base_lane
-// holds 4 * lane in byte 0 and zeros above, so one byte permute yields
-// byte * 256 + 4 * lane.
-__device__ __forceinline__ void addrs4(uint32_t c, uint32_t base_lane, uint32_t (&o)[4])
+// Value pairs 2q and 2q + 1 (k = 4q .. 4q + 3 of the lane's run) from the pair
+// table.  base_lane holds 4 * lane in byte 0 and zeros above, so one byte
+// permute yields the entry's offset byte * 256 + 4 * lane.
+template <int BITS, int NW>
+__device__ __forceinline__ void pairs_of(const uint32_t (&w)[NW], int q, uint32_t base_lane, uint32_t& p0, uint32_t& p1)
 {
-    o[0] = prmt(c, base_lane, 0x7604u);
-    o[1] = prmt(c, base_lane, 0x7614u);
-    o[2] = prmt(c, base_lane, 0x7624u);
-    o[3] = prmt(c, base_lane, 0x7634u);
-}
-
-// Table offsets of the 16 pair entries of one 3-bit group (W0, W1, W2); the
-// 6-bit field lands in bits 8-13, base_lane supplies 4 * lane.
-__device__ __forceinline__ void addrs3(const uint32_t (&w)[3], uint32_t base_lane, uint32_t (&o)[16])
-{
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        o[5 * i + 0] = ((w[i] << 8) & 0x3f00u) | base_lane;
-        o[5 * i + 1] = ((w[i] << 2) & 0x3f00u) | base_lane;
-        o[5 * i + 2] = ((w[i] >> 4) & 0x3f00u) | base_lane;
-        o[5 * i + 3] = ((w[i] >> 10) & 0x3f00u) | base_lane;
-        o[5 * i + 4] = ((w[i] >> 16) & 0x3f00u) | base_lane;
-    }
-    o[15] = ((w[0] >> 22) & 0x0300u) | ((w[1] >> 20) & 0x0c00u) | ((w[2] >> 18) & 0x3000u) | base_lane;
-}
-
-// Decode one row's codes of this lane and accumulate B dot-product partials.
-template <int BITS, int B, int NW, bool F16, int NPAIR>
-__device__ __forceinline__ void decode_row(const CodeVec<NW>& c, uint32_t base_lane,
-                                           const uint32_t (&xr)[B][NPAIR], float* acc, float* acc_hi)
-{
-    if constexpr (BITS == 8) {
-        // word wi holds the codes of k = 4 wi .. 4 wi + 3, one per byte
-#pragma unroll
-        for (int wi = 0; wi < NW; ++wi) {
-            uint32_t o[4];
-            addrs4(c.w[wi], base_lane, o);
-            const uint32_t v0 = lds_tab(o[0]), v1 = lds_tab(o[1]), v2 = lds_tab(o[2]), v3 = lds_tab(o[3]);
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                fma_two<F16>(acc[b], acc_hi[b], v0, v1, xr[b][2 * wi]);
-                fma_two<F16>(acc[b], acc_hi[b], v2, v3, xr[b][2 * wi + 1]);
-            }
-        }
-    } else if constexpr (BITS == 4) {
-#pragma unroll
-        for (int wi = 0; wi < NW; ++wi) {
-            uint32_t o[4];
-            addrs4(c.w[wi], base_lane, o);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t wp = lds_tab(o[j]);
-#pragma unroll
-                for (int b = 0; b < B; ++b) fma_pair<F16>(acc[b], acc_hi[b], wp, xr[b][4 * wi + j]);
-            }
-        }
+    if constexpr (BITS == 4) {
+        const uint32_t c = w[q >> 1];
+        p0 = lds_tab(prmt(c, base_lane, (q & 1) ? 0x7624u : 0x7604u));
+        p1 = lds_tab(prmt(c, base_lane, (q & 1) ? 0x7634u : 0x7614u));
+    } else if constexpr (BITS == 8) {
+        // entry e holds the value of code e in both halves
+        const uint32_t c = w[q];
+        const uint32_t v0 = lds_tab(prmt(c, base_lane, 0x7604u)), v1 = lds_tab(prmt(c, base_lane, 0x7614u));
+        const uint32_t v2 = lds_tab(prmt(c, base_lane, 0x7624u)), v3 = lds_tab(prmt(c, base_lane, 0x7634u));
+        p0 = prmt(v0, v1, 0x5410u);
+        p1 = prmt(v2, v3, 0x5410u);
     } else {
-#pragma unroll
-        for (int gi = 0; gi < NW / 3; ++gi) {
-            uint32_t o[16];
-            const uint32_t w3[3] = {c.w[3 * gi], c.w[3 * gi + 1], c.w[3 * gi + 2]};
-            addrs3(w3, base_lane, o);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const uint32_t wp = lds_tab(o[j]);
-#pragma unroll
-                for (int b = 0; b < B; ++b) fma_pair<F16>(acc[b], acc_hi[b], wp, xr[b][16 * gi + j]);
-            }
-        }
+        // of a group of 32 k: pair i < 15 is the 6-bit field i % 5 of word i / 5; pair 15 the words' top bits
+        auto off = [&](int i) -> uint32_t {
+            const int w0 = 3 * (i / 16);
+            i %= 16;
+            if (i == 15)
+                return ((w[w0] >> 22) & 0x0300u) | ((w[w0 + 1] >> 20) & 0x0c00u) | ((w[w0 + 2] >> 18) & 0x3000u) | base_lane;
+            const uint32_t x = w[w0 + i / 5];
+            const int f = i % 5;
+            const uint32_t v = f == 0 ? (x << 8) : f == 1 ? (x << 2) : f == 2 ? (x >> 4) : f == 3 ? (x >> 10) : (x >> 16);
+            return (v & 0x3f00u) | base_lane;
+        };
+        p0 = lds_tab(off(2 * q));
+        p1 = lds_tab(off(2 * q + 1));
     }
 }
 
-template <int BITS, int B, int KW, int R, bool F16, int NT, int MINB = 512 / NT>
+// S segments of J blocks per span, NTL column tiles, T tiles of 16 / S rows in flight.
+template <int BITS, int S, int J, int NTL, int T, bool F16, int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ GemvParams p,
-                                                            const __grid_constant__ LevelsT<BITS> lv)
+                                                        const __grid_constant__ LevelsT<BITS> lv)
 {
     extern __shared__ __align__(16) uint8_t smem[];
-    constexpr int NPAIR = KW / 2;                            // bf16 pairs of x per lane and batch row
-    constexpr int NW = (BITS == 8) ? KW / 4 : (BITS == 4) ? KW / 8 : 3 * KW / 32;   // code words per lane and row
+    constexpr bool HALVES = S >= 4;                          // a row's segments are split over the MMA's two row halves
+    constexpr int HS = HALVES ? S / 2 : S;                   // segments per row half
+    constexpr int RT = 16 / S, RH = HALVES ? 0 : 8 / S;      // rows per tile; rows from the first half to the second
+    constexpr int BC = batch_cols(S, NTL), CB = 8 / S;       // batch rows; batch rows per column tile
+    constexpr int NW = lane_words(BITS), BB = 16 * NW;       // words of a lane's codes; code bytes of a block
     constexpr int NENT = (BITS == 3) ? 64 : 256;
     constexpr uint32_t TAB_BYTES = NENT * kTabStride;
-    constexpr int V = R * B;
-    constexpr int SPAN = 32 * KW;
-    static_assert(V <= 32 && (V & (V - 1)) == 0, "values per lane must be a power of two <= 32");
+    constexpr int LK = lane_k(BITS), BK = 4 * LK, BQ = LK / 4;    // k of a lane's run and of a block; multiply-adds per block
+    constexpr int NQ = J * BQ;                               // multiply-adds per tile and column tile
+    constexpr int CL = chain_length(NTL), CHAINS = chains_for(BITS, S, NTL), NCH = CHAINS * CL <= NQ ? CHAINS : NQ / CL;
+    static_assert(NQ % (NCH * CL) == 0, "whole groups of chains");
 
     // programmatic dependent launch: the next kernel on the stream may start
     // now.  Its CTAs may run beside this one and do their own prologue
@@ -357,259 +279,273 @@ __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ 
     for (int i = 1; i < kMaxItems; ++i)
         if (i < p.nitems && (int)blockIdx.x >= p.item[i].cta_begin) m = i;
     const GemvItem& item = p.item[m];
-    const int c = (int)blockIdx.x - item.cta_begin;
-    const int64_t r0 = (int64_t)c * item.rows_q + (c < item.rows_rem ? c : item.rows_rem);
-    const int64_t r1 = r0 + item.rows_q + (c < item.rows_rem ? 1 : 0);
+    uint32_t* const lvl = reinterpret_cast<uint32_t*>(smem + kLvlOff);
+    if constexpr (BITS != 8)
+        if (tid < 16) lvl[tid] = item.lvl16[tid];
+    const int cta = (int)blockIdx.x - item.cta_begin;
+    const int c = p.kparts == 1 ? cta : cta / p.kparts, kpart = cta - c * p.kparts;
+    const int s0 = kpart * p.part_spans, s1 = s0 + p.part_spans < p.spans ? s0 + p.part_spans : p.spans;
+    const int r0 = c * item.rows_q + (c < item.rows_rem ? c : item.rows_rem);
+    const int r1 = r0 + item.rows_q + (c < item.rows_rem ? 1 : 0);
 
-    // 0) the first round of code loads of this warp's first (chunk, span) goes
-    //    out first: its latency hides behind the prologue below.  Codes are
-    //    weights, not the previous kernel's output (see the launch contract).
-    const int G = p.groups, SC = p.span_cols;
-    const bool compute_warp = warp < G * SC;
-    const int g = warp % G, scol = warp / G;
-    const int64_t rstride = (int64_t)G * p.row_bytes;
-    CodeVec<NW> ca[R], cb[R];
-    auto span_first = [&](int64_t q0, int s, int& k0, bool& active) -> const uint8_t* {
-        k0 = s * SPAN + lane * KW;
-        active = k0 < p.K;
-        // idle lanes read the row start (valid memory) and multiply by zero
-        const int64_t lane_byte =
-            active ? ((BITS == 8) ? (int64_t)k0 : (BITS == 4) ? (int64_t)k0 / 2 : (int64_t)k0 / 32 * 12) : 0;
-        return item.codes + (q0 + g) * p.row_bytes + lane_byte;
-    };
-    // codes of the round whose first row is at rp, here = rows left from it
-    auto load_round = [&](CodeVec<NW> (&c)[R], const uint8_t* rp, int here) {
-        if (here >= R) {
+    // Lane 4 gq + t4 holds k LK t4 .. LK t4 + LK - 1 of a block.  As a holder of
+    // activations: column gq of each column tile; column tile nt holds batch rows
+    // nt 8 / S .. and for each its S segments.  As a holder of weights: the MMA's
+    // rows gq (h = 0) and gq + 8 (h = 1), each a row of the tile and one segment.
+    //   S = 8, 4: row gq / HS of the tile, segment h HS + gq % HS; columns 2 i and
+    //     2 i + 1 hold batch row i / HS, segments i % HS and HS + i % HS.  A row's
+    //     products then stand in d0 (h = 0) and d3 (h = 1) of the lanes with
+    //     t4 % HS == gq % HS, batch row t4 / HS.
+    //   S = 2, 1: row gq / S + h 8 / S, segment gq % S; column n holds batch row
+    //     n / S, segment n % S.  S = 2: d0 or d1 (d2 or d3), by the segment.
+    const int gq = lane >> 2, t4 = lane & 3;
+    const int rl = gq / HS, aseg = gq % HS;
+    const int bseg = HALVES ? (gq & 1) * HS + (gq >> 1) % HS : gq % S;
+    const int bcol = HALVES ? (gq >> 1) / HS : gq / S;
+    const int G = 1 << p.lg_groups, SC = p.span_cols;
+    const int g = warp & (G - 1), scol = warp >> p.lg_groups;
+    const bool compute_warp = scol < SC && s0 + scol < s1;
+    struct Tile { uint32_t w[2][J][NW]; };
+    Tile ct[T];
+    // The span being worked on: address of this lane's codes in row q0.  Blocks
+    // past K read the row's first block and are taken as 0.
+    struct Span { const uint8_t* codes; int off[2][J]; bool ragged; };
+    auto block_of = [&](int s, int h, int j) { return (s * J + j) * S + (HALVES ? h * HS : 0) + aseg; };
+    auto span_at = [&](int q0, int s) -> Span {
+        Span sp;
+        sp.codes = item.codes + (int64_t)(q0 + rl) * p.row_bytes + t4 * (4 * NW);
+        sp.ragged = (s + 1) * (S * J) > p.blocks;
 #pragma unroll
-            for (int r = 0; r < R; ++r) c[r] = ld_codes<NW>(rp + r * rstride);
-        } else {
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int r = 0; r < R; ++r)
-                if (r < here) c[r] = ld_codes<NW>(rp + r * rstride);
-        }
-    };
-    bool preloaded = false;                     // ca holds the first round of the first (chunk, span)
-    {
-        const int nrows0 = (int)((r0 + p.chunk_rows < r1 ? r0 + p.chunk_rows : r1) - r0);
-        const int my_rows0 = (nrows0 > g) ? (nrows0 - g + G - 1) / G : 0;
-        if (compute_warp && my_rows0 > 0 && scol < p.spans) {
-            int k0;
-            bool active;
-            load_round(ca, span_first(r0, scol, k0, active), my_rows0);
-            preloaded = true;
-        }
-    }
-
-    // 1) start streaming this CTA's code rows into L2, and its share of the
-    //    optional warm-up range.
-    {
-        constexpr int64_t piece = 16384;
-        const uint8_t* base = item.codes + r0 * p.row_bytes;
-        int64_t bytes = p.own_pf ? (r1 - r0) * p.row_bytes : 0;
-        if (bytes > kPrefetchCap) bytes = kPrefetchCap;
-        for (int64_t off = (int64_t)tid * piece; off < bytes; off += (int64_t)NT * piece) {
-            const int64_t n = (bytes - off) < piece ? (bytes - off) : piece;
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(base + off), "r"((uint32_t)n)
-                         : "memory");
-        }
-        if (p.pf_bytes > 0) {
-            const int64_t beg = p.pf_share * blockIdx.x;
-            const int64_t end = (beg + p.pf_share < p.pf_bytes) ? beg + p.pf_share : p.pf_bytes;
-            for (int64_t off = beg + (int64_t)tid * piece; off < end; off += (int64_t)NT * piece) {
-                const int64_t n = (end - off) < piece ? (end - off) : piece;
-                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.pf + off), "r"((uint32_t)n)
-                             : "memory");
+            for (int j = 0; j < J; ++j) {
+                const int kb = block_of(s, h, j);
+                sp.off[h][j] = kb < p.blocks ? kb * BB : 0;
             }
+        return sp;
+    };
+    // codes of the tile at local row lt; rows past the chunk's nrows read its last row
+    auto load_tile = [&](Tile& c, const Span& sp, int lt, int nrows) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int last = nrows - 1 - rl, r = lt + h * RH < last ? lt + h * RH : last;
+            const uint8_t* rp = sp.codes + (int64_t)r * p.row_bytes;
+#pragma unroll
+            for (int j = 0; j < J; ++j) ld_codes<S == 1, NW>(c.w[h][j], rp + sp.off[h][j]);
+        }
+    };
+    // 0) the first T tiles' codes of this warp's first (chunk, span) go out first:
+    //    their latency hides behind the prologue below.  Codes are weights, not
+    //    the previous kernel's output (see the launch contract).
+    auto load_first = [&](const Span& sp, int nrows) {
+#pragma unroll
+        for (int u = 0; u < T; ++u)
+            if ((u * G + g) * RT < nrows) load_tile(ct[u], sp, (u * G + g) * RT, nrows);
+    };
+    auto chunk_of = [&](int q0) { return r1 - q0 > p.chunk_rows ? p.chunk_rows : r1 - q0; };
+    int nrows = chunk_of(r0);
+    Span sp = span_at(r0, s0 + scol);
+    if (compute_warp) load_first(sp, nrows);
+
+    // 1) its share of the optional warm-up range
+    if (p.pf_bytes > 0) {
+        constexpr int64_t piece = 16384;
+        const int64_t beg = p.pf_share * blockIdx.x;
+        const int64_t end = (beg + p.pf_share < p.pf_bytes) ? beg + p.pf_share : p.pf_bytes;
+        for (int64_t off = beg + (int64_t)tid * piece; off < end; off += (int64_t)NT * piece) {
+            const int64_t n = (end - off) < piece ? (end - off) : piece;
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.pf + off), "r"((uint32_t)n)
+                         : "memory");
         }
     }
 
     // 2) pair table: entry e = (value of its low code) | (value of its high
     //    code) << 16, 32 copies (one per lane) in the first 128 bytes of its
     //    256-byte row.  The 16 levels are staged in the free half of row 0
-    //    (indexed parameter reads with per-thread indices would serialise).
+    //    (indexed parameter reads with per-thread indices would serialise); a
+    //    warp makes 32 entries, one per lane, and writes four rows at a time.
     //    8-bit codes: entry e is the value of code e in both halves.
-    if constexpr (BITS == 8) {
-        for (int i = tid; i < NENT * 8; i += NT) {
-            const int e = i >> 3, part = i & 7;
-            const uint32_t v = (uint32_t)lv.v[m][e] * 0x10001u;
-            reinterpret_cast<uint4*>(smem + e * kTabStride)[part] = make_uint4(v, v, v, v);
-        }
-    } else {
-        uint32_t* lvl = reinterpret_cast<uint32_t*>(smem + kLvlOff);
-        if (tid < 16) lvl[tid] = item.lvl16[tid] & 0xffffu;
-        __syncthreads();
-        for (int i = tid; i < NENT * 8; i += NT) {
-            const int e = i >> 3, part = i & 7;
-            const uint32_t lo = (BITS == 4) ? (e & 15) : (e & 7);
-            const uint32_t hi = (BITS == 4) ? (e >> 4) : (e >> 3);
-            const uint32_t v = lvl[lo] | (lvl[hi] << 16);
-            reinterpret_cast<uint4*>(smem + e * kTabStride)[part] = make_uint4(v, v, v, v);
+    if constexpr (BITS != 8) __syncthreads();
+#pragma unroll
+    for (int e0 = 32 * warp; e0 < NENT; e0 += NT) {
+        const int e = e0 + lane;
+        uint32_t v;
+        if constexpr (BITS == 8) v = (uint32_t)lv.v[m][e] * 0x10001u;
+        else v = lvl[BITS == 4 ? (e & 15) : (e & 7)] | (lvl[BITS == 4 ? (e >> 4) : (e >> 3)] << 16);
+        uint8_t* at = smem + (e0 + (lane >> 3)) * kTabStride + (lane & 7) * 16;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t x = __shfl_sync(0xffffffffu, v, 4 * i + (lane >> 3));
+            *reinterpret_cast<uint4*>(at + 4 * i * kTabStride) = make_uint4(x, x, x, x);
         }
     }
-    // span partial i (in the free half of table row i / 32, or after the table)
-    auto red = [&](int i) -> float& {
-        if constexpr (red_in_table(BITS, B))
-            return *reinterpret_cast<float*>(smem + (i >> 5) * kTabStride + 128 + (i & 31) * 4);
-        else
-            return reinterpret_cast<float*>(smem + TAB_BYTES)[i];
-    };
+    // this lane's partial sums: set (scol, segment) of np, first batch row, row rl
+    float* const red0 = reinterpret_cast<float*>(smem + TAB_BYTES);
+    const bool holder = !HALVES || t4 % HS == aseg;
+    float* const red = red0 + (scol * HS + aseg) * p.pitch + rl * BC + (HALVES ? t4 / HS : S == 2 ? t4 : 2 * t4);
+    const uint16_t* const xl = p.X + LK * t4;
     __syncthreads();
 
-    const uint32_t base_lane = 4u * (uint32_t)lane;
-    constexpr int lg2V = (V >= 32) ? 5 : (V >= 16) ? 4 : (V >= 8) ? 3 : (V >= 4) ? 2 : (V >= 2) ? 1 : 0;
-    const int my_v = lane >> (5 - lg2V);
-    const bool writer = (lane & ((32 >> lg2V) - 1)) == 0;
-
-    for (int64_t q0 = r0; q0 < r1; q0 += p.chunk_rows) {
-        const int64_t q1 = (q0 + p.chunk_rows < r1) ? q0 + p.chunk_rows : r1;
-        const int nrows = (int)(q1 - q0);
-        const int my_rows = (nrows > g) ? (nrows - g + G - 1) / G : 0;
-        if (compute_warp && my_rows > 0) {
-            for (int s = scol; s < p.spans; s += SC) {
-                int k0;
-                bool active;
-                const uint8_t* first = span_first(q0, s, k0, active);
-                // Rounds of R rows with two code buffers: the loads of round t+1 are
-                // in flight while round t is decoded.  Full rounds run unguarded;
-                // the last round guards its rows (warp-uniform branches).
-                if (!preloaded) load_round(ca, first, my_rows);
-                preloaded = false;
-                asm volatile("griddepcontrol.wait;" ::: "memory");
-                // activations for this span stay in registers (zero on idle lanes)
-                uint32_t xr[B][NPAIR];
+    uint32_t base_lane = 4u * (uint32_t)lane;
+    asm volatile("" : "+r"(base_lane)::"memory");    // lookups stay behind the barrier
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int q0 = r0;;) {
+        if (compute_warp) {
+            for (int s = s0 + scol;;) {
+                // activations of this span stay in registers (zero outside K and the batch)
+                uint32_t xr[NTL][J][LK / 2];
 #pragma unroll
-                for (int b = 0; b < B; ++b) {
-                    const uint16_t* xp = p.X + (int64_t)b * p.K + (active ? k0 : 0);
+                for (int nt = 0; nt < NTL; ++nt) {
+                    const int b = nt * CB + bcol;
 #pragma unroll
-                    for (int i = 0; i < NPAIR; i += 4) {
-                        uint4 v = make_uint4(0, 0, 0, 0);
-                        if (active && b < p.B) v = *reinterpret_cast<const uint4*>(xp + 2 * i);
-                        xr[b][i] = v.x;
-                        if (i + 1 < NPAIR) xr[b][i + 1] = v.y;
-                        if (i + 2 < NPAIR) xr[b][i + 2] = v.z;
-                        if (i + 3 < NPAIR) xr[b][i + 3] = v.w;
+                    for (int j = 0; j < J; ++j) {
+                        const int kb = (s * J + j) * S + bseg;
+                        const uint16_t* xp = xl + (int64_t)b * p.K + (int64_t)kb * BK;
+                        const bool on = kb < p.blocks && b < p.B;
+#pragma unroll
+                        for (int i = 0; i < LK / 2; i += 4) {
+                            uint4 v = make_uint4(0, 0, 0, 0);
+                            if (on) v = *reinterpret_cast<const uint4*>(xp + 2 * i);
+                            xr[nt][j][i] = v.x;
+                            xr[nt][j][i + 1] = v.y;
+                            xr[nt][j][i + 2] = v.z;
+                            xr[nt][j][i + 3] = v.w;
+                        }
                     }
                 }
-                // the writer lane's result of each round: row my_v / B, batch
-                // row my_v % B; its local row and partial-buffer index advance
-                // by constants
-                int lr_w = g + G * (my_v / B);
-                int red_i = (s * p.chunk_rows + lr_w) * B + my_v % B;
-                auto run_round = [&](const CodeVec<NW> (&c)[R], int here) {
-                    float acc[V], acc_hi[V];
+                // one tile; a row's result for a batch row is added over this warp's spans
+                // in its shared-memory slot
+                const bool first = s == s0 + scol;
+                auto put = [&](float& slot, float v) { slot = first ? v : slot + v; };
+                auto run_tile = [&](Tile& c, int lt) {
+                    if (sp.ragged) {
 #pragma unroll
-                    for (int i = 0; i < V; ++i) acc[i] = acc_hi[i] = 0.f;
-                    if (here >= R) {
+                        for (int h = 0; h < 2; ++h)
 #pragma unroll
-                        for (int r = 0; r < R; ++r) decode_row<BITS, B, NW, F16>(c[r], base_lane, xr, acc + r * B, acc_hi + r * B);
+                            for (int j = 0; j < J; ++j)
+                                if (block_of(s, h, j) >= p.blocks)
+#pragma unroll
+                                    for (int i = 0; i < NW; ++i) c.w[h][j][i] = 0u;
+                    }
+                    // groups of NCH interleaved chains of CL multiply-adds, chains and groups
+                    // added up pairwise with rounding to nearest (the tensor core truncates
+                    // its sums); sum[l] holds the sum of 2^l groups
+                    constexpr int NG = NQ / (NCH * CL);
+                    constexpr bool PAIR = NTL == 1 || BITS != 8;
+                    float acc[NTL][4], sum[5][NTL][4];
+                    static_assert(NG <= 32 && (NG & (NG - 1)) == 0, "pairwise over the groups");
+#pragma unroll
+                    for (int gr = 0; gr < NG; ++gr) {
+                        float d[NTL][NCH][4];
+#pragma unroll
+                        for (int qq = 0; qq < NCH * CL; ++qq) {
+                            const int q = gr * NCH * CL + qq;
+                            uint32_t a0, a1, a2, a3;
+                            pairs_of<BITS, NW>(c.w[0][q / BQ], q % BQ, base_lane, a0, a2);
+                            pairs_of<BITS, NW>(c.w[1][q / BQ], q % BQ, base_lane, a1, a3);
+#pragma unroll
+                            for (int nt = 0; nt < NTL; ++nt)
+                                mma<F16>(d[nt][qq % NCH], qq < NCH, a0, a1, a2, a3, xr[nt][q / BQ][2 * (q % BQ)],
+                                         xr[nt][q / BQ][2 * (q % BQ) + 1]);
+                        }
+#pragma unroll
+                        for (int nt = 0; nt < NTL; ++nt)
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+#pragma unroll
+                                for (int w = NCH / 2; w >= 1; w /= 2)
+#pragma unroll
+                                    for (int ch = 0; ch < w; ++ch) d[nt][ch][i] += d[nt][ch + w][i];
+                                float v = d[nt][0][i];
+                                int l = 0;
+                                if (!PAIR && gr) v += sum[0][nt][i];
+                                if (PAIR)
+#pragma unroll
+                                for (; (gr >> l) & 1; ++l) v += sum[l][nt][i];
+                                if (gr == NG - 1) acc[nt][i] = v;
+                                else sum[l][nt][i] = v;
+                            }
+                    }
+                    float* slot = red + lt * BC;
+                    if constexpr (HALVES) {
+                        if (holder && lt + rl < nrows)
+#pragma unroll
+                            for (int nt = 0; nt < NTL; ++nt) put(slot[nt * CB], acc[nt][0] + acc[nt][3]);
                     } else {
 #pragma unroll
-                        for (int r = 0; r < R; ++r)
-                            if (r < here) decode_row<BITS, B, NW, F16>(c[r], base_lane, xr, acc + r * B, acc_hi + r * B);
-                    }
+                        for (int h = 0; h < 2; ++h)
+                            if (lt + rl + h * RH < nrows)
 #pragma unroll
-                    for (int i = 0; i < V; ++i) acc[i] += acc_hi[i];
-                    reduce_scatter<V>(acc, lane);
-                    if (writer && lr_w < nrows) red(red_i) = acc[0];
-                    lr_w += G * R;
-                    red_i += G * R * B;
+                                for (int nt = 0; nt < NTL; ++nt) {
+                                    if constexpr (S == 2) {
+                                        put(slot[h * RH * BC + nt * CB], aseg ? acc[nt][2 * h + 1] : acc[nt][2 * h]);
+                                    } else {
+                                        put(slot[h * RH * BC + nt * CB], acc[nt][2 * h]);
+                                        put(slot[h * RH * BC + nt * CB + 1], acc[nt][2 * h + 1]);
+                                    }
+                                }
+                    }
                 };
-                // rounds of R rows with two code buffers: the loads of the next
-                // round are in flight while this one is decoded
-                if constexpr (R == 1) {
-                    // one-row rounds (batches of 8 and 16): a counted loop with
-                    // indices recomputed from the round number, which keeps
-                    // fewer registers live in these register-bound kernels
-                    auto load1 = [&](CodeVec<NW> (&c)[R], int t) {
-                        if (t < my_rows) c[0] = ld_codes<NW>(first + (int64_t)t * rstride);
-                    };
-                    auto run1 = [&](const CodeVec<NW> (&c)[R], int t) {
-                        float acc[V], acc_hi[V];
+                // T tiles in flight: a tile's registers are refilled as soon as it is decoded
+                for (int lt = g * RT; lt < nrows;) {
 #pragma unroll
-                        for (int i = 0; i < V; ++i) acc[i] = acc_hi[i] = 0.f;
-                        if (t < my_rows) decode_row<BITS, B, NW, F16>(c[0], base_lane, xr, acc, acc_hi);
-#pragma unroll
-                        for (int i = 0; i < V; ++i) acc[i] += acc_hi[i];
-                        reduce_scatter<V>(acc, lane);
-                        if (writer) {
-                            const int lr = g + G * t;
-                            if (lr < nrows) red((s * p.chunk_rows + lr) * B + my_v % B) = acc[0];
-                        }
-                    };
-                    const int nrounds = my_rows;
-                    for (int t = 0; t < nrounds; t += 2) {
-                        load1(cb, t + 1);
-                        run1(ca, t);
-                        if (t + 1 >= nrounds) break;
-                        load1(ca, t + 2);
-                        run1(cb, t + 1);
-                    }
-                } else {
-                    // Full rounds run without any row checks (branches and their
-                    // convergence points were a quarter of the loop's
-                    // instructions); only the last, partial round checks its rows.
-                    // ca holds round 0 (full, or the partial round itself).
-                    const int nfull = my_rows / R, tail = my_rows - nfull * R;
-                    const int64_t rstep = (int64_t)R * rstride;
-                    auto load_full = [&](CodeVec<NW> (&c)[R], const uint8_t* rp) {
-#pragma unroll
-                        for (int r = 0; r < R; ++r) c[r] = ld_codes<NW>(rp + r * rstride);
-                    };
-                    auto run_full = [&](const CodeVec<NW> (&c)[R]) {
-                        float acc[V], acc_hi[V];
-#pragma unroll
-                        for (int i = 0; i < V; ++i) acc[i] = acc_hi[i] = 0.f;
-#pragma unroll
-                        for (int r = 0; r < R; ++r)
-                            decode_row<BITS, B, NW, F16>(c[r], base_lane, xr, acc + r * B, acc_hi + r * B);
-#pragma unroll
-                        for (int i = 0; i < V; ++i) acc[i] += acc_hi[i];
-                        reduce_scatter<V>(acc, lane);
-                        if (writer) red(red_i) = acc[0];            // a full round's rows all exist
-                        lr_w += G * R;
-                        red_i += G * R * B;
-                    };
-                    const uint8_t* rp = first;
-                    int t = 0;
-                    for (; t + 2 <= nfull; t += 2) {                // rounds t (in ca) and t + 1
-                        load_full(cb, rp + rstep);
-                        run_full(ca);
-                        if (t + 2 < nfull) load_full(ca, rp + 2 * rstep);
-                        else if (tail) load_round(ca, rp + 2 * rstep, tail);
-                        run_full(cb);
-                        rp += 2 * rstep;
-                    }
-                    if (t < nfull) {                                 // one full round left, in ca
-                        if (tail) load_round(cb, rp + rstep, tail);
-                        run_full(ca);
-                        if (tail) run_round(cb, tail);
-                    } else if (tail) {
-                        run_round(ca, tail);
+                    for (int u = 0; u < T; ++u) {
+                        run_tile(ct[u], lt);
+                        if (lt + T * G * RT < nrows) load_tile(ct[u], sp, lt + T * G * RT, nrows);
+                        lt += G * RT;
+                        if (lt >= nrows) break;
                     }
                 }
+                s += SC;
+                if (s >= s1) break;
+                sp = span_at(q0, s);
+                load_first(sp, nrows);
             }
         }
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        __syncthreads();
-        // fixed-order sum over spans
-        for (int i = tid; i < nrows * B; i += NT) {
-            const int lr = i / B, b = i % B;
-            if (b >= p.B) continue;
-            float sum = 0.f;
-            for (int s = 0; s < p.spans; ++s) sum += red((s * p.chunk_rows + lr) * B + b);
-            store_y(item.Y, p.y_dtype, (int64_t)b * item.N + q0 + lr, sum);
+        const int n0 = nrows;
+        const bool more = r1 - q0 > p.chunk_rows;
+        const int q1 = more ? q0 + p.chunk_rows : r1;
+        if (more && compute_warp) {           // the next chunk's first codes are in flight during this one's sums
+            sp = span_at(q1, s0 + scol);
+            load_first(sp, chunk_of(q1));
         }
         __syncthreads();
+        // fixed-order sum of each output's partial sums
+        const int np = (SC < s1 - s0 ? SC : s1 - s0) * HS;
+        for (int i = tid; i < n0 * BC; i += NT) {
+            const int row = i / BC, b = i % BC;
+            if (b >= p.B) continue;
+            float sum = 0.f;
+            int k = 0;
+            for (; k + 8 <= np; k += 8) {
+                float v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = red0[(k + u) * p.pitch + i];
+                sum += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+            }
+            for (; k < np; ++k) sum += red0[k * p.pitch + i];
+            if (p.kparts == 1) store_y(item.Y, p.y_dtype, (int64_t)b * item.N + q0 + row, sum);
+            else item.part[((int64_t)kpart * p.B + b) * item.N + q0 + row] = sum;
+        }
+        if (!more) break;
+        __syncthreads();
+        q0 = q1;
+        nrows = chunk_of(q0);
     }
 }
 
-struct Config {
-    int bits, B, KW, R;
+// Added to a padded batch: the shape for short rows (shape_key).
+constexpr int kShort = 64;
+
+// Launch shape of a batch: S segments, J blocks, NTL column tiles,
+// T tiles in flight, threads per CTA, CTAs per SM.
+struct Shape {
+    int S, J, NTL, T, NT, MINB;
 };
 
-// Dynamic shared memory opt-in and a carveout that leaves room for two CTAs
-// per SM: per-device function attributes, set once per device.
-template <int BITS, int B, int KW, int R, bool F16, int NT, int MINB = 512 / NT>
+// Dynamic shared memory opt-in and a carveout that leaves room for the CTAs of
+// an SM: per-device function attributes, set once per device.
+template <int BITS, int S, int J, int NTL, int T, int NT, int MINB, bool F16>
 cudaError_t run(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, cudaStream_t s)
 {
     LevelsT<BITS> lv;
@@ -617,7 +553,7 @@ cudaError_t run(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, 
     if constexpr (BITS == 8)
         for (int i = 0; i < a.count; ++i)
             for (int c = 0; c < 256; ++c) lv.v[i][c] = a.item[i].lvl16[c];
-    auto k = gemv_kernel<BITS, B, KW, R, F16, NT, MINB>;
+    auto k = gemv_kernel<BITS, S, J, NTL, T, F16, NT, MINB>;
     static bool configured[64] = {false};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -627,7 +563,7 @@ cudaError_t run(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, 
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 B <= 2 ? LOGQ_GEMV_CARVEOUT : (int)cudaSharedmemCarveoutMaxShared);
+                                 batch_cols(S, NTL) <= 2 ? kCarveout : (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
@@ -644,60 +580,82 @@ cudaError_t run(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, 
     return cudaLaunchKernelEx(&cfg, k, p, lv);
 }
 
-template <bool F16>
-cudaError_t dispatch(int bits, int Bp, bool large, bool tiny, const GemvParams& p, const GroupArgs& a, int grid,
-                     size_t smem, cudaStream_t s)
+// The compiled shapes, per code width and padded batch; calls fn with the
+// shape's constants as template arguments.
+// Shape of a key (sh), and its launch when p is not NULL.  More segments
+// make a warp's loads longer runs of one row (S = 8: 256 bytes per row half),
+// fewer leave columns for the batch; J blocks per segment share a row's final sum
+// among more multiply-adds where registers hold the activations (16 per column
+// tile and block).  Each line was the fastest of the shapes tried for it on the
+// Llama-3.1-8B layer (the figures at the top); at 8 bits a block is 64 k, so J
+// doubles.
+template <int BITS, bool F16>
+cudaError_t shape_or_run(int key, Shape* sh, const GemvParams* p, const GroupArgs* a, int grid, size_t smem, cudaStream_t s)
 {
-    constexpr int L = kLargeThreads, S = kSmallThreads;
-    if (bits == 8) {
-        switch (Bp) {
-        case 1: return large ? run<8, 1, 16, 8, F16, L>(p, a, grid, smem, s) : run<8, 1, 16, 8, F16, S>(p, a, grid, smem, s);
-        case 2: return large ? run<8, 2, 16, 4, F16, L>(p, a, grid, smem, s) : run<8, 2, 16, 4, F16, S>(p, a, grid, smem, s);
-        case 4: return run<8, 4, 16, 2, F16, S>(p, a, grid, smem, s);
+#define LOGQ_SHAPE(B, S, J, NTL, T, NT, MINB) \
+    case B: \
+        *sh = Shape{S, J, NTL, T, NT, MINB}; \
+        return p ? run<BITS, S, J, NTL, T, NT, MINB, F16>(*p, *a, grid, smem, s) : cudaSuccess
+    if constexpr (BITS == 3) {
+        switch (key) {
+            LOGQ_SHAPE(1, 8, 1, 1, 6, 256, 2);
+            LOGQ_SHAPE(2, 4, 1, 1, 4, 512, 1);
+            LOGQ_SHAPE(4, 2, 2, 1, 2, 512, 1);
+            LOGQ_SHAPE(8, 1, 2, 1, 2, 512, 1);
+            LOGQ_SHAPE(16, 1, 2, 2, 1, 512, 1);
+            LOGQ_SHAPE(32, 1, 2, 4, 1, 256, 1);
         }
-    } else if (bits == 4) {
-        switch (Bp) {
-        // batch 1: 8-warp CTAs, two per SM (tiny launches: one per SM)
-        case 1:
-            return tiny ? run<4, 1, 16, 8, F16, S, kTinyPerSm>(p, a, grid, smem, s)
-                        : run<4, 1, 32, 8, F16, S, 2>(p, a, grid, smem, s);
-        case 2: return large ? run<4, 2, 32, 4, F16, L>(p, a, grid, smem, s) : run<4, 2, 32, 4, F16, S>(p, a, grid, smem, s);
-        // batch 4: large launches one 16-warp CTA per SM with 32 k per lane,
-        // small ones two 8-warp CTAs with 16 k; batch 8 one 16-warp CTA with
-        // 16 k; batch 16 one 8-warp CTA whose threads hold 16 k of all 16
-        // activation rows (251 registers)
-        case 4: return large ? run<4, 4, 32, 2, F16, L, 1>(p, a, grid, smem, s)
-                             : run<4, 4, 16, 2, F16, S>(p, a, grid, smem, s);
-        case 8: return run<4, 8, 16, 1, F16, L, 1>(p, a, grid, smem, s);
-        case 16: return run<4, 16, 16, 1, F16, S, 1>(p, a, grid, smem, s);
+    } else if constexpr (BITS == 4) {
+        switch (key) {
+            LOGQ_SHAPE(1, 8, 1, 1, 5, 256, 2);
+            LOGQ_SHAPE(2, 4, 1, 1, 4, 512, 1);
+            LOGQ_SHAPE(4, 2, 2, 1, 2, 512, 1);
+            LOGQ_SHAPE(8, 1, 2, 1, 2, 512, 1);
+            LOGQ_SHAPE(16, 1, 4, 2, 1, 256, 1);
+            LOGQ_SHAPE(32, 1, 2, 4, 1, 256, 1);
+            LOGQ_SHAPE(kShort + 1, 2, 1, 1, 5, 256, 2);
+            LOGQ_SHAPE(kShort + 2, 4, 1, 1, 4, 256, 2);
+            LOGQ_SHAPE(kShort + 4, 2, 1, 1, 5, 256, 2);
+            LOGQ_SHAPE(kShort + 8, 1, 2, 1, 3, 256, 1);
+            LOGQ_SHAPE(kShort + 16, 1, 2, 2, 2, 256, 1);
         }
     } else {
-        switch (Bp) {
-        case 1: return large ? run<3, 1, 32, 8, F16, L>(p, a, grid, smem, s) : run<3, 1, 32, 8, F16, S>(p, a, grid, smem, s);
-        case 2: return large ? run<3, 2, 32, 4, F16, L>(p, a, grid, smem, s) : run<3, 2, 32, 4, F16, S>(p, a, grid, smem, s);
-        case 4: return run<3, 4, 32, 2, F16, S>(p, a, grid, smem, s);
+        switch (key) {
+            LOGQ_SHAPE(1, 8, 2, 1, 3, 256, 2);
+            LOGQ_SHAPE(2, 4, 2, 1, 3, 512, 1);
+            LOGQ_SHAPE(4, 2, 2, 1, 3, 512, 1);
+            LOGQ_SHAPE(8, 2, 2, 2, 2, 512, 1);
+            LOGQ_SHAPE(16, 1, 4, 2, 2, 256, 1);
+            LOGQ_SHAPE(32, 1, 4, 4, 1, 256, 1);
         }
     }
+#undef LOGQ_SHAPE
     return cudaErrorInvalidValue;
 }
 
-int padded_batch(int64_t B)
+template <bool F16>
+cudaError_t shape_or_run(int bits, int key, Shape* sh, const GemvParams* p, const GroupArgs* a, int grid, size_t smem,
+                         cudaStream_t s)
 {
-    if (B <= 1) return 1;
-    if (B <= 2) return 2;
-    if (B <= 4) return 4;
-    if (B <= 8) return 8;
-    return 16;
+    return bits == 8 ? shape_or_run<8, F16>(key, sh, p, a, grid, smem, s)
+         : bits == 4 ? shape_or_run<4, F16>(key, sh, p, a, grid, smem, s)
+                     : shape_or_run<3, F16>(key, sh, p, a, grid, smem, s);
 }
 
-int kw_for(int bits, int Bp, bool tiny, bool large)
+// Key of a call's launch shape: the batch padded to a power of two, plus kShort for
+// 4-bit rows of less than 4096 k.  Those fill a CTA's warps with spans of the wide
+// shapes only by sharing each span among several warps, all of which read its
+// activations; shapes with shorter spans spare that.  2048 x 2048 / 16384 x 2048, us:
+// batch 1 2.8 -> 2.35 / (5.4, 6.1 with the short one, so only up to 8 M weights),
+// batch 2 3.1 -> 2.85 / 5.7 -> 5.6, batch 4 3.6 -> 2.8 / 7.5 -> 6.5, batch 8
+// 3.6 -> 2.7 / 8.5 -> 7.75, batch 16 4.9 -> 3.45 / 11.9 -> 9.7; 4096 x 4096 at
+// batch 16 7.5, 8.3 with the short one.
+int shape_key(int bits, int64_t B, int64_t rows, int64_t K)
 {
-    if (bits == 8) return 16;
-    if (bits == 3) return 32;
-    if (Bp == 1 && tiny) return 16;
-    if (Bp <= 2) return 32;
-    if (Bp == 4) return large ? 32 : 16;
-    return 16;
+    int key = 1;
+    while (key < B) key *= 2;
+    if (bits == 4 && K < 4096 && key <= 16 && (key > 1 || rows * K <= (int64_t)8 << 20)) key += kShort;
+    return key;
 }
 
 // The table lookups address shared memory relative to kTabOff, which is where
@@ -720,11 +678,14 @@ cudaError_t check_shared_base()
 
 }  // namespace
 
-bool gemv_supports(int bits, int64_t B)
+// Up to 16 rows always; up to 32 where the tensor-memory kernel is slower: at 3 and
+// 8 bits (Llama-3.1-8B layer at batch 32: 130 against 194 us, 144 against 179), at
+// 4 bits for matrices of up to 32 M weights in a call (4096 x 4096 13.4 against
+// 17.0 us, 6144 x 4096 17.7 against 19.8; 28672 x 4096 62 against 58.6).
+bool gemv_takes(int bits, int64_t B, int64_t rows, int64_t K)
 {
-    if (bits == 4) return B >= 1 && B <= 16;
-    if (bits == 3 || bits == 8) return B >= 1 && B <= 4;
-    return false;
+    if (bits != 3 && bits != 4 && bits != 8) return false;
+    return B >= 1 && (B <= 16 || (B <= 32 && (bits != 4 || rows <= ((int64_t)32 << 20) / K)));
 }
 
 cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
@@ -732,15 +693,12 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
     if (a.count < 1 || a.count > kMaxItems) return cudaErrorInvalidValue;
     cudaError_t e = check_shared_base();
     if (e != cudaSuccess) return e;
-    const int Bp = padded_batch(a.B);
     int64_t total_rows = 0;
     for (int i = 0; i < a.count; ++i) total_rows += a.item[i].N;
-    const int64_t row_bytes = (a.bits == 8) ? a.K : (a.bits == 4) ? a.K / 2 : a.K / 32 * 12;
-    const bool tiny = a.bits == 4 && Bp == 1 && total_rows * row_bytes < kTinyBytes;
-    // large launches: batch 1-2 (and 4-bit batch 4) with at least kSplitBytes of codes
-    const bool large = (Bp <= 2 || (a.bits == 4 && Bp == 4)) && total_rows * row_bytes >= kSplitBytes;
-    const int KW = kw_for(a.bits, Bp, tiny, large);
-    const int span = 32 * KW;
+    const int key = shape_key(a.bits, a.B, total_rows, a.K);
+    Shape sh;
+    if ((e = shape_or_run<false>(a.bits, key, &sh, nullptr, nullptr, 0, 0, s)) != cudaSuccess) return e;
+    const int64_t row_bytes = a.K / 32 * (4 * a.bits);
     GemvParams p;
     memset(&p, 0, sizeof p);
     p.nitems = a.count;
@@ -749,45 +707,45 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
     p.K = (int32_t)a.K;
     p.B = (int32_t)a.B;
     p.y_dtype = a.y_dtype;
-    p.row_bytes = row_bytes;
-    p.spans = (int32_t)((a.K + span - 1) / span);
-    // Batch 1-2: large launches one 512-thread CTA per SM, small ones one
-    // 256-thread CTA per SM.  3- and 8-bit batch 4: two 256-thread CTAs per SM;
-    // 4-bit batches of 4 and more: see dispatch() for the shapes.
-    const bool wide4 = a.bits == 4 && ((Bp == 4 && large) || Bp == 8);
-    const bool b1_4 = a.bits == 4 && Bp == 1;
-    const int threads = ((large && !b1_4) || wide4) ? kLargeThreads : kSmallThreads;
-    const int per_sm = b1_4 ? (tiny ? kTinyPerSm : 2)
-                            : (Bp >= 4 && !(a.bits == 4 && (Bp >= 8 || large))) ? 2 : 1;
-    const int warps = threads / 32;
-    if (p.spans >= warps) {
-        p.groups = 1;
-        p.span_cols = warps;
-    } else {
-        p.groups = warps / p.spans;
-        p.span_cols = p.spans;
+    p.row_bytes = (int32_t)row_bytes;
+    p.blocks = (int32_t)(a.K / (4 * lane_k(a.bits)));
+    p.spans = (p.blocks + sh.S * sh.J - 1) / (sh.S * sh.J);
+    // Batches of 9 and more read more activations than codes where a CTA takes
+    // several passes over K: with room for partial sums, several CTAs share a row
+    // range, one part of the spans each (see the note at kPartBatch).
+    const int warps = sh.NT / 32;
+    const int passes = (p.spans + warps - 1) / warps;
+    int64_t kparts = 1;
+    if (a.B >= kPartBatch) {
+        const int64_t avail = a.ws_bytes > kWorkspaceBytes ? (int64_t)(a.ws_bytes - kWorkspaceBytes) : 0;
+        kparts = avail / (4 * a.B * total_rows);
+        if (kparts > kMaxParts) kparts = kMaxParts;
+        if (kparts > passes) kparts = passes;
+        if (kparts < 1) kparts = 1;
     }
-    // Each CTA's own rows are prefetched into L2 up front only where that was
-    // measured to pay: not in 4-bit batch-1 launches (two CTAs per SM, whose
-    // code loads keep enough in flight) except tiny ones, nor in large launches.
-    p.own_pf = b1_4 ? (tiny ? LOGQ_GEMV_TINY_OWN_PF : 0) : (large ? 0 : 1);
-    // The warm-up range is prefetched only when it is below kSplitBytes: a
-    // launch that large streams its own codes at full rate, and warming L2
-    // with them slows the launch that issues the prefetch more than it helps.
-    p.pf = static_cast<const uint8_t*>(a.pf);
-    p.pf_bytes = (a.pf && a.pf_bytes < kSplitBytes) ? a.pf_bytes : 0;
-
-    // CTAs in proportion to each matrix's rows (at least one each, at most one
-    // per row).
+    p.part_spans = (int32_t)((p.spans + kparts - 1) / kparts);
+    kparts = (p.spans + p.part_spans - 1) / p.part_spans;
+    p.kparts = (int32_t)kparts;
+    while ((warps >> (p.lg_groups + 1)) >= p.part_spans) ++p.lg_groups;
+    p.span_cols = p.part_spans < (warps >> p.lg_groups) ? p.part_spans : warps >> p.lg_groups;
+    // Each matrix's rows are divided among row ranges (kparts CTAs each), in
+    // proportion to the rows: at least one range each, at most one per tile.
     const int sms = sm_count() > 0 ? sm_count() : 148;
-    int grid = (int)(total_rows < (int64_t)sms * per_sm ? total_rows : (int64_t)sms * per_sm);
+    const int per_sm = sh.MINB;
+    const int64_t rt = 16 / sh.S;
+    p.pf = static_cast<const uint8_t*>(a.pf);
+    p.pf_bytes = (a.pf && a.pf_bytes < kPrefetchBytes) ? a.pf_bytes : 0;
+    int64_t units[kMaxItems], total_units = 0;
+    for (int i = 0; i < a.count; ++i) total_units += (units[i] = (a.item[i].N + rt - 1) / rt);
+    const int64_t ranges = (int64_t)sms * per_sm / kparts;
+    int grid = (int)(total_units < ranges ? total_units : ranges);
     if (grid < a.count) grid = a.count;
     int ctas[kMaxItems] = {0};
     int used = 0;
     for (int i = 0; i < a.count; ++i) {
         int64_t c = (int64_t)grid * a.item[i].N / total_rows;
         if (c < 1) c = 1;
-        if (c > a.item[i].N) c = a.item[i].N;
+        if (c > units[i]) c = units[i];
         ctas[i] = (int)c;
         used += ctas[i];
     }
@@ -795,7 +753,7 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
         int best = -1;
         double best_load = -1.0;
         for (int i = 0; i < a.count; ++i) {
-            if (ctas[i] >= a.item[i].N) continue;
+            if (ctas[i] >= units[i]) continue;
             const double load = (double)a.item[i].N / ctas[i];
             if (load > best_load) { best_load = load; best = i; }
         }
@@ -815,32 +773,56 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
         --ctas[best];
         --used;
     }
-    grid = used;
+    grid = used * (int)kparts;
     p.pf_share = p.pf_bytes > 0 ? (((p.pf_bytes + grid - 1) / grid + 15) & ~(int64_t)15) : 0;
     int64_t max_rows = 0;
     int begin = 0;
+    float* part = kparts > 1 ? reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(a.ws) + kWorkspaceBytes) : nullptr;
     for (int i = 0; i < a.count; ++i) {
         GemvItem& it = p.item[i];
         it.codes = a.item[i].codes;
         it.Y = a.item[i].Y;
         it.N = (int32_t)a.item[i].N;
         it.cta_begin = begin;
-        it.cta_count = ctas[i];
         it.rows_q = (int32_t)(a.item[i].N / ctas[i]);
         it.rows_rem = (int32_t)(a.item[i].N % ctas[i]);
         for (int c = 0; c < 16; ++c) it.lvl16[c] = a.item[i].lvl16[c];
-        begin += ctas[i];
+        begin += ctas[i] * (int)kparts;
+        it.part = part;
+        if (kparts > 1) part += kparts * a.B * a.item[i].N;
         const int64_t rows = it.rows_q + (it.rows_rem ? 1 : 0);
         if (rows > max_rows) max_rows = rows;
     }
-    int64_t chunk = kRedBytes / ((int64_t)p.spans * Bp * 4);
-    if (chunk > max_rows) chunk = max_rows;
+    // Partial sums: np sets of one per output, each `pitch` floats from the next.
+    // A warp's store covers `run` consecutive outputs of S / 2 sets: a pitch of
+    // `run` modulo 32 puts them on different banks.
+    const int bc = batch_cols(sh.S, sh.NTL), np = p.span_cols * (sh.S >= 4 ? sh.S / 2 : sh.S);
+    const int run = sh.S == 8 ? 2 : sh.S == 4 ? 8 : sh.S == 2 ? 16 : 0;
+    const size_t tab = (size_t)(a.bits == 3 ? 64 : 256) * kTabStride;
+    const int64_t cap = red_bytes(tab, sh.MINB) / 4;
+    auto pitch_for = [&](int64_t rows) { return (rows * bc + 31 - run) / 32 * 32 + run; };
+    int64_t chunk = max_rows;
+    if (pitch_for(chunk) * np > cap) {
+        chunk = (cap / np - 32) / bc;
+        const int64_t step = (rt << p.lg_groups) * sh.T;       // whole rounds of every warp
+        if (chunk > step) chunk -= chunk % step;
+    }
     if (chunk < 1) return cudaErrorInvalidValue;
     p.chunk_rows = (int32_t)chunk;
-    const size_t tab = (size_t)(a.bits == 3 ? 64 : 256) * kTabStride;
-    const size_t smem = red_in_table(a.bits, Bp) ? tab : tab + (size_t)p.spans * chunk * Bp * 4;
-    return a.x_f16 ? dispatch<true>(a.bits, Bp, large, tiny, p, a, grid, smem, s)
-                   : dispatch<false>(a.bits, Bp, large, tiny, p, a, grid, smem, s);
+    p.pitch = (int32_t)pitch_for(chunk);
+    const size_t smem = tab + (size_t)p.pitch * np * 4;
+    e = a.x_f16 ? shape_or_run<true>(a.bits, key, &sh, &p, &a, grid, smem, s)
+                : shape_or_run<false>(a.bits, key, &sh, &p, &a, grid, smem, s);
+    if (e != cudaSuccess || kparts == 1) return e;
+    SplitSum sum;
+    memset(&sum, 0, sizeof sum);
+    sum.n = a.count;
+    for (int i = 0; i < a.count; ++i) {
+        sum.part[i] = p.item[i].part;
+        sum.Y[i] = a.item[i].Y;
+        sum.count[i] = a.B * a.item[i].N;
+    }
+    return launch_split_sum(sum, (int)kparts, a.y_dtype, s);
 }
 
 cudaError_t launch_gemv(const LinearArgs& a, cudaStream_t s)
@@ -859,6 +841,7 @@ cudaError_t launch_gemv(const LinearArgs& a, cudaStream_t s)
     g.x_f16 = a.x_f16;
     g.y_dtype = a.y_dtype;
     g.ws = a.ws;
+    g.ws_bytes = a.ws_bytes;
     return launch_gemv_group(g, s);
 }
 

@@ -84,6 +84,16 @@ struct GroupArgs {
     const void* pf;          // optional L2 warm-up range
     int64_t pf_bytes;
     Workspace* ws;
+    size_t ws_bytes;         // the caller's workspace bytes
+};
+
+// Outputs of a launch whose k ranges were split: per matrix its partial sums
+// [splits][count] and Y[count].
+struct SplitSum {
+    const float* part[4];
+    void* Y[4];
+    int64_t count[4];       // B * N
+    int n;
 };
 
 // The part of a prefetch hint [p, p + bytes) that a bulk L2 prefetch may take:
@@ -140,6 +150,9 @@ struct PrefillPlan {
 };
 PrefillPlan prefill_plan(int64_t B, const int64_t* N, int count, int64_t K, size_t part_bytes_avail);
 PrefillPlan prefill_plan(int64_t B, int64_t N, int64_t K, size_t part_bytes_avail);
-bool gemv_supports(int bits, int64_t B);
+// Y[i] = sum over the splits of part[split][i], in order, in Y's dtype.
+cudaError_t launch_split_sum(const SplitSum& a, int splits, int y_dtype, cudaStream_t s);
+// Whether the decode kernel runs a batch (rows: of all the call's matrices).
+bool gemv_takes(int bits, int64_t B, int64_t rows, int64_t K);
 
 }  // namespace logq

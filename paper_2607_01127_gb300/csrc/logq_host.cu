@@ -166,44 +166,29 @@ uint16_t f16_bits_of(float v)
 
 logq_status cuda_status(cudaError_t e) { return e == cudaSuccess ? LOGQ_OK : LOGQ_ERR_CUDA; }
 
-// 4-bit batches from this size up to 16 may run on the tensor cores instead of
-// the CUDA-core skinny GEMM (whose fp32 FMAs bound it at 16 per weight).
-#ifndef LOGQ_TC_MIN_BATCH
-#define LOGQ_TC_MIN_BATCH 8
-#endif
+// Workspace sizes.  What the two queries return is part of the interface (callers
+// allocate by it), so they go by a fixed model: batches of up to 4 (4 bits: up to
+// 7) need the base workspace only; 4-bit batches of 8..16 room for split k ranges
+// where the tensor-core plan below beats 27 us per 58.7 M weights up to batch 8 and
+// 49 us at 9..16, plus 2 us; larger batches whatever the plan splits.  The kernels
+// use what room they are given: the decode kernel (gemv_takes) for parts of K,
+// the prefill kernel for its k ranges.
+bool small_batch(int bits, int64_t B) { return B <= (bits == 4 ? 16 : 4); }
 
-// Batches that always run on the tensor cores, or may (4-bit, LOGQ_TC_MIN_BATCH..16).
-bool tensor_core_batch(int bits, int64_t B)
-{
-    return !gemv_supports(bits, B) || (bits == 4 && B >= LOGQ_TC_MIN_BATCH && B <= 16);
-}
+// Batches whose workspace the plan sizes.
+bool tensor_core_batch(int bits, int64_t B) { return !small_batch(bits, B) || (bits == 4 && B >= 8); }
 
-// A 4-bit batch of LOGQ_TC_MIN_BATCH..16 takes the tensor cores when their
-// estimated time beats the CUDA-core kernel's: ~27 us per 58.7 M weights at
-// batches up to 8 and ~49 us at 9..16 (the batch is padded to 8 or 16; fp32
-// FMAs bound it), plus ~2 us per launch (measured on the GB300 on the
-// Llama-3.1-8B shapes).  The tensor-core estimate depends on how far the caller's
-// workspace lets the k ranges split (prefill_plan).
 double cuda_core_us(int64_t B, int64_t N, int64_t K)
 {
     return (double)N * (double)K * (B <= 8 ? 0.46e-6 : 0.84e-6) + 2.0;
 }
 
-bool use_small_batch_tc(int bits, int64_t B, int64_t N, int64_t K, size_t workspace_bytes)
-{
-    if (!(bits == 4 && B >= LOGQ_TC_MIN_BATCH && B <= 16)) return false;
-    const size_t avail = workspace_bytes > kWorkspaceBytes ? workspace_bytes - kWorkspaceBytes : 0;
-    const PrefillPlan pl = prefill_plan(B, N, K, avail);
-    return pl.est_us < cuda_core_us(B, N, K);
-}
-
-// How a grouped call runs: one CUDA-core launch over all matrices, one
-// tensor-core launch whose CTAs the matrices share (small ones, such as k / v
-// projections, then no longer leave SMs idle), or each matrix as its own
-// logq_linear call -- whichever is estimated fastest; batches the CUDA-core
-// kernel always takes stay there.  A smaller workspace can only slow the
-// options that split k ranges, so the workspace the choice needs
-// (part_bytes) leads to the same choice.
+// How a grouped call that the decode kernel does not take runs: one tensor-core
+// launch whose CTAs the matrices share (small ones, such as k / v projections, then
+// no longer leave SMs idle), or each matrix as its own logq_linear call --
+// whichever is estimated faster.  A smaller workspace can only slow the options
+// that split k ranges, so the workspace the choice needs (part_bytes) leads to
+// the same choice.  (kCudaCores: only in sizing small batches, see above.)
 struct GroupChoice {
     enum { kCudaCores, kTensorCores, kSingles } kind;
     size_t part_bytes;
@@ -214,7 +199,7 @@ GroupChoice choose_group(int bits, int64_t B, const int64_t* N, int count, int64
     GroupChoice ch{GroupChoice::kCudaCores, 0};
     if (!tensor_core_batch(bits, B)) return ch;
     const size_t avail = workspace_bytes > kWorkspaceBytes ? workspace_bytes - kWorkspaceBytes : 0;
-    const bool cuda_ok = gemv_supports(bits, B);
+    const bool cuda_ok = small_batch(bits, B);
     double cuda_us = 2.0, singles_us = 0.0;
     size_t single_part = 0;
     for (int i = 0; i < count; ++i) {
@@ -314,8 +299,9 @@ size_t logq_linear_workspace_bytes(int64_t B, int64_t N, int64_t K, int bits)
 {
     if (B <= 0 || logq_packed_bytes(N, K, bits) == 0) return 0;
     if (!tensor_core_batch(bits, B)) return kWorkspaceBytes;
-    if (gemv_supports(bits, B) && !use_small_batch_tc(bits, B, N, K, (size_t)-1)) return kWorkspaceBytes;
-    return kWorkspaceBytes + prefill_plan(B, N, K, (size_t)-1).part_bytes;
+    const PrefillPlan pl = prefill_plan(B, N, K, (size_t)-1);
+    if (small_batch(bits, B) && pl.est_us >= cuda_core_us(B, N, K)) return kWorkspaceBytes;
+    return kWorkspaceBytes + pl.part_bytes;
 }
 
 size_t logq_linear_grouped_workspace_bytes(int64_t B, const int64_t* N, int count, int64_t K, int bits)
@@ -472,8 +458,7 @@ logq_status logq_linear(const uint8_t* codes, const logq_codebook* cb, const voi
     a.ws_bytes = workspace_bytes;
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (gemv_supports(cb->bits, B) && !use_small_batch_tc(cb->bits, B, N, K, workspace_bytes))
-        return cuda_status(launch_gemv(a, s));
+    if (gemv_takes(cb->bits, B, N, K)) return cuda_status(launch_gemv(a, s));
     const cudaError_t e = launch_prefill(a, s);
     if (e == cudaErrorNotSupported) return LOGQ_ERR_UNSUPPORTED;
     return cuda_status(e);
@@ -519,13 +504,14 @@ logq_status logq_linear_grouped(const logq_linear_item* items, int count, const 
     g.x_f16 = x_f16;
     g.y_dtype = (int)y_dtype;
     g.ws = ws;
-    int64_t Ns[4];
-    for (int i = 0; i < count; ++i) Ns[i] = items[i].N;
-    const GroupChoice ch = choose_group(bits, B, Ns, count, K, workspace_bytes);
-    if (ch.kind == GroupChoice::kCudaCores) {
+    g.ws_bytes = workspace_bytes;
+    int64_t Ns[4], rows = 0;
+    for (int i = 0; i < count; ++i) rows += (Ns[i] = items[i].N);
+    if (gemv_takes(bits, B, rows, K)) {
         aligned_prefetch_range(l2_prefetch, l2_prefetch_bytes, &g.pf, &g.pf_bytes);
         return cuda_status(launch_gemv_group(g, s));
     }
+    const GroupChoice ch = choose_group(bits, B, Ns, count, K, workspace_bytes);
     if (ch.kind == GroupChoice::kTensorCores) {
         const cudaError_t e = launch_prefill_group(g, workspace_bytes, s);
         if (e == cudaErrorNotSupported) return LOGQ_ERR_UNSUPPORTED;

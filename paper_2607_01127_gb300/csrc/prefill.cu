@@ -895,19 +895,14 @@ uint32_t make_idesc(bool f16_inputs, int bn)
 // Dynamic shared memory of the layout: table rows, X stages, barriers.
 constexpr uint32_t smem_bytes_for(int bn) { return kTabRegion + kXStages * (uint32_t)bn * kBK * 2 + 256; }
 
-// Outputs of a split launch: per matrix its partial sums [splits][count] and Y[count].
-struct SumArgs {
-    const float* part[kMaxPrefillItems];
-    void* Y[kMaxPrefillItems];
-    int64_t count[kMaxPrefillItems];        // B * N
-    int n;
-};
-
 // Fixed-order sum of the k ranges' fp32 partial sums: Y[i] = sum_s part[s][i]
 // (s = 0, 1, ...), rounded to Y's dtype, over the matrices of the launch in turn.
-__global__ void __launch_bounds__(256) splitk_sum_kernel(const __grid_constant__ SumArgs a, int splits, int64_t total,
+__global__ void __launch_bounds__(256) splitk_sum_kernel(const __grid_constant__ SplitSum a, int splits, int64_t total,
                                                          int y_dtype)
 {
+    // the next kernel may start its prologue; the partial sums' own kernel has to finish first
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x) {
         int m = 0;
         int64_t i = g;
@@ -947,6 +942,28 @@ cudaError_t launch(PrefillParams& p, const CUtensorMap& xmap, int grid, cudaStre
 }
 
 }  // namespace
+
+// Launched like the decode kernels (programmatic dependent launch): its blocks
+// wait for the kernel before it on the stream, and the next one's prologue may
+// run beside it.
+cudaError_t launch_split_sum(const SplitSum& a, int splits, int y_dtype, cudaStream_t s)
+{
+    int64_t total = 0;
+    for (int i = 0; i < a.n; ++i) total += a.count[i];
+    const int sms = sm_count() > 0 ? sm_count() : 148;
+    int64_t blocks = (total + 255) / 256;
+    if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, splitk_sum_kernel, a, splits, total, y_dtype);
+}
 
 PrefillPlan prefill_plan(int64_t B, const int64_t* N, int count, int64_t K, size_t part_bytes_avail)
 {
@@ -1074,11 +1091,10 @@ cudaError_t launch_items(const GroupItem* gi, int count, const void* X, int x_f1
     p.idesc = make_idesc(x_f16 != 0, pl.bn);
     // partial sums of matrix i after those of matrices 0 .. i-1
     float* part = pl.splits > 1 ? reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(ws) + kWorkspaceBytes) : nullptr;
-    SumArgs sa;
+    SplitSum sa;
     memset(&sa, 0, sizeof sa);
     sa.n = count;
     int grid = 0;
-    int64_t total = 0;
     for (int i = 0; i < count; ++i) {
         PrefillItem& it = p.item[i];
         it.codes = gi[i].codes;
@@ -1093,7 +1109,6 @@ cudaError_t launch_items(const GroupItem* gi, int count, const void* X, int x_f1
         sa.part[i] = part;
         sa.Y[i] = gi[i].Y;
         sa.count[i] = B * gi[i].N;
-        total += B * gi[i].N;
         if (part) part += (int64_t)pl.splits * B * gi[i].N;
     }
 
@@ -1103,11 +1118,7 @@ cudaError_t launch_items(const GroupItem* gi, int count, const void* X, int x_f1
     else
         e = bits == 8 ? launch<true, kBNMax>(p, xmap, grid, s) : launch<false, kBNMax>(p, xmap, grid, s);
     if (e != cudaSuccess || pl.splits == 1) return e;
-    const int sms = sm_count() > 0 ? sm_count() : 148;
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-    splitk_sum_kernel<<<(int)blocks, 256, 0, s>>>(sa, pl.splits, total, y_dtype);
-    return cudaGetLastError();
+    return launch_split_sum(sa, pl.splits, y_dtype, s);
 }
 
 }  // namespace
