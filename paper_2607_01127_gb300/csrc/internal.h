@@ -137,11 +137,10 @@ cudaError_t launch_prefill(const LinearArgs& a, cudaStream_t s);
 // workspace, which holds the split k ranges' partial sums).
 cudaError_t launch_prefill_group(const GroupArgs& g, size_t ws_bytes, cudaStream_t s);
 // Tensor-core launch plan of B x N[i] x K products sharing X (count <= 4):
-// token-tile width, k ranges per output tile (the partial sums need part_bytes
-// of workspace beyond kWorkspaceBytes; at most part_bytes_avail are used) and
-// the CTAs each matrix gets.
+// k ranges per output tile (the partial sums need part_bytes of workspace
+// beyond kWorkspaceBytes; at most part_bytes_avail are used) and the CTAs each
+// matrix gets.
 struct PrefillPlan {
-    int bn;
     int splits;
     int ksplit;
     size_t part_bytes;

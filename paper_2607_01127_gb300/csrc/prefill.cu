@@ -3,35 +3,42 @@
 // LUT reads, so here each weight is dequantised once per tile and reused by a
 // dense bf16/fp16 contraction).
 //
-// One persistent CTA per SM walks 128 (weights) x BN (tokens) output tiles, BN
-// = 256 for prefill and 16 for small batches; where there are too few tiles
-// to fill the SMs, each tile's k range is split into ranges taken by
-// different CTAs, which write fp32 partial sums to the caller's workspace and
-// a second kernel adds them in a fixed order.  A launch may cover up to four
-// matrices that read the same X (q/k/v, gate/up): each gets a contiguous
-// range of the CTAs, in proportion to its tiles, and a CTA works on its
-// matrix's tiles only.
+// One persistent CTA per SM walks 128 (weights) x 256 (tokens) output tiles;
+// where there are too few tiles to fill the SMs, each tile's k range is split
+// into ranges taken by different CTAs, which write fp32 partial sums to the
+// caller's workspace and a second kernel adds them in a fixed order.  A launch
+// may cover up to four matrices that read the same X (q/k/v, gate/up): each
+// gets a contiguous range of the CTAs, in proportion to its tiles, and a CTA
+// works on its matrix's tiles only.
 // The dequantised weight tile (the MMA's A operand) lives in tensor memory, not
 // in shared memory: tensor memory holds one fp32 accumulator (256 columns) and
 // eight weight stages (32 columns each), and shared memory holds the pair table
 // and five X stages.
-// Warp roles:
+// Warp roles (28 warps, seven warpgroups; setmaxnreg moves registers from the
+// first to the epilogue):
 //   warp 0     TMA producer: X tiles [256 tokens x 64 k] with 128-byte swizzle.
 //   warp 1     MMA issuer: tcgen05.mma kind::f16, M = 128 (weight rows),
 //              N = 256 (tokens), K = 16, A from tensor memory, B (X) from
 //              shared memory, fp32 accumulator in tensor memory.  Also
-//              allocates TMEM.
-//   warps 2-9  epilogue: two warps per TMEM lane quarter, each draining 128
-//              token columns with tcgen05.ld; 16-bit outputs are rounded into
-//              registers and the accumulator is handed back before the stores
-//              of Y (lane n writes Y[t][n0 + n]).
-//   warps 10-17 decode: two threads per weight row of the tile, each owning 32
+//              allocates TMEM.  (Warps 2 and 3 only fill the warpgroup.)
+//   warps 4-11 epilogue: two warps per TMEM lane quarter, each draining 128
+//              token columns with tcgen05.ld, 32 at a time; the accumulator is
+//              handed back before the last 32 are stored (lane n writes
+//              Y[t][n0 + n]).
+//   warps 12-27 decode: two groups of eight warps that take the stages in turn.
+//              Two threads per weight row of the tile and group, each owning 32
 //              of the stage's 64 k; a thread streams its codes into its own
 //              16-byte slot of a shared ring with cp.async, resolves two codes
 //              per lookup in a per-lane-replicated pair table, and writes the
 //              16 bf16 (or fp16) pairs to its row's TMEM lane with tcgen05.st.
 //              tcgen05.st reaches only the warp's lane quarter (warp % 4), so a
 //              thread's weight row is 32 * (warp % 4) + lane.
+// A decode warp spends ~700 cycles on a stage, most of it waiting (its code
+// copies, the lookups, the free weight stage, the tensor-memory store), so one
+// group cannot feed an MMA that needs 512; two groups overlap those waits.
+// One Llama-3.1-8B layer at 2048 tokens: 8 bits 1176 us with one group, 902 with
+// two; 3 bits 1276 and 1188; 4 bits 775 and 771 (the MMA issuer sets the pace there);
+// Llama-3.2-1B shapes, 517 tokens, 8 bits: 192 and 156.
 // The pair table starts the dynamic shared memory, at the fixed shared address
 // kTabOff, with 256-byte rows: the offset of an entry, byte << 8 | 4 * lane,
 // is one byte permute of the code word and the table base is the load's
@@ -55,28 +62,21 @@ namespace logq {
 namespace {
 
 constexpr int kBM = 128;                 // weight rows per tile (MMA M)
-constexpr int kBNMax = 256;              // widest token tile (MMA N)
+constexpr int kBN = 256;                 // tokens per tile (MMA N)
 constexpr int kBK = 64;                  // k per stage (one 128-byte swizzle atom of bf16)
 constexpr int kMaxPrefillItems = 4;      // matrices of one grouped launch
 constexpr int kXStages = 5;              // X tiles in flight (TMA)
 constexpr int kWStages = 8;              // dequantised weight tiles in flight (tensor memory)
-// Decode warps: four per k slice of a stage (one per TMEM lane quarter), each
-// thread owning one weight row's kSliceK of the stage's 64 k.  Eight (two
-// slices of 32 k) measured faster than sixteen (four of 16 k, 72 registers):
-// the per-stage waits, tensor-memory store and arrive of each warp cost more
-// than the extra warps hide.
-#ifndef LOGQ_PREFILL_DECODE_WARPS
-#define LOGQ_PREFILL_DECODE_WARPS 8
-#endif
-constexpr int kDecodeWarps = LOGQ_PREFILL_DECODE_WARPS;
-static_assert(kDecodeWarps == 4 || kDecodeWarps == 8 || kDecodeWarps == 16, "one, two or four k slices per stage");
-constexpr int kSlices = kDecodeWarps / 4;
-constexpr int kSliceK = 64 / kSlices;            // k per decode thread and stage: 64, 32 or 16
+constexpr int kGroupWarps = 8;                   // decode warps that share a stage: four per k slice, one per TMEM lane quarter
+constexpr int kGroups = 2;                       // groups of decode warps, taking the stages in turn
+constexpr int kDecodeWarps = kGroups * kGroupWarps;
+constexpr int kSlices = kGroupWarps / 4;
+constexpr int kSliceK = 64 / kSlices;            // k per decode thread and stage
 constexpr int kSlicePairs = kSliceK / 2;         // TMEM columns (16-bit pairs) per thread and stage
 constexpr int kDecodeThreads = 32 * kDecodeWarps;
 constexpr int kEpiWarps = 8;                       // two per TMEM lane quarter
-constexpr int kEpi0 = 2, kDec0 = kEpi0 + kEpiWarps;  // first epilogue / decode warp
-constexpr int kThreads = 32 * (kDec0 + kDecodeWarps);  // producer, MMA, epilogue, decode
+constexpr int kEpi0 = 4, kDec0 = kEpi0 + kEpiWarps;  // first epilogue / decode warp (whole warpgroups)
+constexpr int kThreads = 32 * (kDec0 + kDecodeWarps);  // producer and MMA (a warpgroup), epilogue, decode
 constexpr int kCodeSlotBytes = 16;               // ring slot: codes of one thread's slice (<= 16 B)
 constexpr int kCodeStageBytes = kDecodeThreads * kCodeSlotBytes;
 // Shared address at which dynamic shared memory starts in a kernel without
@@ -85,7 +85,7 @@ constexpr uint32_t kTabOff = 1024;
 constexpr uint32_t kTabRow = 256;                // 32 lane copies in the first 128 bytes
 constexpr uint32_t kTabRegion = 256 * kTabRow;   // table rows (the 4-bit table uses all 256)
 constexpr uint32_t kTmemCols = 512;              // accumulator (256) + weight stages (8 x 32)
-constexpr uint32_t kWCol0 = kBNMax;              // first column of weight stage 0 (after the widest accumulator)
+constexpr uint32_t kWCol0 = kBN;                 // first column of weight stage 0 (after the accumulator)
 constexpr uint32_t kWStageCols = kBK / 2;        // 64 k of 16-bit values = 32 columns
 static_assert(kWCol0 + kWStages * kWStageCols <= kTmemCols, "weight stages must fit in tensor memory");
 constexpr long long kWaitLimit = 2000000000LL;   // cycles (~1 s)
@@ -349,20 +349,18 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, ui
 
 // ------------------------------------------------------------------ kernel ---
 
-// EIGHT: 8-bit codes, one per byte: a thread's kSliceK k of a stage are
-// kSliceK bytes (one or two ring slots), each byte resolves to one value (the
-// table holds it in both halves) and two values form a pair with one byte
-// permute.
-template <bool EIGHT, int BN>
+// BITS = 8: one code per byte, a thread's kSliceK k of a stage are kSliceK bytes
+// (two ring slots), each byte resolves to one value (the table holds it in both
+// halves) and two values form a pair with one byte permute.
+template <int BITS>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ CUtensorMap xmap)
 {
-    static_assert(BN >= 16 && BN <= kBNMax && BN % 16 == 0, "MMA N with M = 128");
-    constexpr int XB = BN * kBK * 2;                     // bytes of one X stage
-    constexpr int kChunks = ((BN < 128 ? BN : 128) + 31) / 32;   // 32-column drains per epilogue warp
+    constexpr int XB = kBN * kBK * 2;                    // bytes of one X stage
+    constexpr int kChunks = kBN / 2 / 32;                // 32-column drains per epilogue warp
     // 16-byte ring slots per thread and stage: 8-bit kSliceK bytes; 4-bit kSliceK / 2
     // bytes; 3-bit one 12-byte group per slot (a 16-k slice copies its whole group)
-    constexpr int SLOTS = EIGHT ? (kSliceK >= 16 ? kSliceK / 16 : 1) : (kSliceK == 64 ? 2 : 1);
+    constexpr int SLOTS = BITS == 8 ? (kSliceK >= 16 ? kSliceK / 16 : 1) : (kSliceK == 64 ? 2 : 1);
     // code stages in flight per decode thread: as many as the free halves of the
     // table rows hold, at most 7
     constexpr int RING_FIT = (256 * 128) / (SLOTS * kCodeStageBytes);
@@ -421,7 +419,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
             mbar_init(xempty(s), 1);
         }
         for (int s = 0; s < kWStages; ++s) {
-            mbar_init(wfull(s), kDecodeWarps);
+            mbar_init(wfull(s), kGroupWarps);
             mbar_init(wempty(s), 1);
         }
         mbar_init(accfull, 1);
@@ -433,15 +431,15 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
     }
     // pair table: entry e (two codes) = bf16x2 / f16x2 of their levels, one copy per lane
     {
-        const int nent = (EIGHT || p.bits == 4) ? 256 : 64;
+        const int nent = (BITS != 3) ? 256 : 64;
         for (int i = tid; i < nent * 8; i += kThreads) {
             const int e = i >> 3, part = i & 7;
             uint32_t v;
-            if constexpr (EIGHT) {
+            if constexpr (BITS == 8) {
                 v = (uint32_t)item.lvl16[e] * 0x10001u;
             } else {
-                const uint32_t lo = (p.bits == 4) ? (e & 15) : (e & 7);
-                const uint32_t hi = (p.bits == 4) ? (e >> 4) : (e >> 3);
+                const uint32_t lo = (BITS == 4) ? (e & 15) : (e & 7);
+                const uint32_t hi = (BITS == 4) ? (e >> 4) : (e >> 3);
                 v = (uint32_t)item.lvl16[lo] | ((uint32_t)item.lvl16[hi] << 16);
             }
             sts128(sbase + e * kTabRow + part * 16, v, v, v, v);
@@ -500,6 +498,10 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
                          "r"((uint32_t)(b1 - b0))
                          : "memory");
     };
+    // 896 threads start with 72 registers each: the first warpgroup gives 16 of its
+    // to the two epilogue ones (128 x 16 = 256 x 8)
+    if (warp < kEpi0) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    else if (warp < kDec0) asm volatile("setmaxnreg.inc.sync.aligned.u32 80;");
     if (warp == 0) {
         // ---------------- TMA producer ----------------
         // The whole warp walks the loop (uniform operands); one elected lane issues.
@@ -508,7 +510,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         bool ok = true;
         uint32_t issued = 0, issued_par = 0;           // per stage: used at least once / parity of last load
         for (int tile = cta; tile < ntiles && ok; tile += ncta) {
-            const int t0 = tile_t(tile) * BN;
+            const int t0 = tile_t(tile) * kBN;
             const int kb = k_begin(tile), ke = k_end(tile);
             for (int ks = kb; ks < ke; ++ks) {
                 if (!warp_wait(xempty(stage), phase ^ 1u, abort_flag, p.ws, kWaitProducer)) {
@@ -591,83 +593,54 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         const int row = quarter * 32 + lane;
         const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ehalf * 128);
         int it = 0;
-        // an epilogue warp of the second column half, idle in 16-token tiles
         const bool pf_warp = warp == kEpi0 + 4;
         for (int tile = cta; tile < ntiles; tile += ncta, ++it) {
             if (pf_warp) prefetch_codes(tile + ncta);
             if (!warp_wait(accfull, (uint32_t)it & 1u, abort_flag, p.ws, kWaitEpilogue)) break;
             tc_fence_after();
             const int64_t n = (int64_t)tile_n(tile) * kBM + row;
-            const int tb0 = tile_t(tile) * BN + ehalf * 128;
-            // tokens of this half that exist (may be <= 0: the tile is narrower, or past B)
-            const int hcols = (BN - ehalf * 128) < 128 ? (BN - ehalf * 128) : 128;
-            const int jmax = (p.B - tb0) < hcols ? (p.B - tb0) : hcols;
-            if (hcols <= 0) {
-                // no column of this tile in this half: only hand the accumulator back
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(accempty);
-            } else if (p.splits > 1 || p.y_dtype == LOGQ_F32) {
-                // fp32 out: Y itself, or this k range's partial sums
-                float* yb = p.splits > 1 ? item.part + (int64_t)tile_sp(tile) * p.B * N : static_cast<float*>(item.Y);
+            const int tb0 = tile_t(tile) * kBN + ehalf * 128;
+            // tokens of this half that exist (<= 0 past the end of the batch)
+            const int jmax = (p.B - tb0) < 128 ? (p.B - tb0) : 128;
+            {
+                // 32 tokens at a time; the accumulator is handed back before the last
+                // stores.  Lanes hold consecutive n: each store instruction writes one
+                // contiguous run of Y[t][n0 .. n0+31].
+                const bool f32 = p.splits > 1 || p.y_dtype == LOGQ_F32;       // Y, or this k range's partial sums
+                const bool bf = p.y_dtype == LOGQ_BF16;
+                uint8_t* const yb = p.splits > 1
+                                        ? reinterpret_cast<uint8_t*>(item.part + (int64_t)tile_sp(tile) * p.B * N)
+                                        : static_cast<uint8_t*>(item.Y);
 #pragma unroll 1
                 for (int c = 0; c < kChunks; ++c) {
                     uint32_t v[32];
                     tmem_ld32(tq + (uint32_t)(c * 32), v);
+                    if (c == kChunks - 1) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(accempty);
+                    }
                     const int jm = jmax - 32 * c;
-                    if (n < N && jm > 0) {
-                        float* y = yb + (int64_t)(tb0 + 32 * c) * N + n;
+                    if (n >= N || jm <= 0) continue;
+                    const int64_t at = (int64_t)(tb0 + 32 * c) * N + n;
+                    if (f32) {
+                        float* y = reinterpret_cast<float*>(yb) + at;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (j < jm) y[(int64_t)j * N] = __uint_as_float(v[j]);
-                    }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(accempty);
-            } else {
-                const bool bf = p.y_dtype == LOGQ_BF16;
-                uint32_t pk[64];                        // tokens 2j, 2j+1 rounded to 16 bits
-#pragma unroll
-                for (int c = 0; c < kChunks; ++c) {
-                    uint32_t v[32];
-                    tmem_ld32(tq + (uint32_t)(c * 32), v);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float a = __uint_as_float(v[2 * j]), b = __uint_as_float(v[2 * j + 1]);
-                        if (bf) {
-                            const __nv_bfloat162 h2 = __floats2bfloat162_rn(a, b);
-                            pk[16 * c + j] = *reinterpret_cast<const uint32_t*>(&h2);
-                        } else {
-                            const __half2 h2 = __floats2half2_rn(a, b);
-                            pk[16 * c + j] = *reinterpret_cast<const uint32_t*>(&h2);
-                        }
-                    }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(accempty);
-                if (n < N && jmax > 0) {
-                    // lanes hold consecutive n: each store instruction writes one
-                    // contiguous run of Y[t][n0 .. n0+31]
-                    uint16_t* y = static_cast<uint16_t*>(item.Y) + (int64_t)tb0 * N + n;
-                    if (jmax == 128) {
-#pragma unroll
-                        for (int j = 0; j < 64; ++j) {
-                            y[(int64_t)(2 * j) * N] = (uint16_t)(pk[j] & 0xffffu);
-                            y[(int64_t)(2 * j + 1) * N] = (uint16_t)(pk[j] >> 16);
-                        }
+                        for (int j = 0; j < 32; ++j, y += N)
+                            if (j < jm) *y = __uint_as_float(v[j]);
                     } else {
+                        uint16_t* y = reinterpret_cast<uint16_t*>(yb) + at;
 #pragma unroll
-                        for (int j = 0; j < 64; ++j) {
-                            if (2 * j < jmax) y[(int64_t)(2 * j) * N] = (uint16_t)(pk[j] & 0xffffu);
-                            if (2 * j + 1 < jmax) y[(int64_t)(2 * j + 1) * N] = (uint16_t)(pk[j] >> 16);
+                        for (int j = 0; j < 32; ++j, y += N) {
+                            if (j >= jm) break;
+                            const float a = __uint_as_float(v[j]);
+                            *y = bf ? __bfloat16_as_ushort(__float2bfloat16_rn(a)) : __half_as_ushort(__float2half_rn(a));
                         }
                     }
                 }
             }
         }
-    } else {
+    } else if (warp >= kDec0) {
         // ---------------- decode ----------------
         // tcgen05.st reaches only the warp's TMEM lane quarter (warp % 4), so the
         // weight row of a thread is its TMEM lane: row = 32 * (warp % 4) + lane.
@@ -675,17 +648,19 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         const int dw = warp - kDec0;                    // 0 .. kDecodeWarps-1
         const int d = dw * 32 + lane;                   // code-ring slot, 0 .. kDecodeThreads-1
         const int r = (warp & 3) * 32 + lane;           // weight row within the tile
-        const int h = dw >> 2;                          // slice: k kSliceK*h .. +kSliceK-1 of the stage
+        const int grp = dw / kGroupWarps;               // stages grp, grp + kGroups, ...
+        const int h = (dw % kGroupWarps) >> 2;          // slice: k kSliceK*h .. +kSliceK-1 of the stage
         const uint32_t tw = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + kWCol0 + (uint32_t)(kSlicePairs * h);
         const uint32_t lane4 = 4u * (uint32_t)lane;
         // bytes of one row's codes per stage, and where this thread's slice (for 3-bit:
         // the 32-k group holding it) starts among them
-        const int step_bytes = EIGHT ? 64 : (p.bits == 4) ? 32 : 24;
-        const int slice_off = EIGHT ? kSliceK * h : (p.bits == 4) ? (kSliceK / 2) * h : 12 * ((kSliceK * h) / 32);
-        int stage = 0;
+        const int step_bytes = BITS == 8 ? 64 : (BITS == 4) ? 32 : 24;
+        const int slice_off = BITS == 8 ? kSliceK * h : (BITS == 4) ? (kSliceK / 2) * h : 12 * ((kSliceK * h) / 32);
+        int stage = grp;
         uint32_t phase = 0;
-        int total = 0;                                  // stages this CTA decodes
+        int total = 0;                                  // stages of this CTA, then of this group
         for (int t = cta; t < ntiles; t += ncta) total += k_end(t) - k_begin(t);
+        total = (total - grp + kGroups - 1) / kGroups;
         // Cursor over (tile, k-step) advanced without divisions: one for the
         // copies issued ahead, one for the stage being decoded.
         struct Cursor {
@@ -701,20 +676,28 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
             c.valid = tile < ntiles && n < N;
             c.row = codes + (c.valid ? n : 0) * p.row_bytes + slice_off;
         };
-        auto step = [&](Cursor& c) {
+        auto step1 = [&](Cursor& c) {
             if (++c.ks >= c.ke) set_tile(c, c.tile + ncta);
         };
-        Cursor ahead, cur;
+        auto step = [&](Cursor& c) {
+#pragma unroll
+            for (int i = 0; i < kGroups; ++i) step1(c);
+        };
+        Cursor ahead;
         set_tile(ahead, cta);
-        set_tile(cur, cta);
-        auto issue = [&](int g) {
+        for (int i = 0; i < grp; ++i) step1(ahead);
+        uint32_t exists = 0;                            // bit r: this thread's row exists in ring stage r's tile
+        // copies of stage g of this group into ring stage r
+        auto issue = [&](int g, int r) {
+            exists &= ~(1u << r);
             if (g < total && ahead.valid) {
+                exists |= 1u << r;
                 const uint8_t* src = ahead.row + (int64_t)ahead.ks * step_bytes;
-                const uint32_t dst = ring_slot(g % RING, SLOTS * d);
-                if constexpr (EIGHT) {
+                const uint32_t dst = ring_slot(r, SLOTS * d);
+                if constexpr (BITS == 8) {
 #pragma unroll
                     for (int q = 0; q < SLOTS; ++q) cp_async_16(dst + 16 * q, src + 16 * q);
-                } else if (p.bits == 4) {
+                } else if (BITS == 4) {
                     if constexpr (kSliceK == 16) cp_async_8(dst, src);
                     else {
 #pragma unroll
@@ -734,7 +717,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         };
         // Resolve the codes of one stage (its slot in the ring) into the slice's pair values.
         auto resolve = [&](int slot, bool valid, uint32_t (&pr)[kSlicePairs]) {
-            if constexpr (EIGHT) {
+            if constexpr (BITS == 8) {
                 // word i holds the codes of k = kSliceK h + 4i .. +3: pairs 2i and 2i + 1
                 constexpr int NWD = kSliceK / 4;
                 uint32_t cw8[NWD];
@@ -761,7 +744,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
                     if (valid) cv = lds128(ring_slot(slot, SLOTS * d) + 16 * q);
                     cw[4 * q] = cv.x; cw[4 * q + 1] = cv.y; cw[4 * q + 2] = cv.z; cw[4 * q + 3] = cv.w;
                 }
-                if (p.bits == 4) {
+                if (BITS == 4) {
                     // word i holds k = kSliceK h + 8i .. +7
     #pragma unroll
                     for (int i = 0; i < kSliceK / 8; ++i) {
@@ -804,46 +787,26 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
                 }
             }
         };
-        // Software pipeline: the pairs of stage g+1 are looked up while stage g
-        // waits for its weight slot and is stored.
-        for (int g = 0; g < RING - 1; ++g) issue(g);
-        uint32_t pr_a[kSlicePairs], pr_b[kSlicePairs];
-        int slot = 0;                                   // ring slot of stage g
-        if (total > 0) {
-            issue(RING - 1);
+        // The other group's warps hide this one's latencies: a stage's pairs are looked
+        // up and stored one after the other.
+        for (int g = 0; g < RING; ++g) issue(g, g);
+        int slot = 0;                                   // ring stage of stage g
+        for (int g = 0; g < total; ++g) {
+            uint32_t pr[kSlicePairs];
             cp_async_wait<RING - 1>();
-            resolve(slot, cur.valid, pr_a);
-            step(cur);
-        }
-        // One stage: look up the next stage's pairs into nxt, then store this
-        // stage's (cur) once its weight slot is free.  Called with the two
-        // buffers in alternating roles, so no pairs are copied.
-        bool ok = true;
-        auto stage_step = [&](int g, const uint32_t (&cur_pr)[kSlicePairs], uint32_t (&nxt_pr)[kSlicePairs]) {
+            resolve(slot, (exists >> slot) & 1u, pr);
+            issue(g + RING, slot);                      // this thread's slot has been read
             if (++slot == RING) slot = 0;
-            if (g + 1 < total) {
-                issue(g + RING);
-                cp_async_wait<RING - 1>();
-                resolve(slot, cur.valid, nxt_pr);
-                step(cur);
-            }
-            if (!warp_wait(wempty(stage), phase ^ 1u, abort_flag, p.ws, kWaitDecode)) {
-                ok = false;
-                return;
-            }
+            if (!warp_wait(wempty(stage), phase ^ 1u, abort_flag, p.ws, kWaitDecode)) break;
             tc_fence_after();
             // pair q holds k = kSliceK h + 2q (low half) and + 1: column kSlicePairs h + q of the stage
-            tmem_st_pairs(tw + (uint32_t)stage * kWStageCols, cur_pr);
+            tmem_st_pairs(tw + (uint32_t)stage * kWStageCols, pr);
             tmem_wait_st();
             tc_fence_before();            // this warp's tensor-memory writes -> the MMA issuer
             __syncwarp();
             if (lane == 0) mbar_arrive(wfull(stage));
-            if (++stage == kWStages) { stage = 0; phase ^= 1u; }
-        };
-        for (int g = 0; g < total && ok; g += 2) {
-            stage_step(g, pr_a, pr_b);
-            if (g + 1 >= total || !ok) break;
-            stage_step(g + 1, pr_b, pr_a);
+            stage += kGroups;
+            if (stage >= kWStages) { stage -= kWStages; phase ^= 1u; }
         }
         cp_async_wait<0>();
     }
@@ -879,7 +842,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
     return fn;
 }
 
-uint32_t make_idesc(bool f16_inputs, int bn)
+uint32_t make_idesc(bool f16_inputs)
 {
     uint32_t d = 0;
     d |= 1u << 4;                                   // D format: fp32
@@ -887,13 +850,13 @@ uint32_t make_idesc(bool f16_inputs, int bn)
     d |= ab << 7;
     d |= ab << 10;
     // bits 15, 16: A and B K-major (0)
-    d |= (uint32_t)(bn >> 3) << 17;                 // N / 8
+    d |= (uint32_t)(kBN >> 3) << 17;                 // N / 8
     d |= (uint32_t)(kBM >> 4) << 24;                // M / 16
     return d;
 }
 
 // Dynamic shared memory of the layout: table rows, X stages, barriers.
-constexpr uint32_t smem_bytes_for(int bn) { return kTabRegion + kXStages * (uint32_t)bn * kBK * 2 + 256; }
+constexpr uint32_t kSmemBytes = kTabRegion + kXStages * (uint32_t)kBN * kBK * 2 + 256;
 
 // Fixed-order sum of the k ranges' fp32 partial sums: Y[i] = sum_s part[s][i]
 // (s = 0, 1, ...), rounded to Y's dtype, over the matrices of the launch in turn.
@@ -917,10 +880,9 @@ __global__ void __launch_bounds__(256) splitk_sum_kernel(const __grid_constant__
     }
 }
 
-template <bool EIGHT, int BN>
+template <int BITS>
 cudaError_t launch(PrefillParams& p, const CUtensorMap& xmap, int grid, cudaStream_t s)
 {
-    constexpr uint32_t kSmemBytes = smem_bytes_for(BN);
     static uint32_t configured[64] = {0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -932,12 +894,12 @@ cudaError_t launch(PrefillParams& p, const CUtensorMap& xmap, int grid, cudaStre
         if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
         const uint32_t bytes = kSmemBytes;
         if (reserved != (int)kTabOff || bytes > (uint32_t)optin) return cudaErrorNotSupported;
-        e = cudaFuncSetAttribute(prefill_kernel<EIGHT, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        e = cudaFuncSetAttribute(prefill_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (e != cudaSuccess) return e;
         configured[dev] = bytes;
     }
     p.smem_bytes = configured[dev];
-    prefill_kernel<EIGHT, BN><<<grid, kThreads, configured[dev], s>>>(p, xmap);
+    prefill_kernel<BITS><<<grid, kThreads, configured[dev], s>>>(p, xmap);
     return cudaGetLastError();
 }
 
@@ -969,9 +931,8 @@ PrefillPlan prefill_plan(int64_t B, const int64_t* N, int count, int64_t K, size
 {
     PrefillPlan pl;
     memset(&pl, 0, sizeof pl);
-    pl.bn = B <= 16 ? 16 : kBNMax;
     const int sms = sm_count() > 0 ? sm_count() : 148;
-    const int64_t ttiles = (B + pl.bn - 1) / pl.bn;
+    const int64_t ttiles = (B + kBN - 1) / kBN;
     int64_t tiles[kMaxPrefillItems], sum_n = 0;
     for (int i = 0; i < count; ++i) {
         tiles[i] = ((N[i] + kBM - 1) / kBM) * ttiles;
@@ -1010,8 +971,7 @@ PrefillPlan prefill_plan(int64_t B, const int64_t* N, int count, int64_t K, size
         for (int i = 0; i < count; ++i) r = rounds(i) > r ? rounds(i) : r;
         return r;
     };
-    // Cost in k-step times (~0.5 us each on the GB300, for either tile width:
-    // the roles' hand-offs and the decode threads' code copies, more than the
+    // Cost in k-step times (~0.5 us each on the GB300: the roles' hand-offs and the decode threads' code copies, more than the
     // MMAs, set a stage's time): persistent CTAs take tiles in rounds,
     // a tile of ks k-steps costing ks + 6 (pipeline fill, and the MMA waiting
     // for the epilogue to drain the single accumulator).  A split adds the sum
@@ -1068,7 +1028,7 @@ cudaError_t launch_items(const GroupItem* gi, int count, const void* X, int x_f1
     memset(&xmap, 0, sizeof xmap);
     const cuuint64_t gdim[2] = {(cuuint64_t)K, (cuuint64_t)B};
     const cuuint64_t gstride[1] = {(cuuint64_t)K * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)pl.bn};
+    const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kBN};
     const cuuint32_t estride[2] = {1, 1};
     CUresult r = encode(&xmap, x_f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
                         const_cast<void*>(X), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -1085,10 +1045,10 @@ cudaError_t launch_items(const GroupItem* gi, int count, const void* X, int x_f1
     p.bits = bits;
     p.row_bytes = (bits == 8) ? K : (bits == 4) ? K / 2 : K / 32 * 12;
     p.y_dtype = y_dtype;
-    p.n_tiles_t = (int32_t)((B + pl.bn - 1) / pl.bn);
+    p.n_tiles_t = (int32_t)((B + kBN - 1) / kBN);
     p.splits = pl.splits;
     p.ksplit = pl.ksplit;
-    p.idesc = make_idesc(x_f16 != 0, pl.bn);
+    p.idesc = make_idesc(x_f16 != 0);
     // partial sums of matrix i after those of matrices 0 .. i-1
     float* part = pl.splits > 1 ? reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(ws) + kWorkspaceBytes) : nullptr;
     SplitSum sa;
@@ -1113,10 +1073,7 @@ cudaError_t launch_items(const GroupItem* gi, int count, const void* X, int x_f1
     }
 
     cudaError_t e;
-    if (pl.bn == 16)
-        e = bits == 8 ? launch<true, 16>(p, xmap, grid, s) : launch<false, 16>(p, xmap, grid, s);
-    else
-        e = bits == 8 ? launch<true, kBNMax>(p, xmap, grid, s) : launch<false, kBNMax>(p, xmap, grid, s);
+    e = bits == 8 ? launch<8>(p, xmap, grid, s) : bits == 4 ? launch<4>(p, xmap, grid, s) : launch<3>(p, xmap, grid, s);
     if (e != cudaSuccess || pl.splits == 1) return e;
     return launch_split_sum(sa, pl.splits, y_dtype, s);
 }
