@@ -37,8 +37,16 @@
 // copies, the lookups, the free weight stage, the tensor-memory store), so one
 // group cannot feed an MMA that needs 512; two groups overlap those waits.
 // One Llama-3.1-8B layer at 2048 tokens: 8 bits 1176 us with one group, 902 with
-// two; 3 bits 1276 and 1188; 4 bits 775 and 771 (the MMA issuer sets the pace there);
-// Llama-3.2-1B shapes, 517 tokens, 8 bits: 192 and 156.
+// two; 3 bits 1276 and 1188; Llama-3.2-1B shapes, 517 tokens, 8 bits: 192 and 156.
+// What sets a stage's time otherwise is the issuer's own loop (two barrier polls,
+// each several hundred cycles behind the decode warps' shared-memory accesses, and
+// the issue), so it asks for both barriers at once and its operands are kept
+// uniform (see `warp`): 4 bits, 8B layer at 2048 / 512 / 100 / 33 tokens 771 / 243 /
+// 161 / 148 us before, 579 / 187 / 123 / 111 now (1.55 PFLOP/s at 2048, 0.90 of what
+// cuBLAS holds for seconds under the power limit); 8 bits at 2048 855.  Tried and
+// slower: polling two stages ahead, taking several full stages at a time, resolving
+// 4-bit codes with byte permutes instead of lookups, draining the whole accumulator
+// into registers before the stores (no change).
 // The pair table starts the dynamic shared memory, at the fixed shared address
 // kTabOff, with 256-byte rows: the offset of an entry, byte << 8 | 4 * lane,
 // is one byte permute of the code word and the table base is the load's
@@ -152,6 +160,20 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// The same without waiting.
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(bar), "r"(parity)
@@ -402,7 +424,12 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
     static_assert(8 * (2 * kXStages + 2 * kWStages + 3) + 8 + 4 <= 256, "barrier block overflows");
     volatile int* abort_flag = reinterpret_cast<volatile int*>(gen + tmem_slot + 8);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    // The shuffle tells the compiler that a role's branch is uniform over the warp.
+    // Without it the MMA issuer's operands do not stay in uniform registers, and its
+    // issue of a stage, not the MMAs, sets a stage's time (a loop of nothing but a poll
+    // and the MMAs: 605 cycles a stage, 513 with it).
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     // this CTA's matrix, and its place among that matrix's CTAs
     int m = 0;
 #pragma unroll
@@ -556,10 +583,14 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
             const uint32_t dcol = tmem_base;
             const int kb = k_begin(tile), ke = k_end(tile);
             for (int ks = kb; ks < ke; ++ks) {
-                if (!warp_wait(xfull(xs), xph, abort_flag, p.ws, kWaitMma) ||
-                    !warp_wait(wfull(wsg), wph, abort_flag, p.ws, kWaitMma)) {
-                    ok = false;
-                    break;
+                // lane 0 asks for the X stage, lane 1 for the weights, at once
+                const uint32_t bar = lane ? wfull(wsg) : xfull(xs), ph = lane ? wph : xph;
+                if (__ballot_sync(0xffffffffu, lane < 2 && !mbar_test_wait(bar, ph))) {
+                    const bool full = lane >= 2 || wait_bounded(bar, ph, abort_flag, p.ws, kWaitMma);
+                    if (!__all_sync(0xffffffffu, full)) {
+                        ok = false;
+                        break;
+                    }
                 }
                 tc_fence_after();
                 const uint32_t acol = tmem_base + kWCol0 + (uint32_t)wsg * kWStageCols;
@@ -971,8 +1002,9 @@ PrefillPlan prefill_plan(int64_t B, const int64_t* N, int count, int64_t K, size
         for (int i = 0; i < count; ++i) r = rounds(i) > r ? rounds(i) : r;
         return r;
     };
-    // Cost in k-step times (~0.5 us each on the GB300: the roles' hand-offs and the decode threads' code copies, more than the
-    // MMAs, set a stage's time): persistent CTAs take tiles in rounds,
+    // Cost in k-step times (0.37-0.5 us each on the GB300: the issuer's loop and
+    // the decode warps, more than the MMAs, set a stage's time; est_us keeps to
+    // 0.5, by which the workspace queries are sized): persistent CTAs take tiles in rounds,
     // a tile of ks k-steps costing ks + 6 (pipeline fill, and the MMA waiting
     // for the epilogue to drain the single accumulator).  A split adds the sum
     // kernel (~6) and the partial sums' HBM traffic, written once and read once
