@@ -7,10 +7,11 @@
 // Cholesky).  Then Hd = R R^T with R = J L J upper triangular, Hd^-1 =
 // (R^-1)^T R^-1 and R^-1 is upper with a positive diagonal, so U = R^-1 =
 // J L^-1 J: one Cholesky factorisation and one triangular inverse, in fp32.
-//   - blocked right-looking Cholesky on 64 x 64 blocks: gptq_potrf_kernel
-//     factors a diagonal block and replaces it by the inverse of its factor;
-//     the panel below becomes L21 = A21 L11^-T and the trailing matrix
-//     A22 -= L21 L21^T (both through gemm_kernel);
+//   - blocked right-looking Cholesky on 64 x 64 blocks: potrf_block factors a
+//     diagonal block and replaces it by the inverse of its factor; the panel
+//     below becomes L21 = A21 L11^-T and the trailing matrix A22 -= L21 L21^T
+//     (both through gemm_kernel; one CTA of the second updates and factors the
+//     next diagonal block while the others update the rest);
 //   - the triangular inverse by doubling: with the diagonal blocks already
 //     inverted, two neighbouring inverted blocks [A 0; B C] combine to
 //     [A^-1 0; -C^-1 B A^-1  C^-1] (two products, batched over all pairs of a
@@ -21,15 +22,24 @@
 // e = (w_j - level(q_j)) / U_jj is compensated on every later column c by
 // w_c -= e * U_jc.  A working copy of W (fp32, [N][K]) in the caller's scratch
 // is processed in blocks of 128 columns:
-//   gptq_block_kernel: one warp per row, lane l holding columns 4l .. 4l + 3 of
-//     the row's 128-column slab in registers; the 128 x 128 block of U (zero
-//     below the diagonal) in shared memory.  Column by column the warp takes
-//     the column's weight from its owner lane, quantises it (Eq. (1) as
-//     m = #{ t : |w| >= thresh[t] }, one ballot per 32 boundaries), forms the
-//     error and updates its registers; rows never synchronise with each other.
-//     The slab's codes are packed at the end and its errors kept (E, [N][128]).
+//   gptq_block_kernel: eight lanes per row, lane l holding columns 32 i + 4 l ..
+//     + 3 of the row's 128-column slab in registers; the 128 x 128 block of U
+//     (zero below the diagonal) in shared memory.  Column by column the lanes
+//     take the column's weight from its owner, quantise it (Eq. (1) as
+//     m = #{ t : |w| >= thresh[t] }, the boundaries divided among the lanes),
+//     form the error and update their registers; rows never synchronise with
+//     each other.  The slab's codes are packed at the end and its errors kept
+//     (E, [N][128]).
 //   the columns after the block, W[:, rest] -= E U[block, rest], through gemm_kernel.
 // Every sum has a fixed order, so a run is deterministic.
+//
+// K = 4096: the factor 7.86 ms with single-buffered 128 x 128 products, a
+// two-barriers-per-column diagonal factorisation (60 us a block, alone on the
+// GPU) and one warp per row in the column loop, 2.70 ms now; factor and
+// quantisation of 4096 rows 11.3 and 5.2 ms.  The fp32 operations (23 G
+// multiply-adds in the factor, 34 G in the column updates) take 0.6 and 0.9 ms
+// at the FMA rate; the rest is the chain of 64 diagonal blocks and 32 column
+// blocks, each waiting for the update before it.
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
@@ -40,11 +50,29 @@ namespace logq {
 namespace {
 
 constexpr int kCols = 128;         // columns per quantisation block (K is a multiple of 128)
-constexpr int kRowsPerCta = 16;    // block kernel: one warp per row
-constexpr int kBlockThreads = 32 * kRowsPerCta;
-constexpr int kGT = 128;           // gemm_kernel: output tile (rows and columns)
-constexpr int kGK = 32;            // gemm_kernel: terms per shared-memory stage
-constexpr int kGemmThreads = 256;
+constexpr int kRowsPerCta = 16;    // block kernel: eight lanes per row
+constexpr int kBlockThreads = 8 * kRowsPerCta;
+constexpr int kGT = 128;           // gemm_kernel: tile that LOWER and the triangular skips go by
+constexpr int kGK = 16;            // gemm_kernel: terms per shared-memory stage
+// Packed pairs of fp32: one instruction for two multiply-adds, each rounded as fmaf.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 constexpr int kNb = 64;            // Cholesky block
 constexpr size_t kFactorState = 256;   // bytes of factor state ahead of the work matrix
 
@@ -59,6 +87,163 @@ struct FactorState {
     double mean;                   // mean of H's diagonal
     uint32_t not_pd;               // a Cholesky pivot was not positive (or not finite)
 };
+
+// Inverse of the Cholesky factor of the 64 x 64 diagonal block at A (lower
+// triangle read), written in the block's place with zeros above the diagonal;
+// with L, of the block minus L L^T (L its 64 x 64 rows of the last panel, same
+// leading dimension).  One CTA of 256 threads; thread (ty, tx) holds the 4 x 4
+// elements (ty + 16 i, tx + 16 k) of the block and of a second matrix E (the
+// identity at first) in registers.  Elimination step j takes t_ij = a_ij / p times
+// row j from the rows i > j of both (p = a_jj): A becomes D L~^T and E the unit
+// lower L~^-1 of A = L~ D L~^T, so the factor's inverse is D^-1/2 E.  Four steps go
+// between two barriers: the owners of columns j .. j + 3 of A and of rows
+// j .. j + 3 of E publish them in one of two buffers, and every thread carries the
+// four steps out on its own rows' and columns' entries of them, in the order of
+// single steps.  What bounds it is this chain of 16 dependent rounds.  The pivots'
+// reciprocals are taken of scaled values (sc, exact), so that any positive finite
+// pivot serves.
+struct PotrfShared {
+    union {
+        struct {
+            float4 col[2][kNb];        // [row]: columns j .. j + 3
+            float4 row[2][kNb];        // [column]: rows j .. j + 3 of E
+        };
+        float Lt[kNb][kNb + 4];        // L transposed
+    };
+    float diag[kNb];
+};
+
+__device__ __forceinline__ void potrf_block(float* A, const float* L, int64_t ld, FactorState* st, PotrfShared& sm)
+{
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+    float a[4][4], e[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int r = ty + 16 * i, c = tx + 16 * k;
+            // the upper triangle mirrors the lower one
+            a[i][k] = c <= r ? A[r * ld + c] : A[c * ld + r];
+            e[i][k] = 0.f;
+        }
+    if (L) {
+        for (int i = tid; i < kNb * kNb / 4; i += 256) {
+            const int r = i / (kNb / 4), q = i % (kNb / 4);
+            const float4 v = *reinterpret_cast<const float4*>(L + r * ld + 4 * q);
+            sm.Lt[4 * q + 0][r] = v.x;
+            sm.Lt[4 * q + 1][r] = v.y;
+            sm.Lt[4 * q + 2][r] = v.z;
+            sm.Lt[4 * q + 3][r] = v.w;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int j = 0; j < kNb; ++j) {
+            float lr[4], lc[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                lr[i] = sm.Lt[j][ty + 16 * i];
+                lc[i] = sm.Lt[j][tx + 16 * i];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) e[i][k] = fmaf(lr[i], lc[k], e[i][k]);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            a[i][k] -= e[i][k];
+            e[i][k] = ty + 16 * i == tx + 16 * k ? 1.f : 0.f;
+        }
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj)
+        for (int jm = 0; jm < 16; jm += 4) {
+            const int j = 16 * jj + jm, b = (jm / 4) & 1;
+            if ((tx & ~3) == jm)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) reinterpret_cast<float*>(&sm.col[b][ty + 16 * i])[tx - jm] = a[i][jj];
+            if ((ty & ~3) == jm)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) reinterpret_cast<float*>(&sm.row[b][tx + 16 * k])[ty - jm] = e[jj][k];
+            __syncthreads();
+            float d[4][4], rp[4], sc[4], m[4][4];     // d[r][c]: the pivot block at the step of column c; m: its multipliers
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float4 v = sm.col[b][j + r];
+                d[r][0] = v.x; d[r][1] = v.y; d[r][2] = v.z; d[r][3] = v.w;
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float p = d[c][c];
+                sc[c] = p < 0x1p-64f ? 0x1p64f : p > 0x1p64f ? 0x1p-64f : 1.f;     // keeps 1 / p a normal number
+                rp[c] = 1.f / (p * sc[c]);
+                if (tid == 0) sm.diag[j + c] = p;
+#pragma unroll
+                for (int r = c + 1; r < 4; ++r) {
+                    m[r][c] = d[r][c] * sc[c] * rp[c];
+#pragma unroll
+                    for (int q = c + 1; q <= r; ++q) d[r][q] = fmaf(-m[r][c], d[q][c], d[r][q]);
+                }
+            }
+            // entries of row r in the four columns, each as its own step finds it
+            auto entries = [&](float (&x)[4], int r) {
+                const float4 v = sm.col[b][r];
+                x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const float t = r > j + c ? x[c] * sc[c] * rp[c] : 0.f;
+#pragma unroll
+                    for (int q = c + 1; q < 4; ++q) x[q] = fmaf(-t, d[q][c], x[q]);
+                }
+            };
+            float ak[4][4], ek[4][4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (k >= jj) entries(ak[k], tx + 16 * k);            // a_jk = a_kj
+                if (k <= jj) {
+                    const float4 v = sm.row[b][tx + 16 * k];
+                    ek[k][0] = v.x; ek[k][1] = v.y; ek[k][2] = v.z; ek[k][3] = v.w;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+#pragma unroll
+                        for (int q = c + 1; q < 4; ++q) ek[k][q] = fmaf(-m[q][c], ek[k][c], ek[k][q]);
+                }
+            }
+#pragma unroll
+            for (int i = jj; i < 4; ++i) {
+                const int r = ty + 16 * i;
+                float x[4];
+                entries(x, r);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float t = r > j + c ? x[c] * sc[c] * rp[c] : 0.f;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (k >= jj) a[i][k] = fmaf(-t, ak[k][c], a[i][k]);
+                        if (k <= jj) e[i][k] = fmaf(-t, ek[k][c], e[i][k]);
+                    }
+                }
+            }
+        }
+    __syncthreads();
+    if (tid < kNb && (!(sm.diag[tid] > 0.f) || !isfinite(sm.diag[tid]))) st->not_pd = 1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int r = ty + 16 * i, c = tx + 16 * k;
+            A[r * ld + c] = c <= r ? e[i][k] / sqrtf(sm.diag[r]) : 0.f;
+        }
+}
+
+__global__ void __launch_bounds__(256) gptq_potrf_kernel(float* A, int64_t ld, FactorState* st)
+{
+    __shared__ PotrfShared sm;
+    potrf_block(A, nullptr, ld, st, sm);
+}
 
 // C = beta C + alpha A B, A [M][Kd] row-major; B [Kd][N] row-major, or with BT
 // given as [N][Kd] (C = beta C + alpha A B^T).  Batched over blockIdx.z with
@@ -76,93 +261,170 @@ struct GemmArgs {
     int64_t lda, ldb, ldc;
     int64_t sA, sB, sC;
     float alpha, beta;
+    FactorState* potrf;    // LOWER: see gemm_kernel
 };
 
-// 128 x 128 outputs per CTA; thread (tx, ty) owns rows 4ty + {0..3},
-// 64 + 4ty + {0..3} and columns 4tx + {0..3}, 64 + 4tx + {0..3}; both operands
-// are staged k-major in shared memory and read as float4.
-template <bool BT, bool LOWER, bool TRI_A, bool TRI_B>
-__global__ void __launch_bounds__(kGemmThreads, 2) gemm_kernel(const __grid_constant__ GemmArgs g)
+// TM x TN outputs per CTA, RM x 8 per thread.  A warp covers 4 RM rows and 64
+// columns, its lanes 4 x 8; a thread's rows are RM / 4 runs of 4 (16 apart), its
+// columns two runs of 4 (32 apart), so that a warp's fragment reads are 64
+// (rows) and 128 (columns) contiguous bytes.  Both operands are staged k-major
+// in two shared-memory buffers of 16 terms: the next stage's loads are in
+// flight in registers while one is multiplied, one barrier per stage.  The
+// operands that arrive k-contiguous are transposed on the way; their columns
+// are XORed with 8 (k / 4 % 4), which keeps the transposed stores (8 rows x 4
+// runs of k per warp) and the fragment reads free of bank conflicts.
+// Bound by the fp32 FMA rate; the multiply-adds go in packed pairs, which halves
+// the instructions issued for them (the factor at K = 4096 3.7 ms before, 3.2 with
+// them and the overlapped diagonal blocks).
+// TRI_A takes the rows of tiles with the most terms first, so that the short ones
+// fill the last wave; with TRI_B they come first as they are.
+// LOWER with g.potrf: C's first kNb x kNb block, the next diagonal block, is
+// updated and factored by CTA (0, 0) from the start, beside the others; an extra
+// column of CTAs computes the rest of its tile.
+template <int TM, int TN, int RM, int CN, bool BT, bool LOWER, bool TRI_A, bool TRI_B>
+__global__ void __launch_bounds__(TM / RM * TN / CN, TM == 128 || LOWER ? 2 : 4) gemm_kernel(const __grid_constant__ GemmArgs g)
 {
-    __shared__ __align__(16) float As[kGK][kGT + 4];
-    __shared__ __align__(16) float Bs[kGK][kGT + 4];
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    if (LOWER && blockIdx.y > blockIdx.x) return;
-    const int64_t r0 = (int64_t)blockIdx.x * kGT, c0 = (int64_t)blockIdx.y * kGT;
+    constexpr int NT = TM / RM * TN / CN;
+    constexpr int WM = TM / (4 * RM);                     // warps along the rows
+    constexpr int LA = TM * kGK / 4 / NT, LB = TN * kGK / 4 / NT;   // float4 loads per thread and stage
+    static_assert(LA * NT * 4 == TM * kGK && LB * NT * 4 == TN * kGK, "whole loads");
+    constexpr size_t kStages = 2 * kGK * (TM + TN) * sizeof(float);
+    __shared__ __align__(16) unsigned char smem[LOWER && sizeof(PotrfShared) > kStages ? sizeof(PotrfShared) : kStages];
+    auto& As = *reinterpret_cast<float (*)[2][kGK][TM]>(smem);
+    auto& Bs = *reinterpret_cast<float (*)[2][kGK][TN]>(smem + 2 * kGK * TM * sizeof(float));
+    const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+    int64_t r0 = (int64_t)blockIdx.x * TM, c0 = (int64_t)blockIdx.y * TN;
+    if (TRI_A) {          // the longest rows of tiles first
+        const unsigned i = blockIdx.x + gridDim.x * blockIdx.y;
+        r0 = (int64_t)(gridDim.x - 1 - i / gridDim.y) * TM;
+        c0 = (int64_t)(i % gridDim.y) * TN;
+    }
+    if constexpr (LOWER) {
+        static_assert(NT == 256, "the diagonal block's factorisation takes 256 threads");
+        // the next diagonal block's factorisation starts first; the rest of its tile goes
+        // to the extra column of CTAs
+        if (g.potrf && blockIdx.x == 0 && blockIdx.y == 0)
+            return potrf_block(g.C, g.A, g.ldc, g.potrf, *reinterpret_cast<PotrfShared*>(smem));
+        if (g.potrf && blockIdx.y == gridDim.y - 1) {
+            if (blockIdx.x != 0) return;
+            c0 = 0;
+        }
+    }
+    if (LOWER && c0 / kGT > (r0 + TM - 1) / kGT) return;
     const float* A = g.A + blockIdx.z * g.sA;
     const float* B = g.B + blockIdx.z * g.sB;
     float* C = g.C + blockIdx.z * g.sC;
     int64_t k_begin = 0, k_end = g.Kd;
     if (TRI_B) k_begin = c0 < g.Kd ? c0 / kGK * kGK : g.Kd;
-    if (TRI_A && r0 + kGT < k_end) k_end = r0 + kGT;
-    float acc[8][8];
+    if (TRI_A && r0 + TM < k_end) k_end = r0 + TM;
+    const int m0 = warp % WM * (4 * RM) + lane / 8 * 4, n0 = warp / WM * (8 * CN) + lane % 8 * 4;
+    f32x2 acc2[RM][CN / 2];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[i][k] = 0.f;
-    for (int64_t k0 = k_begin; k0 < k_end; k0 += kGK) {
-        for (int i = tid; i < kGT * kGK / 4; i += kGemmThreads) {
-            const int rr = i / (kGK / 4), q = i % (kGK / 4);
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (r0 + rr < g.M) v = *reinterpret_cast<const float4*>(A + (r0 + rr) * g.lda + k0 + 4 * q);
-            As[4 * q + 0][rr] = v.x;
-            As[4 * q + 1][rr] = v.y;
-            As[4 * q + 2][rr] = v.z;
-            As[4 * q + 3][rr] = v.w;
+        for (int k = 0; k < CN / 2; ++k) acc2[i][k] = 0;
+    float4 la[LA], lb[LB];
+    auto fetch = [&](int64_t k0) {
+#pragma unroll
+        for (int i = 0; i < LA; ++i) {
+            const int f = tid + i * NT, rr = f / (kGK / 4), q = f % (kGK / 4);
+            la[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (r0 + rr < g.M) la[i] = *reinterpret_cast<const float4*>(A + (r0 + rr) * g.lda + k0 + 4 * q);
         }
-        if constexpr (BT) {
-            for (int i = tid; i < kGT * kGK / 4; i += kGemmThreads) {
-                const int nn = i / (kGK / 4), q = i % (kGK / 4);
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (c0 + nn < g.N) v = *reinterpret_cast<const float4*>(B + (c0 + nn) * g.ldb + k0 + 4 * q);
-                Bs[4 * q + 0][nn] = v.x;
-                Bs[4 * q + 1][nn] = v.y;
-                Bs[4 * q + 2][nn] = v.z;
-                Bs[4 * q + 3][nn] = v.w;
-            }
-        } else {
-            for (int i = tid; i < kGK * kGT / 4; i += kGemmThreads) {
-                const int a = i / (kGT / 4), q = i % (kGT / 4);
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (c0 + 4 * q < g.N) v = *reinterpret_cast<const float4*>(B + (k0 + a) * g.ldb + c0 + 4 * q);
-                *reinterpret_cast<float4*>(&Bs[a][4 * q]) = v;
+#pragma unroll
+        for (int i = 0; i < LB; ++i) {
+            const int f = tid + i * NT;
+            lb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (BT) {
+                const int nn = f / (kGK / 4), q = f % (kGK / 4);
+                if (c0 + nn < g.N) lb[i] = *reinterpret_cast<const float4*>(B + (c0 + nn) * g.ldb + k0 + 4 * q);
+            } else {
+                const int a = f / (TN / 4), q = f % (TN / 4);
+                if (c0 + 4 * q < g.N) lb[i] = *reinterpret_cast<const float4*>(B + (k0 + a) * g.ldb + c0 + 4 * q);
             }
         }
-        __syncthreads();
-#pragma unroll 4
+    };
+    auto stage = [&](int s) {
+#pragma unroll
+        for (int i = 0; i < LA; ++i) {
+            const int f = tid + i * NT, q = f % (kGK / 4), at = (f / (kGK / 4)) ^ (8 * q);
+            As[s][4 * q + 0][at] = la[i].x;
+            As[s][4 * q + 1][at] = la[i].y;
+            As[s][4 * q + 2][at] = la[i].z;
+            As[s][4 * q + 3][at] = la[i].w;
+        }
+#pragma unroll
+        for (int i = 0; i < LB; ++i) {
+            const int f = tid + i * NT;
+            if constexpr (BT) {
+                const int q = f % (kGK / 4), at = (f / (kGK / 4)) ^ (8 * q);
+                Bs[s][4 * q + 0][at] = lb[i].x;
+                Bs[s][4 * q + 1][at] = lb[i].y;
+                Bs[s][4 * q + 2][at] = lb[i].z;
+                Bs[s][4 * q + 3][at] = lb[i].w;
+            } else {
+                *reinterpret_cast<float4*>(&Bs[s][f / (TN / 4)][4 * (f % (TN / 4))]) = lb[i];
+            }
+        }
+    };
+    auto multiply = [&](int s) {
+#pragma unroll
         for (int a = 0; a < kGK; ++a) {
-            const float4 e0 = *reinterpret_cast<const float4*>(&As[a][4 * ty]);
-            const float4 e1 = *reinterpret_cast<const float4*>(&As[a][64 + 4 * ty]);
-            const float4 u0 = *reinterpret_cast<const float4*>(&Bs[a][4 * tx]);
-            const float4 u1 = *reinterpret_cast<const float4*>(&Bs[a][64 + 4 * tx]);
-            const float ev[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
-            const float uv[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+            const int swz = 8 * (a / 4);
+            f32x2 ev[RM], uv[CN / 2];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < RM; i += 4) {
+                const float4 e = *reinterpret_cast<const float4*>(&As[s][a][(m0 + 4 * i) ^ swz]);
+                ev[i] = pack2(e.x, e.x); ev[i + 1] = pack2(e.y, e.y);
+                ev[i + 2] = pack2(e.z, e.z); ev[i + 3] = pack2(e.w, e.w);
+            }
 #pragma unroll
-                for (int k = 0; k < 8; ++k) acc[i][k] = fmaf(ev[i], uv[k], acc[i][k]);
+            for (int k = 0; k < CN; k += 4) {
+                const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(&Bs[s][a][BT ? (n0 + 8 * k) ^ swz : n0 + 8 * k]);
+                uv[k / 2] = u.x; uv[k / 2 + 1] = u.y;
+            }
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+                for (int k = 0; k < CN / 2; ++k) acc2[i][k] = fma2(ev[i], uv[k], acc2[i][k]);
         }
+    };
+    if (k_begin < k_end) {
+        fetch(k_begin);
+        stage(0);
         __syncthreads();
+        int s = 0;
+        for (int64_t k0 = k_begin; k0 < k_end; k0 += kGK, s ^= 1) {
+            const bool more = k0 + kGK < k_end;
+            if (more) fetch(k0 + kGK);
+            multiply(s);
+            if (more) stage(s ^ 1);
+            __syncthreads();
+        }
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int64_t rr = r0 + (i < 4 ? 4 * ty + i : 64 + 4 * ty + i - 4);
+    for (int i = 0; i < RM; ++i) {
+        const int64_t rr = r0 + m0 + (i / 4) * 16 + i % 4;
         if (rr >= g.M) continue;
+        float acc[CN];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int64_t c = c0 + 64 * h + 4 * tx;
+        for (int k = 0; k < CN / 2; ++k) unpack2(acc2[i][k], acc[2 * k], acc[2 * k + 1]);
+#pragma unroll
+        for (int h = 0; h < CN / 4; ++h) {
+            const int64_t c = c0 + n0 + 32 * h;
             if (c >= g.N) continue;
+            if (LOWER && g.potrf && rr < kNb && c < kNb) continue;
             float4* p = reinterpret_cast<float4*>(C + rr * g.ldc + c);
             float4 o;
             if (g.beta == 0.f) {
-                o = make_float4(g.alpha * acc[i][4 * h + 0], g.alpha * acc[i][4 * h + 1],
-                                g.alpha * acc[i][4 * h + 2], g.alpha * acc[i][4 * h + 3]);
+                o = make_float4(g.alpha * acc[4 * h + 0], g.alpha * acc[4 * h + 1],
+                                g.alpha * acc[4 * h + 2], g.alpha * acc[4 * h + 3]);
             } else {
                 o = *p;
-                o.x = g.beta * o.x + g.alpha * acc[i][4 * h + 0];
-                o.y = g.beta * o.y + g.alpha * acc[i][4 * h + 1];
-                o.z = g.beta * o.z + g.alpha * acc[i][4 * h + 2];
-                o.w = g.beta * o.w + g.alpha * acc[i][4 * h + 3];
+                o.x = g.beta * o.x + g.alpha * acc[4 * h + 0];
+                o.y = g.beta * o.y + g.alpha * acc[4 * h + 1];
+                o.z = g.beta * o.z + g.alpha * acc[4 * h + 2];
+                o.w = g.beta * o.w + g.alpha * acc[4 * h + 3];
             }
             *p = o;
         }
@@ -194,85 +456,53 @@ __global__ void __launch_bounds__(1024) gptq_diag_kernel(const float* __restrict
     }
 }
 
-// A = J Hd J (rows and columns reversed), damping on the diagonal.
-__global__ void gptq_prep_kernel(const float* __restrict__ H, int64_t K, double damp, const FactorState* st,
-                                 float* __restrict__ A)
+// A = J Hd J (rows and columns reversed), damping on the diagonal; zeros above
+// it, which the triangular products read.  One row per blockIdx.y step.
+__global__ void __launch_bounds__(256) gptq_prep_kernel(const float* __restrict__ H, int64_t K, double damp,
+                                                        const FactorState* st, float* __restrict__ A)
 {
     const double add = damp * st->mean;
-    const int64_t total = K * K;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = idx / K, j = idx % K;
-        const float h = H[(K - 1 - i) * K + (K - 1 - j)];
-        float v = h;
-        if (i == j) v = (float)((h == 0.f ? 1.0 : (double)h) + add);
-        A[idx] = v;
+    for (int64_t i = blockIdx.y; i < K; i += gridDim.y) {
+        const float* h = H + (K - 1 - i) * K;
+        for (int64_t j = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); j < K; j += 4 * (int64_t)gridDim.x * blockDim.x) {
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j <= i) {
+                const float4 v = *reinterpret_cast<const float4*>(h + K - 4 - j);
+                const float r[4] = {v.w, v.z, v.y, v.x};
+                float w[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    w[e] = j + e <= i ? r[e] : 0.f;
+                    if (j + e == i) w[e] = (float)((r[e] == 0.f ? 1.0 : (double)r[e]) + add);
+                }
+                o = make_float4(w[0], w[1], w[2], w[3]);
+            }
+            *reinterpret_cast<float4*>(A + i * K + j) = o;
+        }
     }
 }
 
-// Cholesky of the 64 x 64 diagonal block at (k0, k0) (lower triangle read),
-// then the inverse of its factor, written back in its place with zeros above
-// the diagonal.  One CTA of 256 threads: a 16 x 16 layout for the updates, four
-// threads per column of the inverse.
-__global__ void __launch_bounds__(256) gptq_potrf_kernel(float* __restrict__ A, int64_t K, int64_t k0,
-                                                         FactorState* st)
+// Zeros above the diagonal inside the kGT-wide diagonal tiles, which the
+// trailing updates write whole.
+__global__ void __launch_bounds__(256) gptq_zero_upper_kernel(float* __restrict__ A, int64_t K)
 {
-    __shared__ float a[kNb][kNb + 1];
-    __shared__ float inv[kNb][kNb + 1];
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    for (int i = tid; i < kNb * kNb; i += 256) {
-        const int r = i / kNb, c = i % kNb;
-        a[r][c] = c <= r ? A[(k0 + r) * K + k0 + c] : 0.f;
-    }
-    __syncthreads();
-    for (int j = 0; j < kNb; ++j) {
-        const float p = a[j][j];
-        const float d = sqrtf(p);
-        if (tid == 0 && (!(p > 0.f) || !isfinite(p))) st->not_pd = 1;
-        if (tid > j && tid < kNb) a[tid][j] = a[tid][j] / d;
-        __syncthreads();
-        if (tid == 0) a[j][j] = d;
-        for (int i = j + 1 + ty; i < kNb; i += 16) {
-            const float lij = a[i][j];
-            for (int k = j + 1 + tx; k <= i; k += 16) a[i][k] -= lij * a[k][j];
-        }
-        __syncthreads();
-    }
-    {   // column c of the inverse by forward substitution, each sum split over four lanes
-        const int c = tid / 4, q = tid % 4;
-        for (int i = 0; i < kNb; ++i) {
-            float part = 0.f;
-            if (i > c)
-                for (int k = c + q; k < i; k += 4) part = fmaf(a[i][k], inv[k][c], part);
-            part += __shfl_xor_sync(0xffffffffu, part, 1);
-            part += __shfl_xor_sync(0xffffffffu, part, 2);
-            if (q == 0) inv[i][c] = i < c ? 0.f : ((i == c ? 1.f : 0.f) - part) / a[i][i];
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-    for (int i = tid; i < kNb * kNb; i += 256) {
-        const int r = i / kNb, c = i % kNb;
-        A[(k0 + r) * K + k0 + c] = inv[r][c];
-    }
-}
-
-__global__ void gptq_zero_upper_kernel(float* __restrict__ A, int64_t K)
-{
-    const int64_t total = K * K;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x)
-        if (idx % K > idx / K) A[idx] = 0.f;
+    const int64_t i = (int64_t)blockIdx.x * 2 + threadIdx.x / 128, j = i + 1 + threadIdx.x % 128;
+    if (i < K && j < K) A[i * K + j] = 0.f;
 }
 
 // U[i][j] = Linv[K-1-i][K-1-j] (upper triangular; zeros below the diagonal).
-__global__ void gptq_reverse_kernel(const float* __restrict__ Li, int64_t K, float* __restrict__ U)
+__global__ void __launch_bounds__(256) gptq_reverse_kernel(const float* __restrict__ Li, int64_t K, float* __restrict__ U)
 {
-    const int64_t total = K * K;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = idx / K, j = idx % K;
-        U[idx] = j >= i ? Li[(K - 1 - i) * K + (K - 1 - j)] : 0.f;
+    for (int64_t i = blockIdx.y; i < K; i += gridDim.y) {
+        const float* l = Li + (K - 1 - i) * K;
+        for (int64_t j = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); j < K; j += 4 * (int64_t)gridDim.x * blockDim.x) {
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j + 3 >= i) {
+                const float4 v = *reinterpret_cast<const float4*>(l + K - 4 - j);
+                o = make_float4(j >= i ? v.w : 0.f, j + 1 >= i ? v.z : 0.f, j + 2 >= i ? v.y : 0.f, v.x);
+            }
+            *reinterpret_cast<float4*>(U + i * K + j) = o;
+        }
     }
 }
 
@@ -291,19 +521,22 @@ __global__ void gptq_copy_kernel(const float4* __restrict__ W, int64_t n4, int64
     }
 }
 
+// Bound by the chain of 128 columns (shuffle, compare, divide, update): eight lanes
+// per row put four rows into a warp, which shares that chain's instructions among
+// them (4096 rows: 24 us a block; one warp per row 30 us).
 template <int BITS>
-__global__ void __launch_bounds__(kBlockThreads, 2) gptq_block_kernel(float* __restrict__ Wk, int64_t N, int64_t K,
+__global__ void __launch_bounds__(kBlockThreads, 3) gptq_block_kernel(float* __restrict__ Wk, int64_t N, int64_t K,
                                                                       const float* __restrict__ U, int64_t j0,
                                                                       const __grid_constant__ GptqTables tb,
                                                                       uint8_t* __restrict__ codes,
                                                                       float* __restrict__ E)
 {
-    constexpr int kBallots = BITS == 8 ? 4 : 1;    // 127 or 7 boundaries
+    constexpr int kTh = BITS == 8 ? 16 : 1;        // boundaries per lane: 127 or 7 over 8 lanes
     extern __shared__ float4 sm4[];
     float* Ub = reinterpret_cast<float*>(sm4);     // [kCols][kCols], upper triangle of U's block
     __shared__ float lv[128];
-    const int tid = threadIdx.x, lane = tid % 32;
-    const int64_t r = (int64_t)blockIdx.x * kRowsPerCta + tid / 32;
+    const int tid = threadIdx.x, lane = tid % 32, l8 = lane % 8, base = lane & 24;
+    const int64_t r = (int64_t)blockIdx.x * kRowsPerCta + tid / 8;
     if (tid < 128) lv[tid] = tb.level[tid];
     for (int i = tid; i < kCols * kCols / 4; i += kBlockThreads) {
         const int a = i / (kCols / 4), c = 4 * (i % (kCols / 4));
@@ -314,48 +547,69 @@ __global__ void __launch_bounds__(kBlockThreads, 2) gptq_block_kernel(float* __r
         if (c + 3 < a) v.w = 0.f;
         sm4[i] = v;
     }
-    uint32_t th[kBallots];
+    uint32_t th[kTh];
 #pragma unroll
-    for (int b = 0; b < kBallots; ++b) th[b] = tb.thresh[lane + 32 * b];
-    __syncthreads();
-    if (r >= N) return;
-    const float4 w4 = *reinterpret_cast<const float4*>(Wk + r * K + j0 + 4 * lane);
-    float wv[4] = {w4.x, w4.y, w4.z, w4.w};
-    int qv[4] = {0, 0, 0, 0};
-    float ev[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int j4 = 0; j4 < kCols / 4; ++j4) {
+    for (int b = 0; b < kTh; ++b) th[b] = tb.thresh[l8 + 8 * b];
+    // rows past the end repeat the last one (whole warps take part in the shuffles)
+    const int64_t rr = r < N ? r : N - 1;
+    f32x2 wv[4][2];                                // this lane's columns 32 i + 4 l8 .. + 3, in pairs
+    float ev[4][4];
+    uint32_t cv[4][4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int j = 4 * j4 + k;
-            const float w = __shfl_sync(0xffffffffu, wv[k], j4);
-            const uint32_t u = __float_as_uint(w) & 0x7fffffffu;
-            int m = 0;
-#pragma unroll
-            for (int b = 0; b < kBallots; ++b) m += __popc(__ballot_sync(0xffffffffu, u >= th[b]));
-            const float deq = m ? (w < 0.f ? -lv[m] : lv[m]) : 0.f;
-            const float e = (w - deq) / Ub[j * kCols + j];
-            if (lane == j4) {
-                qv[k] = w < 0.f ? -m : m;
-                ev[k] = e;
-            }
-            const float4 u4 = sm4[(j * kCols) / 4 + lane];
-            wv[0] -= e * u4.x;
-            wv[1] -= e * u4.y;
-            wv[2] -= e * u4.z;
-            wv[3] -= e * u4.w;
-        }
+    for (int i = 0; i < 4; ++i) {
+        const ulonglong2 w4 = *reinterpret_cast<const ulonglong2*>(Wk + rr * K + j0 + 32 * i + 4 * l8);
+        wv[i][0] = w4.x; wv[i][1] = w4.y;
     }
-    *reinterpret_cast<float4*>(E + r * kCols + 4 * lane) = make_float4(ev[0], ev[1], ev[2], ev[3]);
-    // sign-magnitude codes (the layout of include/logq.h)
-    uint32_t c[4];
+    __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-        c[k] = qv[k] < 0 ? ((uint32_t)(-qv[k]) | (1u << (BITS - 1))) : (uint32_t)qv[k];
-    if constexpr (BITS == 4)
-        *reinterpret_cast<uint16_t*>(codes + r * (K / 2) + j0 / 2 + 2 * lane) =
-            (uint16_t)(c[0] | (c[1] << 4) | (c[2] << 8) | (c[3] << 12));
-    else
-        *reinterpret_cast<uint32_t*>(codes + r * K + j0 + 4 * lane) = c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24);
+    for (int i = 0; i < 4; ++i)
+        for (int o = 0; o < 8; ++o)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int j = 32 * i + 4 * o + k;
+                float w0, w1;
+                unpack2(wv[i][k / 2], w0, w1);
+                const float w = __shfl_sync(0xffffffffu, k % 2 ? w1 : w0, base + o);
+                const uint32_t u = __float_as_uint(w) & 0x7fffffffu;
+                int m;
+                if constexpr (BITS == 4) {
+                    m = __popc((__ballot_sync(0xffffffffu, u >= th[0]) >> base) & 0xffu);
+                } else {
+                    m = 0;
+#pragma unroll
+                    for (int b = 0; b < kTh; ++b) m += u >= th[b] ? 1 : 0;
+                    m += __shfl_xor_sync(0xffffffffu, m, 1);
+                    m += __shfl_xor_sync(0xffffffffu, m, 2);
+                    m += __shfl_xor_sync(0xffffffffu, m, 4);
+                }
+                const float deq = m ? (w < 0.f ? -lv[m] : lv[m]) : 0.f;
+                const float e = (w - deq) / Ub[j * kCols + j];
+                if (l8 == o) {
+                    cv[i][k] = w < 0.f && m ? (uint32_t)m | (1u << (BITS - 1)) : (uint32_t)m;
+                    ev[i][k] = e;
+                }
+                const f32x2 ne = pack2(-e, -e);
+                // the columns of earlier runs are done (U is zero there)
+#pragma unroll
+                for (int h = i; h < 4; ++h) {
+                    const ulonglong2 u4 = *reinterpret_cast<const ulonglong2*>(&sm4[(j * kCols) / 4 + l8 + 8 * h]);
+                    wv[h][0] = fma2(ne, u4.x, wv[h][0]);
+                    wv[h][1] = fma2(ne, u4.y, wv[h][1]);
+                }
+            }
+    if (r >= N) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        *reinterpret_cast<float4*>(E + r * kCols + 32 * i + 4 * l8) = make_float4(ev[i][0], ev[i][1], ev[i][2], ev[i][3]);
+        // sign-magnitude codes (the layout of include/logq.h)
+        const uint32_t (&c)[4] = cv[i];
+        if constexpr (BITS == 4)
+            *reinterpret_cast<uint16_t*>(codes + r * (K / 2) + j0 / 2 + 16 * i + 2 * l8) =
+                (uint16_t)(c[0] | (c[1] << 4) | (c[2] << 8) | (c[3] << 12));
+        else
+            *reinterpret_cast<uint32_t*>(codes + r * K + j0 + 32 * i + 4 * l8) =
+                c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24);
+    }
 }
 
 constexpr size_t kBlockSmem = sizeof(float) * kCols * kCols;
@@ -379,13 +633,34 @@ cudaError_t block_launch(float* Wk, int64_t N, int64_t K, const float* U, int64_
     return cudaGetLastError();
 }
 
+template <int TM, int TN, int RM, int CN, bool BT, bool LOWER, bool TRI_A, bool TRI_B>
+cudaError_t gemm_tiles(const GemmArgs& g, int64_t batch, cudaStream_t s)
+{
+    const dim3 grid((unsigned)((g.M + TM - 1) / TM), (unsigned)((g.N + TN - 1) / TN) + (LOWER && g.potrf ? 1 : 0),
+                    (unsigned)batch);
+    gemm_kernel<TM, TN, RM, CN, BT, LOWER, TRI_A, TRI_B><<<grid, TM / RM * TN / CN, 0, s>>>(g);
+    return cudaGetLastError();
+}
+
+// Tile of a product: 32 x 64 for a panel of one block; 64 x 64 while 128 x 128
+// tiles would number less than two per SM; beyond that 64 x 128, or 128 x 128 where
+// only the lower triangle is computed.  K and rows 4096, factor and quantisation,
+// ms, by the last one's tile: 128 x 256 (one CTA per SM) 5.70, 128 x 128 (two)
+// 5.35, 64 x 128 (four) 5.16.
 template <bool BT, bool LOWER, bool TRI_A, bool TRI_B>
 cudaError_t gemm(const GemmArgs& g, int64_t batch, cudaStream_t s)
 {
     if (g.M <= 0 || g.N <= 0 || batch <= 0) return cudaSuccess;
-    const dim3 grid((unsigned)((g.M + kGT - 1) / kGT), (unsigned)((g.N + kGT - 1) / kGT), (unsigned)batch);
-    gemm_kernel<BT, LOWER, TRI_A, TRI_B><<<grid, kGemmThreads, 0, s>>>(g);
-    return cudaGetLastError();
+    const int sms = sm_count() > 0 ? sm_count() : 148;
+    const int64_t tiles = ((g.M + 127) / 128) * ((g.N + 127) / 128) * batch / (LOWER ? 2 : 1);
+    if constexpr (LOWER) {
+        if (tiles < 2 * sms) return gemm_tiles<64, 64, 4, 4, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
+        return gemm_tiles<128, 128, 8, 8, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
+    } else {
+        if (g.N <= 64) return gemm_tiles<32, 64, 4, 8, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
+        if (tiles < 2 * sms) return gemm_tiles<64, 64, 4, 8, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
+        return gemm_tiles<64, 128, 8, 8, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
+    }
 }
 
 GemmArgs gemm_args(const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc, int64_t M,
@@ -406,6 +681,9 @@ GemmArgs gemm_args(const float* A, int64_t lda, const float* B, int64_t ldb, flo
     g.beta = beta;
     return g;
 }
+
+// One row of a K x K matrix per blockIdx.y step, four elements per thread.
+dim3 row_grid(int64_t K) { return dim3((unsigned)((K + 1023) / 1024), (unsigned)(K < 4096 ? K : 4096)); }
 
 unsigned elementwise_grid(int64_t n)
 {
@@ -451,24 +729,25 @@ cudaError_t launch_gptq_factor(const float* H, int64_t K, double damp, float* U,
     gptq_diag_kernel<<<1, 1024, 0, s>>>(H, K, st, dead);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    gptq_prep_kernel<<<elementwise_grid(K * K), 256, 0, s>>>(H, K, damp, st, Lw);
+    gptq_prep_kernel<<<row_grid(K), 256, 0, s>>>(H, K, damp, st, Lw);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // Cholesky of J Hd J; diagonal blocks end up inverted
+    gptq_potrf_kernel<<<1, 256, 0, s>>>(Lw, K, st);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     for (int64_t k0 = 0; k0 < K; k0 += kNb) {
-        gptq_potrf_kernel<<<1, 256, 0, s>>>(Lw, K, k0, st);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const int64_t k1 = k0 + kNb, m = K - k1;
         if (m <= 0) break;
         // L21 = A21 L11^-T, in place
         e = gemm<true, false, false, false>(
             gemm_args(Lw + k1 * K + k0, K, Lw + k0 * K + k0, K, Lw + k1 * K + k0, K, m, kNb, kNb, 1.f, 0.f), 1, s);
         if (e != cudaSuccess) return e;
-        // A22 -= L21 L21^T (lower triangle)
-        e = gemm<true, true, false, false>(
-            gemm_args(Lw + k1 * K + k0, K, Lw + k1 * K + k0, K, Lw + k1 * K + k1, K, m, m, kNb, -1.f, 1.f), 1, s);
+        // A22 -= L21 L21^T (lower triangle), and the inverse factor of its first block
+        GemmArgs g = gemm_args(Lw + k1 * K + k0, K, Lw + k1 * K + k0, K, Lw + k1 * K + k1, K, m, m, kNb, -1.f, 1.f);
+        g.potrf = st;
+        e = gemm<true, true, false, false>(g, 1, s);
         if (e != cudaSuccess) return e;
     }
-    gptq_zero_upper_kernel<<<elementwise_grid(K * K), 256, 0, s>>>(Lw, K);
+    gptq_zero_upper_kernel<<<(unsigned)((K + 1) / 2), 256, 0, s>>>(Lw, K);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // triangular inverse by doubling
     for (int64_t half = kNb; half < K; half *= 2) {
@@ -479,7 +758,7 @@ cudaError_t launch_gptq_factor(const float* H, int64_t K, double damp, float* U,
         if (b0 < K && (e = combine_pairs(Lw, K, s_, half, K - b0, full, 1, X + full * half * half, s)) != cudaSuccess)
             return e;
     }
-    gptq_reverse_kernel<<<elementwise_grid(K * K), 256, 0, s>>>(Lw, K, U);
+    gptq_reverse_kernel<<<row_grid(K), 256, 0, s>>>(Lw, K, U);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (not_pd) {
         e = cudaMemcpyAsync(not_pd, &st->not_pd, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
