@@ -10,8 +10,8 @@
 //   - blocked right-looking Cholesky on 64 x 64 blocks: potrf_block factors a
 //     diagonal block and replaces it by the inverse of its factor; the panel
 //     below becomes L21 = A21 L11^-T and the trailing matrix A22 -= L21 L21^T
-//     (both through gemm_kernel; one CTA of the second updates and factors the
-//     next diagonal block while the others update the rest);
+//     (both through gptq_rank64_kernel; one CTA of the second updates and factors
+//     the next diagonal block while the others update the rest);
 //   - the triangular inverse by doubling: with the diagonal blocks already
 //     inverted, two neighbouring inverted blocks [A 0; B C] combine to
 //     [A^-1 0; -C^-1 B A^-1  C^-1] (two products, batched over all pairs of a
@@ -35,8 +35,8 @@
 //
 // K = 4096: the factor 7.86 ms with single-buffered 128 x 128 products, a
 // two-barriers-per-column diagonal factorisation (60 us a block, alone on the
-// GPU) and one warp per row in the column loop, 2.70 ms now; factor and
-// quantisation of 4096 rows 11.3 and 5.2 ms.  The fp32 operations (23 G
+// GPU) and one warp per row in the column loop, 2.45 ms now; factor and
+// quantisation of 4096 rows 11.3 and 5.0 ms.  The fp32 operations (23 G
 // multiply-adds in the factor, 34 G in the column updates) take 0.6 and 0.9 ms
 // at the FMA rate; the rest is the chain of 64 diagonal blocks and 32 column
 // blocks, each waiting for the update before it.
@@ -52,7 +52,6 @@ namespace {
 constexpr int kCols = 128;         // columns per quantisation block (K is a multiple of 128)
 constexpr int kRowsPerCta = 16;    // block kernel: eight lanes per row
 constexpr int kBlockThreads = 8 * kRowsPerCta;
-constexpr int kGT = 128;           // gemm_kernel: tile that LOWER and the triangular skips go by
 constexpr int kGK = 16;            // gemm_kernel: terms per shared-memory stage
 // Packed pairs of fp32: one instruction for two multiply-adds, each rounded as fmaf.
 using f32x2 = unsigned long long;
@@ -96,17 +95,20 @@ struct FactorState {
 // identity at first) in registers.  Elimination step j takes t_ij = a_ij / p times
 // row j from the rows i > j of both (p = a_jj): A becomes D L~^T and E the unit
 // lower L~^-1 of A = L~ D L~^T, so the factor's inverse is D^-1/2 E.  Four steps go
-// between two barriers: the owners of columns j .. j + 3 of A and of rows
-// j .. j + 3 of E publish them in one of two buffers, and every thread carries the
-// four steps out on its own rows' and columns' entries of them, in the order of
-// single steps.  What bounds it is this chain of 16 dependent rounds.  The pivots'
-// reciprocals are taken of scaled values (sc, exact), so that any positive finite
-// pivot serves.
+// in one round of two barriers: the owners of columns j .. j + 3 of A and of rows
+// j .. j + 3 of E publish them; 64 threads each carry the four steps out on a row
+// of those columns and 64 on a column of those rows, in the order of single steps,
+// and publish what each step finds there; then every thread updates its elements.
+// What bounds it is this chain of 16 dependent rounds.  The pivots' reciprocals
+// are taken of scaled values (sc, exact), so that any positive finite pivot serves.
 struct PotrfShared {
     union {
         struct {
-            float4 col[2][kNb];        // [row]: columns j .. j + 3
-            float4 row[2][kNb];        // [column]: rows j .. j + 3 of E
+            float4 col[kNb];           // [row]: columns j .. j + 3
+            float4 row[kNb];           // [column]: rows j .. j + 3 of E
+            // per step c, [r % 16][r / 16] as a thread reads its four: multipliers t of the
+            // rows, entries of the columns (a_jk = a_kj) and of E's row
+            float t[4][16][4], x[4][16][4], e[4][16][4];
         };
         float Lt[kNb][kNb + 4];        // L transposed
     };
@@ -116,15 +118,15 @@ struct PotrfShared {
 __device__ __forceinline__ void potrf_block(float* A, const float* L, int64_t ld, FactorState* st, PotrfShared& sm)
 {
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    float a[4][4], e[4][4];
+    float a0[4][4], e0[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int r = ty + 16 * i, c = tx + 16 * k;
             // the upper triangle mirrors the lower one
-            a[i][k] = c <= r ? A[r * ld + c] : A[c * ld + r];
-            e[i][k] = 0.f;
+            a0[i][k] = c <= r ? A[r * ld + c] : A[c * ld + r];
+            e0[i][k] = 0.f;
         }
     if (L) {
         for (int i = tid; i < kNb * kNb / 4; i += 256) {
@@ -147,84 +149,91 @@ __device__ __forceinline__ void potrf_block(float* A, const float* L, int64_t ld
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) e[i][k] = fmaf(lr[i], lc[k], e[i][k]);
+                for (int k = 0; k < 4; ++k) e0[i][k] = fmaf(lr[i], lc[k], e0[i][k]);
         }
         __syncthreads();
     }
+    f32x2 a[4][2], e[4][2];            // pairs (k, k + 1)
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            a[i][k] -= e[i][k];
-            e[i][k] = ty + 16 * i == tx + 16 * k ? 1.f : 0.f;
+        for (int k = 0; k < 4; k += 2) {
+            a[i][k / 2] = pack2(a0[i][k] - e0[i][k], a0[i][k + 1] - e0[i][k + 1]);
+            e[i][k / 2] = pack2(ty + 16 * i == tx + 16 * k ? 1.f : 0.f, ty + 16 * i == tx + 16 * (k + 1) ? 1.f : 0.f);
         }
 #pragma unroll
     for (int jj = 0; jj < 4; ++jj)
         for (int jm = 0; jm < 16; jm += 4) {
-            const int j = 16 * jj + jm, b = (jm / 4) & 1;
+            const int j = 16 * jj + jm;
             if ((tx & ~3) == jm)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) reinterpret_cast<float*>(&sm.col[b][ty + 16 * i])[tx - jm] = a[i][jj];
+                for (int i = 0; i < 4; ++i) {
+                    float v[2];
+                    unpack2(a[i][jj / 2], v[0], v[1]);
+                    reinterpret_cast<float*>(&sm.col[ty + 16 * i])[tx - jm] = v[jj % 2];
+                }
             if ((ty & ~3) == jm)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) reinterpret_cast<float*>(&sm.row[b][tx + 16 * k])[ty - jm] = e[jj][k];
+                for (int k = 0; k < 4; k += 2) {
+                    float v[2];
+                    unpack2(e[jj][k / 2], v[0], v[1]);
+                    reinterpret_cast<float*>(&sm.row[tx + 16 * k])[ty - jm] = v[0];
+                    reinterpret_cast<float*>(&sm.row[tx + 16 * (k + 1)])[ty - jm] = v[1];
+                }
             __syncthreads();
-            float d[4][4], rp[4], sc[4], m[4][4];     // d[r][c]: the pivot block at the step of column c; m: its multipliers
+            if (tid < 2 * kNb) {
+                float d[4][4], rp[4], sc[4], m[4][4];     // d[r][c]: the pivot block at the step of column c; m: its multipliers
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float4 v = sm.col[b][j + r];
-                d[r][0] = v.x; d[r][1] = v.y; d[r][2] = v.z; d[r][3] = v.w;
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const float p = d[c][c];
-                sc[c] = p < 0x1p-64f ? 0x1p64f : p > 0x1p64f ? 0x1p-64f : 1.f;     // keeps 1 / p a normal number
-                rp[c] = 1.f / (p * sc[c]);
-                if (tid == 0) sm.diag[j + c] = p;
-#pragma unroll
-                for (int r = c + 1; r < 4; ++r) {
-                    m[r][c] = d[r][c] * sc[c] * rp[c];
-#pragma unroll
-                    for (int q = c + 1; q <= r; ++q) d[r][q] = fmaf(-m[r][c], d[q][c], d[r][q]);
+                for (int r = 0; r < 4; ++r) {
+                    const float4 v = sm.col[j + r];
+                    d[r][0] = v.x; d[r][1] = v.y; d[r][2] = v.z; d[r][3] = v.w;
                 }
-            }
-            // entries of row r in the four columns, each as its own step finds it
-            auto entries = [&](float (&x)[4], int r) {
-                const float4 v = sm.col[b][r];
-                x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const float t = r > j + c ? x[c] * sc[c] * rp[c] : 0.f;
-#pragma unroll
-                    for (int q = c + 1; q < 4; ++q) x[q] = fmaf(-t, d[q][c], x[q]);
-                }
-            };
-            float ak[4][4], ek[4][4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (k >= jj) entries(ak[k], tx + 16 * k);            // a_jk = a_kj
-                if (k <= jj) {
-                    const float4 v = sm.row[b][tx + 16 * k];
-                    ek[k][0] = v.x; ek[k][1] = v.y; ek[k][2] = v.z; ek[k][3] = v.w;
-#pragma unroll
-                    for (int c = 0; c < 3; ++c)
-#pragma unroll
-                        for (int q = c + 1; q < 4; ++q) ek[k][q] = fmaf(-m[q][c], ek[k][c], ek[k][q]);
-                }
-            }
-#pragma unroll
-            for (int i = jj; i < 4; ++i) {
-                const int r = ty + 16 * i;
-                float x[4];
-                entries(x, r);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    const float t = r > j + c ? x[c] * sc[c] * rp[c] : 0.f;
+                    const float p = d[c][c];
+                    sc[c] = p < 0x1p-64f ? 0x1p64f : p > 0x1p64f ? 0x1p-64f : 1.f;     // keeps 1 / p a normal number
+                    rp[c] = 1.f / (p * sc[c]);
+                    if (tid == 0) sm.diag[j + c] = p;
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        if (k >= jj) a[i][k] = fmaf(-t, ak[k][c], a[i][k]);
-                        if (k <= jj) e[i][k] = fmaf(-t, ek[k][c], e[i][k]);
+                    for (int r = c + 1; r < 4; ++r) {
+                        m[r][c] = d[r][c] * sc[c] * rp[c];
+#pragma unroll
+                        for (int q = c + 1; q <= r; ++q) d[r][q] = fmaf(-m[r][c], d[q][c], d[r][q]);
                     }
+                }
+                const int r = tid % kNb;
+                const float4 v = tid < kNb ? sm.col[r] : sm.row[r];
+                float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    float t[4];
+                    if (tid < kNb) {
+                        t[c] = r > j + c ? x[c] * sc[c] * rp[c] : 0.f;
+                        sm.t[c][r % 16][r / 16] = t[c];
+                        sm.x[c][r % 16][r / 16] = x[c];
+#pragma unroll
+                        for (int q = c + 1; q < 4; ++q) x[q] = fmaf(-t[c], d[q][c], x[q]);
+                    } else {
+                        sm.e[c][r % 16][r / 16] = x[c];
+#pragma unroll
+                        for (int q = c + 1; q < 4; ++q) x[q] = fmaf(-m[q][c], x[c], x[q]);
+                    }
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float4 tv = *reinterpret_cast<const float4*>(sm.t[c][ty]);
+                const ulonglong2 xv = *reinterpret_cast<const ulonglong2*>(sm.x[c][tx]);
+                const ulonglong2 ev = *reinterpret_cast<const ulonglong2*>(sm.e[c][tx]);
+                const float t[4] = {tv.x, tv.y, tv.z, tv.w};
+#pragma unroll
+                for (int i = jj; i < 4; ++i) {
+                    const f32x2 nt = pack2(-t[i], -t[i]);
+                    if (jj < 2) a[i][0] = fma2(nt, xv.x, a[i][0]);
+                    a[i][1] = fma2(nt, xv.y, a[i][1]);
+                    e[i][0] = fma2(nt, ev.x, e[i][0]);
+                    if (jj >= 2) e[i][1] = fma2(nt, ev.y, e[i][1]);
                 }
             }
         }
@@ -233,9 +242,12 @@ __device__ __forceinline__ void potrf_block(float* A, const float* L, int64_t ld
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 4; k += 2) {
+            float v[2];
+            unpack2(e[i][k / 2], v[0], v[1]);
             const int r = ty + 16 * i, c = tx + 16 * k;
-            A[r * ld + c] = c <= r ? e[i][k] / sqrtf(sm.diag[r]) : 0.f;
+            A[r * ld + c] = c <= r ? v[0] / sqrtf(sm.diag[r]) : 0.f;
+            A[r * ld + c + 16] = c + 16 <= r ? v[1] / sqrtf(sm.diag[r]) : 0.f;
         }
 }
 
@@ -245,14 +257,12 @@ __global__ void __launch_bounds__(256) gptq_potrf_kernel(float* A, int64_t ld, F
     potrf_block(A, nullptr, ld, st, sm);
 }
 
-// C = beta C + alpha A B, A [M][Kd] row-major; B [Kd][N] row-major, or with BT
-// given as [N][Kd] (C = beta C + alpha A B^T).  Batched over blockIdx.z with
-// element strides sA, sB, sC.  Kd is a multiple of 32; N, the leading
-// dimensions and the batch strides are multiples of 4 and the bases 16-byte
-// aligned.  LOWER: tiles strictly above the diagonal are skipped.  TRI_A: A is
-// lower triangular (A[m][k] = 0 for k > m), TRI_B: B is lower triangular
-// (B[k][n] = 0 for k < n); the stages that hold only such zeros are skipped,
-// the others read the zeros, which must be stored.
+// C = beta C + alpha A B, A [M][Kd] and B [Kd][N] row-major.  Batched over
+// blockIdx.z with element strides sA, sB, sC.  Kd is a multiple of 32; N, the
+// leading dimensions and the batch strides are multiples of 4 and the bases
+// 16-byte aligned.  TRI_A: A is lower triangular (A[m][k] = 0 for k > m), TRI_B:
+// B is lower triangular (B[k][n] = 0 for k < n); the stages that hold only such
+// zeros are skipped, the others read the zeros, which must be stored.
 struct GemmArgs {
     const float* A;
     const float* B;
@@ -261,7 +271,6 @@ struct GemmArgs {
     int64_t lda, ldb, ldc;
     int64_t sA, sB, sC;
     float alpha, beta;
-    FactorState* potrf;    // LOWER: see gemm_kernel
 };
 
 // TM x TN outputs per CTA, RM x 8 per thread.  A warp covers 4 RM rows and 64
@@ -269,29 +278,25 @@ struct GemmArgs {
 // columns two runs of 4 (32 apart), so that a warp's fragment reads are 64
 // (rows) and 128 (columns) contiguous bytes.  Both operands are staged k-major
 // in two shared-memory buffers of 16 terms: the next stage's loads are in
-// flight in registers while one is multiplied, one barrier per stage.  The
-// operands that arrive k-contiguous are transposed on the way; their columns
-// are XORed with 8 (k / 4 % 4), which keeps the transposed stores (8 rows x 4
-// runs of k per warp) and the fragment reads free of bank conflicts.
+// flight in registers while one is multiplied, one barrier per stage.  A, which
+// arrives k-contiguous, is transposed on the way; its columns are XORed with
+// 8 (k / 4 % 4), which keeps the transposed stores (8 rows x 4 runs of k per warp)
+// and the fragment reads free of bank conflicts.
 // Bound by the fp32 FMA rate; the multiply-adds go in packed pairs, which halves
 // the instructions issued for them (the factor at K = 4096 3.7 ms before, 3.2 with
 // them and the overlapped diagonal blocks).
 // TRI_A takes the rows of tiles with the most terms first, so that the short ones
 // fill the last wave; with TRI_B they come first as they are.
-// LOWER with g.potrf: C's first kNb x kNb block, the next diagonal block, is
-// updated and factored by CTA (0, 0) from the start, beside the others; an extra
-// column of CTAs computes the rest of its tile.
-template <int TM, int TN, int RM, int CN, bool BT, bool LOWER, bool TRI_A, bool TRI_B>
-__global__ void __launch_bounds__(TM / RM * TN / CN, TM == 128 || LOWER ? 2 : 4) gemm_kernel(const __grid_constant__ GemmArgs g)
+template <int TM, int TN, int RM, bool TRI_A, bool TRI_B>
+__global__ void __launch_bounds__(TM / RM * TN / 8, 4) gemm_kernel(const __grid_constant__ GemmArgs g)
 {
+    constexpr int CN = 8;
     constexpr int NT = TM / RM * TN / CN;
     constexpr int WM = TM / (4 * RM);                     // warps along the rows
     constexpr int LA = TM * kGK / 4 / NT, LB = TN * kGK / 4 / NT;   // float4 loads per thread and stage
     static_assert(LA * NT * 4 == TM * kGK && LB * NT * 4 == TN * kGK, "whole loads");
-    constexpr size_t kStages = 2 * kGK * (TM + TN) * sizeof(float);
-    __shared__ __align__(16) unsigned char smem[LOWER && sizeof(PotrfShared) > kStages ? sizeof(PotrfShared) : kStages];
-    auto& As = *reinterpret_cast<float (*)[2][kGK][TM]>(smem);
-    auto& Bs = *reinterpret_cast<float (*)[2][kGK][TN]>(smem + 2 * kGK * TM * sizeof(float));
+    __shared__ __align__(16) float As[2][kGK][TM];
+    __shared__ __align__(16) float Bs[2][kGK][TN];
     const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
     int64_t r0 = (int64_t)blockIdx.x * TM, c0 = (int64_t)blockIdx.y * TN;
     if (TRI_A) {          // the longest rows of tiles first
@@ -299,18 +304,6 @@ __global__ void __launch_bounds__(TM / RM * TN / CN, TM == 128 || LOWER ? 2 : 4)
         r0 = (int64_t)(gridDim.x - 1 - i / gridDim.y) * TM;
         c0 = (int64_t)(i % gridDim.y) * TN;
     }
-    if constexpr (LOWER) {
-        static_assert(NT == 256, "the diagonal block's factorisation takes 256 threads");
-        // the next diagonal block's factorisation starts first; the rest of its tile goes
-        // to the extra column of CTAs
-        if (g.potrf && blockIdx.x == 0 && blockIdx.y == 0)
-            return potrf_block(g.C, g.A, g.ldc, g.potrf, *reinterpret_cast<PotrfShared*>(smem));
-        if (g.potrf && blockIdx.y == gridDim.y - 1) {
-            if (blockIdx.x != 0) return;
-            c0 = 0;
-        }
-    }
-    if (LOWER && c0 / kGT > (r0 + TM - 1) / kGT) return;
     const float* A = g.A + blockIdx.z * g.sA;
     const float* B = g.B + blockIdx.z * g.sB;
     float* C = g.C + blockIdx.z * g.sC;
@@ -335,13 +328,8 @@ __global__ void __launch_bounds__(TM / RM * TN / CN, TM == 128 || LOWER ? 2 : 4)
         for (int i = 0; i < LB; ++i) {
             const int f = tid + i * NT;
             lb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if constexpr (BT) {
-                const int nn = f / (kGK / 4), q = f % (kGK / 4);
-                if (c0 + nn < g.N) lb[i] = *reinterpret_cast<const float4*>(B + (c0 + nn) * g.ldb + k0 + 4 * q);
-            } else {
-                const int a = f / (TN / 4), q = f % (TN / 4);
-                if (c0 + 4 * q < g.N) lb[i] = *reinterpret_cast<const float4*>(B + (k0 + a) * g.ldb + c0 + 4 * q);
-            }
+            const int a = f / (TN / 4), q = f % (TN / 4);
+            if (c0 + 4 * q < g.N) lb[i] = *reinterpret_cast<const float4*>(B + (k0 + a) * g.ldb + c0 + 4 * q);
         }
     };
     auto stage = [&](int s) {
@@ -356,15 +344,7 @@ __global__ void __launch_bounds__(TM / RM * TN / CN, TM == 128 || LOWER ? 2 : 4)
 #pragma unroll
         for (int i = 0; i < LB; ++i) {
             const int f = tid + i * NT;
-            if constexpr (BT) {
-                const int q = f % (kGK / 4), at = (f / (kGK / 4)) ^ (8 * q);
-                Bs[s][4 * q + 0][at] = lb[i].x;
-                Bs[s][4 * q + 1][at] = lb[i].y;
-                Bs[s][4 * q + 2][at] = lb[i].z;
-                Bs[s][4 * q + 3][at] = lb[i].w;
-            } else {
-                *reinterpret_cast<float4*>(&Bs[s][f / (TN / 4)][4 * (f % (TN / 4))]) = lb[i];
-            }
+            *reinterpret_cast<float4*>(&Bs[s][f / (TN / 4)][4 * (f % (TN / 4))]) = lb[i];
         }
     };
     auto multiply = [&](int s) {
@@ -380,7 +360,7 @@ __global__ void __launch_bounds__(TM / RM * TN / CN, TM == 128 || LOWER ? 2 : 4)
             }
 #pragma unroll
             for (int k = 0; k < CN; k += 4) {
-                const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(&Bs[s][a][BT ? (n0 + 8 * k) ^ swz : n0 + 8 * k]);
+                const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(&Bs[s][a][n0 + 8 * k]);
                 uv[k / 2] = u.x; uv[k / 2 + 1] = u.y;
             }
 #pragma unroll
@@ -413,7 +393,6 @@ __global__ void __launch_bounds__(TM / RM * TN / CN, TM == 128 || LOWER ? 2 : 4)
         for (int h = 0; h < CN / 4; ++h) {
             const int64_t c = c0 + n0 + 32 * h;
             if (c >= g.N) continue;
-            if (LOWER && g.potrf && rr < kNb && c < kNb) continue;
             float4* p = reinterpret_cast<float4*>(C + rr * g.ldc + c);
             float4 o;
             if (g.beta == 0.f) {
@@ -428,6 +407,98 @@ __global__ void __launch_bounds__(TM / RM * TN / CN, TM == 128 || LOWER ? 2 : 4)
             }
             *p = o;
         }
+    }
+}
+
+// Products of the Cholesky steps, 64 terms long: C -= A B^T (UPDATE) or C = A B^T with
+// A [.][64] and B [.][64] of one leading dimension, TM x 64 outputs per CTA, 4 x 4 per
+// thread.  Everything a CTA reads is requested at once (one trip to L2 instead of
+// one per stage of 16 terms), then multiplied out of shared memory (layout as in
+// gemm_kernel); sizes are multiples of the tile.
+//   UPDATE: the trailing matrix's tiles on and below the diagonal, numbered row by
+//     row.  The first, the next diagonal block, is factored by its CTA while the
+//     others compute.  4032 rows: 47 us with 128 x 128 tiles of four stages.
+//   otherwise the panel below a diagonal block, one row of tiles (C may be A).
+template <int TM, bool UPDATE>
+__global__ void __launch_bounds__(4 * TM, UPDATE ? 3 : 4) gptq_rank64_kernel(const float* A, const float* B, float* C,
+                                                                             int64_t ld,
+                                                                             FactorState* st)
+{
+    constexpr int NT = 4 * TM, WM = TM / 16;
+    constexpr int LB = kNb * 16 / NT;                     // float4 loads of B per thread (4 of A)
+    __shared__ __align__(16) unsigned char smem[sizeof(PotrfShared) > kNb * (TM + kNb) * sizeof(float) && UPDATE
+                                                    ? sizeof(PotrfShared) : kNb * (TM + kNb) * sizeof(float)];
+    auto& As = *reinterpret_cast<float (*)[kNb][TM]>(smem);
+    auto& Bs = *reinterpret_cast<float (*)[kNb][kNb]>(smem + kNb * TM * sizeof(float));
+    int64_t r0 = (int64_t)blockIdx.x * TM, c0 = 0;
+    if constexpr (UPDATE) {
+        static_assert(NT == 256, "the diagonal block's factorisation takes 256 threads");
+        if (blockIdx.x == 0) return potrf_block(C, A, ld, st, *reinterpret_cast<PotrfShared*>(smem));
+        // tile number = row (row + 1) / 2 + column
+        int64_t row = (int64_t)((sqrtf(8.f * blockIdx.x + 1.f) - 1.f) * 0.5f);
+        while (row * (row + 1) / 2 > blockIdx.x) --row;
+        while ((row + 1) * (row + 2) / 2 <= blockIdx.x) ++row;
+        r0 = row * TM;
+        c0 = (blockIdx.x - row * (row + 1) / 2) * kNb;
+    }
+    const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+    const int m0 = warp % WM * 16 + lane / 8 * 4, n0 = warp / WM * 32 + lane % 8 * 4;
+    // a load's row and run of four k: 8 rows x 4 runs per warp
+    float4 la[4], lb[LB], o[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int f = tid + i * NT;
+        la[i] = *reinterpret_cast<const float4*>(A + (r0 + f / 4 % TM) * ld + 4 * (f % 4 + 4 * (f / (4 * TM))));
+    }
+#pragma unroll
+    for (int i = 0; i < LB; ++i) {
+        const int f = tid + i * NT;
+        lb[i] = *reinterpret_cast<const float4*>(B + (c0 + f / 4 % kNb) * ld + 4 * (f % 4 + 4 * (f / (4 * kNb))));
+    }
+    float* c = C + (r0 + m0) * ld + c0 + n0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (UPDATE) o[i] = *reinterpret_cast<const float4*>(c + i * ld);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int f = tid + i * NT, q = f % 4 + 4 * (f / (4 * TM)), at = (f / 4 % TM) ^ (8 * (q % 4));
+        As[4 * q + 0][at] = la[i].x;
+        As[4 * q + 1][at] = la[i].y;
+        As[4 * q + 2][at] = la[i].z;
+        As[4 * q + 3][at] = la[i].w;
+    }
+#pragma unroll
+    for (int i = 0; i < LB; ++i) {
+        const int f = tid + i * NT, q = f % 4 + 4 * (f / (4 * kNb)), at = (f / 4 % kNb) ^ (8 * (q % 4));
+        Bs[4 * q + 0][at] = lb[i].x;
+        Bs[4 * q + 1][at] = lb[i].y;
+        Bs[4 * q + 2][at] = lb[i].z;
+        Bs[4 * q + 3][at] = lb[i].w;
+    }
+    __syncthreads();
+    f32x2 acc[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+#pragma unroll 16
+    for (int a = 0; a < kNb; ++a) {
+        const int swz = 8 * (a / 4 % 4);
+        const float4 e = *reinterpret_cast<const float4*>(&As[a][m0 ^ swz]);
+        const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(&Bs[a][n0 ^ swz]);
+        const f32x2 ev[4] = {pack2(e.x, e.x), pack2(e.y, e.y), pack2(e.z, e.z), pack2(e.w, e.w)};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            acc[i][0] = fma2(ev[i], u.x, acc[i][0]);
+            acc[i][1] = fma2(ev[i], u.y, acc[i][1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float v[4];
+        unpack2(acc[i][0], v[0], v[1]);
+        unpack2(acc[i][1], v[2], v[3]);
+        if constexpr (UPDATE)
+            *reinterpret_cast<float4*>(c + i * ld) = make_float4(o[i].x - v[0], o[i].y - v[1],
+                                                                 o[i].z - v[2], o[i].w - v[3]);
+        else
+            *reinterpret_cast<float4*>(c + i * ld) = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
 
@@ -480,14 +551,6 @@ __global__ void __launch_bounds__(256) gptq_prep_kernel(const float* __restrict_
             *reinterpret_cast<float4*>(A + i * K + j) = o;
         }
     }
-}
-
-// Zeros above the diagonal inside the kGT-wide diagonal tiles, which the
-// trailing updates write whole.
-__global__ void __launch_bounds__(256) gptq_zero_upper_kernel(float* __restrict__ A, int64_t K)
-{
-    const int64_t i = (int64_t)blockIdx.x * 2 + threadIdx.x / 128, j = i + 1 + threadIdx.x % 128;
-    if (i < K && j < K) A[i * K + j] = 0.f;
 }
 
 // U[i][j] = Linv[K-1-i][K-1-j] (upper triangular; zeros below the diagonal).
@@ -633,34 +696,27 @@ cudaError_t block_launch(float* Wk, int64_t N, int64_t K, const float* U, int64_
     return cudaGetLastError();
 }
 
-template <int TM, int TN, int RM, int CN, bool BT, bool LOWER, bool TRI_A, bool TRI_B>
+template <int TM, int TN, int RM, bool TRI_A, bool TRI_B>
 cudaError_t gemm_tiles(const GemmArgs& g, int64_t batch, cudaStream_t s)
 {
-    const dim3 grid((unsigned)((g.M + TM - 1) / TM), (unsigned)((g.N + TN - 1) / TN) + (LOWER && g.potrf ? 1 : 0),
-                    (unsigned)batch);
-    gemm_kernel<TM, TN, RM, CN, BT, LOWER, TRI_A, TRI_B><<<grid, TM / RM * TN / CN, 0, s>>>(g);
+    const dim3 grid((unsigned)((g.M + TM - 1) / TM), (unsigned)((g.N + TN - 1) / TN), (unsigned)batch);
+    gemm_kernel<TM, TN, RM, TRI_A, TRI_B><<<grid, TM / RM * TN / 8, 0, s>>>(g);
     return cudaGetLastError();
 }
 
-// Tile of a product: 32 x 64 for a panel of one block; 64 x 64 while 128 x 128
-// tiles would number less than two per SM; beyond that 64 x 128, or 128 x 128 where
-// only the lower triangle is computed.  K and rows 4096, factor and quantisation,
-// ms, by the last one's tile: 128 x 256 (one CTA per SM) 5.70, 128 x 128 (two)
-// 5.35, 64 x 128 (four) 5.16.
-template <bool BT, bool LOWER, bool TRI_A, bool TRI_B>
+// Tile of a product: 32 x 64 for 64 columns; 64 x 64 while 128 x 128 tiles would
+// number less than two per SM; 64 x 128 beyond that (the column updates of K and
+// rows 4096, whole call: 128 x 256 tiles, one CTA per SM, 5.70 ms, 128 x 128, two,
+// 5.35, 64 x 128, four, 5.16).
+template <bool TRI_A, bool TRI_B>
 cudaError_t gemm(const GemmArgs& g, int64_t batch, cudaStream_t s)
 {
     if (g.M <= 0 || g.N <= 0 || batch <= 0) return cudaSuccess;
     const int sms = sm_count() > 0 ? sm_count() : 148;
-    const int64_t tiles = ((g.M + 127) / 128) * ((g.N + 127) / 128) * batch / (LOWER ? 2 : 1);
-    if constexpr (LOWER) {
-        if (tiles < 2 * sms) return gemm_tiles<64, 64, 4, 4, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
-        return gemm_tiles<128, 128, 8, 8, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
-    } else {
-        if (g.N <= 64) return gemm_tiles<32, 64, 4, 8, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
-        if (tiles < 2 * sms) return gemm_tiles<64, 64, 4, 8, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
-        return gemm_tiles<64, 128, 8, 8, BT, LOWER, TRI_A, TRI_B>(g, batch, s);
-    }
+    const int64_t tiles = ((g.M + 127) / 128) * ((g.N + 127) / 128) * batch;
+    if (g.N <= 64) return gemm_tiles<32, 64, 4, TRI_A, TRI_B>(g, batch, s);
+    if (tiles < 2 * sms) return gemm_tiles<64, 64, 4, TRI_A, TRI_B>(g, batch, s);
+    return gemm_tiles<64, 128, 8, TRI_A, TRI_B>(g, batch, s);
 }
 
 GemmArgs gemm_args(const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc, int64_t M,
@@ -703,14 +759,14 @@ cudaError_t combine_pairs(float* Lw, int64_t K, int64_t s_, int64_t half, int64_
     g.sA = s_ * K + s_;
     g.sB = s_ * K + s_;
     g.sC = c * half;
-    cudaError_t e = gemm<false, false, false, true>(g, count, st);
+    cudaError_t e = gemm<false, true>(g, count, st);
     if (e != cudaSuccess) return e;
     // block (bottom, top) = -C_p^-1 X_p (C_p^-1 lower triangular)
     g = gemm_args(Lw + b0 * K + b0, K, X, half, Lw + b0 * K + t0, K, c, half, c, -1.f, 0.f);
     g.sA = s_ * K + s_;
     g.sB = c * half;
     g.sC = s_ * K + s_;
-    return gemm<false, false, true, false>(g, count, st);
+    return gemm<true, false>(g, count, st);
 }
 
 }  // namespace
@@ -738,17 +794,14 @@ cudaError_t launch_gptq_factor(const float* H, int64_t K, double damp, float* U,
         const int64_t k1 = k0 + kNb, m = K - k1;
         if (m <= 0) break;
         // L21 = A21 L11^-T, in place
-        e = gemm<true, false, false, false>(
-            gemm_args(Lw + k1 * K + k0, K, Lw + k0 * K + k0, K, Lw + k1 * K + k0, K, m, kNb, kNb, 1.f, 0.f), 1, s);
-        if (e != cudaSuccess) return e;
+        float *L11 = Lw + k0 * K + k0, *L21 = Lw + k1 * K + k0, *A22 = Lw + k1 * K + k1;
+        gptq_rank64_kernel<32, false><<<(unsigned)(m / 32), 128, 0, s>>>(L21, L11, L21, K, st);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // A22 -= L21 L21^T (lower triangle), and the inverse factor of its first block
-        GemmArgs g = gemm_args(Lw + k1 * K + k0, K, Lw + k1 * K + k0, K, Lw + k1 * K + k1, K, m, m, kNb, -1.f, 1.f);
-        g.potrf = st;
-        e = gemm<true, true, false, false>(g, 1, s);
-        if (e != cudaSuccess) return e;
+        const int64_t t = m / kNb;
+        gptq_rank64_kernel<64, true><<<(unsigned)(t * (t + 1) / 2), 256, 0, s>>>(L21, L21, A22, K, st);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    gptq_zero_upper_kernel<<<(unsigned)((K + 1) / 2), 256, 0, s>>>(Lw, K);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // triangular inverse by doubling
     for (int64_t half = kNb; half < K; half *= 2) {
         const int64_t s_ = 2 * half;
@@ -805,7 +858,7 @@ cudaError_t launch_gptq(const float* W, int64_t N, int64_t K, const float* U, co
         if (e != cudaSuccess) return e;
         const int64_t c1 = j0 + kCols;
         if (c1 < K) {   // W[:, c1:] -= E U[j0:c1, c1:]
-            e = gemm<false, false, false, false>(
+            e = gemm<false, false>(
                 gemm_args(E, kCols, U + j0 * K + c1, K, Wk + c1, K, N, K - c1, kCols, -1.f, 1.f), 1, s);
             if (e != cudaSuccess) return e;
         }
