@@ -16,13 +16,13 @@
 // and five X stages.
 // Warp roles (28 warps, seven warpgroups; setmaxnreg moves registers from the
 // first to the epilogue):
-//   warp 0     TMA producer: X tiles [256 tokens x 64 k] with 128-byte swizzle.
+//   warp 0     TMA producer: X tiles [tokens x 64 k] with 128-byte swizzle.
 //   warp 1     MMA issuer: tcgen05.mma kind::f16, M = 128 (weight rows),
-//              N = 256 (tokens), K = 16, A from tensor memory, B (X) from
+//              N = tokens of a tile, K = 16, A from tensor memory, B (X) from
 //              shared memory, fp32 accumulator in tensor memory.  Also
 //              allocates TMEM.  (Warps 2 and 3 only fill the warpgroup.)
-//   warps 4-11 epilogue: two warps per TMEM lane quarter, each draining 128
-//              token columns with tcgen05.ld, 32 at a time; the accumulator is
+//   warps 4-11 epilogue: two warps per TMEM lane quarter, each draining half of
+//              the token columns with tcgen05.ld, 32 at a time; the accumulator is
 //              handed back before the last 32 are stored (lane n writes
 //              Y[t][n0 + n]).
 //   warps 12-27 decode: two groups of eight warps that take the stages in turn.
@@ -42,8 +42,9 @@
 // each several hundred cycles behind the decode warps' shared-memory accesses, and
 // the issue), so it asks for both barriers at once and its operands are kept
 // uniform (see `warp`): 4 bits, 8B layer at 2048 / 512 / 100 / 33 tokens 771 / 243 /
-// 161 / 148 us before, 579 / 187 / 123 / 111 now (1.55 PFLOP/s at 2048, 0.90 of what
-// cuBLAS holds for seconds under the power limit); 8 bits at 2048 855.  Tried and
+// 161 / 148 us before, 579 / 187 / 123 / 111 with it (1.55 PFLOP/s at 2048, 0.90 of what
+// cuBLAS holds for seconds under the power limit); 8 bits at 2048 855; 3 bits 1143,
+// and 914 with a slice's codes copied 8 bytes at a time instead of 4.  Tried and
 // slower: polling two stages ahead, taking several full stages at a time, resolving
 // 4-bit codes with byte permutes instead of lookups, draining the whole accumulator
 // into registers before the stores (no change).
@@ -238,11 +239,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
-__device__ __forceinline__ void cp_async_4(uint32_t dst, const void* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
-}
-
 __device__ __forceinline__ void cp_async_8(uint32_t dst, const void* src)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
@@ -379,10 +375,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ CUtensorMap xmap)
 {
     constexpr int XB = kBN * kBK * 2;                    // bytes of one X stage
-    constexpr int kChunks = kBN / 2 / 32;                // 32-column drains per epilogue warp
     // 16-byte ring slots per thread and stage: 8-bit kSliceK bytes; 4-bit kSliceK / 2
-    // bytes; 3-bit one 12-byte group per slot (a 16-k slice copies its whole group)
-    constexpr int SLOTS = BITS == 8 ? (kSliceK >= 16 ? kSliceK / 16 : 1) : (kSliceK == 64 ? 2 : 1);
+    // bytes; 3-bit the 12-byte group of its slice and 4 bytes beside it
+    static_assert(kSliceK == 32, "slices of one 3-bit group, one or two ring slots");
+    constexpr int SLOTS = BITS == 8 ? 2 : 1;
     // code stages in flight per decode thread: as many as the free halves of the
     // table rows hold, at most 7
     constexpr int RING_FIT = (256 * 128) / (SLOTS * kCodeStageBytes);
@@ -620,9 +616,9 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         // columns.  16-bit outputs are read out of tensor memory and rounded into
         // registers first, so the accumulator is handed back before the stores.
         const int quarter = warp & 3;                   // TMEM lanes 32*quarter .. +31
-        const int ehalf = (warp - kEpi0) >> 2;          // token columns 128*ehalf .. +127
+        const int half = kBN / 2, ehalf = (warp - kEpi0) >> 2;          // token columns half*ehalf .. +half-1
         const int row = quarter * 32 + lane;
-        const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ehalf * 128);
+        const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ehalf * half);
         int it = 0;
         const bool pf_warp = warp == kEpi0 + 4;
         for (int tile = cta; tile < ntiles; tile += ncta, ++it) {
@@ -630,9 +626,9 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
             if (!warp_wait(accfull, (uint32_t)it & 1u, abort_flag, p.ws, kWaitEpilogue)) break;
             tc_fence_after();
             const int64_t n = (int64_t)tile_n(tile) * kBM + row;
-            const int tb0 = tile_t(tile) * kBN + ehalf * 128;
+            const int tb0 = tile_t(tile) * kBN + ehalf * half;
             // tokens of this half that exist (<= 0 past the end of the batch)
-            const int jmax = (p.B - tb0) < 128 ? (p.B - tb0) : 128;
+            const int jmax = (p.B - tb0) < half ? (p.B - tb0) : half;
             {
                 // 32 tokens at a time; the accumulator is handed back before the last
                 // stores.  Lanes hold consecutive n: each store instruction writes one
@@ -643,10 +639,10 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
                                         ? reinterpret_cast<uint8_t*>(item.part + (int64_t)tile_sp(tile) * p.B * N)
                                         : static_cast<uint8_t*>(item.Y);
 #pragma unroll 1
-                for (int c = 0; c < kChunks; ++c) {
+                for (int c = 0; c < half / 32; ++c) {
                     uint32_t v[32];
                     tmem_ld32(tq + (uint32_t)(c * 32), v);
-                    if (c == kChunks - 1) {
+                    if (c == half / 32 - 1) {
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(accempty);
@@ -686,7 +682,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         // bytes of one row's codes per stage, and where this thread's slice (for 3-bit:
         // the 32-k group holding it) starts among them
         const int step_bytes = BITS == 8 ? 64 : (BITS == 4) ? 32 : 24;
-        const int slice_off = BITS == 8 ? kSliceK * h : (BITS == 4) ? (kSliceK / 2) * h : 12 * ((kSliceK * h) / 32);
+        const int slice_off = BITS == 8 ? kSliceK * h : (BITS == 4) ? (kSliceK / 2) * h : 8 * h;
         int stage = grp;
         uint32_t phase = 0;
         int total = 0;                                  // stages of this CTA, then of this group
@@ -729,18 +725,11 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
 #pragma unroll
                     for (int q = 0; q < SLOTS; ++q) cp_async_16(dst + 16 * q, src + 16 * q);
                 } else if (BITS == 4) {
-                    if constexpr (kSliceK == 16) cp_async_8(dst, src);
-                    else {
-#pragma unroll
-                        for (int q = 0; q < SLOTS; ++q) cp_async_16(dst + 16 * q, src + 16 * q);
-                    }
+                    cp_async_16(dst, src);
                 } else {
-#pragma unroll
-                    for (int q = 0; q < SLOTS; ++q) {                // group q: 12 bytes into slot q
-                        cp_async_4(dst + 16 * q, src + 12 * q);
-                        cp_async_4(dst + 16 * q + 4, src + 12 * q + 4);
-                        cp_async_4(dst + 16 * q + 8, src + 12 * q + 8);
-                    }
+                    // 8-byte aligned: bytes 0 .. 15 of the stage's 24 for slice 0, 8 .. 23 for slice 1
+                    cp_async_8(dst, src);
+                    cp_async_8(dst + 8, src + 8);
                 }
             }
             if (g < total) step(ahead);
@@ -788,9 +777,8 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
                 } else {
                     // one 12-byte group of 32 k: pair q (k 2q, 2q + 1) is the 6-bit field q % 5
                     // of word q / 5 (q < 15); pair 15 takes the two top bits of each word
-                    // group gi's words are cw[4 gi .. 4 gi + 2] (its ring slot)
-                    auto pair_off = [&](int q, int gi = 0) -> uint32_t {
-                        const uint32_t* g3 = cw + 4 * gi;
+                    const uint32_t g3[3] = {h ? cw[1] : cw[0], h ? cw[2] : cw[1], h ? cw[3] : cw[2]};
+                    auto pair_off = [&](int q) -> uint32_t {
                         if (q == 15)
                             return ((g3[0] >> 22) & 0x0300u) | ((g3[1] >> 20) & 0x0c00u) | ((g3[2] >> 18) & 0x3000u) | lane4;
                         const int f = q % 5;
@@ -799,22 +787,8 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
                                              : f == 3 ? (x >> 10) : (x >> 16);
                         return (field & 0x3f00u) | lane4;
                     };
-                    if constexpr (kSliceK == 64) {
-    #pragma unroll
-                        for (int q = 0; q < 32; ++q) pr[q] = lds_tab(pair_off(q & 15, q >> 4));
-                    } else if constexpr (kSliceK == 32) {
-    #pragma unroll
-                        for (int q = 0; q < 16; ++q) pr[q] = lds_tab(pair_off(q));
-                    } else {
-                        // this slice is half of the group: pairs 8 (h & 1) .. +7
-                        if ((h & 1) == 0) {
-    #pragma unroll
-                            for (int q = 0; q < 8; ++q) pr[q] = lds_tab(pair_off(q));
-                        } else {
-    #pragma unroll
-                            for (int q = 0; q < 8; ++q) pr[q] = lds_tab(pair_off(8 + q));
-                        }
-                    }
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) pr[q] = lds_tab(pair_off(q));
                 }
             }
         };
