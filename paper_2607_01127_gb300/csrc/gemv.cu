@@ -431,7 +431,6 @@ __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ 
                     // added up pairwise with rounding to nearest (the tensor core truncates
                     // its sums); sum[l] holds the sum of 2^l groups
                     constexpr int NG = NQ / (NCH * CL);
-                    constexpr bool PAIR = NTL == 1 || BITS != 8;
                     float acc[NTL][4], sum[5][NTL][4];
                     static_assert(NG <= 32 && (NG & (NG - 1)) == 0, "pairwise over the groups");
 #pragma unroll
@@ -458,8 +457,6 @@ __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ 
                                     for (int ch = 0; ch < w; ++ch) d[nt][ch][i] += d[nt][ch + w][i];
                                 float v = d[nt][0][i];
                                 int l = 0;
-                                if (!PAIR && gr) v += sum[0][nt][i];
-                                if (PAIR)
 #pragma unroll
                                 for (; (gr >> l) & 1; ++l) v += sum[l][nt][i];
                                 if (gr == NG - 1) acc[nt][i] = v;
@@ -678,14 +675,18 @@ cudaError_t check_shared_base()
 
 }  // namespace
 
-// Up to 16 rows always; up to 32 where the tensor-memory kernel is slower: at 3 and
-// 8 bits (Llama-3.1-8B layer at batch 32: 130 against 194 us, 144 against 179), at
-// 4 bits for matrices of up to 32 M weights in a call (4096 x 4096 13.4 against
-// 17.0 us, 6144 x 4096 17.7 against 19.8; 28672 x 4096 62 against 58.6).
+// Up to 16 rows always (28672 x 4096 at 16 rows, 4 bits 27 us against 35 in the
+// tensor-memory kernel).  17..32 where that kernel is slower, by the weights of a
+// call, us at 17 and 32 rows here and there:
+//   4 bits, up to 8 M: 3072 x 2048 6.5-7.6 and 8.9, 4096 x 4096 13.0-14.1 and 12.3;
+//   3 bits, up to 32 M: 16384 x 2048 18.8-20.1 and 20.5, 28672 x 4096 59-62 and 52;
+//   8 bits, up to 16 M: 4096 x 4096 13.7-14.5 and 15.3, 6144 x 4096 18.5-20.0 and 17.7.
 bool gemv_takes(int bits, int64_t B, int64_t rows, int64_t K)
 {
     if (bits != 3 && bits != 4 && bits != 8) return false;
-    return B >= 1 && (B <= 16 || (B <= 32 && (bits != 4 || rows <= ((int64_t)32 << 20) / K)));
+    if (B < 1 || B > 32) return false;
+    const int64_t most = (int64_t)(bits == 4 ? 8 : bits == 3 ? 32 : 16) << 20;
+    return B <= 16 || rows <= most / K;
 }
 
 cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)

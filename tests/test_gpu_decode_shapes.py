@@ -43,10 +43,11 @@ def test_decode_shapes(logq, bits, B, N, K):
     check(logq.logq_linear(codes, cb, X, N, K), *reference(X, q, ocb))
 
 
-@pytest.mark.parametrize("bits,B,N,K", [(4, 17, 8192, 4096), (4, 32, 16384, 2048), (4, 1, 2114, 3968), (4, 1, 65536, 128)])
+@pytest.mark.parametrize("bits,B,N,K", [(4, 17, 2048, 4096), (3, 32, 8192, 4096), (8, 24, 4096, 4096), (4, 1, 2114, 3968), (4, 1, 65536, 128)])
 def test_both_sides_of_a_dispatch_line(logq, bits, B, N, K):
-    """N rows are the most of the one path (4-bit batches above 16: up to 32 M
-    weights; short rows at batch 1: up to 8 M); one more row takes the other."""
+    """N rows are the most of the one path (batches above 16: up to 8 M weights at 4
+    bits, 32 M at 3 and 16 M at 8 bits; short rows at batch 1: up to 8 M); one more
+    row takes the other."""
     codes, cb, ocb, q = make_layer(logq, N + 1, K, bits, BASE[bits], 1)
     X = workloads.activations_torch(B, K, 2, torch.bfloat16, "cuda")
     more = logq.logq_linear(codes, cb, X, N + 1, K)
@@ -96,5 +97,5 @@ def test_non_finite_activations_stay_in_their_row(logq, B):
             keep = [i for i in range(B) if i != b]
             assert torch.equal(Y[keep], clean[keep])
             w = oracle.dequant(q, ocb, oracle.TABLE_BF16)[:, k]
-            want = np.full(N, np.nan) if np.isnan(v) else np.where(w == 0, np.nan, np.sign(w) * np.inf)
+            want = np.full(N, np.nan) if np.isnan(v) else np.where(w == 0, np.nan, np.copysign(np.inf, w))
             np.testing.assert_array_equal(Y[b].double().cpu().numpy(), want)
