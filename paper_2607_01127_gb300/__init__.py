@@ -115,7 +115,7 @@ def _load() -> ctypes.CDLL:
     lib.logq_linear.argtypes = [P, ctypes.POINTER(Codebook), P, c_int, c_i64, c_i64, c_i64, P,
                                 c_int, P, ctypes.c_size_t, P]
     lib.logq_linear.restype = c_int
-    lib.logq_linear_grouped.argtypes = [ctypes.POINTER(LinearItem), c_int, P, c_int, c_i64, c_i64, c_int,
+    lib.logq_linear_grouped.argtypes = [P, c_int, P, c_int, c_i64, c_i64, c_int,      # P: LinearItem[count]
                                         P, ctypes.c_size_t, P, ctypes.c_size_t, P]
     lib.logq_linear_grouped.restype = c_int
     lib.logq_workspace_status.argtypes = [P, P, ctypes.POINTER(ctypes.c_uint32)]
@@ -155,21 +155,49 @@ def _check(status: int, where: str) -> None:
         raise LogqError(status, where)
 
 
-def _stream_ptr(stream):
+# The calls below are as short as the smallest launches they make, so what they
+# do per call is kept to a few attribute reads: pointers are passed as integers
+# (the argument types convert them) and torch's tables are set up once.
+_DTYPE_CODE: dict = {}
+_TORCH_DTYPE: dict = {}
+_raw_stream = None
+
+
+def _bind_torch():
+    global _raw_stream
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    codes = {torch.float32: LOGQ_F32, torch.bfloat16: LOGQ_BF16, torch.float16: LOGQ_F16}
+    _DTYPE_CODE.update(codes)               # whole at once: another thread may be reading
+    _TORCH_DTYPE.update({code: dt for dt, code in codes.items()})
+    stream_of, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+    def raw_stream():
+        return stream_of(device())
+
+    _raw_stream = raw_stream
+
+
+def _stream_ptr(stream):
+    """Address of the stream's cudaStream_t; None: the current device's current stream."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        import torch
+        torch.cuda.init()
+        _bind_torch()
+    return _raw_stream()
 
 
 def _dtype_code(dt) -> int:
-    import torch
-    return {torch.float32: LOGQ_F32, torch.bfloat16: LOGQ_BF16, torch.float16: LOGQ_F16}[dt]
+    if not _DTYPE_CODE:
+        _bind_torch()
+    return _DTYPE_CODE[dt]
 
 
 def _torch_dtype(code: int):
-    import torch
-    return {LOGQ_F32: torch.float32, LOGQ_BF16: torch.bfloat16, LOGQ_F16: torch.float16}[code]
+    if not _TORCH_DTYPE:
+        _bind_torch()
+    return _TORCH_DTYPE[code]
 
 
 def logq_build_codebook(bits: int, base: float, range_: float, flags: int = LOGQ_SHIFT_EXACT) -> Codebook:
@@ -209,19 +237,20 @@ def logq_quantize(W, bits: int, base: float, range_: float = 0.0, flags: int = L
                   codes=None, workspace=None, stream=None):
     """Quantise fp32 device weights W[N, K]; returns (codes uint8 tensor, Codebook)."""
     import torch
-    assert W.dtype == torch.float32 and W.is_cuda and W.dim() == 2 and W.is_contiguous()
+    assert W.dtype is torch.float32 and W.is_cuda and W.dim() == 2 and W.is_contiguous()
     N, K = W.shape
-    nbytes = logq_packed_bytes(N, K, bits)
+    lib = _LIB or _lib()
+    nbytes = lib.logq_packed_bytes(N, K, int(bits))
     if codes is None:
         codes = torch.empty(max(nbytes, 16), dtype=torch.uint8, device=W.device)
     if workspace is None:
         workspace = new_workspace(W.device)
     cb = Codebook()
-    st = _lib().logq_quantize(ctypes.c_void_p(W.data_ptr()), N, K, int(bits), float(base), float(range_),
-                           int(flags), ctypes.c_void_p(codes.data_ptr()), ctypes.byref(cb),
-                           ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream_ptr(stream))
-    _check(st, "logq_quantize")
-    return codes[:nbytes], cb
+    st = lib.logq_quantize(W.data_ptr(), N, K, int(bits), float(base), float(range_), int(flags), codes.data_ptr(),
+                           ctypes.byref(cb), workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
+    if st:
+        _check(st, "logq_quantize")
+    return codes if codes.numel() == nbytes else codes[:nbytes], cb
 
 
 def logq_quantize_noalloc(W, bits: int, base: float, range_: float = 0.0,
@@ -314,24 +343,40 @@ def logq_gptq(W, H, cb: Codebook, damp: float = 0.01, codes=None, scratch=None, 
     return codes[:nbytes]
 
 
+def _output_dtype(y_dtype):
+    """(library code, torch dtype) of an output given as None (fp32), a torch dtype or a code."""
+    if y_dtype is None:
+        return LOGQ_F32, _torch_dtype(LOGQ_F32)
+    if isinstance(y_dtype, int):
+        return y_dtype, _torch_dtype(y_dtype)
+    return _dtype_code(y_dtype), y_dtype
+
+
+def _output(Y, B: int, N: int, dtype, device):
+    """Y after its checks, or a new [B, N] tensor."""
+    if Y is None:
+        import torch
+        return torch.empty((B, N), dtype=dtype, device=device)
+    assert Y.dtype is dtype and Y.is_contiguous() and Y.numel() == B * N, \
+        "Y must be a contiguous [B, N] tensor of the output dtype"
+    return Y
+
+
 def logq_linear(codes, cb: Codebook, X, N: int, K: int, y_dtype=None, Y=None, workspace=None,
                 stream=None):
     """Y[B, N] = X[B, K] @ What^T through the codebook's 16-bit table of X's dtype."""
-    import torch
     assert X.is_cuda and X.dim() == 2 and X.is_contiguous() and X.shape[1] == K
     B = X.shape[0]
     xd = _dtype_code(X.dtype)
-    yd = LOGQ_F32 if y_dtype is None else (_dtype_code(y_dtype) if not isinstance(y_dtype, int) else y_dtype)
-    if Y is None:
-        Y = torch.empty((B, N), dtype=_torch_dtype(yd), device=X.device)
-    assert Y.dtype == _torch_dtype(yd) and Y.is_contiguous() and Y.numel() == B * N, \
-        "Y must be a contiguous [B, N] tensor of the output dtype"
+    yd, dtype = _output_dtype(y_dtype)
+    Y = _output(Y, B, N, dtype, X.device)
     if workspace is None:
         workspace = new_workspace(X.device, logq_linear_workspace_bytes(B, N, K, cb.bits))
-    st = _lib().logq_linear(ctypes.c_void_p(codes.data_ptr()), ctypes.byref(cb), ctypes.c_void_p(X.data_ptr()),
-                         xd, B, int(N), int(K), ctypes.c_void_p(Y.data_ptr()), yd,
-                         ctypes.c_void_p(workspace.data_ptr()), workspace.numel(), _stream_ptr(stream))
-    _check(st, "logq_linear")
+    st = (_LIB or _lib()).logq_linear(codes.data_ptr(), ctypes.byref(cb), X.data_ptr(), xd, B, int(N), int(K),
+                                      Y.data_ptr(), yd, workspace.data_ptr(), workspace.numel(),
+                                      _stream_ptr(stream))
+    if st:
+        _check(st, "logq_linear")
     return Y
 
 
@@ -340,32 +385,25 @@ def logq_linear_grouped(items, X, K: int, y_dtype=None, workspace=None, prefetch
     """Up to four matrices sharing X in one launch: items = [(codes, cb, N, Y or None), ...].
     prefetch: optional device tensor (or (tensor, bytes)) the call warms L2 with.
     Returns the list of outputs."""
-    import torch
     assert X.is_cuda and X.dim() == 2 and X.is_contiguous() and X.shape[1] == K
     B = X.shape[0]
     xd = _dtype_code(X.dtype)
-    yd = LOGQ_F32 if y_dtype is None else (_dtype_code(y_dtype) if not isinstance(y_dtype, int) else y_dtype)
-    arr = (LinearItem * len(items))()
-    outs = []
-    keep = []
-    for i, (codes, cb, N, Y) in enumerate(items):
-        if Y is None:
-            Y = torch.empty((B, N), dtype=_torch_dtype(yd), device=X.device)
-        assert Y.dtype == _torch_dtype(yd) and Y.is_contiguous() and Y.numel() == B * N, \
-            "Y must be a contiguous [B, N] tensor of the output dtype"
+    yd, dtype = _output_dtype(y_dtype)
+    outs, words = [], []
+    for codes, cb, N, Y in items:          # one LinearItem each: codes, codebook, rows, output
+        Y = _output(Y, B, N, dtype, X.device)
         outs.append(Y)
-        keep.append(cb)
-        arr[i] = LinearItem(ctypes.c_void_p(codes.data_ptr()), ctypes.pointer(cb), int(N),
-                            ctypes.c_void_p(Y.data_ptr()))
+        words += (codes.data_ptr(), ctypes.addressof(cb), int(N), Y.data_ptr())
+    arr = (ctypes.c_uint64 * len(words))(*words)
     if workspace is None:
         workspace = new_workspace(X.device, logq_linear_grouped_workspace_bytes(
             B, [int(N) for _, _, N, _ in items], K, items[0][1].bits))
-    pf_ptr = ctypes.c_void_p(prefetch.data_ptr()) if prefetch is not None else None
+    pf_ptr = prefetch.data_ptr() if prefetch is not None else None
     pf_bytes = int(prefetch_bytes) if prefetch is not None else 0
-    st = _lib().logq_linear_grouped(arr, len(items), ctypes.c_void_p(X.data_ptr()), xd, B, int(K), yd, pf_ptr,
-                                    pf_bytes, ctypes.c_void_p(workspace.data_ptr()), workspace.numel(),
-                                    _stream_ptr(stream))
-    _check(st, "logq_linear_grouped")
+    st = (_LIB or _lib()).logq_linear_grouped(arr, len(items), X.data_ptr(), xd, B, int(K), yd, pf_ptr, pf_bytes,
+                                              workspace.data_ptr(), workspace.numel(), _stream_ptr(stream))
+    if st:
+        _check(st, "logq_linear_grouped")
     return outs
 
 
