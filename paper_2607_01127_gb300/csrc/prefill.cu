@@ -386,6 +386,11 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
     constexpr int RING = RING_FIT < 7 ? RING_FIT : 7;
     static_assert(RING * SLOTS * kCodeStageBytes <= 256 * 128, "code ring must fit in the table rows' free halves");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
+    // Programmatic dependent launch: as this launch's CTAs leave, the next one's take
+    // their SMs and set up (pair table, tensor memory, first codes) beside the last
+    // tiles here; what reads X or writes Y or the workspace waits for the launch before.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    auto wait_for_previous = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
     // Layout: pair table (code ring in its rows' free halves) | X stages | barriers
     const uint32_t sbase = smem_u32(smem_raw);
     const uint32_t xs0 = sbase + kTabRegion;
@@ -532,6 +537,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         int stage = 0;
         uint32_t phase = 0;
         bool ok = true;
+        wait_for_previous();
         uint32_t issued = 0, issued_par = 0;           // per stage: used at least once / parity of last load
         for (int tile = cta; tile < ntiles && ok; tile += ncta) {
             const int t0 = tile_t(tile) * p.bn;
@@ -565,6 +571,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         uint32_t xph = 0, wph = 0;
         bool ok = true;
         int it = 0;
+        wait_for_previous();                           // before the first bounded wait
 #ifdef LOGQ_TEST_WAIT_HOOK
         // Test builds only (never the shipped library): when the caller's
         // workspace holds kTestStallWord, the MMA warp first waits on the drain
@@ -622,6 +629,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         const uint32_t tq = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ehalf * half);
         int it = 0;
         const bool pf_warp = warp == kEpi0 + 4;
+        wait_for_previous();
         for (int tile = cta; tile < ntiles; tile += ncta, ++it) {
             if (pf_warp) prefetch_codes(tile + ncta);
             if (!warp_wait(accfull, (uint32_t)it & 1u, abort_flag, p.ws, kWaitEpilogue)) break;
@@ -796,6 +804,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         // The other group's warps hide this one's latencies: a stage's pairs are looked
         // up and stored one after the other.
         for (int g = 0; g < RING; ++g) issue(g, g);
+        wait_for_previous();
         int slot = 0;                                   // ring stage of stage g
         for (int g = 0; g < total; ++g) {
             uint32_t pr[kSlicePairs];
@@ -905,8 +914,17 @@ cudaError_t launch(PrefillParams& p, const CUtensorMap& xmap, int grid, cudaStre
         configured[dev] = bytes;
     }
     p.smem_bytes = configured[dev];
-    prefill_kernel<BITS><<<grid, kThreads, configured[dev], s>>>(p, xmap);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = configured[dev];
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, prefill_kernel<BITS>, p, xmap);
 }
 
 }  // namespace
