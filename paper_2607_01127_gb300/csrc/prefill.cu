@@ -43,8 +43,10 @@
 // the issue), so it asks for both barriers at once and its operands are kept
 // uniform (see `warp`): 4 bits, 8B layer at 2048 / 512 / 100 / 33 tokens 771 / 243 /
 // 161 / 148 us before, 579 / 187 / 123 / 111 with it (1.55 PFLOP/s at 2048, 0.90 of what
-// cuBLAS holds for seconds under the power limit); 8 bits at 2048 855; 3 bits 1143,
-// and 914 with a slice's codes copied 8 bytes at a time instead of 4.  Tried and
+// cuBLAS holds for seconds under the power limit); 8 bits at 2048 855.
+// At 3 and 8 bits the code copies bound it, by the rows an instruction touches: 3 bits
+// 1143 us with three 4-byte copies per thread and stage, 914 with two of 8 bytes;
+// with two lanes per row 895 -> 740 (8 bits 838 -> 716), all at 2048 tokens.  Tried and
 // slower: polling two stages ahead, taking several full stages at a time, resolving
 // 4-bit codes with byte permutes instead of lookups, draining the whole accumulator
 // into registers before the stores (no change).
@@ -683,7 +685,6 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         // The warps of a quarter split the stage's 64 k into kSlices slices.
         const int dw = warp - kDec0;                    // 0 .. kDecodeWarps-1
         const int d = dw * 32 + lane;                   // code-ring slot, 0 .. kDecodeThreads-1
-        const int r = (warp & 3) * 32 + lane;           // weight row within the tile
         const int grp = dw / kGroupWarps;               // stages grp, grp + kGroups, ...
         const int h = (dw % kGroupWarps) >> 2;          // slice: k kSliceK*h .. +kSliceK-1 of the stage
         const uint32_t tw = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + kWCol0 + (uint32_t)(kSlicePairs * h);
@@ -697,20 +698,27 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         int total = 0;                                  // stages of this CTA, then of this group
         for (int t = cta; t < ntiles; t += ncta) total += k_end(t) - k_begin(t);
         total = (total - grp + kGroups - 1) / kGroups;
+        // At 3 and 8 bits a slice takes two copies (8-byte aligned; 3 bits: bytes 0 .. 15 of
+        // the stage's 24 for slice 0, 8 .. 23 for slice 1): two lanes copy a row's, 16 rows
+        // at a time, since a copy instruction costs by the rows it touches (figures at the
+        // top of the file).
+        constexpr bool PAIRED = BITS != 4;
+        const int crow = PAIRED ? lane >> 1 : lane;     // first row of the warp's quarter this lane copies for
+        const int piece = PAIRED ? (lane & 1) * (BITS == 8 ? 16 : 8) : 0;
         // Cursor over (tile, k-step) advanced without divisions: one for the
         // copies issued ahead, one for the stage being decoded.
         struct Cursor {
             int tile, ks, ke;                           // k-step and end of the tile's k range
-            bool valid;                                 // this thread's row exists
-            const uint8_t* row;                         // its codes: slice, stage 0
+            int rows;                                   // rows of the warp's quarter that exist
+            const uint8_t* row;                         // codes of the first row this lane copies: slice, stage 0
         };
         auto set_tile = [&](Cursor& c, int tile) {
             c.tile = tile;
             c.ks = tile < ntiles ? k_begin(tile) : 0;
             c.ke = tile < ntiles ? k_end(tile) : 0;
-            const int64_t n = (int64_t)tile_n(tile) * kBM + r;
-            c.valid = tile < ntiles && n < N;
-            c.row = codes + (c.valid ? n : 0) * p.row_bytes + slice_off;
+            const int64_t n = (int64_t)tile_n(tile) * kBM + 32 * (warp & 3);
+            c.rows = tile < ntiles && n < N ? (N - n < 32 ? (int)(N - n) : 32) : 0;
+            c.row = codes + (n + crow) * p.row_bytes + slice_off + piece;
         };
         auto step1 = [&](Cursor& c) {
             if (++c.ks >= c.ke) set_tile(c, c.tile + ncta);
@@ -726,21 +734,20 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         // copies of stage g of this group into ring stage r
         auto issue = [&](int g, int r) {
             exists &= ~(1u << r);
-            if (g < total && ahead.valid) {
+            if (g < total && lane < ahead.rows) {
                 exists |= 1u << r;
-                const uint8_t* src = ahead.row + (int64_t)ahead.ks * step_bytes;
-                const uint32_t dst = ring_slot(r, SLOTS * d);
-                if constexpr (BITS == 8) {
-#pragma unroll
-                    for (int q = 0; q < SLOTS; ++q) cp_async_16(dst + 16 * q, src + 16 * q);
-                } else if (BITS == 4) {
-                    cp_async_16(dst, src);
-                } else {
-                    // 8-byte aligned: bytes 0 .. 15 of the stage's 24 for slice 0, 8 .. 23 for slice 1
-                    cp_async_8(dst, src);
-                    cp_async_8(dst + 8, src + 8);
-                }
+                if (!PAIRED) cp_async_16(ring_slot(r, d), ahead.row + (int64_t)ahead.ks * step_bytes);
             }
+            if (PAIRED && g < total)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int at = crow + 16 * i;       // row of the quarter
+                    if (at >= ahead.rows) break;
+                    const uint8_t* src = ahead.row + (int64_t)ahead.ks * step_bytes + i * 16 * p.row_bytes;
+                    const uint32_t dst = ring_slot(r, SLOTS * (dw * 32 + at)) + piece;
+                    if constexpr (BITS == 3) cp_async_8(dst, src);
+                    else cp_async_16(dst, src);
+                }
             if (g < total) step(ahead);
             cp_async_commit();
         };
@@ -809,7 +816,9 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         for (int g = 0; g < total; ++g) {
             uint32_t pr[kSlicePairs];
             cp_async_wait<RING - 1>();
+            if (PAIRED) __syncwarp();                   // the other lane's copies are here too
             resolve(slot, (exists >> slot) & 1u, pr);
+            if (PAIRED) __syncwarp();                   // and have been read
             issue(g + RING, slot);                      // this thread's slot has been read
             if (++slot == RING) slot = 0;
             if (!warp_wait(wempty(stage), phase ^ 1u, abort_flag, p.ws, kWaitDecode)) break;
