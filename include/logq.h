@@ -174,9 +174,8 @@ logq_status logq_quantize(const float* W, int64_t N, int64_t K, int bits, double
  *   codes (device): packed as above for cb->bits.  X (device): x_dtype.
  *   Y (device): y_dtype in {LOGQ_F32, x_dtype}; a 16-bit Y is the fp32 sum
  *   rounded to nearest-even.  All device pointers 16-byte aligned.
- *   B <= 16 runs the decode kernel, as does B <= 32 for smaller matrices (up to
- *   8 M weights at 4 bits, 32 M at 3 and 16 M at 8 bits); larger B runs the
- *   prefill GEMM kernel (tcgen05).  Calls sharing a workspace must be ordered on one stream
+ *   B <= 16 runs the decode kernel, as does B <= 32 for matrices of up to 4 M
+ *   weights; larger B runs the prefill GEMM kernel (tcgen05).  Calls sharing a workspace must be ordered on one stream
  *   (partial sums may live in it).
  * Asynchronous.  Errors: LOGQ_ERR_INVALID_ARG, LOGQ_ERR_UNSUPPORTED,
  * LOGQ_ERR_WORKSPACE, LOGQ_ERR_CUDA (launch).  A device-side wait that hit

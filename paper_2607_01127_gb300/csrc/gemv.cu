@@ -33,17 +33,17 @@
 //    its table meanwhile.  At batch 1 two 8-warp CTAs run per SM for that; larger
 //    batches, which hold more activations per lane, fill an SM with one CTA.
 //
-// What bounds it: the lookups (128 bytes of shared memory per 64 weights: 12 us
-// of an SM's shared-memory cycles for the 218 M weights of a Llama-3.1-8B layer,
-// against 16 us of HBM time for their codes at 4 bits) and, per launch, the
-// latency of a CTA's life (activations after the previous launch, first tile,
-// final sum: 2.5-3 us).  Per layer (q+k+v, o, gate+up, down chained, bf16), with
-// fused multiply-adds on the CUDA cores (batches up to 8; 16 as the tcgen05
-// prefill kernel at 3 and 8 bits above 4) before and now:
+// What bounds it: instruction issue (a byte permute, a lookup and 1/8 of an MMA per
+// pair of weights; resolving an eighth of the codes by permutes alone, 7 instructions
+// for 4 codes instead of 4, costs 2 %) and, per launch, the latency of a CTA's life
+// (activations after the previous launch, first tile, final sum: 2.3-3 us).  Per
+// Llama-3.1-8B layer (q+k+v, o, gate+up, down chained, bf16), with fused multiply-adds
+// on the CUDA cores (batches up to 8; 5 and more at 3 and 8 bits and 9 and more at 4 in
+// the prefill kernel) before and now:
 //   4 bits, batch 1 / 2 / 4 / 8 / 16: 31.1 / 45.6 / 57.0 / 109 / 117 us before,
 //     30.7 / 34.3 / 41.8 / 49.1 / 64.4 now;
-//   3 bits, batch 1 / 4 / 16 / 32: 39.0 / 68.7 / 162 / 194 before, 35.8 / 45.5 / 75 / 130 now;
-//   8 bits, batch 1 / 4 / 16 / 32: 52.8 / 85.8 / 157 / 179 before, 48.2 / 64 / 96 / 144 now.
+//   3 bits, batch 1 / 4 / 16: 39.0 / 68.7 / 162 before, 35.8 / 45.5 / 75 now;
+//   8 bits, batch 1 / 4 / 16: 52.8 / 85.8 / 157 before, 48.2 / 64 / 96 now.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -65,7 +65,7 @@ constexpr int kMaxItems = 4;
 // Batches from kPartBatch up may share a row range among kMaxParts CTAs (each a
 // part of K): a CTA that takes several passes over K reads all of X, at batch 16
 // and K = 14336 458 KB against 190 KB of codes.  4096 x 14336 at batch 16 19.8 us
-// instead of 23.3, at batch 32 35.5 instead of 40.4; the partial sums need workspace.
+// instead of 23.3; the partial sums need workspace.
 constexpr int64_t kPartBatch = 9, kMaxParts = 8;
 // Warm-up ranges of this size or more are not prefetched: a launch's end waits for
 // the prefetches it issued, and in a chain of launches that costs more than the
@@ -675,18 +675,16 @@ cudaError_t check_shared_base()
 
 }  // namespace
 
-// Up to 16 rows always (28672 x 4096 at 16 rows, 4 bits 27 us against 35 in the
-// tensor-memory kernel).  17..32 where that kernel is slower, by the weights of a
-// call, us at 17 and 32 rows here and there:
-//   4 bits, up to 8 M: 3072 x 2048 6.5-7.6 and 8.9, 4096 x 4096 13.0-14.1 and 12.3;
-//   3 bits, up to 32 M: 16384 x 2048 18.8-20.1 and 20.5, 28672 x 4096 59-62 and 52;
-//   8 bits, up to 16 M: 4096 x 4096 13.7-14.5 and 15.3, 6144 x 4096 18.5-20.0 and 17.7.
+// Up to 16 rows always (a Llama-3.1-8B layer at 16 rows, here and in the tensor-memory
+// kernel: 4 bits 64 and 74 us, 3 bits 75 and 93, 8 bits 96 and 96).  17..32 for up to
+// 4 M weights in a call: 2048 x 2048 at 17 / 32 rows, 4 bits 5.1 / 6.1 against 6.3 / 6.4,
+// 3 bits 5.2 / 6.0 against 6.7, 8 bits 4.7 / 5.2 against 7.3; 3072 x 2048, 4 bits 6.6 /
+// 7.6 against 6.4 / 6.6; 4096 x 4096 13.0 / 14.0 against 10.5 / 10.7.
 bool gemv_takes(int bits, int64_t B, int64_t rows, int64_t K)
 {
     if (bits != 3 && bits != 4 && bits != 8) return false;
     if (B < 1 || B > 32) return false;
-    const int64_t most = (int64_t)(bits == 4 ? 8 : bits == 3 ? 32 : 16) << 20;
-    return B <= 16 || rows <= most / K;
+    return B <= 16 || rows <= ((int64_t)4 << 20) / K;
 }
 
 cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)

@@ -43,11 +43,10 @@ def test_decode_shapes(logq, bits, B, N, K):
     check(logq.logq_linear(codes, cb, X, N, K), *reference(X, q, ocb))
 
 
-@pytest.mark.parametrize("bits,B,N,K", [(4, 17, 2048, 4096), (3, 32, 8192, 4096), (8, 24, 4096, 4096), (4, 1, 2114, 3968), (4, 1, 65536, 128)])
+@pytest.mark.parametrize("bits,B,N,K", [(4, 17, 1024, 4096), (3, 32, 2048, 2048), (8, 24, 1024, 4096), (4, 1, 2114, 3968), (4, 1, 65536, 128)])
 def test_both_sides_of_a_dispatch_line(logq, bits, B, N, K):
-    """N rows are the most of the one path (batches above 16: up to 8 M weights at 4
-    bits, 32 M at 3 and 16 M at 8 bits; short rows at batch 1: up to 8 M); one more
-    row takes the other."""
+    """N rows are the most of the one path (batches above 16: up to 4 M weights;
+    short rows at batch 1: up to 8 M); one more row takes the other."""
     codes, cb, ocb, q = make_layer(logq, N + 1, K, bits, BASE[bits], 1)
     X = workloads.activations_torch(B, K, 2, torch.bfloat16, "cuda")
     more = logq.logq_linear(codes, cb, X, N + 1, K)
