@@ -813,7 +813,7 @@ def run_ours(args):
                 "us_per_call": round(en["us"], 1), "weights": en["weights"],
                 "gbs_of_w": round(en["weights"] * 4 / (en["us"] * 1e-6) / 1e9, 1),
                 "wmin": en["wmin"], "base": en["base"], "range": en["range"], "eps": 4e-3,
-                "note": "Llama-3.1-8B gate 14336x4096: absmax + 3 selection passes + quantise, "
+                "note": "Llama-3.1-8B gate 14336x4096: 3 selection passes + quantise, "
                         "host sync twice per call"}
         except Exception as e:
             line["energy_quantize"] = {"error": str(e)[:200]}
