@@ -41,7 +41,7 @@
 // on the CUDA cores (batches up to 8; 5 and more at 3 and 8 bits and 9 and more at 4 in
 // the prefill kernel) before and now:
 //   4 bits, batch 1 / 2 / 4 / 8 / 16: 31.1 / 45.6 / 57.0 / 109 / 117 us before,
-//     30.7 / 34.3 / 41.8 / 49.1 / 64.4 now;
+//     30.7 / 34.3 / 41.8 / 49.1 / 63.4 now;
 //   3 bits, batch 1 / 4 / 16: 39.0 / 68.7 / 162 before, 35.8 / 45.5 / 75 now;
 //   8 bits, batch 1 / 4 / 16: 52.8 / 85.8 / 157 before, 48.2 / 64 / 96 now.
 #include <cuda_bf16.h>
@@ -608,7 +608,7 @@ cudaError_t shape_or_run(int key, Shape* sh, const GemvParams* p, const GroupArg
             LOGQ_SHAPE(2, 4, 1, 1, 4, 512, 1);
             LOGQ_SHAPE(4, 2, 2, 1, 2, 512, 1);
             LOGQ_SHAPE(8, 1, 2, 1, 2, 512, 1);
-            LOGQ_SHAPE(16, 1, 4, 2, 1, 256, 1);
+            LOGQ_SHAPE(16, 1, 4, 2, 2, 256, 1);
             LOGQ_SHAPE(32, 1, 2, 4, 1, 256, 1);
             LOGQ_SHAPE(kShort + 1, 2, 1, 1, 5, 256, 2);
             LOGQ_SHAPE(kShort + 2, 4, 1, 1, 4, 256, 2);
