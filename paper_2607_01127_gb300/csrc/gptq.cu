@@ -35,8 +35,8 @@
 //
 // K = 4096: the factor 7.86 ms with single-buffered 128 x 128 products, a
 // two-barriers-per-column diagonal factorisation (60 us a block, alone on the
-// GPU) and one warp per row in the column loop, 2.45 ms now; factor and
-// quantisation of 4096 rows 11.3 and 5.0 ms.  The fp32 operations (23 G
+// GPU) and one warp per row in the column loop, 2.36 ms now; factor and
+// quantisation of 4096 rows 11.3 and 4.66 ms.  The fp32 operations (23 G
 // multiply-adds in the factor, 34 G in the column updates) take 0.6 and 0.9 ms
 // at the FMA rate; the rest is the chain of 64 diagonal blocks and 32 column
 // blocks, each waiting for the update before it.
@@ -70,6 +70,29 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
     f32x2 r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
+}
+
+// Programmatic dependent launch: the next kernel of a chain may start as soon as every
+// CTA of this one has, and waits itself before it touches what this one reads or
+// writes.  The chains here are of 63 x 2 and 32 x 2 kernels of 4-100 us: factor at K =
+// 4096 2.45 -> 2.36 ms, with quantisation 4.97 -> 4.66; K = 128 0.15 -> 0.13.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 constexpr int kNb = 64;            // Cholesky block
@@ -304,6 +327,8 @@ __global__ void __launch_bounds__(TM / RM * TN / 8, 4) gemm_kernel(const __grid_
         r0 = (int64_t)(gridDim.x - 1 - i / gridDim.y) * TM;
         c0 = (int64_t)(i % gridDim.y) * TN;
     }
+    let_next_start();
+    wait_for_previous();
     const float* A = g.A + blockIdx.z * g.sA;
     const float* B = g.B + blockIdx.z * g.sB;
     float* C = g.C + blockIdx.z * g.sC;
@@ -431,6 +456,8 @@ __global__ void __launch_bounds__(4 * TM, UPDATE ? 3 : 4) gptq_rank64_kernel(con
     auto& As = *reinterpret_cast<float (*)[kNb][TM]>(smem);
     auto& Bs = *reinterpret_cast<float (*)[kNb][kNb]>(smem + kNb * TM * sizeof(float));
     int64_t r0 = (int64_t)blockIdx.x * TM, c0 = 0;
+    let_next_start();
+    wait_for_previous();
     if constexpr (UPDATE) {
         static_assert(NT == 256, "the diagonal block's factorisation takes 256 threads");
         if (blockIdx.x == 0) return potrf_block(C, A, ld, st, *reinterpret_cast<PotrfShared*>(smem));
@@ -599,6 +626,7 @@ __global__ void __launch_bounds__(kBlockThreads, 3) gptq_block_kernel(float* __r
     float* Ub = reinterpret_cast<float*>(sm4);     // [kCols][kCols], upper triangle of U's block
     __shared__ float lv[128];
     const int tid = threadIdx.x, lane = tid % 32, l8 = lane % 8, base = lane & 24;
+    let_next_start();
     const int64_t r = (int64_t)blockIdx.x * kRowsPerCta + tid / 8;
     if (tid < 128) lv[tid] = tb.level[tid];
     for (int i = tid; i < kCols * kCols / 4; i += kBlockThreads) {
@@ -613,6 +641,7 @@ __global__ void __launch_bounds__(kBlockThreads, 3) gptq_block_kernel(float* __r
     uint32_t th[kTh];
 #pragma unroll
     for (int b = 0; b < kTh; ++b) th[b] = tb.thresh[l8 + 8 * b];
+    wait_for_previous();                           // the update of these columns (U's block is not its output)
     // rows past the end repeat the last one (whole warps take part in the shuffles)
     const int64_t rr = r < N ? r : N - 1;
     f32x2 wv[4][2];                                // this lane's columns 32 i + 4 l8 .. + 3, in pairs
@@ -692,16 +721,14 @@ cudaError_t block_launch(float* Wk, int64_t N, int64_t K, const float* U, int64_
         configured[dev] = 1;
     }
     const unsigned grid = (unsigned)((N + kRowsPerCta - 1) / kRowsPerCta);
-    gptq_block_kernel<BITS><<<grid, kBlockThreads, kBlockSmem, s>>>(Wk, N, K, U, j0, tb, codes, E);
-    return cudaGetLastError();
+    return launch_chained(gptq_block_kernel<BITS>, dim3(grid), kBlockThreads, kBlockSmem, s, Wk, N, K, U, j0, tb, codes, E);
 }
 
 template <int TM, int TN, int RM, bool TRI_A, bool TRI_B>
 cudaError_t gemm_tiles(const GemmArgs& g, int64_t batch, cudaStream_t s)
 {
     const dim3 grid((unsigned)((g.M + TM - 1) / TM), (unsigned)((g.N + TN - 1) / TN), (unsigned)batch);
-    gemm_kernel<TM, TN, RM, TRI_A, TRI_B><<<grid, TM / RM * TN / 8, 0, s>>>(g);
-    return cudaGetLastError();
+    return launch_chained(gemm_kernel<TM, TN, RM, TRI_A, TRI_B>, grid, TM / RM * TN / 8, 0, s, g);
 }
 
 // Tile of a product: 32 x 64 for 64 columns; 64 x 64 while 128 x 128 tiles would
@@ -795,12 +822,12 @@ cudaError_t launch_gptq_factor(const float* H, int64_t K, double damp, float* U,
         if (m <= 0) break;
         // L21 = A21 L11^-T, in place
         float *L11 = Lw + k0 * K + k0, *L21 = Lw + k1 * K + k0, *A22 = Lw + k1 * K + k1;
-        gptq_rank64_kernel<32, false><<<(unsigned)(m / 32), 128, 0, s>>>(L21, L11, L21, K, st);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_chained(gptq_rank64_kernel<32, false>, dim3((unsigned)(m / 32)), 128, 0, s, L21, L11, L21, K, st);
+        if (e != cudaSuccess) return e;
         // A22 -= L21 L21^T (lower triangle), and the inverse factor of its first block
         const int64_t t = m / kNb;
-        gptq_rank64_kernel<64, true><<<(unsigned)(t * (t + 1) / 2), 256, 0, s>>>(L21, L21, A22, K, st);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_chained(gptq_rank64_kernel<64, true>, dim3((unsigned)(t * (t + 1) / 2)), 256, 0, s, L21, L21, A22, K, st);
+        if (e != cudaSuccess) return e;
     }
     // triangular inverse by doubling
     for (int64_t half = kNb; half < K; half *= 2) {
