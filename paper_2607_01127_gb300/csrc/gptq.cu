@@ -626,7 +626,9 @@ __global__ void __launch_bounds__(kBlockThreads, 3) gptq_block_kernel(float* __r
     float* Ub = reinterpret_cast<float*>(sm4);     // [kCols][kCols], upper triangle of U's block
     __shared__ float lv[128];
     const int tid = threadIdx.x, lane = tid % 32, l8 = lane % 8, base = lane & 24;
-    let_next_start();
+    // not from the last block: what follows the call may read codes before it waits,
+    // as the linear kernels do
+    if (j0 + kCols < K) let_next_start();
     const int64_t r = (int64_t)blockIdx.x * kRowsPerCta + tid / 8;
     if (tid < 128) lv[tid] = tb.level[tid];
     for (int i = tid; i < kCols * kCols / 4; i += kBlockThreads) {

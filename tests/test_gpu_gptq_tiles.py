@@ -54,3 +54,23 @@ def test_rows_do_not_depend_on_the_tiles(logq, bits):
     for r0, n in ((0, 1), (0, 17), (3000, 1000), (N - 1000, 1000)):
         part = logq.logq_gptq(W[r0:r0 + n].contiguous(), H, cb).view(n, -1)
         assert torch.equal(part, codes[r0:r0 + n])
+
+
+@pytest.mark.parametrize("B", [1, 16, 40])
+def test_linear_right_after_gptq(logq, B):
+    """The linear kernels read codes before they wait for the launch before them; the
+    codes GPTQ has just written are complete all the same."""
+    K, N = 256, 9000
+    H = torch.from_numpy(hessian(K, 6, T=2 * K).astype(np.float32)).cuda()
+    W = torch.from_numpy(workloads.weights_np(N, K, seed=10)).cuda()
+    cb = logq.logq_build_codebook(4, 2.0, float(W.abs().max()))
+    X = workloads.activations_torch(B, K, 11, torch.bfloat16, "cuda")
+    codes = logq.logq_gptq(W, H, cb)
+    want = logq.logq_linear(codes, cb, X, N, K)
+    ws = logq.new_workspace(None, logq.logq_linear_workspace_bytes(B, N, K, 4))
+    for _ in range(10):
+        codes.zero_()
+        torch.cuda.synchronize()
+        logq.logq_gptq(W, H, cb, codes=codes)
+        got = logq.logq_linear(codes, cb, X, N, K, workspace=ws)
+        assert torch.equal(got, want)
