@@ -34,11 +34,12 @@
  *   - Every argument is validated before anything is enqueued.  A call that
  *     returns an error other than LOGQ_ERR_CUDA / LOGQ_ERR_NONFINITE has
  *     touched no device memory.
- *   - Decode launches (logq_linear with small B, logq_linear_grouped) use
- *     programmatic dependent launch: they may start while the preceding kernel
- *     on the stream finishes.  They read X and write Y only after that kernel
- *     has completed and its writes are visible, but they read the packed codes
- *     earlier, before that guarantee holds.  So the codes must be complete
+ *   - Linear launches (logq_linear, logq_linear_grouped) use programmatic
+ *     dependent launch: they may start while the preceding kernel on the stream
+ *     finishes.  They read X and write Y only after that kernel has completed
+ *     and its writes are visible, but those of up to 16 rows at 4 bits and 4
+ *     rows at 3 and 8 bits (decode launches) read the packed codes earlier,
+ *     before that guarantee holds.  So for them the codes must be complete
  *     before the call is enqueued, ordered by a host synchronisation after the
  *     kernel that wrote them (of its stream, of an event recorded after it, or
  *     of the device), not by stream order alone.  logq_quantize and

@@ -42,8 +42,8 @@
 // the prefill kernel) before and now:
 //   4 bits, batch 1 / 2 / 4 / 8 / 16: 31.1 / 45.6 / 57.0 / 109 / 117 us before,
 //     30.7 / 34.3 / 41.8 / 49.1 / 63.4 now;
-//   3 bits, batch 1 / 4 / 16: 39.0 / 68.7 / 162 before, 35.8 / 45.5 / 75 now;
-//   8 bits, batch 1 / 4 / 16: 52.8 / 85.8 / 157 before, 48.2 / 64 / 96 now.
+//   3 bits, batch 1 / 4 / 16: 39.0 / 68.7 / 162 before, 35.8 / 45.5 / 78 now;
+//   8 bits, batch 1 / 4 / 16: 52.8 / 85.8 / 157 before, 48.2 / 64 / 100 now.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -101,7 +101,7 @@ struct GemvParams {
     int32_t span_cols;    // warps / G: spans in flight at once
     int32_t chunk_rows;   // rows reduced per shared-memory pass
     int32_t pitch;        // floats from one set of partial sums to the next
-    int32_t _pad;
+    int32_t wait_codes;   // codes are read only after the previous launch (reads_codes_early)
     const uint8_t* pf;    // optional L2 warm-up range (e.g. the next layer's codes)
     int64_t pf_bytes;
     int64_t pf_share;     // bytes of that range per CTA (multiple of 16)
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ 
     };
     // 0) the first T tiles' codes of this warp's first (chunk, span) go out first:
     //    their latency hides behind the prologue below.  Codes are weights, not
-    //    the previous kernel's output (see the launch contract).
+    //    the previous kernel's output (see the launch contract), or wait_codes is set.
     auto load_first = [&](const Span& sp, int nrows) {
 #pragma unroll
         for (int u = 0; u < T; ++u)
@@ -345,6 +345,7 @@ __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ 
     auto chunk_of = [&](int q0) { return r1 - q0 > p.chunk_rows ? p.chunk_rows : r1 - q0; };
     int nrows = chunk_of(r0);
     Span sp = span_at(r0, s0 + scol);
+    if (p.wait_codes) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (compute_warp) load_first(sp, nrows);
 
     // 1) its share of the optional warm-up range
@@ -676,7 +677,7 @@ cudaError_t check_shared_base()
 }  // namespace
 
 // Up to 16 rows always (a Llama-3.1-8B layer at 16 rows, here and in the tensor-memory
-// kernel: 4 bits 64 and 74 us, 3 bits 75 and 93, 8 bits 96 and 96).  17..32 for up to
+// kernel: 4 bits 64 and 74 us, 3 bits 78 and 93, 8 bits 100 and 97).  17..32 for up to
 // 4 M weights in a call: 2048 x 2048 at 17 / 32 rows, 4 bits 5.1 / 6.1 against 6.3 / 6.4,
 // 3 bits 5.2 / 6.0 against 6.7, 8 bits 4.7 / 5.2 against 7.3; 3072 x 2048, 4 bits 6.6 /
 // 7.6 against 6.4 / 6.6; 4096 x 4096 13.0 / 14.0 against 10.5 / 10.7.
@@ -686,6 +687,11 @@ bool gemv_takes(int bits, int64_t B, int64_t rows, int64_t K)
     if (B < 1 || B > 32) return false;
     return B <= 16 || rows <= ((int64_t)4 << 20) / K;
 }
+
+// Launches that may read codes before the launch ahead of them has completed, as
+// include/logq.h says of decode launches.  Larger batches (and 5..16 at 3 and 8 bits)
+// keep to stream order, at 4 % of a layer's time (3 bits at batch 16 75 us without).
+static bool reads_codes_early(int bits, int64_t B) { return B <= (bits == 4 ? 16 : 4); }
 
 cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
 {
@@ -706,6 +712,7 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
     p.K = (int32_t)a.K;
     p.B = (int32_t)a.B;
     p.y_dtype = a.y_dtype;
+    p.wait_codes = reads_codes_early(a.bits, a.B) ? 0 : 1;
     p.row_bytes = (int32_t)row_bytes;
     p.blocks = (int32_t)(a.K / (4 * lane_k(a.bits)));
     p.spans = (p.blocks + sh.S * sh.J - 1) / (sh.S * sh.J);

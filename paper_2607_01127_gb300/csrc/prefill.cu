@@ -389,8 +389,8 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
     static_assert(RING * SLOTS * kCodeStageBytes <= 256 * 128, "code ring must fit in the table rows' free halves");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     // Programmatic dependent launch: as this launch's CTAs leave, the next one's take
-    // their SMs and set up (pair table, tensor memory, first codes) beside the last
-    // tiles here; what reads X or writes Y or the workspace waits for the launch before.
+    // their SMs and set up (pair table, tensor memory, barriers) beside the last tiles
+    // here; what reads codes or X or writes Y or the workspace waits for the launch before.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     auto wait_for_previous = [] { asm volatile("griddepcontrol.wait;" ::: "memory"); };
     // Layout: pair table (code ring in its rows' free halves) | X stages | barriers
@@ -810,8 +810,8 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         };
         // The other group's warps hide this one's latencies: a stage's pairs are looked
         // up and stored one after the other.
+        wait_for_previous();                            // stream order holds for the codes too
         for (int g = 0; g < RING; ++g) issue(g, g);
-        wait_for_previous();
         int slot = 0;                                   // ring stage of stage g
         for (int g = 0; g < total; ++g) {
             uint32_t pr[kSlicePairs];
