@@ -345,7 +345,8 @@ __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ 
     auto chunk_of = [&](int q0) { return r1 - q0 > p.chunk_rows ? p.chunk_rows : r1 - q0; };
     int nrows = chunk_of(r0);
     Span sp = span_at(r0, s0 + scol);
-    if (p.wait_codes) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (BC >= 8 && p.wait_codes)                       // (shapes for up to 4 rows never do)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
     if (compute_warp) load_first(sp, nrows);
 
     // 1) its share of the optional warm-up range
