@@ -689,11 +689,6 @@ bool gemv_takes(int bits, int64_t B, int64_t rows, int64_t K)
     return B <= 16 || rows <= ((int64_t)4 << 20) / K;
 }
 
-// Launches that may read codes before the launch ahead of them has completed, as
-// include/logq.h says of decode launches.  Larger batches (and 5..16 at 3 and 8 bits)
-// keep to stream order, at 4 % of a layer's time (3 bits at batch 16 75 us without).
-static bool reads_codes_early(int bits, int64_t B) { return B <= (bits == 4 ? 16 : 4); }
-
 cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
 {
     if (a.count < 1 || a.count > kMaxItems) return cudaErrorInvalidValue;

@@ -56,18 +56,18 @@ def test_rows_do_not_depend_on_the_tiles(logq, bits):
         assert torch.equal(part, codes[r0:r0 + n])
 
 
-@pytest.mark.parametrize("B", [17, 40])
-def test_linear_right_after_gptq(logq, B):
+@pytest.mark.parametrize("bits,B", [(4, 8), (4, 16), (4, 17), (4, 40), (8, 5), (8, 16), (8, 40)])
+def test_linear_right_after_gptq(logq, bits, B):
     """Batches that keep to stream order read the codes that GPTQ has just written,
     in the decode kernel and in the prefill kernel."""
     K, N = 256, 9000
     H = torch.from_numpy(hessian(K, 6, T=2 * K).astype(np.float32)).cuda()
     W = torch.from_numpy(workloads.weights_np(N, K, seed=10)).cuda()
-    cb = logq.logq_build_codebook(4, 2.0, float(W.abs().max()))
+    cb = logq.logq_build_codebook(bits, {4: 2.0, 8: 1.05}[bits], float(W.abs().max()))
     X = workloads.activations_torch(B, K, 11, torch.bfloat16, "cuda")
     codes = logq.logq_gptq(W, H, cb)
     want = logq.logq_linear(codes, cb, X, N, K)
-    ws = logq.new_workspace(None, logq.logq_linear_workspace_bytes(B, N, K, 4))
+    ws = logq.new_workspace(None, logq.logq_linear_workspace_bytes(B, N, K, bits))
     for _ in range(10):
         codes.zero_()
         torch.cuda.synchronize()
