@@ -225,12 +225,14 @@ __device__ __forceinline__ bool elect_one()
 }
 
 // One lane of the warp polls (a barrier polled by many threads serialises);
-// the outcome is broadcast to the whole warp.
+// the outcome is broadcast to the whole warp.  What that lane acquired is ordered
+// before the other lanes' accesses by __syncwarp; votes and shuffles do not order memory.
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, Workspace* ws,
                                           uint32_t who)
 {
     uint32_t ok = 0;
     if ((threadIdx.x & 31) == 0) ok = wait_bounded(bar, parity, abort_flag, ws, who) ? 1u : 0u;
+    __syncwarp();
     return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
@@ -598,6 +600,7 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
                         break;
                     }
                 }
+                __syncwarp();                          // what lanes 0 and 1 acquired -> the issuing lane
                 tc_fence_after();
                 const uint32_t acol = tmem_base + kWCol0 + (uint32_t)wsg * kWStageCols;
                 const uint64_t bdesc = smem_desc_sw128(xs0 + xs * XB);
