@@ -391,6 +391,8 @@ def logq_linear_grouped(items, X, K: int, y_dtype=None, workspace=None, prefetch
     yd, dtype = _output_dtype(y_dtype)
     outs, words = [], []
     for codes, cb, N, Y in items:          # one LinearItem each: codes, codebook, rows, output
+        if not isinstance(cb, Codebook):   # its address goes in as an integer, unchecked by ctypes
+            raise TypeError(f"codebook expected, not {type(cb).__name__}")
         Y = _output(Y, B, N, dtype, X.device)
         outs.append(Y)
         words += (codes.data_ptr(), ctypes.addressof(cb), int(N), Y.data_ptr())

@@ -274,3 +274,37 @@ def test_linear_rejects_before_launch(logq):
 
 def test_workspace_status_rejects_null(logq):
     assert logq.lib.logq_workspace_status(None, None, None) == logq.LOGQ_ERR_WORKSPACE
+
+
+class _FakeTensor:
+    """What the binding reads of a device tensor; no kernel ever sees it."""
+    is_cuda = True
+
+    def __init__(self, shape, dtype):
+        self.shape, self.dtype, self.device = shape, dtype, "cuda"
+
+    def dim(self):
+        return len(self.shape)
+
+    def is_contiguous(self):
+        return True
+
+    def numel(self):
+        return math.prod(self.shape)
+
+    def data_ptr(self):
+        return 0x10000
+
+
+def test_grouped_refuses_what_is_not_a_codebook(logq):
+    """Any other object in a codebook's place, ctypes objects of its size among them, is a
+    TypeError before the library is called."""
+    import torch
+    X, Y = _FakeTensor((1, 128), torch.bfloat16), _FakeTensor((1, 8), torch.float32)
+    codes, ws = _FakeTensor((512,), torch.uint8), _FakeTensor((256,), torch.uint8)
+    good = logq.Codebook()                     # zeros: refused by the library's own checks
+    wrong = [(ctypes.c_ubyte * ctypes.sizeof(logq.Codebook))(), ctypes.pointer(good), 7, None]
+    for cb in wrong:
+        for items in ([(codes, cb, 8, Y)], [(codes, good, 8, Y), (codes, cb, 8, Y)]):
+            with pytest.raises(TypeError):
+                logq.logq_linear_grouped(items, X, 128, workspace=ws)
