@@ -128,9 +128,11 @@ static uint16_t encode16(double v, int ebits, int mbits)
 uint16_t oracle_bf16_bits(double v) { return encode16(oracle_round_bf16(v), 8, 7); }
 uint16_t oracle_f16_bits(double v)  { return encode16(oracle_round_f16(v), 5, 10); }
 
-/* Smallest fp32 value >= t (t > 0), found by stepping the nearest fp32. */
+/* Smallest fp32 value >= t (t > 0), found by stepping the nearest fp32.  A t of 0
+ * is a positive boundary that underflowed in fp64. */
 static float f32_round_up(double t)
 {
+    if (!(t > 0.0)) return nextafterf(0.0f, 1.0f);
     float f = (float)oracle_round_f32(t);
     while ((double)f < t) f = nextafterf(f, INFINITY);
     while (1) {

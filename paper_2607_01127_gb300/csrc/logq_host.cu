@@ -135,10 +135,12 @@ long floor_log_base(double x, double b)
     return e;
 }
 
-// Smallest fp32 >= t for t > 0.
+// Smallest fp32 >= t for t > 0; a t of 0 is a positive boundary that underflowed in
+// fp64 (no |w| > 0 lies below it).
 float round_up_f32(double t)
 {
     float f = (float)t;
+    if (!(t > 0.0)) return nextafterf(0.0f, 1.0f);
     while ((double)f < t) f = nextafterf(f, INFINITY);
     for (;;) {
         float g = nextafterf(f, 0.0f);

@@ -110,8 +110,12 @@ __device__ __forceinline__ float max_of(const Workspace* ws)
     return ws->nonfinite ? 0.f : __uint_as_float(ws->absmax_bits);
 }
 
-// Boundary j of the codebook whose range is mx.
-__device__ __forceinline__ float boundary(float mx, double factor) { return __double2float_ru((double)mx * factor); }
+// Boundary j of the codebook whose range is mx (at least the smallest positive fp32,
+// as round_up_f32 of logq_host.cu).
+__device__ __forceinline__ float boundary(float mx, double factor)
+{
+    return fmaxf(__double2float_ru((double)mx * factor), __uint_as_float(1u));
+}
 
 // A kernel's boundaries (2 x their bit patterns, NT2 of them, NB real ones) and
 // estimate offset in shared memory.  ONE is the unit of a level in the fixed

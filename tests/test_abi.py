@@ -6,6 +6,8 @@ import ctypes
 import math
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -75,6 +77,18 @@ def test_codebook_invalid(logq, args):
     with pytest.raises(logq.LogqError) as ei:
         logq.logq_build_codebook(*args)
     assert ei.value.status == logq.LOGQ_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("bits,base,mode", [(8, 1e30, 0), (8, 1e30, 1), (4, 1e100, 0), (3, 1e300, 0)])
+def test_codebook_of_boundaries_below_fp64(logq, bits, base, mode):
+    """Boundaries that underflow fp64 to 0 round up to the smallest positive fp32, so that
+    zeros keep code 0 (in a process of its own: the search for them once did not end)."""
+    code = ("import paper_2607_01127_gb300 as m; cb = m.logq_build_codebook(%d, %r, 1.0, %d);"
+            "print([cb.thresh[j] for j in range(cb.qmax)] == sorted(cb.thresh[:cb.qmax]),"
+            " cb.thresh[0], cb.level[cb.qmax])" % (bits, base, mode))
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stderr
+    assert r.stdout.split() == ["True", repr(float(np.nextafter(np.float32(0), np.float32(1)))), "1.0"]
 
 
 def test_codebook_null_out(logq):

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2607_01127_gb300 import workloads
 
 from gpu_common import lib
@@ -31,6 +32,21 @@ def test_reduced_range_equals_given_range(logq, bits, base, scale, N, K):
     want, wcb = logq.logq_quantize(W, bits, base, range_=float(np.abs(w).max()))
     assert torch.equal(codes, want)
     assert bytes(cb) == bytes(wcb)
+
+
+@pytest.mark.parametrize("bits,base", [(8, 1e30), (4, 1e100), (3, 1e300)])
+def test_boundaries_below_fp64(logq, bits, base):
+    """Boundaries that underflow fp64 to 0: zeros keep code 0, the smallest subnormals do not."""
+    w = workloads.weights_np(9, 256, seed=bits)
+    w[0, :4] = [0.0, -0.0, np.nextafter(np.float32(0), np.float32(1)), -1e-40]
+    W = torch.from_numpy(w).cuda()
+    codes, cb = logq.logq_quantize(W, bits, base)
+    want, wcb = logq.logq_quantize(W, bits, base, range_=float(np.abs(w).max()))
+    assert torch.equal(codes, want) and bytes(cb) == bytes(wcb)
+    m = (np.abs(w)[..., None] >= np.array(cb.thresh[:cb.qmax], np.float32)).sum(-1)
+    q = oracle.unpack(codes.cpu().numpy().reshape(9, -1), 9, 256, bits)
+    np.testing.assert_array_equal(q, np.where(w < 0, -m, m))
+    assert q[0, 0] == q[0, 1] == 0 and q[0, 2] > 0 and q[0, 3] < 0
 
 
 @pytest.mark.parametrize("bits", [3, 4, 8])
