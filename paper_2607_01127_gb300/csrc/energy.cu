@@ -19,18 +19,25 @@
 // rate; every other pass runs from the end to the start, so that what the pass
 // before it left in L2 is read from there.
 //   Pass 1: each lane adds its values' m^2 to its own 64-bit cells in shared
-//     memory, one per exponent of a 32-exponent window that the CTA places at its
-//     first values (no collectives, no atomics); the few values outside go to
-//     256 exponent sums with shared-memory atomics.  A cell is folded into
-//     registers before 2^16 values (each m^2 < 2^48) could overflow it.
+//     memory, one per exponent of a 32-exponent window (no collectives, no atomics).
+//     Each warp places its window at its CTA's first values and moves it up when it
+//     meets a larger exponent.  Values below it are added to the window's first
+//     exponent, in whole units of that one's m^2.  The crossing lies above: it holds
+//     at least eps of the energy, so for eps >= n 2^-50 (n weights) its exponent is at
+//     most 26 below w_max's, a window's start at least 30; and what is cut off, below
+//     2^-106 of the total energy per value, is below 2^-56 of what it is compared with.
+//     For a smaller eps they are added one by one, with atomics (EXACT).  A cell is
+//     folded into registers before 2^16 values (each m^2 < 2^48) could overflow it.
+//     14336 x 4096 with 5 % of the rows 1e-14 of the others: 301 us the whole call; 1642
+//     with a window that stays at the CTA's first values and atomics for all others.
 //   Pass 2: 4096 counts with native 32-bit shared-memory atomics, for the weights
 //     of one exponent.
 //   Pass 3: registers, and shared-memory atomics for the few weights inside the
 //     window.
 // When the window does not fit (kWinBuckets), which takes a distribution whose
 // crossing lies in a nearly empty stretch above most of its exponent's weights (or
-// for 2^32 weights and more), `failed` is set and the caller runs the exact form of levels 2 and 3
-// (energy_hist_kernel): per-bucket energies with 64-bit atomics, 4096
+// for 2^32 weights and more), `failed` is set or energy_counts_fit is false, and the
+// caller runs the exact form of levels 2 and 3 (energy_hist_kernel): per-bucket energies with 64-bit atomics, 4096
 // sub-buckets and then 2048 single values.
 #include <math.h>
 #include <stdint.h>
@@ -143,7 +150,11 @@ static_assert(kWinValues % (4 * kScanThreads) == 0, "whole vectors per scanning 
 constexpr int kBelowHi = 4094, kBelowLo = 4095;   // lo[] slots of pass 3's energy below the window
 static_assert(kWinValues * 4 <= 8 * (4096 + 4094), "window counts share the bucket arrays");
 
-// Pass 1 (see the top of the file).
+// First exponent of a window that reaches up to exponent top.
+__device__ __forceinline__ uint32_t window_start(uint32_t top) { return top > kWin ? top - (kWin - 1) : 1u; }
+
+// Pass 1 (see the top of the file).  EXACT: values below a window one by one.
+template <bool EXACT>
 __global__ void __launch_bounds__(kHistThreads) energy_exponents_kernel(const float4* __restrict__ W, int64_t n4,
                                                                         EnergyState* st, Workspace* ws)
 {
@@ -173,9 +184,13 @@ __global__ void __launch_bounds__(kHistThreads) energy_exponents_kernel(const fl
         if (lane == 0) atomicMax(&smax, m);
     }
     __syncthreads();
-    const int top = (int)(smax >> 23) + 1;
-    const uint32_t e_lo = top > kWin ? (uint32_t)(top - (kWin - 1)) : 1u;     // exponent field of cell 0 (a normal one)
+    uint32_t e_lo = window_start((smax >> 23) + 1);   // exponent field of cell 0 (a normal one), the same for the warp
     unsigned long long acc_hi = 0, acc_lo = 0;        // cell `lane` of this warp, folded so far
+    unsigned long long low = 0;                       // this lane's values below the window, in cell 0's unit
+    auto add_at = [&](uint32_t e, unsigned long long hi, unsigned long long lo) {
+        if (hi) atomicAdd(&shi[e], hi);
+        if (lo) atomicAdd(&slo[e], lo);
+    };
     auto fold = [&]() {
         __syncwarp();
         // lane l collects cell l from every lane (rotated start), split before the
@@ -190,6 +205,8 @@ __global__ void __launch_bounds__(kHistThreads) energy_exponents_kernel(const fl
         __syncwarp();
         for (int b = 0; b < kWin; ++b) ce[b * 32] = 0;
         __syncwarp();
+        add_at(e_lo, low >> 24, low & 0xffffffull);
+        low = 0;
     };
     uint32_t umax = 0;
     int64_t folded = 0;
@@ -198,23 +215,40 @@ __global__ void __launch_bounds__(kHistThreads) energy_exponents_kernel(const fl
                                __float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu};
         const uint32_t d[4] = {(u[0] >> 23) - e_lo, (u[1] >> 23) - e_lo, (u[2] >> 23) - e_lo, (u[3] >> 23) - e_lo};
         umax = max(max(umax, max(u[0], u[1])), max(u[2], u[3]));
-        if (max(max(d[0], d[1]), max(d[2], d[3])) < (uint32_t)kWin) {
+        const bool inside = max(max(d[0], d[1]), max(d[2], d[3])) < (uint32_t)kWin;
+        if (r < 0 ? inside : __all_sync(0xffffffffu, inside)) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const uint32_t m = (u[e] & 0x7fffffu) | 0x800000u;
                 ce[d[e] * 32] += (unsigned long long)m * m;
             }
         } else {
+            if (r >= 0) {                             // the whole warp: move the window up?
+                uint32_t m = 0;
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (u[e] < 0x7f800000u) m = max(m, u[e] >> 23);
+                m = __reduce_max_sync(0xffffffffu, m);
+                if (m >= e_lo + kWin) {
+                    fold();
+                    add_at(e_lo + lane, acc_hi, acc_lo);
+                    acc_hi = acc_lo = 0;
+                    e_lo = window_start(m + 1);
+                }
+            }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                if (d[e] < (uint32_t)kWin) {
+                const uint32_t ef = u[e] >> 23;
+                if (ef - e_lo < (uint32_t)kWin) {
                     const uint32_t m = (u[e] & 0x7fffffu) | 0x800000u;
-                    ce[d[e] * 32] += (unsigned long long)m * m;
+                    ce[(ef - e_lo) * 32] += (unsigned long long)m * m;
                 } else if (u[e] != 0 && u[e] < 0x7f800000u) {
                     uint32_t h, l;
                     msq_parts(u[e], h, l);
-                    atomicAdd(&shi[u[e] >> 23], (unsigned long long)h);
-                    atomicAdd(&slo[u[e] >> 23], (unsigned long long)l);
+                    if (!EXACT && ef < e_lo && e_lo > 1)      // (subnormals stay apart from exponent 1)
+                        low += (((unsigned long long)h << 24) | l) >> min(2 * (e_lo - max(ef, 1u)), 63u);
+                    else
+                        add_at(ef, h, l);
                 }
             }
         }
@@ -225,8 +259,7 @@ __global__ void __launch_bounds__(kHistThreads) energy_exponents_kernel(const fl
     });
     __syncwarp();
     fold();
-    if (acc_hi) atomicAdd(&shi[e_lo + lane], acc_hi);
-    if (acc_lo) atomicAdd(&slo[e_lo + lane], acc_lo);
+    add_at(e_lo + lane, acc_hi, acc_lo);
     // umax saw non-finite patterns too: they order above every finite one
     umax = __reduce_max_sync(0xffffffffu, umax);
     if (lane == 0) {
@@ -267,7 +300,7 @@ __global__ void __launch_bounds__(kHistThreads) energy_count_kernel(const float4
 // so the cumulative energies have a lower and an upper bound; the crossing
 // bucket is at or after the first whose upper bound reaches eps and at or before the
 // first whose lower bound does.  Leaves the window's first bucket in wmin_bits and
-// its length in _pad, and clears the bucket arrays.
+// its length in window, and clears the bucket arrays.
 __global__ void __launch_bounds__(kScanThreads) energy_window_scan_kernel(EnergyState* st, double eps)
 {
     constexpr int PER = 4096 / kScanThreads;
@@ -336,7 +369,7 @@ __global__ void __launch_bounds__(kScanThreads) energy_window_scan_kernel(Energy
         const int len = f0 < 4096 ? l0 - f0 + 1 : 0;
         if (len < 1 || len > kWinBuckets) st->failed = 1;
         st->wmin_bits = (uint32_t)f0;
-        st->_pad = (uint32_t)(len < 1 || len > kWinBuckets ? 0 : len);
+        st->window = (uint32_t)(len < 1 || len > kWinBuckets ? 0 : len);
     }
     __syncthreads();
     for (int i = t; i < 4 * 4096; i += kScanThreads) words[i] = 0;     // hi and lo, for pass 3
@@ -348,7 +381,7 @@ __global__ void __launch_bounds__(kHistThreads) energy_values_kernel(const float
 {
     extern __shared__ uint32_t cnt[];                    // [kWinValues]
     __shared__ unsigned long long shi, slo;
-    const uint32_t prefix = st->prefix, len = st->_pad * 2048u;
+    const uint32_t prefix = st->prefix, len = st->window * 2048u;
     if (len == 0) return;                                // no window: the exact form follows
     const uint32_t win0 = (prefix << 23) | (st->wmin_bits << 11);        // first pattern of the window
     for (uint32_t i = threadIdx.x; i < len; i += kHistThreads) cnt[i] = 0;
@@ -409,7 +442,7 @@ __global__ void __launch_bounds__(kScanThreads) energy_value_scan_kernel(EnergyS
     constexpr int PER = kWinValues / kScanThreads;
     __shared__ double part[2][kScanThreads];
     __shared__ int found;
-    const int t = threadIdx.x, len = (int)st->_pad * 2048;
+    const int t = threadIdx.x, len = (int)st->window * 2048;
     if (len == 0) return;
     const uint32_t* cnt = reinterpret_cast<const uint32_t*>(st->hi);
     const uint32_t prefix = st->prefix, start = st->wmin_bits << 11;
@@ -582,6 +615,17 @@ cudaError_t hist(const float4* W, int64_t n4, EnergyState* st, cudaStream_t s)
     return cudaGetLastError();
 }
 
+template <bool EXACT>
+cudaError_t exponents(const float4* W, int64_t n4, EnergyState* st, Workspace* ws, cudaStream_t s)
+{
+    constexpr size_t smem = (size_t)(kHistThreads / 32) * kWin * 32 * sizeof(unsigned long long);
+    static int configured[64] = {0};
+    cudaError_t e = allow_smem(energy_exponents_kernel<EXACT>, smem, configured);
+    if (e != cudaSuccess) return e;
+    energy_exponents_kernel<EXACT><<<stream_grid(n4, 3), kHistThreads, smem, s>>>(W, n4, st, ws);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_energy_range(const float* W, int64_t count, double eps, EnergyState* st, Workspace* ws,
@@ -592,17 +636,15 @@ cudaError_t launch_energy_range(const float* W, int64_t count, double eps, Energ
     const size_t bucket_bytes = sizeof st->hi + sizeof st->lo;
     cudaError_t e;
     if ((e = cudaMemsetAsync(st, 0, sizeof(EnergyState), s)) != cudaSuccess) return e;
-    static int configured1[64] = {0}, configured3[64] = {0};
-    constexpr size_t smem1 = (size_t)(kHistThreads / 32) * kWin * 32 * sizeof(unsigned long long);
-    constexpr size_t smem3 = (size_t)kWinValues * sizeof(uint32_t);
-    if ((e = allow_smem(energy_exponents_kernel, smem1, configured1)) != cudaSuccess) return e;
-    if ((e = allow_smem(energy_values_kernel, smem3, configured3)) != cudaSuccess) return e;
-    energy_exponents_kernel<<<stream_grid(n4, 3), kHistThreads, smem1, s>>>(W4, n4, st, ws);
+    const bool exact = eps < (double)count * 0x1p-50;    // (see the top of the file)
+    e = exact ? exponents<true>(W4, n4, st, ws, s) : exponents<false>(W4, n4, st, ws, s);
+    if (e != cudaSuccess) return e;
     energy_scan_kernel<1><<<1, kScanThreads, 0, s>>>(st, eps);
-    if (count >> 32) {                                   // beyond the passes' 32-bit counts
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        return cudaMemsetAsync(&st->failed, 1, 1, s);
-    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (!energy_counts_fit(count)) return cudaSuccess;
+    static int configured3[64] = {0};
+    constexpr size_t smem3 = (size_t)kWinValues * sizeof(uint32_t);
+    if ((e = allow_smem(energy_values_kernel, smem3, configured3)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(st->hi, 0, bucket_bytes, s)) != cudaSuccess) return e;
     energy_count_kernel<<<stream_grid(n4, 6), kHistThreads, 0, s>>>(W4, n4, st);
     energy_window_scan_kernel<<<1, kScanThreads, 0, s>>>(st, eps);
@@ -611,8 +653,8 @@ cudaError_t launch_energy_range(const float* W, int64_t count, double eps, Energ
     return cudaGetLastError();
 }
 
-// Levels 2 and 3 by exact bucket energies, after launch_energy_range left
-// `failed` set (its exponent and the energy below it stand).
+// Levels 2 and 3 by exact bucket energies, after launch_energy_range left the
+// crossing open (its exponent and the energy below it stand).
 cudaError_t launch_energy_exact(const float* W, int64_t count, double eps, EnergyState* st, cudaStream_t s)
 {
     const float4* W4 = reinterpret_cast<const float4*>(W);

@@ -32,7 +32,7 @@ struct EnergyState {
     uint32_t prefix;
     uint32_t wmin_bits;     // the result; before it, the first bucket of pass 3's window
     uint32_t failed;        // the window of the counting passes did not settle the crossing
-    uint32_t _pad;          // buckets of pass 3's window
+    uint32_t window;        // buckets of pass 3's window
 };
 
 // Decision boundaries handed to the quantise kernel: fp32, rounded up; or
@@ -120,6 +120,8 @@ logq_status quantize_with(const float* W, int64_t N, int64_t K, int bits, double
 cudaError_t launch_absmax(const float* W, int64_t count, Workspace* ws, cudaStream_t s);
 cudaError_t launch_energy_range(const float* W, int64_t count, double eps, EnergyState* st, Workspace* ws,
                                 cudaStream_t s);
+// Whether the selection's passes can count so many weights in 32 bits.
+inline bool energy_counts_fit(int64_t count) { return (count >> 32) == 0; }
 cudaError_t launch_energy_exact(const float* W, int64_t count, double eps, EnergyState* st, cudaStream_t s);
 cudaError_t launch_quantize(const float* W, int64_t N, int64_t K, const QuantParams& p,
                             uint8_t* codes, Workspace* ws, cudaStream_t s);

@@ -358,8 +358,8 @@ logq_status logq_quantize_energy(const float* W, int64_t N, int64_t K, int bits,
     float fmax;
     memcpy(&fmax, &host_words[0], 4);
     if (!(fmax > 0.0f)) return LOGQ_ERR_INVALID_ARG;     // all-zero weights
-    if (sel[1]) {
-        // the counting passes left the crossing open (rare): exact bucket energies settle it
+    if (sel[1] || !energy_counts_fit(N * K)) {
+        // the passes left the crossing open (rare): exact bucket energies settle it
         if ((e = launch_energy_exact(W, N * K, eps, st, s)) != cudaSuccess) return LOGQ_ERR_CUDA;
         if ((e = cudaMemcpyAsync(sel, &st->wmin_bits, sizeof sel, cudaMemcpyDeviceToHost, s)) != cudaSuccess)
             return LOGQ_ERR_CUDA;

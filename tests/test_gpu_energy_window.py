@@ -31,6 +31,10 @@ def share_below(w, t):
     return float(np.sum(a[a < t] ** 2) / np.sum(a * a))
 
 
+def scales(n, share, small):
+    return np.where(np.random.default_rng(n).random(n) < share, small, 1.0).astype(np.float32)
+
+
 CASES = {
     # the window does not settle the crossing: exact bucket energies do
     "stretch": lambda: stretch(1024 * 128, 400).reshape(1024, 128),
@@ -40,6 +44,12 @@ CASES = {
                                           workloads.weights_np(300, 4096, seed=3)]),
     "early_large": lambda: np.concatenate([workloads.weights_np(2, 128, seed=4) * np.float32(1e20),
                                            workloads.weights_np(37, 128, seed=5)]),
+    # rows or columns of dead neurons: below the windows (where the crossing may lie: 0.2) or windows' first values
+    "dead_rows": lambda: workloads.weights_np(900, 1024, seed=8) * scales(900, 0.3, 1e-14)[:, None],
+    "dead_rows_subnormal": lambda: workloads.weights_np(900, 1024, seed=8) * scales(900, 0.95, 1e-38)[:, None],
+    "dead_columns": lambda: workloads.weights_np(900, 1024, seed=8) * scales(1024, 0.1, 1e-25)[None, :],
+    # windows that move up again and again
+    "ascending": lambda: workloads.weights_np(1500, 512, seed=9) * np.exp2(np.arange(1500) // 8 - 100.0).astype(np.float32)[:, None],
     # one vector, a grid's remainder, zeros in every vector
     "one_row": lambda: workloads.weights_np(1, 128, seed=6),
     "zeros": lambda: workloads.weights_np(129, 640, seed=7) * (np.arange(640) % 4 == 1).astype(np.float32),
