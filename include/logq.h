@@ -37,16 +37,17 @@
  *   - Linear launches (logq_linear, logq_linear_grouped) use programmatic
  *     dependent launch: they may start while the preceding kernel on the stream
  *     finishes.  They read X and write Y only after that kernel has completed
- *     and its writes are visible, but those of up to 7 rows at 4 bits and 4 rows
- *     at 3 and 8 bits (small decode launches) read the packed codes earlier,
- *     before that guarantee holds.  So for them the codes must be complete
+ *     and its writes are visible, but small decode launches read the packed codes
+ *     earlier, before that guarantee holds: up to 4 rows at 3 and 8 bits; at 4
+ *     bits up to 7 rows, 8 rows of matrices of up to 32 M weights in the call, and
+ *     16 rows of up to 8 M.  So for them the codes must be complete
  *     before the call is enqueued, ordered by a host synchronisation after the
  *     kernel that wrote them (of its stream, of an event recorded after it, or
  *     of the device), not by stream order alone.  logq_quantize and
  *     logq_quantize_energy end with such a synchronisation; after logq_gptq
  *     the caller synchronises.  Weights quantised once and reused (the decode
- *     case) meet this.  Launches of more rows keep to stream order for their
- *     codes too.
+ *     case) meet this.  All other launches keep to stream order for their codes
+ *     too.
  *   - Device code never traps.  Conditions found on the device (non-finite
  *     weights, a pipeline wait that exceeded its bound) are written to the
  *     caller's workspace and reported by logq_quantize or logq_workspace_status.

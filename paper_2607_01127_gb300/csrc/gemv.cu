@@ -708,7 +708,7 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
     p.K = (int32_t)a.K;
     p.B = (int32_t)a.B;
     p.y_dtype = a.y_dtype;
-    p.wait_codes = reads_codes_early(a.bits, a.B) ? 0 : 1;
+    p.wait_codes = reads_codes_early(a.bits, a.B, total_rows * a.K) ? 0 : 1;
     p.row_bytes = (int32_t)row_bytes;
     p.blocks = (int32_t)(a.K / (4 * lane_k(a.bits)));
     p.spans = (p.blocks + sh.S * sh.J - 1) / (sh.S * sh.J);

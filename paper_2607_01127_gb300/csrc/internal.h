@@ -156,9 +156,16 @@ cudaError_t launch_split_sum(const SplitSum& a, int splits, int y_dtype, cudaStr
 // Whether the decode kernel runs a batch (rows: of all the call's matrices).
 bool gemv_takes(int bits, int64_t B, int64_t rows, int64_t K);
 // Decode launches that may read codes before the launch ahead of them has completed,
-// as include/logq.h says: up to 7 rows at 4 bits, 4 at 3 and 8 bits.  Larger batches
-// keep to stream order for their codes, as prefill launches do, at 4 to 5 % of a layer's
-// time (batch 16: 4 bits 66.6 us, 63.2 without; 3 bits 78, 75 without).
-inline bool reads_codes_early(int bits, int64_t B) { return B <= (bits == 4 ? 7 : 4); }
+// as include/logq.h says (weights: of all the call's matrices).  They are those that the
+// library has never run in a kernel that keeps to stream order for its codes: 3 and 8
+// bits up to 4 rows, 4 bits up to 7, and up to 16 where the model that the workspace is
+// sized by (prefill_plan against 0.46e-6 us a weight at 8 rows, 0.84e-6 beyond, plus 2)
+// keeps off the tensor-core launch whatever the shape: its estimate is at least
+// 6 + 0.4e-6 us a weight.  All others wait, at 4 to 5 % of a layer's time.
+inline bool reads_codes_early(int bits, int64_t B, int64_t weights)
+{
+    if (bits != 4) return B <= 4;
+    return B <= 7 || (B == 8 && weights <= (int64_t)32 << 20) || (B <= 16 && weights <= (int64_t)8 << 20);
+}
 
 }  // namespace logq

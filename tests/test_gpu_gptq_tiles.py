@@ -56,11 +56,13 @@ def test_rows_do_not_depend_on_the_tiles(logq, bits):
         assert torch.equal(part, codes[r0:r0 + n])
 
 
-@pytest.mark.parametrize("bits,B", [(4, 8), (4, 16), (4, 17), (4, 40), (8, 5), (8, 16), (8, 40)])
-def test_linear_right_after_gptq(logq, bits, B):
-    """Batches that keep to stream order read the codes that GPTQ has just written,
-    in the decode kernel and in the prefill kernel."""
-    K, N = 256, 9000
+@pytest.mark.parametrize("bits,B,N", [(4, 8, 132000), (4, 16, 33000), (4, 17, 9000), (4, 40, 9000), (8, 5, 9000),
+                                      (8, 16, 9000), (8, 40, 9000)])
+def test_linear_right_after_gptq(logq, bits, B, N):
+    """Launches that keep to stream order (4 bits: 8 rows of more than 32 M weights, 16 of
+    more than 8 M) read the codes that GPTQ has just written, in the decode kernel and in
+    the prefill kernel."""
+    K = 256
     H = torch.from_numpy(hessian(K, 6, T=2 * K).astype(np.float32)).cuda()
     W = torch.from_numpy(workloads.weights_np(N, K, seed=10)).cuda()
     cb = logq.logq_build_codebook(bits, {4: 2.0, 8: 1.05}[bits], float(W.abs().max()))
