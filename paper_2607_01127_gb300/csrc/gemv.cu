@@ -304,7 +304,8 @@ __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ 
     const int bcol = HALVES ? (gq >> 1) / HS : gq / S;
     const int G = 1 << p.lg_groups, SC = p.span_cols;
     const int g = warp & (G - 1), scol = warp >> p.lg_groups;
-    const bool compute_warp = scol < SC && s0 + scol < s1;
+    // (a warp whose first tile starts past the rows would only load activations)
+    const bool compute_warp = scol < SC && s0 + scol < s1 && g * RT < r1 - r0;
     struct Tile { uint32_t w[2][J][NW]; };
     Tile ct[T];
     // The span being worked on: address of this lane's codes in row q0.  Blocks
@@ -534,7 +535,9 @@ __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ 
 }
 
 // Added to a padded batch: the shape for short rows (shape_key).
-constexpr int kShort = 64;
+constexpr int kShort = 64, kMid = 128;
+// Launches of up to this many weights keep to one CTA per SM (per_sm).
+constexpr int64_t kOneCta = (int64_t)4 << 20;
 
 // Launch shape of a batch: S segments, J blocks, NTL column tiles,
 // T tiles in flight, threads per CTA, CTAs per SM.
@@ -603,6 +606,9 @@ cudaError_t shape_or_run(int key, Shape* sh, const GemvParams* p, const GroupArg
             LOGQ_SHAPE(8, 1, 2, 1, 2, 512, 1);
             LOGQ_SHAPE(16, 1, 2, 2, 1, 512, 1);
             LOGQ_SHAPE(32, 1, 2, 4, 1, 256, 1);
+            LOGQ_SHAPE(kShort + 1, 4, 1, 1, 4, 256, 2);
+            LOGQ_SHAPE(kShort + 2, 4, 1, 1, 4, 256, 2);
+            LOGQ_SHAPE(kShort + 4, 2, 1, 1, 4, 256, 2);
         }
     } else if constexpr (BITS == 4) {
         switch (key) {
@@ -612,7 +618,8 @@ cudaError_t shape_or_run(int key, Shape* sh, const GemvParams* p, const GroupArg
             LOGQ_SHAPE(8, 1, 2, 1, 2, 512, 1);
             LOGQ_SHAPE(16, 1, 4, 2, 2, 256, 1);
             LOGQ_SHAPE(32, 1, 2, 4, 1, 256, 1);
-            LOGQ_SHAPE(kShort + 1, 2, 1, 1, 5, 256, 2);
+            LOGQ_SHAPE(kShort + 1, 2, 1, 1, 4, 256, 2);
+            LOGQ_SHAPE(kMid + 1, 4, 1, 1, 4, 256, 2);
             LOGQ_SHAPE(kShort + 2, 4, 1, 1, 4, 256, 2);
             LOGQ_SHAPE(kShort + 4, 2, 1, 1, 5, 256, 2);
             LOGQ_SHAPE(kShort + 8, 1, 2, 1, 3, 256, 1);
@@ -626,6 +633,10 @@ cudaError_t shape_or_run(int key, Shape* sh, const GemvParams* p, const GroupArg
             LOGQ_SHAPE(8, 2, 2, 2, 2, 512, 1);
             LOGQ_SHAPE(16, 1, 4, 2, 2, 256, 1);
             LOGQ_SHAPE(32, 1, 4, 4, 1, 256, 1);
+            LOGQ_SHAPE(kShort + 1, 4, 1, 1, 5, 256, 2);
+            LOGQ_SHAPE(kShort + 2, 4, 1, 1, 5, 256, 2);
+            LOGQ_SHAPE(kMid + 2, 4, 2, 1, 3, 256, 2);
+            LOGQ_SHAPE(kShort + 4, 2, 2, 1, 3, 256, 2);
         }
     }
 #undef LOGQ_SHAPE
@@ -641,21 +652,44 @@ cudaError_t shape_or_run(int bits, int key, Shape* sh, const GemvParams* p, cons
                      : shape_or_run<3, F16>(key, sh, p, a, grid, smem, s);
 }
 
-// Key of a call's launch shape: the batch padded to a power of two, plus kShort for
-// 4-bit rows of less than 4096 k.  Those fill a CTA's warps with spans of the wide
-// shapes only by sharing each span among several warps, all of which read its
-// activations; shapes with shorter spans spare that.  2048 x 2048 / 16384 x 2048, us:
-// batch 1 2.8 -> 2.35 / (5.4, 6.1 with the short one, so only up to 8 M weights),
-// batch 2 3.1 -> 2.85 / 5.7 -> 5.6, batch 4 3.6 -> 2.8 / 7.5 -> 6.5, batch 8
-// 3.6 -> 2.7 / 8.5 -> 7.75, batch 16 4.9 -> 3.45 / 11.9 -> 9.7; 4096 x 4096 at
-// batch 16 7.5, 8.3 with the short one.
+// Key of a call's launch shape: the batch padded to a power of two, plus kShort or kMid for
+// short rows.  Those fill a CTA's warps with spans of the wide shapes only by sharing each
+// span among several warps, all of which read its activations; shapes with shorter spans
+// spare that.  Single launches, us, wide shape / this one (rows x k, batch in brackets):
+//   3 bits: 512 x 2048 (1) 2.38 / 1.86, (2) 2.65 / 1.95; 8192 x 512 (1) 2.86 / 2.27, (4) 3.39 /
+//     2.5; 2048 x 2048 (2) 3.14 / 2.4, (4) 3.66 / 2.6; 16384 x 2048 (2) 6.6 / 6.35;
+//   4 bits: 8192 x 512 (2) 2.42 here, 4096 k (2): 1024 rows 3.0 / 2.4, 28672 rows 14.9 / 14.3;
+//     1000 x 3968 (1) 2.32 (kMid), 3.25 with the kShort shape, whose spans take two passes
+//     from K = 2176 on; 2048 x 2048 (8) 3.6 / 2.7, (16) 4.9 / 3.45; 4096 x 4096 (16) 7.5, 8.3
+//     with the short one;
+//   8 bits: 8192 x 512 (1) 3.46 / 2.7; 512 x 2048 (2) 2.84 / 1.9; 16384 x 2048 (2) 9.1 / 8.6, (4)
+//     10.8 / 10.0; 6144 x 4096 (2, kMid) 7.6 / 7.2; 2048 x 2048 (1) 2.65 / 2.73, so batch 1
+//     only up to 1024 k.
+// Batch 1 at 3 and 4 bits: up to 8 M weights (16384 x 2048 in a chain of the 1B shapes 0.06 us
+// slower with the short shape, 32768 x 2048 at 3 bits 9.8 / 10.3).
 int shape_key(int bits, int64_t B, int64_t rows, int64_t K)
 {
     int key = 1;
     while (key < B) key *= 2;
-    if (bits == 4 && K < 4096 && key <= 16 && (key > 1 || rows * K <= (int64_t)8 << 20)) key += kShort;
+    const bool few = rows * K <= (int64_t)8 << 20;
+    if (bits == 4) {
+        if (key == 1 && K < 4096 && few) key += K <= 2048 ? kShort : kMid;
+        else if (key == 2 ? K <= 4096 : key == 4 ? K <= 2048 : K < 4096 && key >= 8 && key <= 16) key += kShort;
+    } else if (bits == 3) {
+        if (key == 1 ? K < 4096 && few : key == 2 ? K <= 4096 : key == 4 && K <= 2048) key += kShort;
+    } else {
+        if (key == 1 ? K <= 1024 : key <= 4 && K <= 2048) key += kShort;
+        else if (key == 2 && K <= 4096) key += kMid;
+    }
     return key;
 }
+
+// CTAs of a launch per SM: as many as fit, but one for small launches of the shapes that
+// fit twice, so that the next launch's CTAs find room on every SM from the start (their
+// table and first code loads then run beside this launch).  1B step, one CTA per SM for no
+// launch / up to 4 M weights (o) / up to 8 M (q/k/v too): batch 1 233.2 / 232.4 / 235.6 us,
+// batch 2 265.3 / 256.6 / 258.9, batch 4 286.7 / 279.5 / 284.4.
+int per_sm(const Shape& sh, int64_t weights) { return weights <= kOneCta ? 1 : sh.MINB; }
 
 // The table lookups address shared memory relative to kTabOff, which is where
 // dynamic shared memory starts when a kernel has no static shared memory.
@@ -733,13 +767,12 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
     // Each matrix's rows are divided among row ranges (kparts CTAs each), in
     // proportion to the rows: at least one range each, at most one per tile.
     const int sms = sm_count() > 0 ? sm_count() : 148;
-    const int per_sm = sh.MINB;
     const int64_t rt = 16 / sh.S;
     p.pf = static_cast<const uint8_t*>(a.pf);
     p.pf_bytes = (a.pf && a.pf_bytes < kPrefetchBytes) ? a.pf_bytes : 0;
     int64_t units[kMaxItems], total_units = 0;
     for (int i = 0; i < a.count; ++i) total_units += (units[i] = (a.item[i].N + rt - 1) / rt);
-    const int64_t ranges = (int64_t)sms * per_sm / kparts;
+    const int64_t ranges = (int64_t)sms * per_sm(sh, total_rows * a.K) / kparts;
     int grid = (int)(total_units < ranges ? total_units : ranges);
     if (grid < a.count) grid = a.count;
     int ctas[kMaxItems] = {0};

@@ -43,10 +43,12 @@ def test_decode_shapes(logq, bits, B, N, K):
     check(logq.logq_linear(codes, cb, X, N, K), *reference(X, q, ocb))
 
 
-@pytest.mark.parametrize("bits,B,N,K", [(4, 17, 1024, 4096), (3, 32, 2048, 2048), (8, 24, 1024, 4096), (4, 1, 2114, 3968), (4, 1, 65536, 128)])
+@pytest.mark.parametrize("bits,B,N,K", [(4, 17, 1024, 4096), (3, 32, 2048, 2048), (8, 24, 1024, 4096), (4, 1, 2114, 3968), (4, 1, 65536, 128),
+                                           (3, 1, 2114, 3968), (4, 2, 1024, 4096), (8, 1, 32768, 128)])
 def test_both_sides_of_a_dispatch_line(logq, bits, B, N, K):
-    """N rows are the most of the one path (batches above 16: up to 4 M weights;
-    short rows at batch 1: up to 8 M); one more row takes the other."""
+    """N rows are the most of the one path (batches above 16: up to 4 M weights; one CTA
+    per SM: up to 4 M; short rows at batch 1, 3 and 4 bits: up to 8 M); one more row takes
+    the other."""
     codes, cb, ocb, q = make_layer(logq, N + 1, K, bits, BASE[bits], 1)
     X = workloads.activations_torch(B, K, 2, torch.bfloat16, "cuda")
     more = logq.logq_linear(codes, cb, X, N + 1, K)
@@ -58,6 +60,18 @@ def test_both_sides_of_a_dispatch_line(logq, bits, B, N, K):
         check(more[:, rows], Yr, A)
     else:          # the tensor-memory kernel's chains truncate K / 16 times
         assert np.all(np.abs(more[:, rows].double().cpu().numpy() - Yr) <= (K / 16 + 60) * 2.0 ** -23 * A)
+
+
+# k on both sides of the lines between the shapes for short rows; fewer rows than a CTA's
+# warps have tiles for, and more
+@pytest.mark.parametrize("bits", [3, 4, 8])
+@pytest.mark.parametrize("B", [1, 2, 4])
+@pytest.mark.parametrize("K", [1024, 1152, 2048, 2176, 4096, 4224])
+def test_short_rows(logq, bits, B, K):
+    for N in (3, 2000):
+        codes, cb, ocb, q = make_layer(logq, N, K, bits, BASE[bits], K + B)
+        X = workloads.activations_torch(B, K, B, torch.bfloat16, "cuda")
+        check(logq.logq_linear(codes, cb, X, N, K), *reference(X, q, ocb))
 
 
 @pytest.mark.parametrize("bits", [3, 4, 8])
