@@ -151,14 +151,21 @@ __host__ __device__ constexpr int chains_for(int bits, int S, int NTL)
     return NTL == 1 ? (bits == 4 && S <= 2 ? 4 : 8) : NTL == 2 ? 2 : 1;
 }
 constexpr int kMaxSmem = 226 * 1024;
-// Shared memory of partial sums after a table of tab bytes, per_sm CTAs on an SM.
-constexpr int64_t red_bytes(size_t tab, int per_sm) { return (int64_t)227 * 1024 / per_sm - 1024 - (int64_t)tab; }
-// Shared-memory carveout of the batch-1/2 kernels, in percent of the maximum:
-// 58 % is 132 KiB, room for two CTAs of 64 KiB (plus their reserved 1 KiB).
-// The rest of the 256 KiB per SM is L1, which also holds the data of the code
-// loads in flight; one setting for all of them spares the SMs a
-// reconfiguration between launches.
-constexpr int kCarveout = 58;
+// Shared-memory carveout of every shape, in percent of the maximum, which gives 164 KiB:
+// room for two CTAs of a 64 KiB table and 17 KiB of partial sums (red_bytes; rows that
+// need more are taken in chunks).  The rest of the 256 KiB per SM is L1, which holds
+// activations that several warps read and the code loads in flight; one setting for all
+// of them spares the SMs a reconfiguration between launches.  8B layer, 58 / 66 / 72 /
+// 86 % and the maximum: batch 1 31.7 / 31.6 / 31.9 / 33.6 / 33.4 us, 4 39.6 / 39.6 / 39.7 /
+// 42.0 / 41.9, 8 49.4 / 49.5 / 49.5 / 52.9 / 52.9, 16 63.0 / 63.0 / 63.6 / 66.7 / 66.8;
+// 8 bits at batch 16 95.2 / 95.2 / 96.2 / 100.2 / 100.1.
+constexpr int kCarveout = 66;
+// Shared memory of partial sums after a table of tab bytes, per_sm CTAs on an SM: two stay
+// within the carveout; one may ask for more.
+constexpr int64_t red_bytes(size_t tab, int per_sm)
+{
+    return (int64_t)(per_sm > 1 ? 164 : 227) * 1024 / per_sm - 1024 - (int64_t)tab;
+}
 
 // A lane's codes of a block: 16 bytes, or (3-bit) the three words of a 12-byte
 // group.  ALLOC: through L1 as usual; else without an L1 line.
@@ -564,8 +571,7 @@ cudaError_t run(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, 
     if (!configured[dev]) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 batch_cols(S, NTL) <= 2 ? kCarveout : (int)cudaSharedmemCarveoutMaxShared);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, kCarveout);
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
@@ -839,8 +845,10 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
     int64_t chunk = max_rows;
     if (pitch_for(chunk) * np > cap) {
         chunk = (cap / np - 32) / bc;
-        const int64_t step = (rt << p.lg_groups) * sh.T;       // whole rounds of every warp
+        const int64_t step = rt << p.lg_groups;                // a tile of every warp
+        const int64_t equal = (max_rows + (max_rows + chunk - 1) / chunk - 1) / ((max_rows + chunk - 1) / chunk);
         if (chunk > step) chunk -= chunk % step;
+        if ((equal + step - 1) / step * step < chunk) chunk = (equal + step - 1) / step * step;
     }
     if (chunk < 1) return cudaErrorInvalidValue;
     p.chunk_rows = (int32_t)chunk;

@@ -74,6 +74,19 @@ def test_short_rows(logq, bits, B, K):
         check(logq.logq_linear(codes, cb, X, N, K), *reference(X, q, ocb))
 
 
+@pytest.mark.parametrize("bits,B,N,K", [(4, 3, 21001, 2048), (4, 4, 33000, 2048), (8, 4, 47001, 1024), (4, 16, 60011, 128)])
+def test_rows_of_a_cta_in_chunks(logq, bits, B, N, K):
+    """More rows per CTA than its partial sums have room for: equal chunks, ragged ends."""
+    codes, cb, ocb, q = make_layer(logq, N, K, bits, BASE[bits], 9)
+    X = workloads.activations_torch(B, K, 3, torch.bfloat16, "cuda")
+    Y = logq.logq_linear(codes, cb, X, N, K)
+    rows = np.r_[0:400, N // 2:N // 2 + 300, N - 300:N]
+    Yr, A = reference(X, q[rows], ocb)
+    check(Y[:, rows], Yr, A)
+    part = logq.logq_linear(codes[:logq.logq_packed_bytes(999, K, bits)].clone(), cb, X, 999, K)
+    assert torch.equal(Y[:, :999], part)             # a row's sums do not depend on the chunks
+
+
 @pytest.mark.parametrize("bits", [3, 4, 8])
 @pytest.mark.parametrize("B", [9, 16, 32])
 @pytest.mark.parametrize("sets", [0, 1, 2, 3, 8])
