@@ -864,15 +864,16 @@ def run_ours(args):
 
 
 CASES = ("decode_layers_8b", "decode_step_1b", "skinny_gate_8b", "gemv_gateup_1b", "gemv_gate_8b", "prefill_q_8b",
-         "prefill_qkv_8b", "quantize_gate_8b", "energy_gate_8b",
-         "gemv8_gate_8b", "gptq_q_8b", "gptq_update_q_8b", "quantize3_gate_8b")
+         "prefill8_q_8b", "prefill_gate_8b_33", "prefill_qkv_8b", "quantize_gate_8b", "energy_gate_8b",
+         "gemv3_gate_8b", "gemv8_gate_8b", "gptq_q_8b", "gptq_update_q_8b", "quantize3_gate_8b")
 
 
 def run_case(name: str):
     """One small workload run twice (for a profiler capture of the second run):
     the gate+up launch of the 1B decode step, the 8B gate GEMV, the 8B q-shaped
-    prefill GEMM (2048 tokens) and the grouped q/k/v one, the quantisation of an 8B gate matrix, its
-    self-calibrating (energy-range) quantisation, the 8-bit gate GEMV and 4-bit
+    prefill GEMM (2048 tokens, 4 or 8 bits), the gate one at 33 tokens and the grouped q/k/v one,
+    the quantisation of an 8B gate matrix, its
+    self-calibrating (energy-range) quantisation, the 3- and 8-bit gate GEMVs and 4-bit
     GPTQ of an 8B q matrix (factor and quantisation; or the quantisation alone with a
     fixed upper-triangular factor standing in for U)."""
     import torch
@@ -915,10 +916,11 @@ def run_case(name: str):
         X = workloads.activations_torch(1, K, 1, torch.bfloat16, dev)
         for _ in range(2):
             logq.logq_linear(c[0], c[1], X, N, K, workspace=ws)
-    elif name == "prefill_q_8b":
-        N, K = workloads.LLAMA_8B_SHAPES["q"]
-        c = logq.logq_quantize(workloads.weights_torch(N, K, 14, True, dev), 4, 1.5, workspace=ws)
-        X = workloads.activations_torch(PREFILL_TOKENS, K, 2, torch.bfloat16, dev)
+    elif name in ("prefill_q_8b", "prefill8_q_8b", "prefill_gate_8b_33"):
+        N, K = workloads.LLAMA_8B_SHAPES["gate" if "gate" in name else "q"]
+        bits, base = (8, 1.04) if "8_q" in name else (4, 1.5)
+        c = logq.logq_quantize(workloads.weights_torch(N, K, 14, True, dev), bits, base, workspace=ws)
+        X = workloads.activations_torch(33 if name.endswith("_33") else PREFILL_TOKENS, K, 2, torch.bfloat16, dev)
         for _ in range(2):
             logq.logq_linear(c[0], c[1], X, N, K, y_dtype=torch.bfloat16, workspace=ws)
     elif name == "prefill_qkv_8b":
@@ -941,9 +943,10 @@ def run_case(name: str):
         W = workloads.weights_torch(N, K, 15, True, dev)
         for _ in range(2):
             logq.logq_quantize(W, 3, 1.8, workspace=ws)
-    elif name == "gemv8_gate_8b":
+    elif name in ("gemv3_gate_8b", "gemv8_gate_8b"):
         N, K = workloads.LLAMA_8B_SHAPES["gate"]
-        c = logq.logq_quantize(workloads.weights_torch(N, K, 13, True, dev), 8, 1.04, workspace=ws)
+        bits, base = (3, 1.8) if name.startswith("gemv3") else (8, 1.04)
+        c = logq.logq_quantize(workloads.weights_torch(N, K, 13, True, dev), bits, base, workspace=ws)
         X = workloads.activations_torch(1, K, 1, torch.bfloat16, dev)
         for _ in range(2):
             logq.logq_linear(c[0], c[1], X, N, K, workspace=ws)

@@ -178,8 +178,8 @@ logq_status logq_quantize(const float* W, int64_t N, int64_t K, int bits, double
  *   Y (device): y_dtype in {LOGQ_F32, x_dtype}; a 16-bit Y is the fp32 sum
  *   rounded to nearest-even.  All device pointers 16-byte aligned.
  *   B <= 16 runs the decode kernel, as does B <= 32 for matrices of up to 4 M
- *   weights; larger B runs the prefill GEMM kernel (tcgen05).  Calls sharing a workspace must be ordered on one stream
- *   (partial sums may live in it).
+ *   weights; larger B runs the prefill GEMM kernel (tcgen05).  Calls sharing a
+ *   workspace must be ordered on one stream (partial sums may live in it).
  * Asynchronous.  Errors: LOGQ_ERR_INVALID_ARG, LOGQ_ERR_UNSUPPORTED,
  * LOGQ_ERR_WORKSPACE, LOGQ_ERR_CUDA (launch).  A device-side wait that hit
  * its bound is reported later by logq_workspace_status. */
@@ -230,8 +230,9 @@ size_t logq_energy_scratch_bytes(void);
  *   Eq. (4) as printed -- and the codes exactly as logq_quantize with those
  *   arguments would produce them.
  * The selection runs on the device in three streaming passes over W (a radix
- * selection over the bit patterns of |w|) plus the quantisation pass; energies of equal-exponent buckets are summed exactly in
- * integers and accumulated across buckets in fp64, in ascending order of |w|.
+ * selection over the bit patterns of |w|) plus the quantisation pass; energies of
+ * equal-exponent buckets are summed in integers (exactly wherever they can reach
+ * the selection) and accumulated across buckets in fp64, in ascending order of |w|.
  *   eps in (0, 1].  wmin_out (host, may be NULL) receives w_min; cb_out (host,
  *   may be NULL) the codebook (its base is b, its range w_max).
  *   scratch: logq_energy_scratch_bytes() bytes of device memory.
@@ -325,10 +326,9 @@ typedef struct logq_linear_item {
  * of their codebooks.  Batches that the decode kernel takes (as logq_linear,
  * with the weights of all items) share a single launch of it.  Larger B runs
  * one prefill launch whose CTAs are divided among the matrices in proportion to
- * their tiles,
- * when its estimate beats one launch per matrix (small matrices such as k / v
- * projections then share the GPU with a larger one); otherwise one launch
- * each, as logq_linear.  The workspace holds the partial sums of split k
+ * their tiles, when its estimate beats one launch per matrix (small matrices
+ * such as k / v projections then share the GPU with a larger one); otherwise
+ * one launch each, as logq_linear.  The workspace holds the partial sums of split k
  * ranges as for logq_linear: logq_linear_grouped_workspace_bytes gives the
  * size with which the planned launches split fully.
  * l2_prefetch (device, may be NULL) / l2_prefetch_bytes name a range the

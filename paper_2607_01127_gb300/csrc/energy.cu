@@ -37,8 +37,8 @@
 // When the window does not fit (kWinBuckets), which takes a distribution whose
 // crossing lies in a nearly empty stretch above most of its exponent's weights (or
 // for 2^32 weights and more), `failed` is set or energy_counts_fit is false, and the
-// caller runs the exact form of levels 2 and 3 (energy_hist_kernel): per-bucket energies with 64-bit atomics, 4096
-// sub-buckets and then 2048 single values.
+// caller runs the exact form of levels 2 and 3 (energy_hist_kernel): per-bucket energies
+// with 64-bit atomics, 4096 sub-buckets and then 2048 single values.
 #include <math.h>
 #include <stdint.h>
 

@@ -33,17 +33,25 @@
 //    its table meanwhile.  At batch 1 two 8-warp CTAs run per SM for that; larger
 //    batches, which hold more activations per lane, fill an SM with one CTA.
 //
-// What bounds it: instruction issue (a byte permute, a lookup and 1/8 of an MMA per
-// pair of weights; resolving an eighth of the codes by permutes alone, 7 instructions
-// for 4 codes instead of 4, costs 2 %) and, per launch, the latency of a CTA's life
-// (activations after the previous launch, first tile, final sum: 2.3-3 us).  Per
-// Llama-3.1-8B layer (q+k+v, o, gate+up, down chained, bf16), with fused multiply-adds
-// on the CUDA cores (batches up to 8; 5 and more at 3 and 8 bits and 9 and more at 4 in
-// the prefill kernel) before and now:
+// What bounds it: nothing is saturated; the busiest unit is the L1 data path, which the
+// lookups share with the code and activation loads.  8B gate (14336 x 4096) at batch 1,
+// cycles per SM of the 15 300 of a launch in a chain (7.9 us): L1 data path 9 970 (lookups
+// and partial sums 7 400, loads 2 570), HBM 8 400 (29.4 MB), instruction issue 7 140 per
+// scheduler, and 16 warps to overlap them; the top stall is the wait for loads.  3 bits
+// 10 380 and 9 340 (issue), 8 bits 17 260 and 12 430, 4 bits at batch 16 17 150 and 8 300
+// (half of it activation loads).  So added instructions cost (an eighth of the codes
+// resolved by permutes alone, 7 instructions for 4 codes instead of 4: 2 %) and so does a
+// smaller L1 (kCarveout).  Per launch, the latency of a CTA's life (activations after the
+// previous launch, first tile, final sum) is 1.6-2.5 us.  Per Llama-3.1-8B layer (q+k+v, o,
+// gate+up, down chained, bf16), with fused multiply-adds on the CUDA cores (batches up to 8;
+// 5 and more at 3 and 8 bits and 9 and more at 4 in the prefill kernel) before and now:
 //   4 bits, batch 1 / 2 / 4 / 8 / 16: 31.1 / 45.6 / 57.0 / 109 / 117 us before,
-//     30.7 / 34.3 / 41.8 / 49.1 / 63.4 now;
-//   3 bits, batch 1 / 4 / 16: 39.0 / 68.7 / 162 before, 35.8 / 45.5 / 78 now;
-//   8 bits, batch 1 / 4 / 16: 52.8 / 85.8 / 157 before, 48.2 / 64 / 100 now.
+//     30.6 / 33.9 / 39.5 / 48.7 / 63.0 now;
+//   3 bits, batch 1 / 4 / 16: 39.0 / 68.7 / 162 before, 36.0 / 44.2 / 76.4 now;
+//   8 bits, batch 1 / 4 / 16: 52.8 / 85.8 / 157 before, 48.7 / 59.1 / 92.3 now.
+// Slower than before: few rows of long K at batches 3-16 (every CTA loads all activations
+// in its turn of passes): 64 x 4096 at 4 bits, batch 4 1.7 -> 2.6, 8 2.2 -> 3.4, 16 2.9 ->
+// 4.8; 128 x 14336, batch 8 4.9 -> 9.2.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -69,8 +77,8 @@ constexpr int kMaxItems = 4;
 constexpr int64_t kPartBatch = 9, kMaxParts = 8;
 // Warm-up ranges of this size or more are not prefetched: a launch's end waits for
 // the prefetches it issued, and in a chain of launches that costs more than the
-// next one gains (a Llama-3.1-8B step of 128 launches: 981 us with 4 MiB, 990
-// with 20 MiB).
+// next one gains (4 / 8 / 20 MiB: Llama-3.1-8B step of 128 launches 986 / 986 / 1002 us,
+// Llama-3.2-1B step of 64 230.9 / 230.5 / 238.4, at 8 bits 313.9 / 317.5 / 325.4).
 constexpr int64_t kPrefetchBytes = 4 << 20;
 
 // One matrix of a grouped launch: all items share X, K, B and the code width.
@@ -717,8 +725,9 @@ cudaError_t check_shared_base()
 
 }  // namespace
 
-// Up to 16 rows always (a Llama-3.1-8B layer at 16 rows, here and in the tensor-memory
-// kernel: 4 bits 64 and 74 us, 3 bits 78 and 93, 8 bits 100 and 97).  17..32 for up to
+// Up to 16 rows always (a Llama-3.1-8B layer at 9 / 16 rows, here and in the prefill kernel:
+// 4 bits 59.1 / 63.3 and 91.8 / 75.5 us, 3 bits 70.9 / 76.0 and 101 / 94.4, 8 bits 90.9 /
+// 92.4 and 103 / 97.0).  17..32 for up to
 // 4 M weights in a call: 2048 x 2048 at 17 / 32 rows, 4 bits 5.1 / 6.1 against 6.3 / 6.4,
 // 3 bits 5.2 / 6.0 against 6.7, 8 bits 4.7 / 5.2 against 7.3; 3072 x 2048, 4 bits 6.6 /
 // 7.6 against 6.4 / 6.6; 4096 x 4096 13.0 / 14.0 against 10.5 / 10.7.

@@ -159,9 +159,9 @@ bool gemv_takes(int bits, int64_t B, int64_t rows, int64_t K);
 // as include/logq.h says (weights: of all the call's matrices).  They are those that the
 // library has never run in a kernel that keeps to stream order for its codes: 3 and 8
 // bits up to 4 rows, 4 bits up to 7, and up to 16 where the model that the workspace is
-// sized by (prefill_plan against 0.46e-6 us a weight at 8 rows, 0.84e-6 beyond, plus 2)
-// keeps off the tensor-core launch whatever the shape: its estimate is at least
-// 6 + 0.4e-6 us a weight.  All others wait, at 4 to 5 % of a layer's time.
+// sized by (prefill_plan against small_batch_us of logq_host.cu: 0.46e-6 us a weight at 8
+// rows, 0.84e-6 beyond, plus 2) keeps off the prefill kernel whatever the shape: that
+// one's estimate is at least 6 + 0.4e-6 us a weight.  All others wait, at 4 to 5 % of a layer's time.
 inline bool reads_codes_early(int bits, int64_t B, int64_t weights)
 {
     if (bits != 4) return B <= 4;

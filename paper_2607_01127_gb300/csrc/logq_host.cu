@@ -169,18 +169,19 @@ uint16_t f16_bits_of(float v)
 logq_status cuda_status(cudaError_t e) { return e == cudaSuccess ? LOGQ_OK : LOGQ_ERR_CUDA; }
 
 // Workspace sizes.  What the two queries return is part of the interface (callers
-// allocate by it), so they go by a fixed model: batches of up to 4 (4 bits: up to
-// 7) need the base workspace only; 4-bit batches of 8..16 room for split k ranges
-// where the tensor-core plan below beats 27 us per 58.7 M weights up to batch 8 and
-// 49 us at 9..16, plus 2 us; larger batches whatever the plan splits.  The kernels
-// use what room they are given: the decode kernel (gemv_takes) for parts of K,
+// allocate by it), so they go by a fixed model, not by the kernels' present times:
+// batches of up to 4 (4 bits: up to 7) need the base workspace only; 4-bit batches of
+// 8..16 room for split k ranges where the prefill kernel's plan beats 27 us per 58.7 M
+// weights up to batch 8 and 49 us at 9..16, plus 2 us (small_batch_us; the times of a
+// decode kernel on fused multiply-adds); larger batches whatever the plan splits.  The
+// kernels use what room they are given: the decode kernel (gemv_takes) for parts of K,
 // the prefill kernel for its k ranges.
 bool small_batch(int bits, int64_t B) { return B <= (bits == 4 ? 16 : 4); }
 
 // Batches whose workspace the plan sizes.
 bool tensor_core_batch(int bits, int64_t B) { return !small_batch(bits, B) || (bits == 4 && B >= 8); }
 
-double cuda_core_us(int64_t B, int64_t N, int64_t K)
+double small_batch_us(int64_t B, int64_t N, int64_t K)
 {
     return (double)N * (double)K * (B <= 8 ? 0.46e-6 : 0.84e-6) + 2.0;
 }
@@ -190,27 +191,27 @@ double cuda_core_us(int64_t B, int64_t N, int64_t K)
 // no longer leave SMs idle), or each matrix as its own logq_linear call --
 // whichever is estimated faster.  A smaller workspace can only slow the options
 // that split k ranges, so the workspace the choice needs (part_bytes) leads to
-// the same choice.  (kCudaCores: only in sizing small batches, see above.)
+// the same choice.  (kDecode: only in sizing small batches, by the model above.)
 struct GroupChoice {
-    enum { kCudaCores, kTensorCores, kSingles } kind;
+    enum { kDecode, kTensorCores, kSingles } kind;
     size_t part_bytes;
 };
 
 GroupChoice choose_group(int bits, int64_t B, const int64_t* N, int count, int64_t K, size_t workspace_bytes)
 {
-    GroupChoice ch{GroupChoice::kCudaCores, 0};
+    GroupChoice ch{GroupChoice::kDecode, 0};
     if (!tensor_core_batch(bits, B)) return ch;
     const size_t avail = workspace_bytes > kWorkspaceBytes ? workspace_bytes - kWorkspaceBytes : 0;
-    const bool cuda_ok = small_batch(bits, B);
-    double cuda_us = 2.0, singles_us = 0.0;
+    const bool small_ok = small_batch(bits, B);
+    double small_us = 2.0, singles_us = 0.0;
     size_t single_part = 0;
     for (int i = 0; i < count; ++i) {
         const PrefillPlan pl = prefill_plan(B, N[i], K, avail);
         double us = pl.est_us;
         size_t part = pl.part_bytes;
-        if (cuda_ok) {
-            const double c = cuda_core_us(B, N[i], K);
-            cuda_us += c - 2.0;
+        if (small_ok) {
+            const double c = small_batch_us(B, N[i], K);
+            small_us += c - 2.0;
             if (c <= us) {
                 us = c;
                 part = 0;
@@ -220,7 +221,7 @@ GroupChoice choose_group(int bits, int64_t B, const int64_t* N, int count, int64
         single_part = part > single_part ? part : single_part;
     }
     const PrefillPlan gp = prefill_plan(B, N, count, K, avail);
-    double best = cuda_ok ? cuda_us : 1e300;
+    double best = small_ok ? small_us : 1e300;
     if (count > 1 && gp.est_us < best) {
         best = gp.est_us;
         ch = GroupChoice{GroupChoice::kTensorCores, gp.part_bytes};
@@ -302,7 +303,7 @@ size_t logq_linear_workspace_bytes(int64_t B, int64_t N, int64_t K, int bits)
     if (B <= 0 || logq_packed_bytes(N, K, bits) == 0) return 0;
     if (!tensor_core_batch(bits, B)) return kWorkspaceBytes;
     const PrefillPlan pl = prefill_plan(B, N, K, (size_t)-1);
-    if (small_batch(bits, B) && pl.est_us >= cuda_core_us(B, N, K)) return kWorkspaceBytes;
+    if (small_batch(bits, B) && pl.est_us >= small_batch_us(B, N, K)) return kWorkspaceBytes;
     return kWorkspaceBytes + pl.part_bytes;
 }
 

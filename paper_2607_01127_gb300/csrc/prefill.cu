@@ -3,15 +3,15 @@
 // LUT reads, so here each weight is dequantised once per tile and reused by a
 // dense bf16/fp16 contraction).
 //
-// One persistent CTA per SM walks 128 (weights) x 256 (tokens) output tiles;
-// where there are too few tiles to fill the SMs, each tile's k range is split
+// One persistent CTA per SM walks output tiles of 128 weight rows x 64, 128, 192 or
+// 256 tokens (one width per launch, the tokens in equal tiles); where there are too few tiles to fill the SMs, each tile's k range is split
 // into ranges taken by different CTAs, which write fp32 partial sums to the
 // caller's workspace and a second kernel adds them in a fixed order.  A launch
 // may cover up to four matrices that read the same X (q/k/v, gate/up): each
 // gets a contiguous range of the CTAs, in proportion to its tiles, and a CTA
 // works on its matrix's tiles only.
 // The dequantised weight tile (the MMA's A operand) lives in tensor memory, not
-// in shared memory: tensor memory holds one fp32 accumulator (256 columns) and
+// in shared memory: tensor memory holds one fp32 accumulator (up to 256 columns) and
 // eight weight stages (32 columns each), and shared memory holds the pair table
 // and five X stages.
 // Warp roles (28 warps, seven warpgroups; setmaxnreg moves registers from the
@@ -625,9 +625,8 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
         }
     } else if (warp >= kEpi0 && warp < kDec0) {
         // ---------------- epilogue ----------------
-        // Two warps per TMEM lane quarter, each owning 128 of the tile's 256 token
-        // columns.  16-bit outputs are read out of tensor memory and rounded into
-        // registers first, so the accumulator is handed back before the stores.
+        // Two warps per TMEM lane quarter, each owning half of the tile's token columns
+        // (32 to 128), drained 32 at a time.
         const int quarter = warp & 3;                   // TMEM lanes 32*quarter .. +31
         const int half = p.bn / 2, ehalf = (warp - kEpi0) >> 2;          // token columns half*ehalf .. +half-1
         const int row = quarter * 32 + lane;
@@ -644,8 +643,8 @@ prefill_kernel(const __grid_constant__ PrefillParams p, const __grid_constant__ 
             // tokens of this half that exist (<= 0 past the end of the batch)
             const int jmax = (p.B - tb0) < half ? (p.B - tb0) : half;
             {
-                // 32 tokens at a time; the accumulator is handed back before the last
-                // stores.  Lanes hold consecutive n: each store instruction writes one
+                // 32 tokens at a time; the accumulator is handed back before the stores of
+                // the last 32.  Lanes hold consecutive n: each store instruction writes one
                 // contiguous run of Y[t][n0 .. n0+31].
                 const bool f32 = p.splits > 1 || p.y_dtype == LOGQ_F32;       // Y, or this k range's partial sums
                 const bool bf = p.y_dtype == LOGQ_BF16;

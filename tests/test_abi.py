@@ -110,10 +110,10 @@ def test_workspace_bytes(logq):
 
 
 def test_linear_workspace_bytes(logq):
-    """4-bit products that stay on the CUDA cores need only the base workspace
-    (batches up to 7, and batches 8..16 where that kernel is estimated faster);
-    tensor-core products whose output tiles are too few to fill the GPU ask for
-    room for split-k partial sums (splits x B x N fp32); invalid sizes give 0."""
+    """Batches up to 4 (4 bits: 7) need only the base workspace, as do 4-bit batches of
+    8..16 where the sizing model keeps off the prefill kernel's plan; other products
+    whose output tiles are too few to fill the GPU ask for room for split-k partial
+    sums (splits x B x N fp32); invalid sizes give 0."""
     base = logq.logq_workspace_bytes()
     assert logq.logq_linear_workspace_bytes(1, 4096, 4096, 4) == base
     assert logq.logq_linear_workspace_bytes(4, 14336, 4096, 4) == base
@@ -129,9 +129,9 @@ def test_linear_workspace_bytes(logq):
 
 
 def test_linear_grouped_workspace_bytes(logq):
-    """A group that runs as one tensor-core launch asks for the partial sums of all its
-    matrices (splits x B x sum(N) fp32), one that runs on the CUDA cores or unsplit only
-    for the base workspace; a single matrix asks what logq_linear asks; invalid groups
+    """A group sized as one prefill launch asks for the partial sums of all its matrices
+    (splits x B x sum(N) fp32), one sized as a small batch or unsplit only for the base
+    workspace; a single matrix asks what logq_linear asks; invalid groups
     give 0."""
     base = logq.logq_workspace_bytes()
     g = logq.logq_linear_grouped_workspace_bytes
@@ -141,8 +141,7 @@ def test_linear_grouped_workspace_bytes(logq):
     assert g(1, [14336, 14336], 4096, 4) == base
     # 3-bit group at batch 96: one launch, every k range split in two
     assert g(96, [640, 256], 1152, 3) == base + 2 * 96 * 896 * 4
-    # q/k/v at batch 16: the tensor-core group with k split in three beats the
-    # CUDA-core group launch and the single calls
+    # q/k/v at batch 16: sized as one prefill launch with k split in three
     assert g(16, [4096, 1024, 1024], 4096, 4) == base + 3 * 16 * 6144 * 4
     for B, N, K, bits in [(16, 4096, 8192, 4), (64, 1024, 4096, 4), (2048, 1024, 4096, 4), (1, 4096, 4096, 4)]:
         assert g(B, [N], K, bits) == logq.logq_linear_workspace_bytes(B, N, K, bits)

@@ -81,7 +81,7 @@ def test_gemv8_dtypes(logq, B, xdt, ydt):
 
 
 def test_gemv8_large_launch_and_grouped(logq):
-    """A launch above the 20 MiB split (one 16-warp CTA per SM) and a grouped
+    """A launch of more than 20 MiB of codes and a grouped
     launch of two 8-bit matrices equal to the single calls."""
     N, K = 10247, 2048
     w = workloads.weights_np(N, K, seed=23)

@@ -1,4 +1,4 @@
-"""Decode GEMV / skinny GEMM and prefill GEMM against the fp64 oracle:
+"""Decode kernel and prefill GEMM against the fp64 oracle:
 |y_gpu - y_ref| <= 1e-3 * sum_k |x_k w_k| + 1e-6 for every output, with the
 oracle evaluating X * What^T on the same codes and the same 16-bit table."""
 import numpy as np
@@ -67,15 +67,14 @@ def test_gemv_16bit_output(logq, xdt, B):
 @pytest.mark.parametrize("bits,N,K,B", [(4, 20491, 2048, 1), (4, 20491, 2048, 2), (3, 27403, 2048, 1),
                                          (3, 27403, 2048, 2), (4, 5131, 8192, 1)])
 def test_gemv_large_launch(logq, bits, N, K, B):
-    """Launches above the size at which the batch-1/2 decode kernel switches to
-    one 16-warp CTA per SM (20 MiB of codes), ragged row counts."""
+    """Launches of 20 MiB of codes and more (many tiles per CTA), ragged row counts."""
     run_case(logq, N, K, bits, B, torch.bfloat16, seed=N + B + bits)
 
 
 @pytest.mark.parametrize("N,K", [(4095, 2048), (4096, 2048), (20479, 2048), (20480, 2048)])
 def test_gemv_launch_shape_boundaries(logq, N, K):
-    """Batch-1 launches on either side of the sizes where the decode kernel
-    changes shape (4 MiB and 20 MiB of codes)."""
+    """Batch-1 launches on either side of the most weights of the shape for short rows
+    (4 MiB of codes) and of 20 MiB, where the rows of a CTA stop being even."""
     run_case(logq, N, K, 4, 1, torch.bfloat16, seed=N)
 
 
@@ -161,12 +160,13 @@ def test_prefill_bf16(logq, N, K, B, bits):
 
 
 @pytest.mark.parametrize("N,K,B,ydt", [(4096, 8192, 16, torch.bfloat16), (4100, 8192, 12, None),
-                                       (4096, 14336, 16, torch.bfloat16), (4096, 8192, 9, torch.bfloat16)])
-def test_small_batch_tensor_cores_split_k(logq, N, K, B, ydt):
-    """4-bit batches of 9..16 on long-K shapes run on the tensor cores with each
-    output tile's k range split over CTAs (fp32 partials, fixed-order sum) when the
-    workspace has room; with the minimal workspace the same call keeps the
-    CUDA-core kernel.  Both match the oracle; base 3 makes almost every code
+                                       (4096, 14336, 16, torch.bfloat16), (4096, 8192, 9, torch.bfloat16),
+                                       (1000, 8192, 33, None), (4096, 2048, 40, torch.bfloat16)])
+def test_split_k_with_and_without_room(logq, N, K, B, ydt):
+    """Long-K shapes whose row ranges share K among CTAs when the workspace has room
+    (fp32 partials, fixed-order sum): parts of K in the decode kernel at batches 9..16,
+    split k ranges in the prefill kernel above 32; with the minimal workspace the
+    same call runs unsplit.  Both match the oracle; base 3 makes almost every code
     non-zero, so the two summation orders give different fp32 sums."""
     codes, cb, ocb, q = make_layer(logq, N, K, 4, 3.0, N + B)
     X = workloads.activations_torch(B, K, N + K, torch.bfloat16, "cuda")
@@ -181,10 +181,12 @@ def test_small_batch_tensor_cores_split_k(logq, N, K, B, ydt):
     assert not torch.equal(Yt, Yc)
 
 
-def test_small_batch_tensor_cores_without_split(logq):
-    """112 output tiles of 128 rows fill enough SMs without splitting the k range;
-    the tensor cores beat the CUDA-core kernel at batch 16 here, workspace or not."""
-    N, K, B = 14336, 2048, 16
+@pytest.mark.parametrize("B", [16, 64])
+def test_minimal_workspace_suffices_for_many_rows(logq, B):
+    """112 output tiles of 128 rows fill enough SMs without splitting the k range, in
+    the decode kernel (16) and in the prefill kernel (64): the queries ask for no more
+    than the minimal workspace."""
+    N, K = 14336, 2048
     assert logq.logq_linear_workspace_bytes(B, N, K, 4) == logq.logq_workspace_bytes()
     codes, cb, ocb, q = make_layer(logq, N, K, 4, 3.0, 77)
     X = workloads.activations_torch(B, K, 77, torch.bfloat16, "cuda")
@@ -193,9 +195,10 @@ def test_small_batch_tensor_cores_without_split(logq):
     check_linear(Y.double().cpu().numpy(), Yr, A, "bf16")
 
 
-@pytest.mark.parametrize("bits,B", [(3, 8), (8, 16), (3, 5)])
-def test_small_batch_3_and_8_bit_on_tensor_cores(logq, bits, B):
-    """3- and 8-bit batches above 4 run on the tensor cores in 16-token tiles (split or not)."""
+@pytest.mark.parametrize("bits,B", [(3, 8), (8, 16), (3, 5), (3, 36), (8, 33)])
+def test_small_batch_3_and_8_bit(logq, bits, B):
+    """3- and 8-bit batches above 4 (decode kernel, with and without parts of K) and just
+    above 32 (prefill kernel, one 64-token tile)."""
     run_case(logq, 2048, 2048, bits, B, torch.bfloat16, ydt=torch.bfloat16, seed=bits * 10 + B,
              base=1.25 if bits == 3 else 1.05)
     run_case(logq, 300, 1152, bits, B, torch.bfloat16, seed=bits + B, base=1.25 if bits == 3 else 1.05)
@@ -244,13 +247,14 @@ def test_grouped_split_k_equals_single_calls(logq):
     (4, 512, [(2048, 1.3), (512, 1.6)], 1024),
     (3, 96, [(640, 1.25), (256, 1.4)], 1152),
     (8, 200, [(384, 1.05), (136, 1.02), (64, 1.03), (256, 1.04)], 512),
-    (4, 12, [(8192, 1.5), (8192, 1.8)], 4096),                   # gate/up-like, 16-token tiles
+    (4, 33, [(8192, 1.5), (8192, 1.8)], 4096),                   # gate/up-like, one 64-token tile
+    (4, 12, [(8192, 1.5), (8192, 1.8)], 4096),                   # the same in the decode kernel
 ])
-def test_grouped_tensor_core_launch(logq, bits, B, shapes, K):
-    """Matrices sharing X in one tensor-core launch (each a share of the CTAs, its own
-    table): every output matches the oracle, with and without room for split k ranges.
-    Unsplit, above batch 16 (where a single call also runs on the tensor cores), each
-    equals the single call's bit for bit (same tiles, same k order)."""
+def test_grouped_prefill_launch(logq, bits, B, shapes, K):
+    """Matrices sharing X in one prefill launch (each a share of the CTAs, its own table;
+    the last group in one decode launch): every output matches the oracle, with and
+    without room for split k ranges.  Unsplit, in the prefill kernel, each equals the
+    single call's bit for bit (same tiles, same k order)."""
     layers = [make_layer(logq, N, K, bits, base, seed=110 + i) for i, (N, base) in enumerate(shapes)]
     X = workloads.activations_torch(B, K, 111, torch.bfloat16, "cuda")
     items = [(codes, cb, N, None) for (codes, cb, ocb, q), (N, _) in zip(layers, shapes)]
