@@ -1,4 +1,4 @@
-// Decode kernel: Y[b][n] = sum_k X[b][k] * table[code(n, k)] for batches up to 32
+// Decode kernels: Y[b][n] = sum_k X[b][k] * table[code(n, k)] for batches up to 32
 // (paper Sec. 3.3: dequantisation by lookup table instead of exponentiation).
 //
 //  * Pair table in shared memory.  Two codes (one byte at 4 bits, one 6-bit
@@ -49,9 +49,7 @@
 //     30.6 / 33.9 / 39.5 / 48.7 / 63.0 now;
 //   3 bits, batch 1 / 4 / 16: 39.0 / 68.7 / 162 before, 36.0 / 44.2 / 76.4 now;
 //   8 bits, batch 1 / 4 / 16: 52.8 / 85.8 / 157 before, 48.7 / 59.1 / 92.3 now.
-// Slower than before: few rows of long K at batches 3-16 (every CTA loads all activations
-// in its turn of passes): 64 x 4096 at 4 bits, batch 4 1.7 -> 2.6, 8 2.2 -> 3.4, 16 2.9 ->
-// 4.8; 128 x 14336, batch 8 4.9 -> 9.2.
+// Few rows of long K at batches 3-16 have a kernel of their own (few_rows_kernel).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -549,6 +547,195 @@ __global__ void __launch_bounds__(NT, MINB) gemv_kernel(const __grid_constant__ 
     }
 }
 
+// ------------------------------------------------------------ few rows ---
+
+// acc_lo / acc_hi += the low / high 16-bit value of w times that of x.
+template <bool F16>
+__device__ __forceinline__ void fma_pair(float& lo, float& hi, uint32_t w, uint32_t x)
+{
+    if constexpr (F16)
+        asm("{.reg .b16 wl, wh, xl, xh;\n\tmov.b32 {wl, wh}, %2;\n\tmov.b32 {xl, xh}, %3;\n\t"
+            "fma.rn.f32.f16 %0, wl, xl, %0;\n\tfma.rn.f32.f16 %1, wh, xh, %1;}"
+            : "+f"(lo), "+f"(hi) : "r"(w), "r"(x));
+    else
+        asm("{.reg .b16 wl, wh, xl, xh;\n\tmov.b32 {wl, wh}, %2;\n\tmov.b32 {xl, xh}, %3;\n\t"
+            "fma.rn.f32.bf16 %0, wl, xl, %0;\n\tfma.rn.f32.bf16 %1, wh, xh, %1;}"
+            : "+f"(lo), "+f"(hi) : "r"(w), "r"(x));
+}
+
+// Sum of each of V per-lane values over the 32 lanes; lane l returns that of value
+// l >> (5 - log2 V) (V a power of two up to 32).
+template <int V>
+__device__ __forceinline__ float reduce_scatter(float (&a)[V], int lane)
+{
+    int count = V;
+#pragma unroll
+    for (int m = 16; m >= 1; m >>= 1) {
+        if (count > 1) {
+            const int half = count / 2;
+            const bool upper = (lane & m) != 0;
+#pragma unroll
+            for (int i = 0; i < V / 2; ++i)
+                if (i < half) {
+                    const float send = upper ? a[i] : a[i + half];
+                    const float keep = upper ? a[i + half] : a[i];
+                    a[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+                }
+            count = half;
+        } else {
+            a[0] += __shfl_xor_sync(0xffffffffu, a[0], m);
+        }
+    }
+    return a[0];
+}
+
+// The pair table, and this CTA's share of the warm-up range below it, as in gemv_kernel.
+// (Not shared with it: as functions they cost its batch-1 4-bit instance a spilled register
+// and the 8B step 4 %, 979 -> 1018 us.)
+template <int BITS, int NT>
+__device__ __forceinline__ void build_table(uint8_t* smem, const uint32_t* lvl, const LevelsT<BITS>& lv, int m)
+{
+    constexpr int NENT = (BITS == 3) ? 64 : 256;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (BITS != 8) __syncthreads();
+#pragma unroll
+    for (int e0 = 32 * warp; e0 < NENT; e0 += NT) {
+        const int e = e0 + lane;
+        uint32_t v;
+        if constexpr (BITS == 8) v = (uint32_t)lv.v[m][e] * 0x10001u;
+        else v = lvl[BITS == 4 ? (e & 15) : (e & 7)] | (lvl[BITS == 4 ? (e >> 4) : (e >> 3)] << 16);
+        uint8_t* at = smem + (e0 + (lane >> 3)) * kTabStride + (lane & 7) * 16;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t x = __shfl_sync(0xffffffffu, v, 4 * i + (lane >> 3));
+            *reinterpret_cast<uint4*>(at + 4 * i * kTabStride) = make_uint4(x, x, x, x);
+        }
+    }
+}
+
+template <int NT>
+__device__ __forceinline__ void warm_share(const GemvParams& p)
+{
+    if (p.pf_bytes <= 0) return;
+    constexpr int64_t piece = 16384;
+    const int64_t beg = p.pf_share * blockIdx.x;
+    const int64_t end = (beg + p.pf_share < p.pf_bytes) ? beg + p.pf_share : p.pf_bytes;
+    for (int64_t off = beg + (int64_t)threadIdx.x * piece; off < end; off += (int64_t)NT * piece) {
+        const int64_t n = (end - off) < piece ? (end - off) : piece;
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.pf + off), "r"((uint32_t)n) : "memory");
+    }
+}
+
+// k of a lane's run in the few-rows kernel: 8 bytes of 4-bit codes, 16 of 8-bit ones, a
+// 3-bit group.
+__host__ __device__ constexpr int few_k(int bits) { return bits == 3 ? 32 : 16; }
+
+// Few rows of long K (few_rows), batches 3 to 16 padded to B: one row at a time per group
+// of warps, fused multiply-adds on the CUDA cores.  Each warp owns spans of 32 runs of
+// consecutive k; a row's products are summed over its lanes, then over the spans in
+// order.  Against the matrix-instruction kernel, whose tiles of 16 / S rows leave most SMs
+// idle here while each CTA loads all activations with 64 bytes between its lanes: a row per
+// CTA, and activation loads at half the cost in the L1 path (figures at few_rows).  Bound by
+// those loads and by latency.
+template <int BITS, int B, bool F16, int NT>
+__global__ void __launch_bounds__(NT, 1) few_rows_kernel(const __grid_constant__ GemvParams p,
+                                                         const __grid_constant__ LevelsT<BITS> lv)
+{
+    extern __shared__ __align__(16) uint8_t smem[];
+    constexpr int LK = few_k(BITS), NW = BITS == 8 ? LK / 4 : BITS == 4 ? LK / 8 : 3;
+    constexpr uint32_t TAB_BYTES = (BITS == 3 ? 64 : 256) * kTabStride;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");      // (see gemv_kernel)
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if ((uint32_t)__cvta_generic_to_shared(smem) != kTabOff) {   // table addressing relies on it
+        if (tid == 0) atomicExch(p.err, (uint32_t)LOGQ_ERR_UNSUPPORTED);
+        return;
+    }
+    int m = 0;
+#pragma unroll
+    for (int i = 1; i < kMaxItems; ++i)
+        if (i < p.nitems && (int)blockIdx.x >= p.item[i].cta_begin) m = i;
+    const GemvItem& item = p.item[m];
+    uint32_t* const lvl = reinterpret_cast<uint32_t*>(smem + kLvlOff);
+    if constexpr (BITS != 8)
+        if (tid < 16) lvl[tid] = item.lvl16[tid];
+    const int cta = (int)blockIdx.x - item.cta_begin;
+    const int r0 = cta * item.rows_q + (cta < item.rows_rem ? cta : item.rows_rem);
+    const int rows = item.rows_q + (cta < item.rows_rem ? 1 : 0);
+    const int G = 1 << p.lg_groups, g = warp & (G - 1), scol = warp >> p.lg_groups;
+    const bool compute_warp = scol < p.span_cols && g < rows;
+    struct Codes { uint32_t w[NW]; };
+    // this lane's codes of row r0 + r, span s; runs past K count as 0
+    auto load = [&](Codes& c, int r, int s) {
+        const int k0 = (s * 32 + lane) * LK;
+        const uint8_t* at = item.codes + (int64_t)(r0 + r) * p.row_bytes + k0 / 32 * (4 * BITS) + k0 % 32 * BITS / 8;
+        if (k0 >= p.K) {
+#pragma unroll
+            for (int i = 0; i < NW; ++i) c.w[i] = 0u;
+        } else if constexpr (NW == 2) {
+            asm volatile("ld.global.nc.L1::no_allocate.v2.b32 {%0,%1}, [%2];" : "=r"(c.w[0]), "=r"(c.w[1]) : "l"(at));
+        } else {
+            ld_codes<false, NW>(c.w, at);
+        }
+    };
+    if (p.wait_codes) asm volatile("griddepcontrol.wait;" ::: "memory");
+    Codes cur;
+    if (compute_warp) load(cur, g, scol);
+    warm_share<NT>(p);
+    build_table<BITS, NT>(smem, lvl, lv, m);
+    __syncthreads();
+    uint32_t base_lane = 4u * (uint32_t)lane;
+    asm volatile("" : "+r"(base_lane)::"memory");    // lookups stay behind the barrier
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    float* const red = reinterpret_cast<float*>(smem + TAB_BYTES);       // [span][row][B]
+    if (compute_warp)
+        for (int s = scol; s < p.spans; s += p.span_cols) {
+            const int k0 = (s * 32 + lane) * LK;
+            uint32_t xr[B][LK / 2];
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+#pragma unroll
+                for (int i = 0; i < LK / 2; i += 4) {
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (k0 < p.K && b < p.B) v = *reinterpret_cast<const uint4*>(p.X + (int64_t)b * p.K + k0 + 2 * i);
+                    xr[b][i] = v.x;
+                    xr[b][i + 1] = v.y;
+                    xr[b][i + 2] = v.z;
+                    xr[b][i + 3] = v.w;
+                }
+            for (int r = g; r < rows; r += G) {
+                Codes next;                          // the next row's, or the next span's first
+                const bool same = r + G < rows;
+                if (same || s + p.span_cols < p.spans) load(next, same ? r + G : g, same ? s : s + p.span_cols);
+                float lo[B], hi[B];
+#pragma unroll
+                for (int b = 0; b < B; ++b) lo[b] = hi[b] = 0.f;
+#pragma unroll
+                for (int q = 0; q < LK / 4; ++q) {
+                    uint32_t p0, p1;
+                    pairs_of<BITS, NW>(cur.w, q, base_lane, p0, p1);
+#pragma unroll
+                    for (int b = 0; b < B; ++b) {
+                        fma_pair<F16>(lo[b], hi[b], p0, xr[b][2 * q]);
+                        fma_pair<F16>(lo[b], hi[b], p1, xr[b][2 * q + 1]);
+                    }
+                }
+#pragma unroll
+                for (int b = 0; b < B; ++b) lo[b] += hi[b];
+                const float sum = reduce_scatter<B>(lo, lane);
+                if (lane % (32 / B) == 0) red[(s * rows + r) * B + lane / (32 / B)] = sum;
+                cur = next;
+            }
+        }
+    __syncthreads();
+    for (int i = tid; i < rows * B; i += NT) {
+        const int row = i / B, b = i % B;
+        if (b >= p.B) continue;
+        float sum = 0.f;
+        for (int s = 0; s < p.spans; ++s) sum += red[s * rows * B + i];
+        store_y(item.Y, p.y_dtype, (int64_t)b * item.N + r0 + row, sum);
+    }
+}
+
 // Added to a padded batch: the shape for short rows (shape_key).
 constexpr int kShort = 64, kMid = 128;
 // Launches of up to this many weights keep to one CTA per SM (per_sm).
@@ -560,18 +747,17 @@ struct Shape {
     int S, J, NTL, T, NT, MINB;
 };
 
-// Dynamic shared memory opt-in and a carveout that leaves room for the CTAs of
-// an SM: per-device function attributes, set once per device.
-template <int BITS, int S, int J, int NTL, int T, int NT, int MINB, bool F16>
-cudaError_t run(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, cudaStream_t s)
+// Launch of a decode kernel k.  Dynamic shared memory opt-in and carveout: per-device
+// function attributes, set once per device.
+template <int BITS, typename Kernel>
+cudaError_t run_kernel(Kernel k, bool (&configured)[64], const GemvParams& p, const GroupArgs& a, int grid, int threads,
+                       size_t smem, cudaStream_t s)
 {
     LevelsT<BITS> lv;
     memset(&lv, 0, sizeof lv);
     if constexpr (BITS == 8)
         for (int i = 0; i < a.count; ++i)
             for (int c = 0; c < 256; ++c) lv.v[i][c] = a.item[i].lvl16[c];
-    auto k = gemv_kernel<BITS, S, J, NTL, T, F16, NT, MINB>;
-    static bool configured[64] = {false};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -585,7 +771,7 @@ cudaError_t run(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, 
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(NT);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -594,6 +780,20 @@ cudaError_t run(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, p, lv);
+}
+
+template <int BITS, int S, int J, int NTL, int T, int NT, int MINB, bool F16>
+cudaError_t run(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, cudaStream_t s)
+{
+    static bool configured[64] = {false};
+    return run_kernel<BITS>(gemv_kernel<BITS, S, J, NTL, T, F16, NT, MINB>, configured, p, a, grid, NT, smem, s);
+}
+
+template <int BITS, int B, int NT, bool F16>
+cudaError_t run_few(const GemvParams& p, const GroupArgs& a, int grid, size_t smem, cudaStream_t s)
+{
+    static bool configured[64] = {false};
+    return run_kernel<BITS>(few_rows_kernel<BITS, B, F16, NT>, configured, p, a, grid, NT, smem, s);
 }
 
 // The compiled shapes, per code width and padded batch; calls fn with the
@@ -705,6 +905,61 @@ int shape_key(int bits, int64_t B, int64_t rows, int64_t K)
 // batch 2 265.3 / 256.6 / 258.9, batch 4 286.7 / 279.5 / 284.4.
 int per_sm(const Shape& sh, int64_t weights) { return weights <= kOneCta ? 1 : sh.MINB; }
 
+// Whether few_rows_kernel runs a launch.  us, matrix-instruction kernel / few_rows_kernel
+// (rows x k, batch in brackets; the line lies where they meet):
+//   4 bits: 64 x 4096 (4) 2.58 / 1.85, (8) 3.25 / 2.29, (16) 4.46 / 2.86; 128 x 8192 (8) 5.60 /
+//     2.94; 128 x 14336 (16) 13.9 / 7.5; 256 x 4096 (4) 2.68 / 2.22; 384 rows at 3072, 8192 and
+//     14336 k (4) 2.42 / 2.37, 3.40 / 3.07, 5.60 / 5.78, (8) 3.30 / 3.00, 5.71 / 4.01, 10.1 / 7.3,
+//     (16) 4.42 / 3.65, 8.75 / 6.83, 15.1 / 13.4; 512 x 4096 (8) 3.45 / 3.51; 192 x 2048 (8) 2.28 /
+//     2.31;
+//   3 bits: 128 x 4096 (4) 2.77 / 2.43, 192 x 8192 3.46 / 3.81;
+//   8 bits: 128 x 3072 (4) 2.17 / 2.08, 192 x 3072 2.17 / 2.23, 256 x 4096 2.41 / 2.41, 256 x 14336
+//     7.5 / 4.9, 384 x 4096 2.42 / 2.77.
+bool few_rows(int bits, int64_t B, int64_t rows, int64_t K)
+{
+    if (B < 3 || B > (bits == 4 ? 16 : 4) || K <= 2048) return false;
+    return rows <= (bits == 4 ? (B <= 4 ? 256 : 384) : bits == 3 || K < 4096 ? 128 : 256);
+}
+
+// CTAs per matrix in proportion to the rows, about `grid` in all: at least one each, at
+// most one per unit.  Returns their number.
+int share_ctas(const GroupArgs& a, int64_t total_rows, const int64_t* units, int grid, int* ctas)
+{
+    int used = 0;
+    for (int i = 0; i < a.count; ++i) {
+        int64_t c = (int64_t)grid * a.item[i].N / total_rows;
+        if (c < 1) c = 1;
+        if (c > units[i]) c = units[i];
+        ctas[i] = (int)c;
+        used += ctas[i];
+    }
+    while (used < grid) {               // hand out what rounding left, largest rows per CTA first
+        int best = -1;
+        double best_load = -1.0;
+        for (int i = 0; i < a.count; ++i) {
+            if (ctas[i] >= units[i]) continue;
+            const double load = (double)a.item[i].N / ctas[i];
+            if (load > best_load) { best_load = load; best = i; }
+        }
+        if (best < 0) break;
+        ++ctas[best];
+        ++used;
+    }
+    while (used > grid) {               // too many (minimums): take from the lightest
+        int best = -1;
+        double best_load = 1e300;
+        for (int i = 0; i < a.count; ++i) {
+            if (ctas[i] <= 1) continue;
+            const double load = (double)a.item[i].N / ctas[i];
+            if (load < best_load) { best_load = load; best = i; }
+        }
+        if (best < 0) break;
+        --ctas[best];
+        --used;
+    }
+    return used;
+}
+
 // The table lookups address shared memory relative to kTabOff, which is where
 // dynamic shared memory starts when a kernel has no static shared memory.
 cudaError_t check_shared_base()
@@ -738,17 +993,9 @@ bool gemv_takes(int bits, int64_t B, int64_t rows, int64_t K)
     return B <= 16 || rows <= ((int64_t)4 << 20) / K;
 }
 
-cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
+// Fields that every decode launch shares.
+static GemvParams common_params(const GroupArgs& a, int64_t total_rows)
 {
-    if (a.count < 1 || a.count > kMaxItems) return cudaErrorInvalidValue;
-    cudaError_t e = check_shared_base();
-    if (e != cudaSuccess) return e;
-    int64_t total_rows = 0;
-    for (int i = 0; i < a.count; ++i) total_rows += a.item[i].N;
-    const int key = shape_key(a.bits, a.B, total_rows, a.K);
-    Shape sh;
-    if ((e = shape_or_run<false>(a.bits, key, &sh, nullptr, nullptr, 0, 0, s)) != cudaSuccess) return e;
-    const int64_t row_bytes = a.K / 32 * (4 * a.bits);
     GemvParams p;
     memset(&p, 0, sizeof p);
     p.nitems = a.count;
@@ -758,7 +1005,74 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
     p.B = (int32_t)a.B;
     p.y_dtype = a.y_dtype;
     p.wait_codes = reads_codes_early(a.bits, a.B, total_rows * a.K) ? 0 : 1;
-    p.row_bytes = (int32_t)row_bytes;
+    p.row_bytes = (int32_t)(a.K / 32 * (4 * a.bits));
+    p.kparts = 1;
+    p.pf = static_cast<const uint8_t*>(a.pf);
+    p.pf_bytes = (a.pf && a.pf_bytes < kPrefetchBytes) ? a.pf_bytes : 0;
+    for (int i = 0; i < a.count; ++i) {
+        GemvItem& it = p.item[i];
+        it.codes = a.item[i].codes;
+        it.Y = a.item[i].Y;
+        it.N = (int32_t)a.item[i].N;
+        for (int c = 0; c < 16; ++c) it.lvl16[c] = a.item[i].lvl16[c];
+    }
+    return p;
+}
+
+// The launch of few_rows_kernel: warps 8 at batches above 8, else 16, as registers allow.
+static cudaError_t launch_few(const GroupArgs& a, int64_t total_rows, cudaStream_t s)
+{
+    GemvParams p = common_params(a, total_rows);
+    const int Bp = a.B <= 4 ? 4 : a.B <= 8 ? 8 : 16, warps = Bp == 16 ? 8 : 16;
+    p.spans = (int32_t)((a.K + 32 * few_k(a.bits) - 1) / (32 * few_k(a.bits)));
+    while ((warps >> (p.lg_groups + 1)) >= p.spans) ++p.lg_groups;
+    p.span_cols = p.spans < (warps >> p.lg_groups) ? p.spans : warps >> p.lg_groups;
+    const int sms = sm_count() > 0 ? sm_count() : 148;
+    int64_t units[kMaxItems];
+    for (int i = 0; i < a.count; ++i) units[i] = a.item[i].N;
+    int grid = (int)(total_rows < sms ? total_rows : sms), ctas[kMaxItems] = {0}, begin = 0;
+    if (grid < a.count) grid = a.count;
+    grid = share_ctas(a, total_rows, units, grid, ctas);
+    p.pf_share = p.pf_bytes > 0 ? (((p.pf_bytes + grid - 1) / grid + 15) & ~(int64_t)15) : 0;
+    int64_t max_rows = 0;
+    for (int i = 0; i < a.count; ++i) {
+        GemvItem& it = p.item[i];
+        it.cta_begin = begin;
+        it.rows_q = (int32_t)(a.item[i].N / ctas[i]);
+        it.rows_rem = (int32_t)(a.item[i].N % ctas[i]);
+        begin += ctas[i];
+        const int64_t rows = it.rows_q + (it.rows_rem ? 1 : 0);
+        if (rows > max_rows) max_rows = rows;
+    }
+    const size_t smem = (size_t)(a.bits == 3 ? 64 : 256) * kTabStride + (size_t)p.spans * max_rows * Bp * 4;
+    if (smem > (size_t)kMaxSmem) return cudaErrorNotSupported;
+#define LOGQ_FEW(BITS, B, NT) \
+    if (a.bits == BITS && Bp == B) \
+        return a.x_f16 ? run_few<BITS, B, NT, true>(p, a, grid, smem, s) : run_few<BITS, B, NT, false>(p, a, grid, smem, s)
+    LOGQ_FEW(4, 4, 512);
+    LOGQ_FEW(4, 8, 512);
+    LOGQ_FEW(4, 16, 256);
+    LOGQ_FEW(3, 4, 512);
+    LOGQ_FEW(8, 4, 512);
+#undef LOGQ_FEW
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
+{
+    if (a.count < 1 || a.count > kMaxItems) return cudaErrorInvalidValue;
+    cudaError_t e = check_shared_base();
+    if (e != cudaSuccess) return e;
+    int64_t total_rows = 0;
+    for (int i = 0; i < a.count; ++i) total_rows += a.item[i].N;
+    if (few_rows(a.bits, a.B, total_rows, a.K)) {
+        e = launch_few(a, total_rows, s);
+        if (e != cudaErrorNotSupported) return e;        // (its sums do not fit shared memory)
+    }
+    const int key = shape_key(a.bits, a.B, total_rows, a.K);
+    Shape sh;
+    if ((e = shape_or_run<false>(a.bits, key, &sh, nullptr, nullptr, 0, 0, s)) != cudaSuccess) return e;
+    GemvParams p = common_params(a, total_rows);
     p.blocks = (int32_t)(a.K / (4 * lane_k(a.bits)));
     p.spans = (p.blocks + sh.S * sh.J - 1) / (sh.S * sh.J);
     // Batches of 9 and more read more activations than codes where a CTA takes
@@ -783,46 +1097,13 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
     // proportion to the rows: at least one range each, at most one per tile.
     const int sms = sm_count() > 0 ? sm_count() : 148;
     const int64_t rt = 16 / sh.S;
-    p.pf = static_cast<const uint8_t*>(a.pf);
-    p.pf_bytes = (a.pf && a.pf_bytes < kPrefetchBytes) ? a.pf_bytes : 0;
     int64_t units[kMaxItems], total_units = 0;
     for (int i = 0; i < a.count; ++i) total_units += (units[i] = (a.item[i].N + rt - 1) / rt);
     const int64_t ranges = (int64_t)sms * per_sm(sh, total_rows * a.K) / kparts;
     int grid = (int)(total_units < ranges ? total_units : ranges);
     if (grid < a.count) grid = a.count;
     int ctas[kMaxItems] = {0};
-    int used = 0;
-    for (int i = 0; i < a.count; ++i) {
-        int64_t c = (int64_t)grid * a.item[i].N / total_rows;
-        if (c < 1) c = 1;
-        if (c > units[i]) c = units[i];
-        ctas[i] = (int)c;
-        used += ctas[i];
-    }
-    while (used < grid) {               // hand out what rounding left, largest rows per CTA first
-        int best = -1;
-        double best_load = -1.0;
-        for (int i = 0; i < a.count; ++i) {
-            if (ctas[i] >= units[i]) continue;
-            const double load = (double)a.item[i].N / ctas[i];
-            if (load > best_load) { best_load = load; best = i; }
-        }
-        if (best < 0) break;
-        ++ctas[best];
-        ++used;
-    }
-    while (used > grid) {               // too many (minimums): take from the lightest
-        int best = -1;
-        double best_load = 1e300;
-        for (int i = 0; i < a.count; ++i) {
-            if (ctas[i] <= 1) continue;
-            const double load = (double)a.item[i].N / ctas[i];
-            if (load < best_load) { best_load = load; best = i; }
-        }
-        if (best < 0) break;
-        --ctas[best];
-        --used;
-    }
+    const int used = share_ctas(a, total_rows, units, grid, ctas);
     grid = used * (int)kparts;
     p.pf_share = p.pf_bytes > 0 ? (((p.pf_bytes + grid - 1) / grid + 15) & ~(int64_t)15) : 0;
     int64_t max_rows = 0;
@@ -830,13 +1111,9 @@ cudaError_t launch_gemv_group(const GroupArgs& a, cudaStream_t s)
     float* part = kparts > 1 ? reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(a.ws) + kWorkspaceBytes) : nullptr;
     for (int i = 0; i < a.count; ++i) {
         GemvItem& it = p.item[i];
-        it.codes = a.item[i].codes;
-        it.Y = a.item[i].Y;
-        it.N = (int32_t)a.item[i].N;
         it.cta_begin = begin;
         it.rows_q = (int32_t)(a.item[i].N / ctas[i]);
         it.rows_rem = (int32_t)(a.item[i].N % ctas[i]);
-        for (int c = 0; c < 16; ++c) it.lvl16[c] = a.item[i].lvl16[c];
         begin += ctas[i] * (int)kparts;
         it.part = part;
         if (kparts > 1) part += kparts * a.B * a.item[i].N;

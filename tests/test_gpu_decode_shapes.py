@@ -62,6 +62,36 @@ def test_both_sides_of_a_dispatch_line(logq, bits, B, N, K):
         assert np.all(np.abs(more[:, rows].double().cpu().numpy() - Yr) <= (K / 16 + 60) * 2.0 ** -23 * A)
 
 
+# few rows of long K (the rows that each CTA takes one by one) and one more than the most of
+# them at each width; k of whole spans, of a ragged last one and on both sides of the line
+@pytest.mark.parametrize("bits,B", [(4, 3), (4, 4), (4, 5), (4, 8), (4, 9), (4, 16), (3, 3), (3, 4), (8, 3), (8, 4)])
+@pytest.mark.parametrize("N,K", [(1, 14336), (2, 2048), (3, 2176), (128, 4224), (129, 3968), (256, 4096), (257, 4096), (384, 8576),
+                                 (385, 8576)])
+def test_few_rows(logq, bits, B, N, K):
+    codes, cb, ocb, q = make_layer(logq, N, K, bits, BASE[bits], N + K)
+    X = workloads.activations_torch(B, K, B, torch.float16 if B % 2 else torch.bfloat16, "cuda")
+    Y = logq.logq_linear(codes, cb, X, N, K)
+    check(Y, *reference(X, q, ocb))
+    # grouped: the same rows as three matrices
+    if N == 128:
+        row = logq.logq_packed_bytes(1, K, bits)
+        parts = [(codes[a * row:b * row].clone(), cb, b - a, None) for a, b in ((0, 1), (1, 100), (100, 128))]
+        assert torch.equal(torch.cat(logq.logq_linear_grouped(parts, X, K), 1), Y)
+
+
+@pytest.mark.parametrize("bits", [3, 4, 8])
+def test_infinite_levels_stay_out_of_the_ragged_end(logq, bits):
+    """fp16 levels that overflow: outputs over a last span that K leaves ragged are those
+    of the infinities in the matrix, not NaN from lanes past K."""
+    N, K = 5, 4224
+    cb = logq.logq_build_codebook(bits, 1.3, 1e6)
+    codes = torch.zeros(logq.logq_packed_bytes(N, K, bits), dtype=torch.uint8, device="cuda")
+    codes.view(N, -1)[:, 0] = cb.qmax                       # k = 0: the largest level, +inf in fp16
+    for B in (4, 16):
+        X = torch.ones(B, K, dtype=torch.float16, device="cuda")
+        assert bool((logq.logq_linear(codes, cb, X, N, K) == float("inf")).all())
+
+
 # k on both sides of the lines between the shapes for short rows; fewer rows than a CTA's
 # warps have tiles for, and more
 @pytest.mark.parametrize("bits", [3, 4, 8])
@@ -106,12 +136,13 @@ def test_parts_of_k_use_the_workspace_given(logq, bits, B, sets):
     assert st == logq.LOGQ_OK
 
 
+@pytest.mark.parametrize("K", [1152, 4224])
 @pytest.mark.parametrize("B", [1, 2, 4, 8, 16, 32])
-def test_non_finite_activations_stay_in_their_row(logq, B):
+def test_non_finite_activations_stay_in_their_row(logq, B, K):
     """A NaN or an infinity reaches every output of its own batch row (an infinity as
     NaN where the level is 0) and no other row, although rows and parts of K share
     one matrix instruction."""
-    N, K = 70, 1152
+    N = 70
     codes, cb, ocb, q = make_layer(logq, N, K, 4, 1.5, 6)
     X = workloads.activations_torch(B, K, 7, torch.bfloat16, "cuda")
     clean = logq.logq_linear(codes, cb, X, N, K)
