@@ -43,7 +43,9 @@
 // the issue), so it asks for both barriers at once and its operands are kept
 // uniform (see `warp`): 4 bits, 8B layer at 2048 / 512 / 100 / 33 tokens 771 / 243 /
 // 161 / 148 us before, 579 / 187 / 123 / 111 with it (1.55 PFLOP/s at 2048, 0.90 of what
-// cuBLAS holds for seconds under the power limit); 8 bits at 2048 855.
+// cuBLAS holds for seconds under the power limit); 8 bits at 2048 855.  (These are a
+// layer's launches repeated as a captured chain; made as four calls it takes 619 us at
+// 2048 tokens now, 1.44 PFLOP/s.)
 // At 3 and 8 bits the code copies bound it, by the rows an instruction touches: 3 bits
 // 1143 us with three 4-byte copies per thread and stage, 914 with two of 8 bytes;
 // with two lanes per row 895 -> 740 (8 bits 838 -> 716), all at 2048 tokens.  Tried and
