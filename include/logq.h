@@ -39,9 +39,9 @@
  *     finishes.  They read X and write Y only after that kernel has completed
  *     and its writes are visible, but small decode launches read the packed codes
  *     earlier, before that guarantee holds: up to 4 rows at 3 and 8 bits; at 4
- *     bits up to 7 rows, 8 rows of matrices of up to 32 M weights in the call, and
- *     16 rows of up to 8 M.  So for them the codes must be complete
- *     before the call is enqueued, ordered by a host synchronisation after the
+ *     bits up to 7 rows, 8 rows where the call's matrices hold up to 2^25 weights,
+ *     and 9 to 16 rows where they hold up to 2^23.  So for them the codes must be
+ *     complete before the call is enqueued, ordered by a host synchronisation after the
  *     kernel that wrote them (of its stream, of an event recorded after it, or
  *     of the device), not by stream order alone.  logq_quantize and
  *     logq_quantize_energy end with such a synchronisation; after logq_gptq

@@ -130,8 +130,8 @@ def test_energy_range_8bit(logq):
                                    (512, 4096, 2048)])
 @pytest.mark.parametrize("ydt", [None, torch.bfloat16])
 def test_prefill8(logq, N, K, B, ydt):
-    """Batches above 4 run the tensor-core prefill with 8-bit codes (ragged
-    token tiles and weight-row tiles included)."""
+    """8-bit codes in the prefill kernel (ragged token tiles and weight-row tiles
+    included), and at 5 rows in the decode kernel."""
     w = workloads.weights_np(N, K, seed=N + K + B)
     codes, cb = logq.logq_quantize(torch.from_numpy(w).cuda(), 8, 1.05)
     ocb = oracle.build_codebook(8, 1.05, cb.range)
